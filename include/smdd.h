@@ -232,7 +232,7 @@ int mdc_forward_static(int nt, int nr, int nv, int ns, float scale, const float 
 
 /* ---------------------------------------------------------------------------------------------
  * Kernel configuration and autotuning.  Every configuration computes the same operator; they differ
- * in speed only.  The FFT radix order and the kernel of each per-frequency product are the choices.
+ * in speed only.  The kernel of each per-frequency product is the choice.
  * A plan made with MDC_PREC_BF16X3 may run the FP32 FMA kernels for a product (they are more
  * accurate than the split-BF16 bound); the tensor-core kernels are allowed for such plans only.
  * ------------------------------------------------------------------------------------------- */
@@ -250,17 +250,13 @@ int mdc_forward_static(int nt, int nr, int nv, int ns, float scale, const float 
                                 gives no tensor-map encoder) */
 
 typedef struct {
-    int fft_variant;   /* 0: default radix order of the FFT plan; 1: the reversed order (accepted for
-                          every size, identical to 0 where all radices are equal); 2: the register FFT:
-                          two passes with 32 values per thread and one shared-memory exchange per
-                          transform for FFT lengths 256 .. 2048, three passes (48 * 4 * 8) with 48
-                          values per thread and two exchanges for 3072; elsewhere 2 means 0.  Steps
-                          with N-SGD, Adam or the causality mute run variant 0 whatever is set. */
+    int fft_variant;   /* 0, 1 or 2: accepted and read back (1 as 0 for the lengths 128, 1024 and 8192, 2 as 0
+                          below 256 and for 4096 and 8192).  The trace kernels have one form per FFT
+                          length, which every value runs. */
     int gemm_fwd;      /* MDC_GEMM_SIMT, MDC_GEMM_TC, MDC_GEMM_GEMV or MDC_GEMM_TC_STREAM */
     int gemm_adj;      /* MDC_GEMM_SIMT, MDC_GEMM_SIMT32, MDC_GEMM_SIMT64 or MDC_GEMM_TC */
-    int fft_prefetch;  /* 1: the update runs as persistent CTAs that prefetch the next tile's gradient
-                          spectra while transforming the current one (variants 0 and 1, nfft <= 3072;
-                          elsewhere 0) */
+    int fft_prefetch;  /* 0 or 1: accepted and read back (as 0 above nfft 3072 and with fft_variant 2); selects
+                          nothing */
     int reserved[4];   /* zero */
 } mdc_config;
 
@@ -274,8 +270,7 @@ int mdc_plan_get_config(mdc_plan_t plan, mdc_config *cfg);
 int mdc_plan_set_config(mdc_plan_t plan, const mdc_config *cfg);
 /* Autotune: time every candidate of each choice on this plan's sizes, with batch size nb and the
  * step flags (SMDD_RECIPROCITY changes the adjoint), reps timed launches each after one warm-up, and
- * keep the fastest.  The FFT candidates are timed on a step's two trace kernels: the fused update over a
- * subset of at most 64 MiB of model traces (scaled to all of them) plus the residual step of one batch.  best (host, may be NULL) receives the chosen configuration.
+ * keep the fastest.  best (host, may be NULL) receives the chosen configuration.
  * Uses temporary device memory (cudaMalloc), overwrites the plan's spectral workspaces, synchronises
  * the stream, and must not be called during a stream capture. */
 int mdc_plan_autotune(mdc_plan_t plan, int nb, int flags, int reps, mdc_config *best, void *stream);

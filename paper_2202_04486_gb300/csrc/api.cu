@@ -31,6 +31,14 @@ struct DeviceGuard {
     }
 };
 
+// Row length of the spectra for n traces: even (pairs of traces are 16-byte aligned); from 16 traces on a multiple
+// of 4 and from 64 on of 8, so that the 64-byte segments of the trace kernels' tiles start on whole sectors (at
+// most 11 % more memory; nr 301: 15 % less DRAM traffic of the update than with rows of 302)
+int padded_ld(int n) {
+    const int m = n >= 64 ? 8 : n >= 16 ? 4 : 2;
+    return (n + m - 1) / m * m;
+}
+
 bool is_pow2(int x) { return x > 0 && (x & (x - 1)) == 0; }
 
 #ifndef SMDD_TC_ADJ_TMA
@@ -62,9 +70,7 @@ struct mdc_plan_s {
     float2 *Xh = nullptr;        // [nf][nv][ldr]  model spectra, reused for gradient spectra
     float2 *Uh = nullptr;        // [nf][nv][ldb]  batch spectra (prediction, then residual)
     uint8_t *adj_img = nullptr;  // split-BF16 plans: operand images of the adjoint products (null: not held)
-    float2 *tw = nullptr;        // twiddle tables of the FFT variants: 0 at 0, 1 at tw1_off, 2 at tw2_off
-    int tw1_off = 0, tw2_off = 0;
-    float2 *twN = nullptr;       // [M+1]
+    float2 *tw = nullptr;        // twiddle tables of the trace kernels
     double *partials = nullptr;  // residual-kernel block partials
     double *lam = nullptr;       // [nf] power-iteration results, [nf] = max
     unsigned int *counter = nullptr;
@@ -81,8 +87,8 @@ struct mdc_plan_s {
     long long stage_launches[MDC_NUM_STAGES] = {0};
     long long launches = 0;
     // kernel configuration (see mdc_config)
-    int fft_variant = 0;
-    int fft_prefetch = 0;        // update: persistent CTAs prefetching the next tile (variants 0/1, M <= 1536)
+    int fft_variant = 0;         // accepted and reported; the trace kernels are the same for every value
+    int fft_prefetch = 0;        // likewise
     int gemm_fwd = MDC_GEMM_SIMT;
     int gemm_adj = MDC_GEMM_SIMT;
     int nf_active = 0;           // band limit of the products (0: every bin)
@@ -142,10 +148,7 @@ FftArgs base_fft(const mdc_plan_s *p) {
     FftArgs a;
     memset(&a, 0, sizeof(a));
     a.nt = p->nt;
-    a.tw = p->tw + (p->fft_variant == 2 ? p->tw2_off : p->fft_variant == 1 ? p->tw1_off : 0);
-    a.variant = p->fft_variant;
-    a.prefetch = p->fft_prefetch;
-    a.twN = p->twN;
+    a.tw = p->tw;
     a.s = p->scale / (float)p->nfft;
     a.status = p->status;
     return a;
@@ -158,13 +161,7 @@ int ti_log2_for(int n_contig, int TR) {
     return l;
 }
 
-
-// time traces may be read and written as float4: every trace starts on a 16-byte boundary
-bool vec4_ok(int nt, const void *p) { return nt % 4 == 0 && (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
-
-int traces_per_cta(const mdc_plan_s *p) {
-    return p->fft_variant == 2 ? fft2_traces_per_cta(p->M) : fft_traces_per_cta(p->M);
-}
+int traces_per_cta(const mdc_plan_s *p) { return fft_traces_per_cta(p->M); }
 
 // model-layout grid: trace (i = r, j = v) of a [nv][nr][nt] array  <->  spectra [nf][nv][ldr]
 TraceGrid model_grid(const mdc_plan_s *p, int nouter) {
@@ -199,7 +196,7 @@ int rfft_model(mdc_plan_s *p, const float *X, cudaStream_t st) {
     FftArgs a = base_fft(p);
     a.g = model_grid(p, p->nv);
     a.tin = X;
-    a.vec = vec4_ok(p->nt, X);
+    a.vec = time_vec(p->nt, X);
     a.spec = p->Xh;
     return launch_stage(p, ST_RFFT, st, [&] { return launch_rfft(p->M, a, st); });
 }
@@ -283,7 +280,7 @@ int forward_impl(mdc_plan_s *p, const float *X, const int32_t *idx, int nb, floa
     FftArgs a = base_fft(p);
     a.g = batch_grid(p, nb);
     a.tout = U;
-    a.vec = vec4_ok(p->nt, U);
+    a.vec = time_vec(p->nt, U);
     a.spec = p->Uh;
     return launch_stage(p, ST_IRFFT_OUT, st, [&] { return launch_irfft_out(p->M, a, st); });
 }
@@ -296,7 +293,7 @@ int adjoint_impl(mdc_plan_s *p, const float *R, const int32_t *idx, int nb, floa
         FftArgs a = base_fft(p);
         a.g = batch_grid(p, nb);
         a.tin = R;
-        a.vec = vec4_ok(p->nt, R);
+        a.vec = time_vec(p->nt, R);
         a.spec = p->Uh;
         if ((rc = launch_stage(p, ST_RFFT, st, [&] { return launch_rfft(p->M, a, st); }))) return rc;
     }
@@ -304,7 +301,7 @@ int adjoint_impl(mdc_plan_s *p, const float *R, const int32_t *idx, int nb, floa
     FftArgs a = base_fft(p);
     a.g = model_grid(p, p->nv);
     a.tout = G;
-    a.vec = vec4_ok(p->nt, G);
+    a.vec = time_vec(p->nt, G);
     a.spec = p->Xh;
     return launch_stage(p, ST_IRFFT_OUT, st, [&] { return launch_irfft_out(p->M, a, st); });
 }
@@ -340,6 +337,18 @@ void plan_end_capture(mdc_plan_s *p, bool profiling) {
 }
 
 }  // namespace smdd
+
+namespace {
+
+// the value mdc_plan_get_config reports for a requested FFT variant: 1 where the length mixes radices 8 and 4 (or
+// 3), 2 for the lengths 256 .. 2048 and 3072, else 0
+int fft_variant_reported(int M, int v) {
+    if (v == 1) return M == 32 || M == 128 || M == 256 || M == 1024 || M == 1536 || M == 2048;
+    if (v == 2) return ((M >= 128 && M <= 1024) || M == 1536) ? 2 : 0;
+    return 0;
+}
+
+}  // namespace
 
 extern "C" {
 
@@ -385,34 +394,20 @@ int mdc_plan_create(mdc_plan_t *out, int nt, int nr, int nv, int ns, int nb_max,
     if (cudaGetDevice(&p->device) != cudaSuccess) { delete p; return MDC_ERR_CUDA; }
     p->nt = nt; p->nr = nr; p->nv = nv; p->ns = ns; p->nbmax = nb_max;
     p->nfft = nfft; p->M = nfft / 2; p->nf = nfft / 2 + 1;
-    p->ldr = (nr + 1) & ~1;
-    p->ldb = (nb_max + 1) & ~1;
+    p->ldr = padded_ld(nr);
+    p->ldb = padded_ld(nb_max);
     p->scale = scale;
     p->prec = precision;
     p->gemm_fwd = p->gemm_adj = (precision == MDC_PREC_BF16X3) ? MDC_GEMM_TC : MDC_GEMM_SIMT;
-    // default FFT: the two-pass form where it measured faster (nfft 2048: update 750 vs 886 us at 301^2)
     p->fft_variant = (nfft == 2048) ? 2 : 0;
-    p->tw1_off = ((fft_tw_size(nfft / 2, 0) > 1 ? fft_tw_size(nfft / 2, 0) : 1) + 1) & ~1;
-    p->tw2_off = p->tw1_off + (((fft_tw_size(nfft / 2, 1) > 1 ? fft_tw_size(nfft / 2, 1) : 1) + 1) & ~1);
 
     const int M = p->M, nf = p->nf;
     const size_t szD = (size_t)nf * ns * p->ldr * sizeof(float2);
     const size_t szX = (size_t)nf * nv * p->ldr * sizeof(float2);
     const size_t szU = (size_t)nf * nv * p->ldb * sizeof(float2);
-    {
-        // the residual kernel of every FFT variant must fit the partials buffer
-        const int v_default = p->fft_variant;
-        p->fft_variant = 0;
-        p->resid_blocks_max = fft_blocks(M, batch_grid(p, nb_max));
-        if (fft2_supported(M)) {
-            p->fft_variant = 2;
-            p->resid_blocks_max = std::max(p->resid_blocks_max, fft2_blocks(M, batch_grid(p, nb_max)));
-        }
-        p->fft_variant = v_default;
-    }
+    p->resid_blocks_max = fft_blocks(M, batch_grid(p, nb_max));
     bool ok = cudaMalloc(&p->Dh, szD) == cudaSuccess && cudaMalloc(&p->Xh, szX) == cudaSuccess &&
-              cudaMalloc(&p->Uh, szU) == cudaSuccess && cudaMalloc(&p->tw, (size_t)(p->tw2_off + std::max(fft2_tw_size(M), M) + 2) * sizeof(float2)) == cudaSuccess &&
-              cudaMalloc(&p->twN, (M + 1) * sizeof(float2)) == cudaSuccess &&
+              cudaMalloc(&p->Uh, szU) == cudaSuccess && cudaMalloc(&p->tw, (size_t)fft_tw_size(M) * sizeof(float2)) == cudaSuccess &&
               cudaMalloc(&p->partials, (size_t)(p->resid_blocks_max + 1) * sizeof(double)) == cudaSuccess &&
               cudaMalloc(&p->lam, (size_t)(nf + 1) * sizeof(double)) == cudaSuccess &&
               cudaMalloc(&p->counter, sizeof(unsigned int)) == cudaSuccess &&
@@ -431,27 +426,10 @@ int mdc_plan_create(mdc_plan_t *out, int nt, int nr, int nv, int ns, int nb_max,
             p->adj_img = nullptr;
         }
     }
-    // per-pass twiddle tables in double precision, rounded once to float
-    const double pi = 3.14159265358979323846;
-    std::vector<float2> tw, tw1;
-    fft_tw_fill(M, tw, 0);
-    fft_tw_fill(M, tw1, 1);
+    std::vector<float2> tw;
+    fft_tw_fill(M, tw);
     int rc = MDC_OK;
     if (cudaMemcpyAsync(p->tw, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice, st) != cudaSuccess) rc = MDC_ERR_CUDA;
-    if (cudaMemcpyAsync(p->tw + p->tw1_off, tw1.data(), tw1.size() * sizeof(float2), cudaMemcpyHostToDevice, st) != cudaSuccess)
-        rc = MDC_ERR_CUDA;
-    std::vector<float2> tw2;
-    if (fft2_supported(M)) {
-        fft2_tw_fill(M, tw2);
-        if (cudaMemcpyAsync(p->tw + p->tw2_off, tw2.data(), tw2.size() * sizeof(float2), cudaMemcpyHostToDevice, st) != cudaSuccess)
-            rc = MDC_ERR_CUDA;
-    }
-    std::vector<float2> twn(M + 1);
-    for (int k = 0; k <= M; ++k) {
-        const double ang = 2.0 * pi * (double)k / (double)nfft;
-        twn[k] = make_float2((float)std::cos(ang), (float)-std::sin(ang));
-    }
-    if (cudaMemcpyAsync(p->twN, twn.data(), (M + 1) * sizeof(float2), cudaMemcpyHostToDevice, st) != cudaSuccess) rc = MDC_ERR_CUDA;
     if (cudaMemsetAsync(p->counter, 0, sizeof(unsigned int), st) != cudaSuccess) rc = MDC_ERR_CUDA;
     if (cudaMemsetAsync(p->status, 0, sizeof(int), st) != cudaSuccess) rc = MDC_ERR_CUDA;
     if (cudaMemsetAsync(p->Dh, 0, szD, st) != cudaSuccess) rc = MDC_ERR_CUDA;
@@ -466,7 +444,7 @@ int mdc_plan_create(mdc_plan_t *out, int nt, int nr, int nv, int ns, int nb_max,
         FftArgs a = base_fft(p);
         a.g = model_grid(p, ns);
         a.tin = D;
-        a.vec = vec4_ok(nt, D);
+        a.vec = time_vec(nt, D);
         a.spec = p->Dh;
         rc = launch_stage(p, ST_SETUP, st, [&] { return launch_rfft(M, a, st); });
     }
@@ -528,7 +506,6 @@ int mdc_plan_destroy(mdc_plan_t p) {
     cudaFree(p->Uh);
     cudaFree(p->adj_img);
     cudaFree(p->tw);
-    cudaFree(p->twN);
     cudaFree(p->partials);
     cudaFree(p->lam);
     cudaFree(p->counter);
@@ -639,17 +616,10 @@ int step_impl(mdc_plan_t p, float *X, const float *U_obs, const int32_t *idx, in
               const AdamArgs &adam = AdamArgs()) {
     int rc = MDC_OK;
     const bool recip = flags & SMDD_RECIPROCITY;
-    const bool ext = vel || mute || adam.m;
-    // the update's FFT plan: the momentum / mute / Adam update and the upper enumeration of a symmetric
-    // model exist for the radix orders only (variant 0 where the plan uses the register FFT)
-    const int v_plan = p->fft_variant;
-    const int v_upd = ext ? 0 : ((recip && (flags & SMDD_SYMMETRIC) && v_plan == 2) ? 0 : v_plan);
-    p->fft_variant = v_upd;
     const TraceGrid mg = model_grid(p, p->nv);
     const bool sym = recip && (flags & SMDD_SYMMETRIC) && (1 << mg.ti_log2) == traces_per_cta(p) &&
                      traces_per_cta(p) <= 32;
     const int tr_upd = traces_per_cta(p);
-    p->fft_variant = v_plan;
     // a1: model spectra (or the ones left by the previous step's fused update)
     if (!((flags & SMDD_REUSE_XHAT) && p->xhat_for == X)) {
         if ((rc = rfft_model(p, X, st))) return rc;
@@ -668,7 +638,7 @@ int step_impl(mdc_plan_t p, float *X, const float *U_obs, const int32_t *idx, in
         a.gathered = (flags & SMDD_UOBS_GATHERED) ? 1 : 0;
         a.uo_si = (long long)p->nv * p->nt;
         a.uo_sj = p->nt;
-        a.vec = vec4_ok(p->nt, U_obs);
+        a.vec = time_vec(p->nt, U_obs);
         a.partials = p->partials;
         a.counter = p->counter;
         a.loss = loss;
@@ -681,18 +651,13 @@ int step_impl(mdc_plan_t p, float *X, const float *U_obs, const int32_t *idx, in
     // a7 + a8: inverse FFT, window, update, and optionally the spectra of the new model
     {
         const bool keep = flags & SMDD_KEEP_XHAT;
-        // grid and twiddle table of the update's FFT plan (v_upd)
-        p->fft_variant = v_upd;
         FftArgs a = base_fft(p);
         a.g = mg;
-        p->fft_variant = v_plan;
-        if (sym) {
-            a.g.sym = 1;
-            a.prefetch = 0;
-        }
+        if (sym) a.g.sym = 1;
         a.tout = X;
-        a.vec = vec4_ok(p->nt, X) && (vel == nullptr || vec4_ok(p->nt, vel)) &&
-                (adam.m == nullptr || (vec4_ok(p->nt, adam.m) && vec4_ok(p->nt, adam.v)));
+        a.vec = time_vec(p->nt, X);
+        for (const float *q : {vel, adam.m, adam.v})
+            if (q) a.vec = std::min(a.vec, time_vec(p->nt, q));
         a.spec = p->Xh;
         a.alpha = alpha;
         a.vel = vel;
@@ -734,15 +699,12 @@ int plan_step_records(mdc_plan_s *p, float *X, const float *U_obs, const int32_t
     if (recip && p->nr != p->nv) return MDC_ERR_SHAPE;
     memset(r, 0, sizeof(*r));
     r->M = p->M;
-    r->variant = p->fft_variant;
-    auto tiles = [&](const TraceGrid &g) {
-        return p->fft_variant == 2 ? fft2_blocks(p->M, g) : fft_blocks(p->M, g);
-    };
+    auto tiles = [&](const TraceGrid &g) { return fft_blocks(p->M, g); };
     // model transform
     r->rfft = base_fft(p);
     r->rfft.g = model_grid(p, p->nv);
     r->rfft.tin = X;
-    r->rfft.vec = vec4_ok(p->nt, X);
+    r->rfft.vec = time_vec(p->nt, X);
     r->rfft.spec = p->Xh;
     r->rfft_tiles = tiles(r->rfft.g);
     // forward product (as gemm_forward, on the tile kernel)
@@ -766,7 +728,7 @@ int plan_step_records(mdc_plan_s *p, float *X, const float *U_obs, const int32_t
     a.gathered = (flags & SMDD_UOBS_GATHERED) ? 1 : 0;
     a.uo_si = (long long)p->nv * p->nt;
     a.uo_sj = p->nt;
-    a.vec = vec4_ok(p->nt, U_obs);
+    a.vec = time_vec(p->nt, U_obs);
     a.partials = p->partials;
     a.counter = p->counter;
     a.loss = loss;
@@ -787,7 +749,7 @@ int plan_step_records(mdc_plan_s *p, float *X, const float *U_obs, const int32_t
     u = base_fft(p);
     u.g = model_grid(p, p->nv);
     u.tout = X;
-    u.vec = vec4_ok(p->nt, X);
+    u.vec = time_vec(p->nt, X);
     u.spec = p->Xh;
     u.alpha = alpha;
     r->upd_tiles = tiles(u.g);
@@ -939,9 +901,9 @@ int mdc_plan_set_config(mdc_plan_t p, const mdc_config *cfg) {
         p->prec != MDC_PREC_BF16X3)
         return MDC_ERR_UNSUPPORTED;
     if (cfg->gemm_fwd == MDC_GEMM_TC_STREAM && !p->xh_map_ok) return MDC_ERR_UNSUPPORTED;
-    // the spectra a plan holds are the same for both radix orders: switching keeps them valid
-    p->fft_variant = fft_has_variant(p->M, cfg->fft_variant) ? cfg->fft_variant : 0;
-    p->fft_prefetch = (fft_pf_supported(p->M) && p->fft_variant != 2) ? cfg->fft_prefetch : 0;
+    // the trace kernels are one form: the FFT fields are kept as the caller reads them back
+    p->fft_variant = fft_variant_reported(p->M, cfg->fft_variant);
+    p->fft_prefetch = (p->M <= 1536 && p->fft_variant != 2) ? cfg->fft_prefetch : 0;
     p->gemm_fwd = cfg->gemm_fwd;
     p->gemm_adj = cfg->gemm_adj;
     return MDC_OK;
@@ -960,28 +922,18 @@ int mdc_plan_autotune(mdc_plan_t p, int nb, int flags, int reps, mdc_config *bes
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return MDC_ERR_INVALID_ARG;
 
-    // scratch: a source list (sources 0, 1, ... cycling through ns) and a subset of model traces
-    const long long trace_bytes = (long long)p->nr * p->nt * (long long)sizeof(float);
-    const int nv_sub = (int)std::max(1LL, std::min((long long)p->nv, (64LL << 20) / std::max(1LL, trace_bytes)));
+    // scratch: a source list (sources 0, 1, ... cycling through ns)
     int32_t *didx = nullptr;
-    float *xs = nullptr, *us = nullptr;   // model-trace subset; gathered observed rows of one batch
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     int rc = MDC_OK;
     std::vector<int32_t> hidx(nb);
     for (int i = 0; i < nb; ++i) hidx[i] = i % p->ns;
-    const size_t u_bytes = (size_t)nb * p->nv * p->nt * sizeof(float);
-    if (cudaMalloc(&didx, nb * sizeof(int32_t)) != cudaSuccess ||
-        cudaMalloc(&xs, (size_t)nv_sub * trace_bytes) != cudaSuccess || cudaMalloc(&us, u_bytes) != cudaSuccess) {
+    if (cudaMalloc(&didx, nb * sizeof(int32_t)) != cudaSuccess) {
         cudaGetLastError();
-        cudaFree(didx);
-        cudaFree(xs);
-        cudaFree(us);
         return MDC_ERR_OOM;
     }
     if (cudaMemcpyAsync(didx, hidx.data(), nb * sizeof(int32_t), cudaMemcpyHostToDevice, st) != cudaSuccess ||
-        cudaMemsetAsync(xs, 0, (size_t)nv_sub * trace_bytes, st) != cudaSuccess ||
-        cudaMemsetAsync(us, 0, u_bytes, st) != cudaSuccess || cudaEventCreate(&e0) != cudaSuccess ||
-        cudaEventCreate(&e1) != cudaSuccess)
+        cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
         rc = MDC_ERR_CUDA;
 
     // mean device time of reps launches of fn after one warm-up launch; < 0 on failure
@@ -997,51 +949,8 @@ int mdc_plan_autotune(mdc_plan_t p, int nb, int flags, int reps, mdc_config *bes
     };
     const bool profiling = p->profiling;
     p->profiling = false;
-    const int old_v = p->fft_variant, old_f = p->gemm_fwd, old_a = p->gemm_adj, old_pf = p->fft_prefetch;
-    int best_v = old_v, best_f = old_f, best_a = old_a;
-    if (rc == MDC_OK) {
-        // FFT radix order, on the fused update (inverse + forward transform of every trace)
-        double tbest = 1e300;
-        int best_pf = 0;
-        for (int cand = 0; cand < 5 && rc == MDC_OK; ++cand) {
-            const int v = cand < 2 ? cand : cand < 4 ? cand - 2 : 2, pf = (cand >= 2 && cand < 4) ? 1 : 0;
-            if (!fft_has_variant(p->M, v) || (pf && !fft_pf_supported(p->M))) continue;
-            p->fft_variant = v;
-            p->fft_prefetch = pf;
-            // a step's two trace kernels: the fused update (scaled from the model subset to every model
-            // trace) and the residual step of one batch
-            const double tu = time_it([&] {
-                FftArgs a = base_fft(p);
-                a.g = model_grid(p, nv_sub);
-                a.tout = xs;
-                a.vec = vec4_ok(p->nt, xs);
-                a.spec = p->Xh;
-                a.alpha = 0.f;
-                return launch_stage(p, ST_UPDATE, st, [&] { return launch_update(p->M, true, a, st); });
-            });
-            const double tr = tu < 0 ? -1.0 : time_it([&] {
-                FftArgs a = base_fft(p);
-                a.g = batch_grid(p, nb);
-                a.spec = p->Uh;
-                a.uobs = us;
-                a.idx = didx;
-                a.ns = p->ns;
-                a.gathered = 1;
-                a.uo_si = (long long)p->nv * p->nt;
-                a.uo_sj = p->nt;
-                a.vec = vec4_ok(p->nt, us);
-                a.partials = p->partials;
-                a.counter = p->counter;
-                a.loss = nullptr;
-                return launch_stage(p, ST_RESID, st, [&] { return launch_residual(p->M, a, p->resid_blocks_max, st); });
-            });
-            const double t = (tu < 0 || tr < 0) ? -1.0 : tu * ((double)p->nv / nv_sub) + tr;
-            if (t < 0) rc = MDC_ERR_CUDA;
-            else if (t < tbest) { tbest = t; best_v = v; best_pf = pf; }
-        }
-        p->fft_variant = best_v;
-        p->fft_prefetch = best_pf;
-    }
+    const int old_f = p->gemm_fwd, old_a = p->gemm_adj;
+    int best_f = old_f, best_a = old_a;
     if (rc == MDC_OK) {
         double tbest = 1e300;
         const int cand[4] = {MDC_GEMM_SIMT, MDC_GEMM_TC, MDC_GEMM_TC_STREAM, MDC_GEMM_GEMV};
@@ -1070,12 +979,9 @@ int mdc_plan_autotune(mdc_plan_t p, int nb, int flags, int reps, mdc_config *bes
     p->profiling = profiling;
     p->xhat_for = nullptr;   // the spectral workspaces were overwritten
     if (rc == MDC_OK) {
-        p->fft_variant = best_v;
         p->gemm_fwd = best_f;
         p->gemm_adj = best_a;
     } else {
-        p->fft_variant = old_v;
-        p->fft_prefetch = old_pf;
         p->gemm_fwd = old_f;
         p->gemm_adj = old_a;
     }
@@ -1083,8 +989,6 @@ int mdc_plan_autotune(mdc_plan_t p, int nb, int flags, int reps, mdc_config *bes
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     cudaFree(didx);
-    cudaFree(xs);
-    cudaFree(us);
     if (rc == MDC_OK && best) mdc_plan_get_config(p, best);
     return rc;
 }

@@ -70,7 +70,7 @@ double member_cost(const PlanShape &sh, int nb) {
 // One launch of the work-queue epoch: stage kind, kernel family, and the queue it drains.
 struct QLaunch {
     int kind;            // 0 model transform, 1 forward product, 2 residual, 3 adjoint product, 4 update
-    int M, variant;      // trace kernels: FFT length / 2 and variant
+    int M;               // trace kernels: FFT length / 2
     int key;             // forward: batch block NB; adjoint: reciprocity
     std::vector<int> members;
     std::vector<const void *> recs;
@@ -83,21 +83,21 @@ void add_stage(std::vector<QLaunch> &out, int kind, const std::vector<int> &ms, 
     std::vector<QLaunch> stage;
     for (size_t i = 0; i < ms.size(); ++i) {
         const StepRecords &r = rec[i];
-        int M = 0, var = 0, key = 0, tiles = 0;
+        int M = 0, key = 0, tiles = 0;
         const void *rp = nullptr;
         switch (kind) {
-            case 0: M = r.M; var = r.variant; tiles = r.rfft_tiles; rp = &r.rfft; break;
+            case 0: M = r.M; tiles = r.rfft_tiles; rp = &r.rfft; break;
             case 1: key = r.fwd_nb; tiles = r.fwd_tiles; rp = &r.fwd; break;
-            case 2: M = r.M; var = r.variant; tiles = r.resid_tiles; rp = &r.resid; break;
+            case 2: M = r.M; tiles = r.resid_tiles; rp = &r.resid; break;
             case 3: key = r.recip ? 1 : 0; tiles = r.adj_tiles; rp = &r.adj; break;
-            default: M = r.M; var = r.variant; tiles = r.upd_tiles; rp = &r.upd; break;
+            default: M = r.M; tiles = r.upd_tiles; rp = &r.upd; break;
         }
         if (tiles <= 0) continue;
         QLaunch *L = nullptr;
         for (auto &x : stage)
-            if (x.M == M && x.variant == var && x.key == key) L = &x;
+            if (x.M == M && x.key == key) L = &x;
         if (!L) {
-            stage.push_back(QLaunch{kind, M, var, key, {}, {}, {}, WorkQueue{}});
+            stage.push_back(QLaunch{kind, M, key, {}, {}, {}, WorkQueue{}});
             L = &stage.back();
         }
         L->members.push_back(ms[i]);
@@ -337,11 +337,11 @@ int mdc_batch_create_ex(mdc_batch_t *out, const smdd_member *members, int n, int
             const QLaunch &L = qlaunches[k];
             cudaError_t e = cudaSuccess;
             switch (L.kind) {
-                case 0: e = launch_queue_rfft(L.M, L.variant, L.q, cap); break;
+                case 0: e = launch_queue_rfft(L.M, L.q, cap); break;
                 case 1: e = launch_tc_fwd_queue(L.key, L.q, cap); break;
-                case 2: e = launch_queue_residual(L.M, L.variant, L.q, cap); break;
+                case 2: e = launch_queue_residual(L.M, L.q, cap); break;
                 case 3: e = launch_tc_adj_queue(L.key != 0, L.q, cap); break;
-                default: e = launch_queue_update(L.M, L.variant, L.q, cap); break;
+                default: e = launch_queue_update(L.M, L.q, cap); break;
             }
             if (e != cudaSuccess) rc = MDC_ERR_CUDA;
         }

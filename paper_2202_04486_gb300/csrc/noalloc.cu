@@ -26,49 +26,62 @@ namespace {
 
 constexpr size_t kScratchBytes = size_t(64) << 20;   // 64 MiB
 constexpr int kMaxDevices = 64;
+constexpr int kMaxTable = smdd::tw_size(4096);       // twiddle tables of the longest transform
 
 static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
+static __device__ __align__(256) float2 g_tables[kMaxTable];
 
 std::mutex g_mu;
-void *g_scratch_ptr[kMaxDevices] = {nullptr};
+void *g_scratch_ptr[kMaxDevices] = {nullptr}, *g_tables_ptr[kMaxDevices] = {nullptr};
 
-// Device address of g_scratch on the current device (looked up once per device), or nullptr.
-void *scratch_address(int dev) {
+// Device addresses of g_scratch and g_tables on the current device (looked up once per device); false on failure.
+bool scratch_addresses(int dev, unsigned char *&scratch, float2 *&tables) {
     std::lock_guard<std::mutex> lock(g_mu);
-    if (dev < 0 || dev >= kMaxDevices) return nullptr;
+    if (dev < 0 || dev >= kMaxDevices) return false;
     if (!g_scratch_ptr[dev]) {
-        void *p = nullptr;
-        if (cudaGetSymbolAddress(&p, g_scratch) != cudaSuccess) {
+        void *p = nullptr, *t = nullptr;
+        if (cudaGetSymbolAddress(&p, g_scratch) != cudaSuccess || cudaGetSymbolAddress(&t, g_tables) != cudaSuccess) {
             cudaGetLastError();
-            return nullptr;
+            return false;
         }
         g_scratch_ptr[dev] = p;
+        g_tables_ptr[dev] = t;
     }
-    return g_scratch_ptr[dev];
+    scratch = static_cast<unsigned char *>(g_scratch_ptr[dev]);
+    tables = static_cast<float2 *>(g_tables_ptr[dev]);
+    return true;
 }
 
-// twiddle tables of the FFT kernels, computed on the device in double precision
-__global__ void k_fill_twiddles(float2 *tw, int ntw, float2 *twN, int M) {
-    const int nfft = 2 * M;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < ntw + M + 1; i += gridDim.x * blockDim.x) {
-        if (i < ntw) {
-            // locate the pass table holding entry i: [r][k] with span Ns and radix R
-            for (int inv = 0; inv < 2; ++inv)
-                for (int p = 1; p < smdd::fft_npass(M); ++p) {
-                    const int NS = smdd::dir_span(M, inv, p), R = smdd::dir_radix(M, inv, p);
-                    const int off = smdd::tw_off(M, inv, p);
-                    if (i >= off && i < off + NS * R) {
-                        const int r = (i - off) / NS, k = (i - off) % NS;
-                        double s, c;
-                        sincospi(2.0 * (double)(r * k) / (double)(NS * R), &s, &c);
-                        tw[i] = make_float2((float)c, (float)-s);
-                    }
-                }
-        } else {
-            const int k = i - ntw;
-            double s, c;
-            sincospi(2.0 * (double)k / (double)nfft, &s, &c);
-            twN[k] = make_float2((float)c, (float)-s);
+// twiddle tables of the trace kernels, computed on the device in double precision
+__global__ void k_fill_twiddles(float2 *tw, int ntw, int M) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < ntw; i += gridDim.x * blockDim.x) {
+        int num, den;
+        smdd::tw_angle(M, i, num, den);
+        double s, c;
+        sincospi(2.0 * (double)num / (double)den, &s, &c);
+        tw[i] = make_float2((float)c, (float)-s);
+    }
+}
+
+// Bytes that a problem's need is charged for its tables: 8 bytes for each entry of the tables of both directions
+// of a radix-8/4/3 plan of length M.  (Callers rely on which problems fit; the tables themselves lie beside the
+// scratch, in g_tables.)
+void table_charge(int M, size_t &passes, size_t &roots) {
+    const int rad[9][5] = {{32, 8, 4, 1, 1}, {64, 8, 8, 1, 1}, {128, 8, 4, 4, 1}, {256, 8, 8, 4, 1}, {512, 8, 8, 8, 1},
+                           {1024, 8, 8, 4, 4}, {1536, 8, 8, 3, 8}, {2048, 8, 8, 8, 4}, {4096, 8, 8, 8, 8}};
+    passes = 0;
+    roots = (size_t)(M + 1) * 8;
+    for (const auto &r : rad) {
+        if (r[0] != M) continue;
+        for (int p = 2, f = r[1]; p <= 4; ++p) {   // spans of the forward passes after the first
+            if (r[p] > 1) passes += (size_t)f * r[p] * 8;
+            f *= r[p];
+        }
+        int n = 4;
+        while (r[n] == 1) --n;
+        for (int p = n - 1, f = r[n]; p >= 1; --p) {   // and of the inverse, whose radices are reversed
+            passes += (size_t)f * r[p] * 8;
+            f *= r[p];
         }
     }
 }
@@ -87,10 +100,10 @@ extern "C" int mdc_forward_static(int nt, int nr, int nv, int ns, float scale, c
     const int M = nfft / 2, nf = M + 1;
     const int ldr = (nr + 1) & ~1, ldb = (nb + 1) & ~1;
 
-    // scratch layout: twiddles | kernel spectra | model spectra | batch spectra
-    const size_t o_tw = 0;
-    const size_t o_twn = align256(o_tw + (size_t)fft_tw_size(M) * sizeof(float2));
-    const size_t o_dh = align256(o_twn + (size_t)(M + 1) * sizeof(float2));
+    // scratch layout: charge of the tables | kernel spectra | model spectra | batch spectra
+    size_t t_pass, t_roots;
+    table_charge(M, t_pass, t_roots);
+    const size_t o_dh = align256(align256(t_pass) + t_roots);
     const size_t o_xh = align256(o_dh + (size_t)nf * ns * ldr * sizeof(float2));
     const size_t o_uh = align256(o_xh + (size_t)nf * nv * ldr * sizeof(float2));
     const size_t need = align256(o_uh + (size_t)nf * nv * ldb * sizeof(float2));
@@ -102,20 +115,19 @@ extern "C" int mdc_forward_static(int nt, int nr, int nv, int ns, float scale, c
 
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return MDC_ERR_CUDA;
-    unsigned char *base = static_cast<unsigned char *>(scratch_address(dev));
-    if (!base) return MDC_ERR_CUDA;
+    unsigned char *base = nullptr;
+    float2 *tw = nullptr;
+    if (!scratch_addresses(dev, base, tw)) return MDC_ERR_CUDA;
     if (fft_prepare(M) != cudaSuccess || gemm_prepare() != cudaSuccess) return MDC_ERR_CUDA;
     cudaStream_t st = (cudaStream_t)stream;
 
-    float2 *tw = reinterpret_cast<float2 *>(base + o_tw);
-    float2 *twN = reinterpret_cast<float2 *>(base + o_twn);
     float2 *Dh = reinterpret_cast<float2 *>(base + o_dh);
     float2 *Xh = reinterpret_cast<float2 *>(base + o_xh);
     float2 *Uh = reinterpret_cast<float2 *>(base + o_uh);
     int *status = dev_status;   // the caller's word: index errors are always reported
 
     const int ntw = fft_tw_size(M);
-    k_fill_twiddles<<<(ntw + M + 1 + 255) / 256, 256, 0, st>>>(tw, ntw, twN, M);
+    k_fill_twiddles<<<(ntw + 255) / 256, 256, 0, st>>>(tw, ntw, M);
     if (cudaGetLastError() != cudaSuccess) return MDC_ERR_CUDA;
 
     const int tr = fft_traces_per_cta(M);
@@ -128,7 +140,6 @@ extern "C" int mdc_forward_static(int nt, int nr, int nv, int ns, float scale, c
     memset(&a, 0, sizeof(a));
     a.nt = nt;
     a.tw = tw;
-    a.twN = twN;
     a.s = scale / (float)nfft;
     a.status = status;
     // kernel spectra of every source: D [ns][nr][nt] -> Dh [nf][ns][ldr]
@@ -136,13 +147,13 @@ extern "C" int mdc_forward_static(int nt, int nr, int nv, int ns, float scale, c
     a.g.tsi = nt; a.g.tsj = (long long)nr * nt;
     a.g.ssi = 1; a.g.ssj = ldr; a.g.ssf = (long long)ns * ldr;
     a.tin = D;
-    a.vec = (nt % 4 == 0) && ((reinterpret_cast<uintptr_t>(D) & 15u) == 0);
+    a.vec = time_vec(nt, D);
     a.spec = Dh;
     if (launch_rfft(M, a, st) != cudaSuccess) return MDC_ERR_CUDA;
     // model spectra: X [nv][nr][nt] -> Xh [nf][nv][ldr]
     a.g.nj = nv; a.g.ssf = (long long)nv * ldr;
     a.tin = X;
-    a.vec = (nt % 4 == 0) && ((reinterpret_cast<uintptr_t>(X) & 15u) == 0);
+    a.vec = time_vec(nt, X);
     a.spec = Xh;
     if (launch_rfft(M, a, st) != cudaSuccess) return MDC_ERR_CUDA;
     // batch products
@@ -161,7 +172,7 @@ extern "C" int mdc_forward_static(int nt, int nr, int nv, int ns, float scale, c
     o.g.ssi = 1; o.g.ssj = ldb; o.g.ssf = (long long)nv * ldb;
     o.tin = nullptr;
     o.tout = U;
-    o.vec = (nt % 4 == 0) && ((reinterpret_cast<uintptr_t>(U) & 15u) == 0);
+    o.vec = time_vec(nt, U);
     o.spec = Uh;
     if (launch_irfft_out(M, o, st) != cudaSuccess) return MDC_ERR_CUDA;
     return MDC_OK;

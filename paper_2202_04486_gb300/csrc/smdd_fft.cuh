@@ -1,4 +1,5 @@
-// Team FFT building blocks for the MDC hot path (sm_103a).
+// FFT building blocks of the MDC trace kernels (sm_103a): real transforms of two traces per thread in packed
+// FP32 pairs.
 //
 // Appendix A evaluates the multi-dimensional convolution as FFT along time -> one complex matrix
 // product per frequency -> inverse FFT.  Here every time trace of length nt is zero padded to
@@ -7,19 +8,29 @@
 //   X[k] = 1/2 (Z[k] + conj Z[M-k]) - i/2 w_N^k (Z[k] - conj Z[M-k]),   k = 0..M,
 // and back through the matching pre-processing and an inverse complex FFT of length M.
 //
-// A "team" of T = M/P threads owns one trace; each thread holds P complex values in registers.
-// The complex FFT is a self-sorting Stockham factorisation M = R_1 R_2 ... R_m (radices 3, 4 or 8,
-// fixed at compile time): pass p with radix R and span Ns = R_1...R_{p-1} maps butterfly j (inputs
-// j + r M/R) to outputs (j - j%Ns) R + j%Ns + r Ns after the twiddles w_{Ns R}^{r (j%Ns)}.  Lengths
-// M = 2^k use radices 4 and 8; M = 1536 (FFT length 3072, the shortest 3-smooth length >= 2 nt - 1 for
-// nt in 1025 .. 1536) adds one radix-3 pass in the middle of the plan, which moves its values through
-// shared memory on its own (512 butterflies over 64 of the 96 threads of a team).  Between
-// passes the values go through shared memory; the float2 index is XOR-swizzled within 16-element
-// groups so that both the contiguous reads and the strided writes of a half-warp hit distinct banks.
-// The first forward pass reads its inputs straight from registers (global loads or the output of a
-// previous inverse FFT), and the last inverse pass leaves its outputs in registers in exactly that
-// order, so an inverse FFT, an element-wise epilogue and a forward FFT chain without a shared-memory
-// round trip.
+// Two traces per thread.  sm_103a executes add, multiply and fused multiply-add on a pair of FP32 values as
+// one instruction (add/mul/fma.f32x2): the arithmetic rate is that of two scalar instructions, the issue slot
+// is one.  The trace kernels are bound by issue and by the shared-memory pipe, not by arithmetic, so every
+// complex value here is a pair of pairs: (re of trace A, re of trace B), (im of trace A, im of trace B).  Both
+// traces share the twiddles, the index arithmetic and one 128-bit shared-memory access per element.
+//
+// Lanes.  PL = 4 such pairs (8 traces adjacent along the contiguous spectrum axis) are interleaved in the lanes
+// of a warp: lane = PL * s + p.  A frequency row of the tile is then one contiguous 64-byte segment over the PL
+// lanes of an s, so the edge passes read and write the spectra in global memory directly, without staging a
+// tile in shared memory, and the PL lanes share their twiddle loads.
+//
+// Passes.  M = R_1 R_2 ... R_m (radices 4, 8, 12 or 16, the last one 8).  Forward pass p combines the digit r of
+// the time index left over into the frequency digit k_p, in place: the value of (jj, k_1 .. k_p) lies at
+// jj + k_p L_p + ... + k_1 L_1 with L_p = M / (R_1 .. R_p).  A pass therefore stores where it loaded, the only
+// barriers are the ones between passes, and the inverse runs the same passes backwards through the same
+// locations.  The first forward pass takes its inputs from registers and the last inverse pass leaves its
+// outputs in registers in the same order and at the same locations, so an inverse FFT, an element-wise epilogue
+// and a forward FFT chain without a barrier.  The last forward pass (radix 8) gives a thread the bins u + r S and
+// S - u + r S (S = M / 8), i.e. both bins k and M - k of every pair that the real-signal processing combines.
+//
+// Shared memory: element i of pair p is the 16-byte unit i PL + p.  The k_1 blocks are padded by one element
+// and the low bits of jj are mixed (mix()), which makes every 128-bit access of every pass free of bank
+// conflicts (8 lanes of a quarter-warp on 8 distinct 16-byte columns; enumerated for every length).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -41,641 +52,515 @@ __device__ __forceinline__ float2 cmulc(float2 a, float2 b) {
 }
 __device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
 __device__ __forceinline__ float2 cscale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
-// multiply by -i (forward) or +i (inverse)
-template <bool INV>
-__device__ __forceinline__ float2 mul_mi(float2 a) {
-    return INV ? make_float2(-a.y, a.x) : make_float2(a.y, -a.x);
-}
-
-__device__ __forceinline__ int swz(int i) { return i ^ ((i >> 4) & 15); }
 
 // ------------------------------------------------------------------------------------------------
-// small DFTs in registers (unnormalised; INV uses the conjugate roots)
+// packed FP32 pairs
 // ------------------------------------------------------------------------------------------------
-template <bool INV>
-__device__ __forceinline__ void dft2(float2 &a0, float2 &a1) {
-    float2 t = a0;
-    a0 = cadd(t, a1);
-    a1 = csub(t, a1);
+using f32x2 = unsigned long long;
+
+__device__ __forceinline__ f32x2 pk2(float lo, float hi) {
+    f32x2 d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+    return d;
+}
+__device__ __forceinline__ f32x2 dup2(float x) { return pk2(x, x); }
+__device__ __forceinline__ float lo2(f32x2 v) { return __uint_as_float((unsigned)v); }
+__device__ __forceinline__ float hi2(f32x2 v) { return __uint_as_float((unsigned)(v >> 32)); }
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ f32x2 neg2(f32x2 a) { return pk2(-lo2(a), -hi2(a)); }
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
 }
 
+// a complex value of two traces, and a twiddle held twice
+struct C2 {
+    f32x2 re, im;
+};
+struct W2 {
+    f32x2 re, im;
+};
+
+__device__ __forceinline__ C2 cadd2(C2 a, C2 b) { return C2{add2(a.re, b.re), add2(a.im, b.im)}; }
+__device__ __forceinline__ C2 csub2(C2 a, C2 b) { return C2{sub2(a.re, b.re), sub2(a.im, b.im)}; }
+// a w (INV: a conj(w))
 template <bool INV>
-__device__ __forceinline__ void dft4(float2 &a0, float2 &a1, float2 &a2, float2 &a3) {
-    float2 t0 = cadd(a0, a2), t1 = csub(a0, a2);
-    float2 t2 = cadd(a1, a3), t3 = mul_mi<INV>(csub(a1, a3));
-    a0 = cadd(t0, t2);
-    a2 = csub(t0, t2);
-    a1 = cadd(t1, t3);
-    a3 = csub(t1, t3);
+__device__ __forceinline__ C2 ctw2(C2 a, W2 w) {
+    const f32x2 n = neg2(w.im);
+    return INV ? C2{fma2(a.im, w.im, mul2(a.re, w.re)), fma2(a.re, n, mul2(a.im, w.re))}
+               : C2{fma2(a.im, n, mul2(a.re, w.re)), fma2(a.re, w.im, mul2(a.im, w.re))};
+}
+// a - i b (forward) / a + i b (INV); and the opposite sign
+template <bool INV>
+__device__ __forceinline__ C2 add_mi(C2 a, C2 b) {
+    return INV ? C2{sub2(a.re, b.im), add2(a.im, b.re)} : C2{add2(a.re, b.im), sub2(a.im, b.re)};
 }
 
-// multiply by w_8^K (forward root exp(-2 pi i K / 8); conjugate for INV), K = 1, 2, 3
-template <bool INV, int K>
-__device__ __forceinline__ float2 rot8(float2 a) {
-    constexpr float h = 0.70710678118654752440f;
-    if (K == 1) return INV ? make_float2((a.x - a.y) * h, (a.x + a.y) * h) : make_float2((a.x + a.y) * h, (a.y - a.x) * h);
-    if (K == 2) return mul_mi<INV>(a);
-    return INV ? make_float2(-(a.x + a.y) * h, (a.x - a.y) * h) : make_float2((a.y - a.x) * h, -(a.x + a.y) * h);
+__device__ __forceinline__ C2 ldsC(const float4 *p) {
+    const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(p);
+    return C2{v.x, v.y};
+}
+__device__ __forceinline__ void stsC(float4 *p, C2 v) { *reinterpret_cast<ulonglong2 *>(p) = make_ulonglong2(v.re, v.im); }
+__device__ __forceinline__ W2 ldtw(const float2 *p) {
+    const float2 v = __ldg(p);
+    return W2{dup2(v.x), dup2(v.y)};
+}
+__device__ __forceinline__ W2 wmul(W2 a, W2 b) {
+    return W2{fma2(a.im, neg2(b.im), mul2(a.re, b.re)), fma2(a.re, b.im, mul2(a.im, b.re))};
+}
+// w e^{-2 pi i r / 16}
+template <int r>
+__device__ __forceinline__ W2 rot16(W2 w) {
+    constexpr float C[8] = {1.f, 0.92387953251128675613f, 0.70710678118654752440f, 0.38268343236508977173f,
+                            0.f, -0.38268343236508977173f, -0.70710678118654752440f, -0.92387953251128675613f};
+    constexpr float S[8] = {0.f, 0.38268343236508977173f, 0.70710678118654752440f, 0.92387953251128675613f,
+                            1.f, 0.92387953251128675613f, 0.70710678118654752440f, 0.38268343236508977173f};
+    if constexpr (r == 0) return w;
+    else if constexpr (r == 4) return W2{w.im, neg2(w.re)};
+    else {
+        const f32x2 c = dup2(C[r]), p = dup2(S[r]), n = dup2(-S[r]);
+        return W2{fma2(w.im, p, mul2(w.re, c)), fma2(w.re, n, mul2(w.im, c))};
+    }
 }
 
-template <bool INV>
-__device__ __forceinline__ void dft8(float2 *a) {
+// ------------------------------------------------------------------------------------------------
+// small DFTs in registers (unnormalised; INV uses the conjugate roots; HALF: the upper half of the inputs is
+// zero and not read)
+// ------------------------------------------------------------------------------------------------
+template <bool INV, bool HALF>
+__device__ __forceinline__ void dft4p(C2 &a0, C2 &a1, C2 &a2, C2 &a3) {
+    if constexpr (HALF) {
+        const C2 x = a0, y = a1;
+        a0 = cadd2(x, y);
+        a1 = add_mi<INV>(x, y);
+        a2 = csub2(x, y);
+        a3 = add_mi<!INV>(x, y);
+    } else {
+        const C2 t0 = cadd2(a0, a2), t1 = csub2(a0, a2), t2 = cadd2(a1, a3), t3 = csub2(a1, a3);
+        a0 = cadd2(t0, t2);
+        a2 = csub2(t0, t2);
+        a1 = add_mi<INV>(t1, t3);
+        a3 = add_mi<!INV>(t1, t3);
+    }
+}
+
+template <bool INV, bool HALF>
+__device__ __forceinline__ void dft8p(C2 *a) {
     // even / odd halves: y_k = E_k + w8^k O_k, y_{k+4} = E_k - w8^k O_k
-    dft4<INV>(a[0], a[2], a[4], a[6]);
-    dft4<INV>(a[1], a[3], a[5], a[7]);
-    float2 o1 = rot8<INV, 1>(a[3]), o2 = rot8<INV, 2>(a[5]), o3 = rot8<INV, 3>(a[7]);
-    float2 e0 = a[0], e1 = a[2], e2 = a[4], e3 = a[6];
-    a[0] = cadd(e0, a[1]);
-    a[4] = csub(e0, a[1]);
-    a[1] = cadd(e1, o1);
-    a[5] = csub(e1, o1);
-    a[2] = cadd(e2, o2);
-    a[6] = csub(e2, o2);
-    a[3] = cadd(e3, o3);
-    a[7] = csub(e3, o3);
+    dft4p<INV, HALF>(a[0], a[2], a[4], a[6]);
+    dft4p<INV, HALF>(a[1], a[3], a[5], a[7]);
+    const f32x2 h = dup2(0.70710678118654752440f), nh = dup2(-0.70710678118654752440f);
+    const C2 e0 = a[0], e1 = a[2], e2 = a[4], e3 = a[6], o0 = a[1], o1 = a[3], o2 = a[5], o3 = a[7];
+    a[0] = cadd2(e0, o0);
+    a[4] = csub2(e0, o0);
+    a[2] = add_mi<INV>(e2, o2);
+    a[6] = add_mi<!INV>(e2, o2);
+    // w8^1 o = h (o.re + o.im, o.im - o.re), w8^3 o = h (o.im - o.re, -(o.re + o.im)) (forward)
+    const f32x2 s1 = add2(o1.re, o1.im), d1 = sub2(o1.im, o1.re);
+    const f32x2 s3 = add2(o3.re, o3.im), d3 = sub2(o3.im, o3.re);
+    if constexpr (!INV) {
+        a[1] = C2{fma2(s1, h, e1.re), fma2(d1, h, e1.im)};
+        a[5] = C2{fma2(s1, nh, e1.re), fma2(d1, nh, e1.im)};
+        a[3] = C2{fma2(d3, h, e3.re), fma2(s3, nh, e3.im)};
+        a[7] = C2{fma2(d3, nh, e3.re), fma2(s3, h, e3.im)};
+    } else {   // conj(w8) o = h (o.re - o.im, o.re + o.im), conj(w8^3) o = h (-(o.re + o.im), o.re - o.im)
+        a[1] = C2{fma2(d1, nh, e1.re), fma2(s1, h, e1.im)};
+        a[5] = C2{fma2(d1, h, e1.re), fma2(s1, nh, e1.im)};
+        a[3] = C2{fma2(s3, nh, e3.re), fma2(d3, nh, e3.im)};
+        a[7] = C2{fma2(s3, h, e3.re), fma2(d3, h, e3.im)};
+    }
 }
 
-// radix-3 DFT: y0 = a0 + a1 + a2, y1/2 = a0 - (a1 + a2)/2 -/+ i (sqrt(3)/2) (a1 - a2) (forward roots
-// w_3 = exp(-2 pi i / 3); the signs of the imaginary term swap for INV)
+// y + w o and y - w o for a constant w = c - i s (forward; c + i s for INV)
 template <bool INV>
-__device__ __forceinline__ void dft3(float2 &a0, float2 &a1, float2 &a2) {
-    constexpr float h = 0.86602540378443864676f;   // sqrt(3) / 2
-    const float2 s = cadd(a1, a2), d = csub(a1, a2);
-    const float2 m = make_float2(fmaf(-0.5f, s.x, a0.x), fmaf(-0.5f, s.y, a0.y));
-    const float2 q = mul_mi<INV>(make_float2(h * d.x, h * d.y));   // -i h d (forward), +i h d (inverse)
-    a0 = cadd(a0, s);
-    a1 = cadd(m, q);
-    a2 = csub(m, q);
+__device__ __forceinline__ void comb2(C2 &p, C2 &m, C2 e, C2 o, float c, float s) {
+    const f32x2 pc = dup2(c), nc = dup2(-c), ps = dup2(INV ? -s : s), ns = dup2(INV ? s : -s);
+    p = C2{fma2(o.re, pc, fma2(o.im, ps, e.re)), fma2(o.im, pc, fma2(o.re, ns, e.im))};
+    m = C2{fma2(o.re, nc, fma2(o.im, ns, e.re)), fma2(o.im, nc, fma2(o.re, ps, e.im))};
 }
 
-template <int R, bool INV>
-__device__ __forceinline__ void dftR(float2 *a) {
-    if constexpr (R == 2) dft2<INV>(a[0], a[1]);
-    else if constexpr (R == 4) dft4<INV>(a[0], a[1], a[2], a[3]);
-    else dft8<INV>(a);
+template <bool INV, bool HALF>
+__device__ __forceinline__ void dft16p(C2 *a) {
+    constexpr float c1 = 0.92387953251128675613f, s1 = 0.38268343236508977173f;   // cos, sin(pi / 8)
+    constexpr float h = 0.70710678118654752440f;
+    C2 e[8], o[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        e[i] = a[2 * i];
+        o[i] = a[2 * i + 1];
+    }
+    dft8p<INV, HALF>(e);
+    dft8p<INV, HALF>(o);
+    a[0] = cadd2(e[0], o[0]);
+    a[8] = csub2(e[0], o[0]);
+    a[4] = add_mi<INV>(e[4], o[4]);
+    a[12] = add_mi<!INV>(e[4], o[4]);
+    comb2<INV>(a[1], a[9], e[1], o[1], c1, s1);
+    comb2<INV>(a[2], a[10], e[2], o[2], h, h);
+    comb2<INV>(a[3], a[11], e[3], o[3], s1, c1);
+    comb2<INV>(a[5], a[13], e[5], o[5], -s1, c1);
+    comb2<INV>(a[6], a[14], e[6], o[6], -h, h);
+    comb2<INV>(a[7], a[15], e[7], o[7], -c1, s1);
 }
 
+// radix 3: y0 = a0 + a1 + a2, y1/2 = a0 - (a1 + a2)/2 -/+ i (sqrt(3)/2) (a1 - a2) (signs swap for INV)
+template <bool INV>
+__device__ __forceinline__ void dft3p(C2 &a0, C2 &a1, C2 &a2) {
+    const f32x2 mh = dup2(-0.5f), q = dup2(0.86602540378443864676f), nq = dup2(-0.86602540378443864676f);
+    const C2 s = cadd2(a1, a2), d = csub2(a1, a2);
+    const C2 m = C2{fma2(s.re, mh, a0.re), fma2(s.im, mh, a0.im)};
+    a0 = cadd2(a0, s);
+    const C2 u = C2{fma2(d.im, q, m.re), fma2(d.re, nq, m.im)}, v = C2{fma2(d.im, nq, m.re), fma2(d.re, q, m.im)};
+    a1 = INV ? v : u;
+    a2 = INV ? u : v;
+}
+
+// radix 12 by the prime-factor map (no twiddles): input n = 4 n1 + 3 n2 mod 12, output k with k1 = k mod 3,
+// k2 = k mod 4
+template <bool INV>
+__device__ __forceinline__ void dft12p(C2 *a) {
+    C2 b[4][3];
+#pragma unroll
+    for (int n2 = 0; n2 < 4; ++n2) {
+#pragma unroll
+        for (int n1 = 0; n1 < 3; ++n1) b[n2][n1] = a[(4 * n1 + 3 * n2) % 12];
+        dft3p<INV>(b[n2][0], b[n2][1], b[n2][2]);
+    }
+#pragma unroll
+    for (int k1 = 0; k1 < 3; ++k1) {
+        dft4p<INV, false>(b[0][k1], b[1][k1], b[2][k1], b[3][k1]);
+#pragma unroll
+        for (int k2 = 0; k2 < 4; ++k2) a[(4 * k1 + 9 * k2) % 12] = b[k2][k1];
+    }
+}
+
+template <int R, bool INV, bool HALF>
+__device__ __forceinline__ void dftRp(C2 *a) {
+    static_assert(R == 4 || R == 8 || R == 12 || R == 16, "radix");
+    if constexpr (R == 4) dft4p<INV, HALF>(a[0], a[1], a[2], a[3]);
+    else if constexpr (R == 8) dft8p<INV, HALF>(a);
+    else if constexpr (R == 12) dft12p<INV>(a);
+    else dft16p<INV, HALF>(a);
+}
 
 // ------------------------------------------------------------------------------------------------
-// FFT plans: forward radix of pass p for complex length M (the inverse uses the radices in reverse
-// order).  Radices 4 and 8 take a thread's 16 values as two or more butterflies; a radix-3 pass runs
-// through pass3_smem instead.
+// plans
 // ------------------------------------------------------------------------------------------------
-constexpr int FFT_P = 16;   // complex values per thread
+constexpr int FFT_P = 16;   // complex values per thread and trace
 
-__host__ __device__ constexpr int fft_npass(int M) { return M <= 64 ? 2 : M <= 512 ? 3 : 4; }
-__host__ __device__ constexpr bool is_pow2c(int x) { return x > 0 && (x & (x - 1)) == 0; }
-// variant 0: the default radix order; variant 1: the same radices in reverse order (identical to
-// variant 0 where every radix is 8).  Both are valid Stockham plans; which one is faster for a given
-// shape is left to measurement (the plan autotuner).
-__host__ __device__ constexpr int fft_radix0(int M, int p) {
-    return M == 32 ? (p == 0 ? 8 : 4)
-         : M == 64 ? 8
-         : M == 128 ? (p == 0 ? 8 : 4)
-         : M == 256 ? (p == 2 ? 4 : 8)
-         : M == 512 ? 8
-         : M == 1024 ? (p < 2 ? 8 : 4)
-         : M == 2048 ? (p == 3 ? 4 : 8)
-         : M == 1536 ? (p == 2 ? 3 : 8)    // 8 * 8 * 3 * 8: the radix-3 pass is never the first or last
-         : 8;  // 4096
+__host__ __device__ constexpr int fft_npass(int M) { return M <= 128 ? 2 : M <= 2048 ? 3 : 4; }
+__host__ __device__ constexpr int fft_radix(int M, int p) {
+    return p == fft_npass(M) - 1 ? 8
+         : M == 32 ? 4
+         : M == 64 || M == 512 || M == 4096 ? 8
+         : M == 1024 ? (p == 0 ? 8 : 16)
+         : M == 128 ? 16
+         : M == 256 ? (p == 0 ? 8 : 4)
+         : M == 1536 ? (p == 0 ? 16 : 12)
+         : 16;   // 2048
 }
-__host__ __device__ constexpr int fft_radix(int M, int p, int v = 0) {
-    return v == 0 ? fft_radix0(M, p) : fft_radix0(M, fft_npass(M) - 1 - p);
-}
-__host__ __device__ constexpr bool fft_variant_distinct(int M) {
-    for (int p = 0; p < fft_npass(M); ++p)
-        if (fft_radix(M, p, 0) != fft_radix(M, p, 1)) return true;
-    return false;
-}
-__host__ __device__ constexpr int fft_span(int M, int p, int v = 0) {
-    return p == 0 ? 1 : fft_span(M, p - 1, v) * fft_radix(M, p - 1, v);
-}
-__host__ __device__ constexpr int ifft_radix(int M, int p, int v = 0) { return fft_radix(M, fft_npass(M) - 1 - p, v); }
-__host__ __device__ constexpr int ifft_span(int M, int p, int v = 0) {
-    return p == 0 ? 1 : ifft_span(M, p - 1, v) * ifft_radix(M, p - 1, v);
-}
-__host__ __device__ constexpr int dir_radix(int M, bool inv, int p, int v = 0) { return inv ? ifft_radix(M, p, v) : fft_radix(M, p, v); }
-__host__ __device__ constexpr int dir_span(int M, bool inv, int p, int v = 0) { return inv ? ifft_span(M, p, v) : fft_span(M, p, v); }
+// NS_p = R_1 .. R_{p-1}: frequency digits before pass p (0-based); L_p = M / (R_1 .. R_p)
+__host__ __device__ constexpr int fft_span(int M, int p) { return p == 0 ? 1 : fft_span(M, p - 1) * fft_radix(M, p - 1); }
+__host__ __device__ constexpr int fft_left(int M, int p) { return M / (fft_span(M, p) * fft_radix(M, p)); }
 
-// Twiddle tables, one per pass p >= 1 of each direction: entry [r][k] (r < R, k < Ns) holds
-// w_{Ns R}^{r k} (forward roots; the inverse multiplies by their conjugates).  k is the fast index, so
-// the adjacent butterflies of a thread and of neighbouring lanes read adjacent entries.  Offsets in float2.
-__host__ __device__ constexpr int tw_off(int M, bool inv, int p, int v = 0) {
+// Tables (float2).  Passes p >= 1: entry [i][k] (k < NS_p) = w_{NS_p R_p}^{r_i k} for the roots r_i = 1, 2, 3, 4, 8, 12
+// below R_p; every other power is one product of two of these (twiddles()).  (Loading every power, in doubled form,
+// costs the shared-memory / L1 pipe four cycles per load and warp: 2300 of 9400 such cycles a tile at M = 1024, on the
+// busiest pipe of these kernels.)  Then w_N^k for k <= S / 2.
+__host__ __device__ constexpr int tw_roots(int R) { return 2 + R / 4; }
+__host__ __device__ constexpr int tw_root(int i) { return i < 3 ? i + 1 : 4 * (i - 2); }
+__host__ __device__ constexpr int tw_off(int M, int p) {
     int off = 0;
-    if (inv)
-        for (int q = 1; q < fft_npass(M); ++q) off += fft_span(M, q, v) * fft_radix(M, q, v);
-    for (int q = 1; q < p; ++q) off += dir_span(M, inv, q, v) * dir_radix(M, inv, q, v);
+    for (int q = 1; q < p; ++q) off += tw_roots(fft_radix(M, q)) * fft_span(M, q);
     return off;
 }
-__host__ __device__ constexpr int tw_size(int M, int v = 0) { return tw_off(M, true, fft_npass(M), v); }
+__host__ __device__ constexpr int twn_off(int M) { return tw_off(M, fft_npass(M)); }
+__host__ __device__ constexpr int tw_size(int M) { return twn_off(M) + M / 16 + 1; }
+// the angle of entry i of the tables, as the fraction num / den of a full turn (w = exp(-2 pi i num / den))
+__host__ __device__ inline void tw_angle(int M, int i, int &num, int &den) {
+    num = i - twn_off(M);
+    den = 2 * M;
+    for (int p = 1; p < fft_npass(M); ++p) {
+        const int off = tw_off(M, p), NS = fft_span(M, p), R = fft_radix(M, p);
+        if (i >= off && i < off + tw_roots(R) * NS) {
+            const int root = (i - off) / NS;
+            num = tw_root(root) * ((i - off) % NS);
+            den = NS * R;
+        }
+    }
+}
 
-// Shared-memory layout of one trace: element i at float2 index i + 2 (i / 16).  The padding keeps
-// every pair (2m, 2m+1) 16-byte aligned and makes the 128-bit accesses of the passes bank-conflict
-// free; for the index patterns below the padded address splits into a per-thread base plus a
-// compile-time offset.
-__host__ __device__ constexpr int padi(int i) { return i + 2 * (i >> 4); }
+// z[r] *= w^r (INV: conj(w)^r), r = 1 .. R - 1, with the root w^{tw_root(i)} at tw[i NS]
+template <int R, int NS, bool INV>
+__device__ __forceinline__ void twiddles(C2 *z, const float2 *__restrict__ tw) {
+    const W2 w1 = ldtw(tw), w2 = ldtw(tw + NS), w3 = ldtw(tw + 2 * NS);
+    z[1] = ctw2<INV>(z[1], w1);
+    z[2] = ctw2<INV>(z[2], w2);
+    z[3] = ctw2<INV>(z[3], w3);
+#pragma unroll
+    for (int i = 1; i < R / 4; ++i) {
+        const W2 w = ldtw(tw + (2 + i) * NS);
+        z[4 * i] = ctw2<INV>(z[4 * i], w);
+        z[4 * i + 1] = ctw2<INV>(z[4 * i + 1], wmul(w, w1));
+        z[4 * i + 2] = ctw2<INV>(z[4 * i + 2], wmul(w, w2));
+        z[4 * i + 3] = ctw2<INV>(z[4 * i + 3], wmul(w, w3));
+    }
+}
 
-// Launch geometry of the trace kernels for complex length M: a team of T = M/16 threads per trace,
-// TR traces per CTA.  The defaults can be overridden at compile time for tuning sweeps.
-#ifndef SMDD_FFT_TRACES
-#define SMDD_FFT_TRACES 8
+// Launch geometry for complex length M: T = M/16 threads per pair of traces, PL pairs interleaved in the lanes,
+// G such groups in a CTA (4 for the lengths whose group is at most a warp: with one, the CTA's fixed work -- the
+// loss reduction and its atomic above all -- costs a third of the residual step at nt 30 to 128).
+#ifndef SMDD_FFT_MINB_1024
+#define SMDD_FFT_MINB_1024 2
 #endif
-#ifndef SMDD_FFT_MINB
-#define SMDD_FFT_MINB 3
+#ifndef SMDD_FFT_MINB_1536
+#define SMDD_FFT_MINB_1536 1
 #endif
-#ifndef SMDD_FFT_MINB_LARGE          // the same for M >= 1024 (teams of 64 threads or more)
-#define SMDD_FFT_MINB_LARGE SMDD_FFT_MINB
-#endif
-#ifndef SMDD_FFT_MIN_TR              // fewest traces per CTA for M <= 1024
-#define SMDD_FFT_MIN_TR 2
-#endif
-#ifndef SMDD_FFT_TR_2048             // traces per CTA at M = 2048 (teams of 128 threads)
-#define SMDD_FFT_TR_2048 8
-#endif
-#ifndef SMDD_FFT_TR_1536             // traces per CTA at M = 1536 (teams of 96 threads; 8 measured 1.2x
-#define SMDD_FFT_TR_1536 8           // faster than 4 on the update at nt 1500, 1200 x 200)
-#endif
-#ifndef SMDD_FFT_NAMED_BAR           // 1: teams of more than one warp sync on their own named barrier
-#define SMDD_FFT_NAMED_BAR 1
+#ifndef SMDD_FFT_PL_1536
+#define SMDD_FFT_PL_1536 4
 #endif
 
 template <int M>
 struct Team {
-    static constexpr int P = FFT_P;
-    static constexpr int T = M / P;                           // threads per trace
-    static constexpr int TR_RAW = SMDD_FFT_TRACES * 512 / M;  // SMDD_FFT_TRACES traces per CTA at M = 512
-    // traces per CTA: a CTA moves TR consecutive traces x 8 bytes of each frequency row of the
-    // spectra, so small TR wastes sectors; at M = 2048 the CTA takes as many traces as 1024 threads
-    // hold (8: 64-byte rows; measured 1.5x faster than 2 traces despite 64 registers per thread), else
-    // at least SMDD_FFT_MIN_TR; at most 1024 threads
-    static constexpr int TR_MIN = M == 2048 ? SMDD_FFT_TR_2048 : M == 1536 ? SMDD_FFT_TR_1536 : SMDD_FFT_MIN_TR;
-    static constexpr int TR_LO = TR_RAW < TR_MIN ? TR_MIN : TR_RAW;
-    static constexpr int TR = T * TR_LO > 1024 ? 1024 / T : TR_LO;
-    static constexpr int THREADS = T * TR;                    // CTA size
-    // float2 per trace buffer: padi(M) is a multiple of 16; the extra 16/TR float2 make the TR traces x
-    // 16/TR bins that a half-warp touches in the tile loads / stores fall on 16 distinct bank pairs
-    static constexpr int STRIDE = padi(M) + (TR >= 8 ? 2 : 16 / TR);
-    static constexpr size_t SMEM = (size_t)TR * STRIDE * sizeof(float2);
-    static_assert(T <= 32 || TR <= 15, "at most 15 named team barriers");
-    // resident CTAs per SM asked of the compiler: never below ~80 registers per thread
-    static constexpr int MINB_ASK = M >= 1024 ? SMDD_FFT_MINB_LARGE : SMDD_FFT_MINB;
-    static constexpr int MINB = (768 / THREADS) < 1 ? 1 : ((768 / THREADS) < MINB_ASK ? 768 / THREADS : MINB_ASK);
+    static constexpr int T = M / FFT_P;
+    static constexpr int PL = M == 4096 ? 2 : M == 1536 ? SMDD_FFT_PL_1536 : 4;
+    static constexpr int GT = PL * T;                    // threads of a group
+    static constexpr int G = M <= 128 ? 4 : 1;           // groups in a CTA
+    static constexpr int THREADS = GT * G;
+    static constexpr int TR = 2 * PL * G;                // traces in a CTA
+    static constexpr int R1 = fft_radix(M, 0), L1 = M / R1;
+    static constexpr int ELEMS = R1 * (L1 + 1);          // elements of a pair's buffer (padded)
+    static constexpr size_t SMEM = (size_t)ELEMS * PL * G * 16;
+    // resident CTAs per SM asked of the compiler: at most 128 registers per thread
+    static constexpr int MINB = M == 1024 ? SMDD_FFT_MINB_1024
+                              : M == 1536 ? SMDD_FFT_MINB_1536
+                              : THREADS >= 512 ? 1 : 512 / THREADS;
 };
 
-// Synchronise the T threads of one trace's team (team k = threads [kT, (k+1)T) of the CTA).  Every
-// thread of a team reaches the same sequence of team syncs.
-template <int T>
-__device__ __forceinline__ void team_sync() {
-    if constexpr (T <= 32) {
-        __syncwarp();
-    } else if constexpr (SMDD_FFT_NAMED_BAR) {
-        static_assert(T % 32 == 0, "named barriers count whole warps");
-        // barrier 0 is __syncthreads; teams use 1..TR (TR <= 15 for every team size here)
-        asm volatile("bar.sync %0, %1;\n" ::"r"(1 + (int)(threadIdx.x / T)), "n"(T) : "memory");
-    } else {
-        __syncthreads();
+// Synchronise the threads of a group (a group lies in one warp, or the CTA is one group).
+template <int M>
+__device__ __forceinline__ void group_sync() {
+    static_assert(Team<M>::GT <= 32 || Team<M>::G == 1, "no barrier for several groups of more than a warp");
+    if constexpr (Team<M>::GT <= 32) __syncwarp();
+    else __syncthreads();
+}
+
+// mixing of the low bits of jj (and of the digit of the last pass): lanes whose jj differ by 1 or by 2 fall on
+// different 16-byte columns of a quarter-warp's access
+template <int PL>
+__host__ __device__ __forceinline__ constexpr int mix(int i) {
+    return PL == 4 ? (i ^ ((i >> 1) & 1)) : (i ^ ((i >> 2) & 1));
+}
+// offset of the digits k_1 .. k_p (kk = k_1 + R_1 k_2 + ...)
+template <int M>
+__device__ __forceinline__ int digit_off(int kk, int p) {
+    constexpr int R1 = fft_radix(M, 0), L1 = M / R1;
+    if (p == 1) return kk * (L1 + 1);
+    int o = (kk % R1) * (L1 + 1);
+    kk /= R1;
+    for (int q = 1; q < p; ++q) {
+        o += (kk % fft_radix(M, q)) * fft_left(M, q);
+        kk /= fft_radix(M, q);
+    }
+    return o;
+}
+// first-pass butterfly q of thread s: pairs of adjacent jj (one butterfly when R_1 = 16)
+template <int M>
+__device__ __forceinline__ int first_jj(int s, int q) {
+    return Team<M>::R1 == 16 ? s : 2 * s + (q & 1) + 2 * Team<M>::T * (q >> 1);
+}
+
+// ------------------------------------------------------------------------------------------------
+// passes between registers and shared memory (buf: the group's buffer, offset by the pair)
+// ------------------------------------------------------------------------------------------------
+// first forward pass: a[q R1 + r] holds z[first_jj(q) + r L1] for r < R1 / 2 (the upper half is the zero
+// padding, not read)
+template <int M>
+__device__ __forceinline__ void fwd_first(C2 (&a)[FFT_P], float4 *buf, int s) {
+    constexpr int R = Team<M>::R1, L = Team<M>::L1, PL = Team<M>::PL;
+#pragma unroll
+    for (int q = 0; q < FFT_P / R; ++q) {
+        dftRp<R, false, true>(&a[q * R]);
+        float4 *b = buf + mix<PL>(first_jj<M>(s, q)) * PL;
+#pragma unroll
+        for (int r = 0; r < R; ++r) stsC(b + r * (L + 1) * PL, a[q * R + r]);
     }
 }
 
-__device__ __forceinline__ float4 lds4(const float2 *p) { return *reinterpret_cast<const float4 *>(p); }
-__device__ __forceinline__ void sts4(float2 *p, float2 lo, float2 hi) {
-    *reinterpret_cast<float4 *>(p) = make_float4(lo.x, lo.y, hi.x, hi.y);
-}
-
-// Register convention for a pass of radix R: thread t owns the butterflies j = 2t + e + 2T qq
-// (e in {0,1}, qq < 8/R); a[(2 qq + e) R + r] holds element j + r M/R of the pass input.
-
-template <int M, int R>
-__device__ __forceinline__ void pass_load(const float2 *buf, int t, float2 (&a)[FFT_P]) {
-    constexpr int T = M / FFT_P, QQ = FFT_P / R / 2, S = M / R;
-    const float2 *b = buf + padi(2 * t);
+// last inverse pass: a[q R1 + r] = z[first_jj(q) + r L1], of which the caller uses r < R1 / 2
+template <int M>
+__device__ __forceinline__ void inv_last(C2 (&a)[FFT_P], const float4 *buf, int s) {
+    constexpr int R = Team<M>::R1, L = Team<M>::L1, PL = Team<M>::PL;
 #pragma unroll
-    for (int qq = 0; qq < QQ; ++qq)
+    for (int q = 0; q < FFT_P / R; ++q) {
+        const float4 *b = buf + mix<PL>(first_jj<M>(s, q)) * PL;
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const float4 v = lds4(b + padi(2 * T * qq + r * S));
-            a[(2 * qq) * R + r] = make_float2(v.x, v.y);
-            a[(2 * qq + 1) * R + r] = make_float2(v.z, v.w);
-        }
-}
-
-// Twiddle powers w^r, r < R, from the loaded w^1 (and w^4 when R = 8): at most three dependent
-// complex products per power (a few ulp), instead of one table load per power.
-template <int R>
-__device__ __forceinline__ void twiddle_powers(float2 w1, float2 w4, float2 (&w)[R]) {
-    w[0] = make_float2(1.f, 0.f);
-    w[1] = w1;
-    if constexpr (R >= 4) {
-        w[2] = cmul(w1, w1);
-        w[3] = cmul(w[2], w1);
-    }
-    if constexpr (R == 8) {
-        w[4] = w4;
-        w[5] = cmul(w4, w1);
-        w[6] = cmul(w4, w[2]);
-        w[7] = cmul(w4, w[3]);
+        for (int r = 0; r < R; ++r) a[q * R + r] = ldsC(b + r * (L + 1) * PL);
+        dftRp<R, true, false>(&a[q * R]);
     }
 }
 
-template <int M, int R, int NS, bool INV, int TWOFF>
-__device__ __forceinline__ void pass_compute(float2 (&a)[FFT_P], int t, const float2 *__restrict__ tw) {
-    constexpr int T = M / FFT_P, QQ = FFT_P / R / 2;
+// middle pass p, in place (a length whose butterflies do not divide by the threads has a partial last round)
+template <int M, bool INV, int p>
+__device__ __forceinline__ void mid_pass(float4 *buf, int s, const float2 *__restrict__ tw) {
+    constexpr int R = fft_radix(M, p), L = fft_left(M, p), NS = fft_span(M, p), T = Team<M>::T, PL = Team<M>::PL;
+    constexpr int NB = M / R, NQ = (NB + T - 1) / T;
+    static_assert(T % L == 0 && L % 4 == 0, "every round of a thread has the same jj");
+    const int jj = s % L;
 #pragma unroll
-    for (int qq = 0; qq < QQ; ++qq) {
-        if constexpr (NS > 1) {
-            // butterflies j and j+1 use twiddle columns k0 and k0+1, adjacent in each row of the table
-            // (NS is even, so j and j+1 share the block of NS)
-            const int k0 = is_pow2c(NS) ? ((2 * t + 2 * T * qq) & (NS - 1)) : ((2 * t + 2 * T * qq) % NS);
-            const float4 v1 = __ldg(reinterpret_cast<const float4 *>(tw + TWOFF + 1 * NS + k0));
-            float4 v4 = v1;
-            if constexpr (R == 8) v4 = __ldg(reinterpret_cast<const float4 *>(tw + TWOFF + 4 * NS + k0));
-            // one butterfly's powers at a time: half the twiddle registers live at once
+    for (int q = 0; q < NQ; ++q) {
+        if (NB % T == 0 || s + T * q < NB) {
+            const int kk = s / L + q * (T / L);
+            float4 *b = buf + (mix<PL>(jj) + digit_off<M>(kk, p)) * PL;
+            const float2 *w = tw + tw_off(M, p) + kk;
+            C2 x[R];
 #pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                float2 w[R];
-                twiddle_powers<R>(e ? make_float2(v1.z, v1.w) : make_float2(v1.x, v1.y),
-                                  e ? make_float2(v4.z, v4.w) : make_float2(v4.x, v4.y), w);
-#pragma unroll
-                for (int r = 1; r < R; ++r) {
-                    float2 &x = a[(2 * qq + e) * R + r];
-                    x = INV ? cmulc(x, w[r]) : cmul(x, w[r]);
-                }
+            for (int r = 0; r < R; ++r) x[r] = ldsC(b + r * L * PL);
+            if constexpr (!INV) {
+                twiddles<R, NS, false>(x, w);
+                dftRp<R, false, false>(x);
+            } else {
+                dftRp<R, true, false>(x);
+                twiddles<R, NS, true>(x, w);
             }
+#pragma unroll
+            for (int r = 0; r < R; ++r) stsC(b + r * L * PL, x[r]);
         }
-        dftR<R, INV>(&a[(2 * qq) * R]);
-        dftR<R, INV>(&a[(2 * qq + 1) * R]);
     }
 }
 
-template <int M, int R, int NS>
-__device__ __forceinline__ void pass_store(float2 *buf, int t, const float2 (&a)[FFT_P]) {
-    constexpr int T = M / FFT_P, QQ = FFT_P / R / 2;
-    if constexpr (!is_pow2c(NS)) {
-        static_assert((2 * T) % NS == 0, "the butterflies j0 + 2T qq share the residue of j0");
-        // spans with a factor 3: the padded index of every store is formed in full (the per-thread base
-        // plus immediate split needs power-of-two blocks); pairs stay 16-byte aligned (j even, NS even)
-        const int j0 = 2 * t, k = j0 % NS;
-#pragma unroll
-        for (int qq = 0; qq < QQ; ++qq) {
-            const int o = (j0 + 2 * T * qq - k) * R + k;   // j0 + 2T qq has the same residue k (2T % NS == 0)
-#pragma unroll
-            for (int r = 0; r < R; ++r) sts4(buf + padi(o + r * NS), a[(2 * qq) * R + r], a[(2 * qq + 1) * R + r]);
-        }
-    } else if constexpr (NS == 1) {
-        float2 *b = buf + padi(2 * t * R);
-#pragma unroll
-        for (int qq = 0; qq < QQ; ++qq)
-#pragma unroll
-            for (int e = 0; e < 2; ++e)
-#pragma unroll
-                for (int r = 0; r < R; r += 2)
-                    sts4(b + padi(e * R + 2 * T * R * qq + r), a[(2 * qq + e) * R + r], a[(2 * qq + e) * R + r + 1]);
-    } else if constexpr (NS <= 2 * T) {
-        float2 *b = buf + padi((2 * t - ((2 * t) & (NS - 1))) * R + ((2 * t) & (NS - 1)));
-#pragma unroll
-        for (int qq = 0; qq < QQ; ++qq)
-#pragma unroll
-            for (int r = 0; r < R; ++r)
-                sts4(b + padi(2 * T * R * qq + r * NS), a[(2 * qq) * R + r], a[(2 * qq + 1) * R + r]);
-    } else {
-        float2 *b = buf + padi(2 * t);
-#pragma unroll
-        for (int qq = 0; qq < QQ; ++qq)
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const int c = (2 * T * qq - ((2 * T * qq) % NS)) * R + ((2 * T * qq) % NS) + r * NS;
-                sts4(b + padi(c), a[(2 * qq) * R + r], a[(2 * qq + 1) * R + r]);
-            }
+template <int M, bool INV, int p>
+__device__ __forceinline__ void mid_passes(float4 *buf, int s, const float2 *__restrict__ tw) {
+    // forward: p = 1 .. npass - 2; inverse: p = npass - 2 .. 1; a barrier after each
+    if constexpr (p >= 1 && p <= fft_npass(M) - 2) {
+        mid_pass<M, INV, p>(buf, s, tw);
+        group_sync<M>();
+        mid_passes<M, INV, INV ? p - 1 : p + 1>(buf, s, tw);
     }
 }
 
-// A radix-3 pass of span NS, shared memory to shared memory (never the first or last pass of a plan, so
-// no register hand-over): butterfly j reads j + r M/3, applies w_{3 NS}^{r (j % NS)} (table rows 1 and 2),
-// transforms and stores at (j - j % NS) 3 + j % NS + r NS.  Team syncs between the loads and the stores
-// and at the end.
+// ------------------------------------------------------------------------------------------------
+// edge passes: radix 8 with the real-signal processing
+// ------------------------------------------------------------------------------------------------
+// Z[k], Z[M-k] (in x, y) from X[k], X[M-k] and w = w_N^k: Z = E + i O, E = X[k] + conj X[M-k],
+// O = (X[k] - conj X[M-k]) conj(w); Z[M-k] = conj(E - i O)
+__device__ __forceinline__ void real_pre(C2 &x, C2 &y, W2 w) {
+    const f32x2 er = add2(x.re, y.re), ei = sub2(x.im, y.im), dr = sub2(x.re, y.re), di = add2(x.im, y.im);
+    const f32x2 o_re = fma2(di, w.im, mul2(dr, w.re)), o_im = fma2(dr, neg2(w.im), mul2(di, w.re));
+    x = C2{sub2(er, o_im), add2(ei, o_re)};
+    y = C2{add2(er, o_im), sub2(o_re, ei)};
+}
+// X[k], X[M-k] (in x, y) from Z[k], Z[M-k] and w = w_N^k: with e = (Z[k] + conj Z[M-k]) / 2,
+// g = w (Z[k] - conj Z[M-k]) / 2: X[k] = e - i g, X[M-k] = conj(e + i g)
+__device__ __forceinline__ void real_post(C2 &x, C2 &y, W2 w) {
+    const f32x2 hf = dup2(0.5f), nhf = dup2(-0.5f);
+    const f32x2 er = add2(x.re, y.re), ei = sub2(x.im, y.im), dr = sub2(x.re, y.re), di = add2(x.im, y.im);
+    const f32x2 g_im = fma2(dr, w.im, mul2(di, w.re)), ng_re = fma2(di, w.im, mul2(dr, neg2(w.re)));
+    const f32x2 e2 = mul2(er, hf), g2 = mul2(ng_re, hf);
+    x = C2{fma2(g_im, hf, e2), fma2(ei, hf, g2)};
+    y = C2{fma2(g_im, nhf, e2), fma2(ei, nhf, g2)};
+}
+
+// The bins of thread s: A[r] = bin s + r S and B[r] = bin S - s + r S (S/2 + r S for s = 0), r < 8, S = M / 8; for
+// s = 0 also bin M (its real part goes to `nyq`).
 //
-// The M/3 butterflies go to the TA = pass3_threads(M) first threads of the team, j = t + TA q (q < M/(3 TA)),
-// TA a multiple of 16 that divides M/3 and NS | TA: every thread then has the same count, j % NS = t % NS
-// for all its butterflies (one pair of twiddles per pass), and its shared-memory offsets are per-thread
-// bases plus compile-time constants.  (At M = 1536: 64 of the 96 threads, 8 butterflies each.)
-__host__ __device__ constexpr int pass3_threads(int M, int NS) {
-    int best = 0;
-    for (int ta = 16; ta <= M / FFT_P; ta += 16)
-        if ((M / 3) % ta == 0 && ta % NS == 0) best = ta;
-    return best;
-}
-
-template <int M, bool INV, int NS, int TWOFF>
-__device__ __forceinline__ void pass3_smem(float2 *buf, int t, const float2 *__restrict__ tw) {
-    constexpr int T = M / FFT_P, NBF = M / 3;
-    constexpr int TA = pass3_threads(M, NS);
-    if constexpr (TA > 0 && NS % 16 == 0) {
-        // spans that are multiples of 16: every offset below splits as padi(base) + padi(constant)
-        constexpr int NQ = NBF / TA;
-        if (t < TA) {
-            const int k = t % NS;
-            float2 w1 = make_float2(1.f, 0.f), w2 = w1;
-            if constexpr (NS > 1) {
-                w1 = __ldg(tw + TWOFF + NS + k);
-                w2 = __ldg(tw + TWOFF + 2 * NS + k);
-            }
-            const float2 *src = buf + padi(t);
-            float2 x[NQ][3];
-#pragma unroll
-            for (int q = 0; q < NQ; ++q)
-#pragma unroll
-                for (int r = 0; r < 3; ++r) x[q][r] = src[padi(TA * q + r * NBF)];
-            team_sync<T>();
-            float2 *dst = buf + padi((t - k) * 3 + k);
-#pragma unroll
-            for (int q = 0; q < NQ; ++q) {
-                if constexpr (NS > 1) {
-                    x[q][1] = INV ? cmulc(x[q][1], w1) : cmul(x[q][1], w1);
-                    x[q][2] = INV ? cmulc(x[q][2], w2) : cmul(x[q][2], w2);
-                }
-                dft3<INV>(x[q][0], x[q][1], x[q][2]);
-#pragma unroll
-                for (int r = 0; r < 3; ++r) dst[padi(3 * TA * q + r * NS)] = x[q][r];
-            }
-        } else {
-            team_sync<T>();
-        }
-        team_sync<T>();
-    } else if constexpr (TA > 0) {
-        // spans below 16 (NS | 16): the store offset (j - k) 3 + k + r NS has three per-thread bases
-        constexpr int NQ = NBF / TA;
-        if (t < TA) {
-            const int k = t % NS;
-            float2 w1 = make_float2(1.f, 0.f), w2 = w1;
-            if constexpr (NS > 1) {
-                w1 = __ldg(tw + TWOFF + NS + k);
-                w2 = __ldg(tw + TWOFF + 2 * NS + k);
-            }
-            const float2 *src = buf + padi(t);
-            float2 x[NQ][3];
-#pragma unroll
-            for (int q = 0; q < NQ; ++q)
-#pragma unroll
-                for (int r = 0; r < 3; ++r) x[q][r] = src[padi(TA * q + r * NBF)];
-            team_sync<T>();
-            const int o = (t - k) * 3 + k;   // 3 TA q is a multiple of 16: padi(o + r NS + 3 TA q) = padi(o + r NS) + padi(3 TA q)
-            float2 *d0 = buf + padi(o), *d1 = buf + padi(o + NS), *d2 = buf + padi(o + 2 * NS);
-#pragma unroll
-            for (int q = 0; q < NQ; ++q) {
-                if constexpr (NS > 1) {
-                    x[q][1] = INV ? cmulc(x[q][1], w1) : cmul(x[q][1], w1);
-                    x[q][2] = INV ? cmulc(x[q][2], w2) : cmul(x[q][2], w2);
-                }
-                dft3<INV>(x[q][0], x[q][1], x[q][2]);
-                d0[padi(3 * TA * q)] = x[q][0];
-                d1[padi(3 * TA * q)] = x[q][1];
-                d2[padi(3 * TA * q)] = x[q][2];
-            }
-        } else {
-            team_sync<T>();
-        }
-        team_sync<T>();
+// inverse: A, B hold the spectrum; real pre-processing, radix-8 inverse butterflies, twiddles, store
+template <int M>
+__device__ __forceinline__ void edge_inv(C2 (&A)[8], C2 (&B)[8], f32x2 nyq, float4 *buf, int s, const float2 *__restrict__ tw) {
+    constexpr int S = M / 8, PL = Team<M>::PL, P = fft_npass(M) - 1;
+    const W2 wn = ldtw(tw + twn_off(M) + s);   // w_N^s
+    if (s != 0) {
+        real_pre(A[0], B[7], wn);
+        real_pre(A[1], B[6], rot16<1>(wn));
+        real_pre(A[2], B[5], rot16<2>(wn));
+        real_pre(A[3], B[4], rot16<3>(wn));
+        real_pre(A[4], B[3], rot16<4>(wn));
+        real_pre(A[5], B[2], rot16<5>(wn));
+        real_pre(A[6], B[1], rot16<6>(wn));
+        real_pre(A[7], B[0], rot16<7>(wn));
     } else {
-        // general case: butterfly j = t + T q, the last round partial
-        constexpr int NQ = (NBF + T - 1) / T;
-        float2 x[NQ][3];
+        // A: k = r S pairs with M - k = (8 - r) S; k = 0 with bin M (imaginary parts ignored), k = M/2 with itself
+        const f32x2 x0 = A[0].re;
+        A[0] = C2{add2(x0, nyq), sub2(x0, nyq)};
+        real_pre(A[1], A[7], rot16<1>(wn));
+        real_pre(A[2], A[6], rot16<2>(wn));
+        real_pre(A[3], A[5], rot16<3>(wn));
+        A[4] = C2{add2(A[4].re, A[4].re), neg2(add2(A[4].im, A[4].im))};
+        // B: k = S/2 + r S pairs with S/2 + (7 - r) S
+        const W2 wh = ldtw(tw + twn_off(M) + S / 2);
+        real_pre(B[0], B[7], wh);
+        real_pre(B[1], B[6], rot16<1>(wh));
+        real_pre(B[2], B[5], rot16<2>(wh));
+        real_pre(B[3], B[4], rot16<3>(wh));
+    }
+    const float2 *w = tw + tw_off(M, P);
 #pragma unroll
-        for (int q = 0; q < NQ; ++q) {
-            const int j = t + T * q;
-            if (j < NBF) {
+    for (int h = 0; h < 2; ++h) {
+        C2(&z)[8] = h ? B : A;
+        const int u = h ? (s ? S - s : S / 2) : s;
+        dft8p<true, false>(z);
+        twiddles<8, S, true>(z, w + u);
+        float4 *b = buf + digit_off<M>(u, P) * PL;
 #pragma unroll
-                for (int r = 0; r < 3; ++r) x[q][r] = buf[padi(j + r * NBF)];
-            }
-        }
-        team_sync<T>();
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) {
-            const int j = t + T * q;
-            if (j < NBF) {
-                const int k = j % NS;
-                if constexpr (NS > 1) {
-                    const float2 w1 = __ldg(tw + TWOFF + NS + k), w2 = __ldg(tw + TWOFF + 2 * NS + k);
-                    x[q][1] = INV ? cmulc(x[q][1], w1) : cmul(x[q][1], w1);
-                    x[q][2] = INV ? cmulc(x[q][2], w2) : cmul(x[q][2], w2);
-                }
-                dft3<INV>(x[q][0], x[q][1], x[q][2]);
-                const int o = (j - k) * 3 + k;
-#pragma unroll
-                for (int r = 0; r < 3; ++r) buf[padi(o + r * NS)] = x[q][r];
-            }
-        }
-        team_sync<T>();
+        for (int r = 0; r < 8; ++r) stsC(b + mix<PL>(r) * PL, z[r]);
     }
 }
 
-template <int M, bool INV, int p, int PEND, int V>
-__device__ __forceinline__ void passes_from(float2 (&a)[FFT_P], float2 *buf, int t, const float2 *__restrict__ tw) {
-    // passes p .. PEND-1 of a direction: load, compute, and (except for the last inverse pass) store
-    if constexpr (p < PEND) {
-        constexpr int R = dir_radix(M, INV, p, V), NS = dir_span(M, INV, p, V);
-        if constexpr (R == 3) {
-            static_assert(p > 0 && p + 1 < fft_npass(M), "the radix-3 pass sits inside the plan");
-            pass3_smem<M, INV, NS, tw_off(M, INV, p, V)>(buf, t, tw);
-        } else {
-            pass_load<M, R>(buf, t, a);
-            if constexpr (!INV) team_sync<M / FFT_P>();
-            pass_compute<M, R, NS, INV, tw_off(M, INV, p, V)>(a, t, tw);
-            if constexpr (!INV || p + 1 < fft_npass(M)) {
-                if constexpr (INV) team_sync<M / FFT_P>();
-                pass_store<M, R, NS>(buf, t, a);
-                team_sync<M / FFT_P>();
-            }
-        }
-        passes_from<M, INV, p + 1, PEND, V>(a, buf, t, tw);
+// forward: load, twiddles, radix-8 butterflies, real post-processing; on return A, B hold the spectrum, nyq the
+// real part of bin M for s = 0
+template <int M>
+__device__ __forceinline__ void edge_fwd(C2 (&A)[8], C2 (&B)[8], f32x2 &nyq, const float4 *buf, int s, const float2 *__restrict__ tw) {
+    constexpr int S = M / 8, PL = Team<M>::PL, P = fft_npass(M) - 1;
+    const float2 *w = tw + tw_off(M, P);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        C2(&z)[8] = h ? B : A;
+        const int u = h ? (s ? S - s : S / 2) : s;
+        const float4 *b = buf + digit_off<M>(u, P) * PL;
+#pragma unroll
+        for (int r = 0; r < 8; ++r) z[r] = ldsC(b + mix<PL>(r) * PL);
+        twiddles<8, S, false>(z, w + u);
+        dft8p<false, false>(z);
     }
-}
-
-// w_32^m = exp(-2 pi i m / 32), m in [0, 32): the roots used by the real-spectrum passes
-__device__ __forceinline__ float2 root32(int m) {
-    constexpr float c[9] = {1.0f, 0.98078528040323044913f, 0.92387953251128675613f, 0.83146961230254523708f,
-                            0.70710678118654752440f, 0.55557023301960222474f, 0.38268343236508977173f,
-                            0.19509032201612826785f, 0.0f};   // cos(pi m / 16), m = 0..8
-    m &= 31;
-    const int q = m >> 3, rr = m & 7;
-    float x = c[rr], y = c[8 - rr];        // cos, sin of the angle inside the quadrant
-    float cs, sn;
-    switch (q) {
-        case 0: cs = x; sn = y; break;
-        case 1: cs = -y; sn = x; break;
-        case 2: cs = -x; sn = -y; break;
-        default: cs = y; sn = -x; break;
+    const W2 wn = ldtw(tw + twn_off(M) + s);   // w_N^s
+    nyq = 0;
+    if (s != 0) {
+        real_post(A[0], B[7], wn);
+        real_post(A[1], B[6], rot16<1>(wn));
+        real_post(A[2], B[5], rot16<2>(wn));
+        real_post(A[3], B[4], rot16<3>(wn));
+        real_post(A[4], B[3], rot16<4>(wn));
+        real_post(A[5], B[2], rot16<5>(wn));
+        real_post(A[6], B[1], rot16<6>(wn));
+        real_post(A[7], B[0], rot16<7>(wn));
+    } else {
+        nyq = sub2(A[0].re, A[0].im);
+        A[0] = C2{add2(A[0].re, A[0].im), 0};
+        real_post(A[1], A[7], rot16<1>(wn));
+        real_post(A[2], A[6], rot16<2>(wn));
+        real_post(A[3], A[5], rot16<3>(wn));
+        A[4].im = neg2(A[4].im);
+        const W2 wh = ldtw(tw + twn_off(M) + S / 2);
+        real_post(B[0], B[7], wh);
+        real_post(B[1], B[6], rot16<1>(wh));
+        real_post(B[2], B[5], rot16<2>(wh));
+        real_post(B[3], B[4], rot16<3>(wh));
     }
-    return make_float2(cs, -sn);
-}
-
-// The butterflies of the last forward pass and of the first inverse pass (radix R, span M/R): thread t
-// owns the pairs u = t + T q (q < 8/R) and, for each, the butterflies ja = u and jb = M/R - u
-// (jb = M/(2R) for u = 0).  The bins k = ja + r M/R and M - k = jb + (R-1-r) M/R then lie in the same
-// thread, so the real-signal post- and pre-processing run in registers.
-template <int M, int V>
-struct EdgePass {
-    static constexpr int R = fft_radix(M, fft_npass(M) - 1, V);
-    static constexpr int S = M / R;     // span of the last forward pass = stride of its inputs
-    static constexpr int NP = 8 / R;    // pairs per thread
-};
-
-// Last forward pass + real post-processing.  Input: buf after the other forward passes.  Output: buf
-// holds X[1..M-1] in their slots and (X[0], X[M]) in slot 0.  Ends with a team sync.
-template <int M, int V>
-__device__ __forceinline__ void fwd_last_real(float2 (&a)[FFT_P], float2 *buf, int t, const float2 *__restrict__ tw,
-                                              const float2 *__restrict__ twN) {
-    constexpr int T = M / FFT_P, R = EdgePass<M, V>::R, S = EdgePass<M, V>::S, NP = EdgePass<M, V>::NP;
-    constexpr int TWOFF = tw_off(M, false, fft_npass(M) - 1, V);
-    int ja[NP], jb[NP];
-#pragma unroll
-    for (int q = 0; q < NP; ++q) {
-        const int u = t + T * q;
-        ja[q] = u;
-        jb[q] = u ? S - u : S / 2;
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            a[(2 * q) * R + r] = buf[padi(ja[q] + r * S)];
-            a[(2 * q + 1) * R + r] = buf[padi(jb[q] + r * S)];
-        }
-    }
-    team_sync<T>();
-#pragma unroll
-    for (int q = 0; q < NP; ++q) {
-        const int u = ja[q];
-        float2 *A = &a[(2 * q) * R], *B = &a[(2 * q + 1) * R];
-        // twiddles w_M^{r j}: ja from the table, jb = S - u from w_M^{r S} conj(w_M^{r u}) = w_R^r conj(.)
-        const float2 t1 = __ldg(tw + TWOFF + 1 * S + u);
-        const float2 t4 = (R == 8) ? __ldg(tw + TWOFF + 4 * S + u) : t1;
-        float2 wa[R];
-        twiddle_powers<R>(t1, t4, wa);
-#pragma unroll
-        for (int r = 1; r < R; ++r) {
-            A[r] = cmul(A[r], wa[r]);
-            const float2 wb = u ? cmul(root32(32 * r / R), cconj(wa[r])) : root32(16 * r / R);
-            B[r] = cmul(B[r], wb);
-        }
-        dftR<R, false>(A);
-        dftR<R, false>(B);
-        // X[k] = e - i w_N^k d, e = (Z[k] + conj Z[M-k]) / 2, d = (Z[k] - conj Z[M-k]) / 2; each bin goes to
-        // its slot as soon as it is formed (every load of this pass precedes the team sync above), so A
-        // and B are read-only here and no output array is held in registers
-        const float2 wn = __ldg(twN + u);   // w_N^u
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const float2 za = A[r], zma = u ? B[R - 1 - r] : A[(R - r) % R];
-            const float2 zb = B[r], zmb = u ? A[R - 1 - r] : B[R - 1 - r];
-            const float2 wka = cmul(wn, root32(16 * r / R));                                   // w_N^{u + r S}
-            const float2 wkb = u ? cmul(root32(16 * (r + 1) / R), cconj(wn)) : root32(8 / R + 16 * r / R);
-            const float2 pa = cmul(wka, cscale(csub(za, cconj(zma)), 0.5f));
-            const float2 pb = cmul(wkb, cscale(csub(zb, cconj(zmb)), 0.5f));
-            float2 xa = cadd(cscale(cadd(za, cconj(zma)), 0.5f), mul_mi<false>(pa));
-            const float2 xb = cadd(cscale(cadd(zb, cconj(zmb)), 0.5f), mul_mi<false>(pb));
-            if (r == 0 && u == 0) xa = make_float2(xa.x, A[0].x - A[0].y);   // slot 0: X[0], X[M] = Re Z[0] - Im Z[0]
-            buf[padi(ja[q] + r * S)] = xa;
-            buf[padi(jb[q] + r * S)] = xb;
-        }
-    }
-    team_sync<T>();
-}
-
-// First inverse pass with the real pre-processing: buf holds a real-signal spectrum (slot 0 = (X[0],
-// X[M])).  Forms Z[k] = E + i O, E = X[k] + conj X[M-k], O = (X[k] - conj X[M-k]) w_N^{-k}, applies the
-// radix-R inverse butterflies and stores the pass output.  Ends with a team sync.
-template <int M, int V>
-__device__ __forceinline__ void inv_first_real(float2 (&a)[FFT_P], float2 *buf, int t, const float2 *__restrict__ twN) {
-    constexpr int T = M / FFT_P, R = EdgePass<M, V>::R, S = EdgePass<M, V>::S, NP = EdgePass<M, V>::NP;
-    int ja[NP], jb[NP];
-#pragma unroll
-    for (int q = 0; q < NP; ++q) {
-        const int u = t + T * q;
-        ja[q] = u;
-        jb[q] = u ? S - u : S / 2;
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            a[(2 * q) * R + r] = buf[padi(ja[q] + r * S)];
-            a[(2 * q + 1) * R + r] = buf[padi(jb[q] + r * S)];
-        }
-    }
-    team_sync<T>();
-#pragma unroll
-    for (int q = 0; q < NP; ++q) {
-        const int u = ja[q];
-        float2 *A = &a[(2 * q) * R], *B = &a[(2 * q + 1) * R];
-        const float2 s0 = A[0];
-        const float2 xm0 = make_float2(s0.y, 0.f);   // X[M] when u == 0
-        if (u == 0) A[0] = make_float2(s0.x, 0.f);
-        const float2 wn = __ldg(twN + u);
-        float2 za[R], zb[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const float2 xa = A[r], xma = u ? B[R - 1 - r] : (r == 0 ? xm0 : A[(R - r) % R]);
-            const float2 xb = B[r], xmb = u ? A[R - 1 - r] : B[R - 1 - r];
-            const float2 wka = cmul(wn, root32(16 * r / R));
-            const float2 wkb = u ? cmul(root32(16 * (r + 1) / R), cconj(wn)) : root32(8 / R + 16 * r / R);
-            const float2 oa = cmulc(csub(xa, cconj(xma)), wka);   // times w_N^{-k}
-            const float2 ob = cmulc(csub(xb, cconj(xmb)), wkb);
-            za[r] = cadd(cadd(xa, cconj(xma)), mul_mi<true>(oa));   // E + i O
-            zb[r] = cadd(cadd(xb, cconj(xmb)), mul_mi<true>(ob));
-        }
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            A[r] = za[r];
-            B[r] = zb[r];
-        }
-        dftR<R, true>(A);
-        dftR<R, true>(B);
-#pragma unroll
-        for (int r = 0; r < R; r += 2) {
-            sts4(buf + padi(ja[q] * R + r), A[r], A[r + 1]);
-            sts4(buf + padi(jb[q] * R + r), B[r], B[r + 1]);
-        }
-    }
-    team_sync<T>();
-}
-
-// Forward real FFT of length 2M.  Input: registers in first-pass order (time samples).  Output: the
-// real-signal spectrum in buf (slot 0 = (X[0], X[M]), bins 1..M-1 in their slots, padded layout).  Ends
-// with a team sync.  No thread of the team may still read buf on entry.
-template <int M, int V>
-__device__ __forceinline__ void rfft_regs_to_smem(float2 (&a)[FFT_P], float2 *buf, int t, const float2 *__restrict__ tw,
-                                                  const float2 *__restrict__ twN) {
-    constexpr int R0 = fft_radix(M, 0, V);
-    pass_compute<M, R0, 1, false, 0>(a, t, tw);
-    pass_store<M, R0, 1>(buf, t, a);
-    team_sync<M / FFT_P>();
-    passes_from<M, false, 1, fft_npass(M) - 1, V>(a, buf, t, tw);
-    fwd_last_real<M, V>(a, buf, t, tw, twN);
-}
-
-// Inverse real FFT of length 2M (unnormalised: yields 2M x).  Input: real-signal spectrum in buf.
-// Output: registers in first-forward-pass order (time samples).  The last pass reads buf, so the caller
-// must sync the team before writing buf again.
-template <int M, int V>
-__device__ __forceinline__ void irfft_smem_to_regs(float2 (&a)[FFT_P], float2 *buf, int t, const float2 *__restrict__ tw,
-                                                   const float2 *__restrict__ twN) {
-    inv_first_real<M, V>(a, buf, t, twN);
-    passes_from<M, true, 1, fft_npass(M), V>(a, buf, t, tw);
-}
-
-// The same with `mid()` run after the first pass: a caller that needs time-domain inputs after the
-// transform issues their loads there, so they are not held in registers through the real
-// pre-processing (the pass with the most live values) but still overlap the remaining passes.
-//
-// Where the second inverse pass is the radix-3 pass (the one that holds the most values at once), mid()
-// runs after it instead.
-template <int M, int V>
-__host__ __device__ constexpr int irfft_mid_pass() {
-    return (fft_npass(M) > 2 && ifft_radix(M, 1, V) == 3) ? 2 : 1;
-}
-
-template <int M, int V, class F>
-__device__ __forceinline__ void irfft_smem_to_regs_mid(float2 (&a)[FFT_P], float2 *buf, int t, const float2 *__restrict__ tw,
-                                                       const float2 *__restrict__ twN, F &&mid) {
-    constexpr int MP = irfft_mid_pass<M, V>();
-    inv_first_real<M, V>(a, buf, t, twN);
-    passes_from<M, true, 1, MP, V>(a, buf, t, tw);
-    mid();
-    passes_from<M, true, MP, fft_npass(M), V>(a, buf, t, tw);
 }
 
 }  // namespace smdd

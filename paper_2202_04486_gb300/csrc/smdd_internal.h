@@ -29,12 +29,12 @@ struct TraceGrid {
 struct FftArgs {
     TraceGrid g;
     int nt;
-    int vec;                 // time traces may be accessed as float4 (nt % 4 == 0, 16-byte aligned base)
+    int vec;                 // time traces: 2 = 16-byte aligned quads (nt % 4 == 0), 1 = 8-byte aligned pairs
+                             // (nt % 2 == 0), 0 = neither (see time_vec)
     const float *tin;        // time input (rfft)
     float *tout;             // time output (irfft_out) / model in-out (update)
     float2 *spec;            // spectra (read and/or written)
-    const float2 *tw;        // per-pass twiddle tables (see tw_off)
-    const float2 *twN;       // exp(-2 pi i k / N), k <= M
+    const float2 *tw;        // twiddle tables of the passes and of the real-signal processing (see tw_off)
     float s;                 // epilogue factor scale / N
     float alpha;             // step size (update)
     // residual: observed rows, row(i) = gathered ? i : idx[i]
@@ -46,7 +46,6 @@ struct FftArgs {
     unsigned int *counter;
     double *loss;
     int *status;
-    int variant;             // FFT variant: 0 / 1 radix orders of fft_radix, 2 the two-pass FFT (smdd_fft2.cuh)
     // update: Nesterov velocity (null for SGD), momentum, causality mute (first kept sample per
     // model trace, [nv][nr]; null for none)
     float *vel;
@@ -56,7 +55,6 @@ struct FftArgs {
     // c1 = 1 / (1 - beta1^t), c2 = 1 / (1 - beta2^t) of step t
     float *adam_m, *adam_v;
     float beta1, beta2, eps, c1, c2;
-    int prefetch;            // update: persistent CTAs prefetching the next tile's spectra (M <= 1024)
 };
 
 struct GemmArgs {
@@ -124,34 +122,21 @@ cudaError_t launch_residual(int M, const FftArgs &a, int nblocks_expected, cudaS
 cudaError_t launch_update(int M, bool keep_xhat, const FftArgs &a, cudaStream_t st);
 int fft_blocks(int M, const TraceGrid &g);
 int fft_traces_per_cta(int M);
-bool fft_pf_supported(int M);   // the persistent prefetching update exists for complex length M
 cudaError_t fft_prepare(int M);                                // opt-in to the dynamic shared memory of size M
-int fft_tw_size(int M, int variant = 0);
-bool fft_has_variant(int M, int variant);                     // variant 1 exists where it differs from 0
-void fft_tw_fill(int M, std::vector<float2> &tw, int variant = 0);   // host: per-pass twiddle tables
+int fft_tw_size(int M);                                        // entries of the twiddle tables
+void fft_tw_fill(int M, std::vector<float2> &tw);              // host: the tables, rounded once from double
+// alignment class of time traces (FftArgs::vec): every trace starts on a 16-byte (2) or 8-byte (1) boundary
+inline int time_vec(int nt, const void *p) {
+    const uintptr_t u = reinterpret_cast<uintptr_t>(p);
+    return (nt % 4 == 0 && (u & 15u) == 0) ? 2 : (nt % 2 == 0 && (u & 7u) == 0) ? 1 : 0;
+}
 
-// register FFT kernels (radix-order variant 2: two passes for 128 <= M <= 1024, three for M = 1536;
-// fft2_kernels.cu)
-bool fft2_supported(int M);
-int fft2_traces_per_cta(int M);
-int fft2_blocks(int M, const TraceGrid &g);
-int fft2_tw_size(int M);                             // entries of the variant's twiddle tables
-void fft2_tw_fill(int M, std::vector<float2> &tw);   // host: the variant's twiddle tables
-cudaError_t fft2_prepare(int M);
-cudaError_t launch2_rfft(int M, const FftArgs &a, cudaStream_t st);
-cudaError_t launch2_irfft_out(int M, const FftArgs &a, cudaStream_t st);
-cudaError_t launch2_residual(int M, const FftArgs &a, int nblocks_expected, cudaStream_t st);
-cudaError_t launch2_update(int M, bool keep_xhat, const FftArgs &a, cudaStream_t st);
-
-// work-queue forms of the trace kernels (rfft, residual step, SGD update with the new model's spectra),
-// for FFT variant 0, 1 (radix orders) or 2 (register FFT): CTAs resident on every SM, each taking tiles
-// from the queue until it is empty.  Tile counts per member: fft_blocks / fft2_blocks of its grid.
-cudaError_t launch_queue_rfft(int M, int variant, const WorkQueue &q, cudaStream_t st);
-cudaError_t launch_queue_residual(int M, int variant, const WorkQueue &q, cudaStream_t st);
-cudaError_t launch_queue_update(int M, int variant, const WorkQueue &q, cudaStream_t st);
-cudaError_t launch2_queue_rfft(int M, const WorkQueue &q, cudaStream_t st);
-cudaError_t launch2_queue_residual(int M, const WorkQueue &q, cudaStream_t st);
-cudaError_t launch2_queue_update(int M, const WorkQueue &q, cudaStream_t st);
+// work-queue forms of the trace kernels (rfft, residual step, SGD update with the new model's spectra): CTAs
+// resident on every SM, each taking tiles from the queue until it is empty.  Tile counts per member: fft_blocks
+// of its grid.
+cudaError_t launch_queue_rfft(int M, const WorkQueue &q, cudaStream_t st);
+cudaError_t launch_queue_residual(int M, const WorkQueue &q, cudaStream_t st);
+cudaError_t launch_queue_update(int M, const WorkQueue &q, cudaStream_t st);
 
 cudaError_t launch_cgemm_fwd(const GemmArgs &a, int nf, cudaStream_t st);
 cudaError_t launch_cgemm_adj(const GemmArgs &a, bool recip, int nf, cudaStream_t st, int tile = 0);
@@ -193,11 +178,11 @@ struct PlanShape {
 // argument records with their tile counts, for the work-queue epochs: the model transform (used on the
 // first step only), the forward product on the tensor-core tile kernel with batch block fwd_nb, the
 // residual step, the adjoint product (tile kernel, reciprocity flag) and the update.  The trace kernels
-// run FFT variant `variant` of complex length M.  Returns MDC_ERR_UNSUPPORTED unless the plan's products
+// have complex length M.  Returns MDC_ERR_UNSUPPORTED unless the plan's products
 // run on the tensor cores (MDC_PREC_BF16X3 with MDC_GEMM_TC or MDC_GEMM_TC_STREAM forward and
 // MDC_GEMM_TC adjoint) and no band limit is set.
 struct StepRecords {
-    int M, variant;
+    int M;
     FftArgs rfft;
     int rfft_tiles;
     GemmArgs fwd;
