@@ -14,6 +14,9 @@ using namespace smdd;
 
 namespace {
 
+constexpr int SPEC_FL2 = 2;
+static_assert(SPEC_F == 1 << SPEC_FL2, "SPEC_F is a power of two");
+
 struct PendingTiming {
     int stage;
     cudaEvent_t e0, e1;
@@ -31,9 +34,8 @@ struct DeviceGuard {
     }
 };
 
-// Row length of the spectra for n traces: even (pairs of traces are 16-byte aligned); from 16 traces on a multiple
-// of 4 and from 64 on of 8, so that the 64-byte segments of the trace kernels' tiles start on whole sectors (at
-// most 11 % more memory; nr 301: 15 % less DRAM traffic of the update than with rows of 302)
+// Row length of the kernel spectra for n receivers: even (pairs of traces are 16-byte aligned); from 16 traces on a multiple
+// of 4 and from 64 on of 8, so that rows start on whole sectors (at most 11 % more memory from 64 on)
 int padded_ld(int n) {
     const int m = n >= 64 ? 8 : n >= 16 ? 4 : 2;
     return (n + m - 1) / m * m;
@@ -63,12 +65,12 @@ int default_nfft(int nt) {
 struct mdc_plan_s {
     int device = 0;
     int nt = 0, nr = 0, nv = 0, ns = 0, nbmax = 0, nfft = 0, M = 0, nf = 0;
-    int ldr = 0, ldb = 0;
+    int ldr = 0, ldb = 0, ldd = 0;   // columns per row of the model, batch and kernel spectra
     int prec = MDC_PREC_FP32;
     float scale = 1.f;
-    float2 *Dh = nullptr;        // [nf][ns][ldr]
-    float2 *Xh = nullptr;        // [nf][nv][ldr]  model spectra, reused for gradient spectra
-    float2 *Uh = nullptr;        // [nf][nv][ldb]  batch spectra (prediction, then residual)
+    float2 *Dh = nullptr;        // [nf][ns][ldd]
+    float2 *Xh = nullptr;        // model spectra, reused for gradient spectra (rows of ldr, SPEC_F layout)
+    float2 *Uh = nullptr;        // batch spectra (prediction, then residual; rows of ldb, SPEC_F layout)
     uint8_t *adj_img = nullptr;  // split-BF16 plans: operand images of the adjoint products (null: not held)
     float2 *tw = nullptr;        // twiddle tables of the trace kernels
     double *partials = nullptr;  // residual-kernel block partials
@@ -104,7 +106,7 @@ struct mdc_plan_s {
         cudaStream_t copy = nullptr;
         int next = 0;
     } *hs = nullptr;
-    alignas(64) unsigned char xh_map[128] = {0};   // tensor map of Xh for the streamed forward product
+    TcMaps maps;                 // tensor maps of Xh (split-BF16 plans)
     bool xh_map_ok = false;
     LsqrWork *lsqr = nullptr;    // full-gradient solver workspace, allocated by the first smdd_lsqr
 };
@@ -163,7 +165,7 @@ int ti_log2_for(int n_contig, int TR) {
 
 int traces_per_cta(const mdc_plan_s *p) { return fft_traces_per_cta(p->M); }
 
-// model-layout grid: trace (i = r, j = v) of a [nv][nr][nt] array  <->  spectra [nf][nv][ldr]
+// model-layout grid: trace (i = r, j = v) of a [nv][nr][nt] array  <->  its spectra (rows of ldr, SPEC_F layout)
 TraceGrid model_grid(const mdc_plan_s *p, int nouter) {
     TraceGrid g;
     g.ni = p->nr;
@@ -171,13 +173,22 @@ TraceGrid model_grid(const mdc_plan_s *p, int nouter) {
     g.ti_log2 = ti_log2_for(p->nr, traces_per_cta(p));
     g.tsi = p->nt;
     g.tsj = (long long)p->nr * p->nt;
-    g.ssi = 1;
-    g.ssj = p->ldr;
-    g.ssf = (long long)nouter * p->ldr;
+    g.fl2 = SPEC_FL2;
+    g.ssj = (long long)p->ldr * SPEC_F;
+    g.ssf = (long long)nouter * g.ssj;
     return g;
 }
 
-// batch-layout grid: trace (i = b, j = v) of a [nb][nv][nt] array  <->  spectra [nf][nv][ldb]
+// the same for the kernel spectra: [ns][nr][nt] <-> [nf][ns][ldd], rows of one bin contiguous
+TraceGrid kernel_grid(const mdc_plan_s *p) {
+    TraceGrid g = model_grid(p, p->ns);
+    g.fl2 = 0;
+    g.ssj = p->ldd;
+    g.ssf = (long long)p->ns * p->ldd;
+    return g;
+}
+
+// batch-layout grid: trace (i = b, j = v) of a [nb][nv][nt] array  <->  its spectra (rows of ldb, SPEC_F layout)
 TraceGrid batch_grid(const mdc_plan_s *p, int nb) {
     TraceGrid g;
     g.ni = nb;
@@ -185,9 +196,9 @@ TraceGrid batch_grid(const mdc_plan_s *p, int nb) {
     g.ti_log2 = ti_log2_for(nb, traces_per_cta(p));
     g.tsi = (long long)p->nv * p->nt;
     g.tsj = p->nt;
-    g.ssi = 1;
-    g.ssj = p->ldb;
-    g.ssf = (long long)p->nv * p->ldb;
+    g.fl2 = SPEC_FL2;
+    g.ssj = (long long)p->ldb * SPEC_F;
+    g.ssf = (long long)p->nv * g.ssj;
     return g;
 }
 
@@ -201,6 +212,15 @@ int rfft_model(mdc_plan_s *p, const float *X, cudaStream_t st) {
     return launch_stage(p, ST_RFFT, st, [&] { return launch_rfft(p->M, a, st); });
 }
 
+void set_shape(GemmArgs &g, const mdc_plan_s *p, int nb) {
+    g.nv = p->nv; g.nr = p->nr; g.ns = p->ns; g.nb = nb;
+    g.ldr = p->ldr; g.ldb = p->ldb; g.ldd = p->ldd;
+    g.sDf = (long long)p->ns * p->ldd;
+}
+
+// the split-BF16 forward products read the part of a symmetric model's spectra below the block diagonal transposed
+bool reads_transposed(const mdc_plan_s *p) { return p->gemm_fwd == MDC_GEMM_TC || p->gemm_fwd == MDC_GEMM_TC_STREAM; }
+
 int gemm_forward(mdc_plan_s *p, const int32_t *idx, int nb, cudaStream_t st) {
     GemmArgs g;
     memset(&g, 0, sizeof(g));
@@ -208,32 +228,32 @@ int gemm_forward(mdc_plan_s *p, const int32_t *idx, int nb, cudaStream_t st) {
     g.Dh = p->Dh;
     g.idx = idx;
     g.C = p->Uh;
-    g.nv = p->nv; g.nr = p->nr; g.ns = p->ns; g.nb = nb; g.ldr = p->ldr; g.ldb = p->ldb;
-    g.sAf = (long long)p->nv * p->ldr;
-    g.sDf = (long long)p->ns * p->ldr;
-    g.sCf = (long long)p->nv * p->ldb;
+    set_shape(g, p, nb);
+    g.sAf = (long long)p->nv * p->ldr * SPEC_F;
+    g.sCf = (long long)p->nv * p->ldb * SPEC_F;
     g.outscale = 1.f;
     g.status = p->status;
     g.nf_active = p->nf_active;
     g.wait_probe = p->wait_probe;
     if (p->xhat_upper_tr > 0) {
-        // the spectra below the block diagonal of a symmetric model: read transposed by the tile kernel,
+        // the spectra below the block diagonal of a symmetric model: read transposed by the split-BF16 kernels,
         // else copied into place first
-        if (p->gemm_fwd == MDC_GEMM_TC) {
+        if (reads_transposed(p)) {
             g.sym_tr = p->xhat_upper_tr;
         } else {
             const int tr = p->xhat_upper_tr;
             p->xhat_upper_tr = 0;
             const int rc = launch_stage(p, ST_GEMM_FWD, st, [&] {
-                return launch_mirror_lower(p->Xh, p->nv, p->ldr, (long long)p->nv * p->ldr, p->nf, tr, st);
+                return launch_mirror_lower(p->Xh, p->nv, p->ldr, p->nf, tr, st);
             });
             if (rc) return rc;
         }
     }
-    if (p->gemm_fwd == MDC_GEMM_TC)
-        return launch_stage(p, ST_GEMM_FWD, st, [&] { return launch_tc_fwd(g, p->nf, st); });
-    if (p->gemm_fwd == MDC_GEMM_TC_STREAM && p->xh_map_ok)
-        return launch_stage(p, ST_GEMM_FWD, st, [&] { return launch_tc_fwd_stream(g, p->xh_map, p->nf, st); });
+    if (p->gemm_fwd == MDC_GEMM_TC_STREAM) g.wait_probe = 0;   // (the failure-path check is MDC_GEMM_TC's)
+    if (p->gemm_fwd == MDC_GEMM_TC || p->gemm_fwd == MDC_GEMM_TC_STREAM)
+        return launch_stage(p, ST_GEMM_FWD, st, [&] {
+            return p->xh_map_ok ? launch_tc_fwd_p(g, p->maps, p->nf, st) : launch_tc_fwd(g, p->nf, st);
+        });
     if (p->gemm_fwd == MDC_GEMM_GEMV && gemv_supported(p->nv) && p->nf_active == 0)
         return launch_stage(p, ST_GEMM_FWD, st, [&] { return launch_gemv_fwd(g, p->nf, st); });
     return launch_stage(p, ST_GEMM_FWD, st, [&] { return launch_cgemm_fwd(g, p->nf, st); });
@@ -246,10 +266,9 @@ int gemm_adjoint(mdc_plan_s *p, const int32_t *idx, int nb, bool recip, cudaStre
     g.Dh = p->Dh;
     g.idx = idx;
     g.C = p->Xh;
-    g.nv = p->nv; g.nr = p->nr; g.ns = p->ns; g.nb = nb; g.ldr = p->ldr; g.ldb = p->ldb;
-    g.sAf = (long long)p->nv * p->ldb;
-    g.sDf = (long long)p->ns * p->ldr;
-    g.sCf = (long long)p->nv * p->ldr;
+    set_shape(g, p, nb);
+    g.sAf = (long long)p->nv * p->ldb * SPEC_F;
+    g.sCf = (long long)p->nv * p->ldr * SPEC_F;
     g.outscale = recip ? 0.5f : 1.f;
     g.status = p->status;
     g.nf_active = p->nf_active;
@@ -264,7 +283,7 @@ int gemm_adjoint(mdc_plan_s *p, const int32_t *idx, int nb, bool recip, cudaStre
                 g.img = p->adj_img;
                 g.img_nkc = (nb + 31) / 32;
             }
-            return launch_tc_adj(g, recip, p->nf, st, (SMDD_TC_ADJ_TMA && p->xh_map_ok) ? p->xh_map : nullptr);
+            return launch_tc_adj(g, recip, p->nf, st, (SMDD_TC_ADJ_TMA && p->xh_map_ok) ? p->maps.adj : nullptr);
         });
     if (p->gemm_adj == MDC_GEMM_GEMV && gemv_supported(p->nv) && !recip && p->nf_active == 0 && nb <= 1024)
         return launch_stage(p, ST_GEMM_ADJ, st, [&] { return launch_gemv_adj(g, p->nf, st); });
@@ -394,17 +413,18 @@ int mdc_plan_create(mdc_plan_t *out, int nt, int nr, int nv, int ns, int nb_max,
     if (cudaGetDevice(&p->device) != cudaSuccess) { delete p; return MDC_ERR_CUDA; }
     p->nt = nt; p->nr = nr; p->nv = nv; p->ns = ns; p->nbmax = nb_max;
     p->nfft = nfft; p->M = nfft / 2; p->nf = nfft / 2 + 1;
-    p->ldr = padded_ld(nr);
-    p->ldb = padded_ld(nb_max);
+    p->ldr = (nr + 7) & ~7;
+    p->ldb = (nb_max + 7) & ~7;
+    p->ldd = padded_ld(nr);
     p->scale = scale;
     p->prec = precision;
     p->gemm_fwd = p->gemm_adj = (precision == MDC_PREC_BF16X3) ? MDC_GEMM_TC : MDC_GEMM_SIMT;
     p->fft_variant = (nfft == 2048) ? 2 : 0;
 
     const int M = p->M, nf = p->nf;
-    const size_t szD = (size_t)nf * ns * p->ldr * sizeof(float2);
-    const size_t szX = (size_t)nf * nv * p->ldr * sizeof(float2);
-    const size_t szU = (size_t)nf * nv * p->ldb * sizeof(float2);
+    const size_t szD = (size_t)nf * ns * p->ldd * sizeof(float2);
+    const size_t szX = (size_t)spec_blocks(nf) * SPEC_F * nv * p->ldr * sizeof(float2);
+    const size_t szU = (size_t)spec_blocks(nf) * SPEC_F * nv * p->ldb * sizeof(float2);
     p->resid_blocks_max = fft_blocks(M, batch_grid(p, nb_max));
     bool ok = cudaMalloc(&p->Dh, szD) == cudaSuccess && cudaMalloc(&p->Xh, szX) == cudaSuccess &&
               cudaMalloc(&p->Uh, szU) == cudaSuccess && cudaMalloc(&p->tw, (size_t)fft_tw_size(M) * sizeof(float2)) == cudaSuccess &&
@@ -438,11 +458,11 @@ int mdc_plan_create(mdc_plan_t *out, int nt, int nr, int nv, int ns, int nb_max,
     if (rc == MDC_OK && (fft_prepare(M) != cudaSuccess || gemm_prepare() != cudaSuccess)) rc = MDC_ERR_CUDA;
     if (rc == MDC_OK && precision == MDC_PREC_BF16X3 && tc_prepare() != cudaSuccess) rc = MDC_ERR_CUDA;
     if (rc == MDC_OK && precision == MDC_PREC_BF16X3)   // without a map, MDC_GEMM_TC_STREAM is unsupported
-        p->xh_map_ok = tc_encode_fwd_map(p->xh_map, p->Xh, nr, nv, p->ldr, p->nf) == cudaSuccess;
+        p->xh_map_ok = tc_encode_maps(&p->maps, p->Xh, nr, nv, p->ldr, p->nf) == cudaSuccess;
     if (rc == MDC_OK) {
-        // kernel spectra: D [ns][nr][nt] -> Dh [nf][ns][ldr] (same layout rule as the model)
+        // kernel spectra: D [ns][nr][nt] -> Dh [nf][ns][ldd]
         FftArgs a = base_fft(p);
-        a.g = model_grid(p, ns);
+        a.g = kernel_grid(p);
         a.tin = D;
         a.vec = time_vec(nt, D);
         a.spec = p->Dh;
@@ -533,7 +553,7 @@ int mdc_plan_sigma2_max(mdc_plan_t p, int n_iter, double *sigma2, void *stream) 
     DeviceGuard dg(p->device);
     cudaStream_t st = (cudaStream_t)stream;
     int rc = launch_stage(p, ST_SETUP, st, [&] {
-        return launch_power_iter(p->Dh, p->ns, p->nr, p->ldr, (long long)p->ns * p->ldr, p->nf, n_iter, p->lam, st);
+        return launch_power_iter(p->Dh, p->ns, p->nr, p->ldd, (long long)p->ns * p->ldd, p->nf, n_iter, p->lam, st);
     });
     if (rc) return rc;
     rc = launch_stage(p, ST_SETUP, st, [&] { return launch_max_reduce(p->lam, p->nf, p->lam + p->nf, st); });
@@ -672,11 +692,11 @@ int step_impl(mdc_plan_t p, float *X, const float *U_obs, const int32_t *idx, in
         a.c2 = adam.c2;
         // a symmetric model's spectra below the block diagonal are copies of the ones above it: the tile
         // forward product of the next step reads them transposed, any other kernel needs the copy
-        const bool mirror = keep && sym && p->gemm_fwd != MDC_GEMM_TC;
+        const bool mirror = keep && sym && !reads_transposed(p);
         if ((rc = launch_stage(p, ST_UPDATE, st, [&] {
                  const cudaError_t e = launch_update(p->M, keep, a, st);
                  if (e != cudaSuccess || !mirror) return e;
-                 return launch_mirror_lower(p->Xh, p->nv, p->ldr, (long long)p->nv * p->ldr, p->nf, tr_upd, st);
+                 return launch_mirror_lower(p->Xh, p->nv, p->ldr, p->nf, tr_upd, st);
              })))
             return rc;
         if (keep) p->xhat_for = X;
@@ -710,8 +730,8 @@ int plan_step_records(mdc_plan_s *p, float *X, const float *U_obs, const int32_t
     // forward product (as gemm_forward, on the tile kernel)
     GemmArgs &g = r->fwd;
     g.A = p->Xh; g.Dh = p->Dh; g.idx = idx; g.C = p->Uh;
-    g.nv = p->nv; g.nr = p->nr; g.ns = p->ns; g.nb = nb; g.ldr = p->ldr; g.ldb = p->ldb;
-    g.sAf = (long long)p->nv * p->ldr; g.sDf = (long long)p->ns * p->ldr; g.sCf = (long long)p->nv * p->ldb;
+    set_shape(g, p, nb);
+    g.sAf = (long long)p->nv * p->ldr * SPEC_F; g.sCf = (long long)p->nv * p->ldb * SPEC_F;
     g.outscale = 1.f;
     g.status = p->status;
     g.wait_probe = p->wait_probe;
@@ -737,8 +757,8 @@ int plan_step_records(mdc_plan_s *p, float *X, const float *U_obs, const int32_t
     // adjoint product
     GemmArgs &h = r->adj;
     h.A = p->Uh; h.Dh = p->Dh; h.idx = idx; h.C = p->Xh;
-    h.nv = p->nv; h.nr = p->nr; h.ns = p->ns; h.nb = nb; h.ldr = p->ldr; h.ldb = p->ldb;
-    h.sAf = (long long)p->nv * p->ldb; h.sDf = (long long)p->ns * p->ldr; h.sCf = (long long)p->nv * p->ldr;
+    set_shape(h, p, nb);
+    h.sAf = (long long)p->nv * p->ldb * SPEC_F; h.sCf = (long long)p->nv * p->ldr * SPEC_F;
     h.outscale = recip ? 0.5f : 1.f;
     h.status = p->status;
     h.wait_probe = p->wait_probe;

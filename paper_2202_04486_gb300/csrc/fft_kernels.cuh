@@ -8,10 +8,11 @@
 // convolution (forward) and the linear cross-correlation at non-negative lags (adjoint, Eq. 6).
 //
 // Memory behaviour: a CTA owns TR traces whose spectra are adjacent along the contiguous axis; its threads
-// read and write the bins of those traces straight from the edge passes of the FFT (smdd_fft.cuh), one
-// contiguous segment of 8 PL bytes times two traces per frequency row, all loads of a thread issued together.
+// read and write the bins of those traces straight from the edge passes of the FFT (smdd_fft.cuh): 8 traces x
+// SPEC_F bins are 256 contiguous bytes (smdd_internal.h), all loads of a thread are issued together.
 // Time-domain inputs needed after an inverse FFT (the model for the update, the observed data for the
-// residual) are loaded into registers before its middle passes, so their latency overlaps them.
+// residual) are loaded into registers before its middle passes, so their latency overlaps them (after the inverse
+// where the registers do not reach, Team::LATE).
 //
 // This header holds the device code and the per-length launchers FftLaunch<M>; each complex length M is
 // instantiated in a translation unit of its own (fft_m*.cu) so the library compiles in parallel, and
@@ -87,10 +88,17 @@ __device__ __forceinline__ PairCtx<M> pair_ctx(const TraceGrid &g, int bid) {
     return x;
 }
 
-// The pair's traces are adjacent along the contiguous spectrum axis and 16-byte aligned: one 16-byte access per
-// bin (a grid with a single trace along i, or odd strides, takes two 8-byte accesses).
-__device__ __forceinline__ bool pair_io(const TraceGrid &g) {
-    return g.ti_log2 >= 1 && g.ssi == 1 && (g.ssj % 2) == 0 && (g.ssf % 2) == 0;
+// The pair's traces are adjacent along the contiguous spectrum axis and 16-byte aligned (rows have an even
+// length): one 16-byte access per bin (a grid with a single trace along i takes two 8-byte accesses).
+__device__ __forceinline__ bool pair_io(const TraceGrid &g) { return g.ti_log2 >= 1; }
+
+// bin 0 of a trace
+__device__ __forceinline__ long long spec_trace(const TraceGrid &g, const TileCoord &c) {
+    return (((long long)(c.i >> 3) << (3 + g.fl2)) + (c.i & 7)) + (long long)c.j * g.ssj;
+}
+// bin f of a trace relative to its bin 0
+__device__ __forceinline__ long long spec_at(const TraceGrid &g, int f) {
+    return (long long)(f >> g.fl2) * g.ssf + ((f & ((1 << g.fl2) - 1)) << 3);
 }
 
 __device__ __forceinline__ C2 join(float2 a, float2 b) { return C2{pk2(a.x, b.x), pk2(a.y, b.y)}; }
@@ -100,8 +108,8 @@ __device__ __forceinline__ C2 join(float2 a, float2 b) { return C2{pk2(a.x, b.x)
 template <int M>
 __device__ __forceinline__ void bins_load(C2 (&z)[8], const float2 *__restrict__ spec, const TraceGrid &g, const PairCtx<M> &x,
                                           int f0, int fs) {
-    const float2 *a = spec + (long long)x.c[0].i * g.ssi + (long long)x.c[0].j * g.ssj + (long long)f0 * g.ssf;
-    const long long st = (long long)fs * g.ssf;
+    const float2 *a = spec + spec_trace(g, x.c[0]) + spec_at(g, f0);
+    const long long st = spec_at(g, fs);   // fs is a multiple of the bins of a block
     if (pair_io(g)) {
         float4 v[8];
 #pragma unroll
@@ -111,7 +119,7 @@ __device__ __forceinline__ void bins_load(C2 (&z)[8], const float2 *__restrict__
         for (int r = 0; r < 8; ++r)
             z[r] = join(make_float2(v[r].x, v[r].y), x.c[1].valid ? make_float2(v[r].z, v[r].w) : make_float2(0.f, 0.f));
     } else {
-        const float2 *b = spec + (long long)x.c[1].i * g.ssi + (long long)x.c[1].j * g.ssj + (long long)f0 * g.ssf;
+        const float2 *b = spec + spec_trace(g, x.c[1]) + spec_at(g, f0);
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
             const float2 va = x.c[0].valid ? __ldcs(a + r * st) : make_float2(0.f, 0.f);
@@ -124,14 +132,14 @@ __device__ __forceinline__ void bins_load(C2 (&z)[8], const float2 *__restrict__
 template <int M>
 __device__ __forceinline__ void bins_store(const C2 (&z)[8], float2 *__restrict__ spec, const TraceGrid &g, const PairCtx<M> &x,
                                            int f0, int fs) {
-    float2 *a = spec + (long long)x.c[0].i * g.ssi + (long long)x.c[0].j * g.ssj + (long long)f0 * g.ssf;
-    const long long st = (long long)fs * g.ssf;
+    float2 *a = spec + spec_trace(g, x.c[0]) + spec_at(g, f0);
+    const long long st = spec_at(g, fs);
     if (pair_io(g) && x.c[1].valid) {   // (the first trace of a pair is valid if the second is)
 #pragma unroll
         for (int r = 0; r < 8; ++r)
             *reinterpret_cast<float4 *>(a + r * st) = make_float4(lo2(z[r].re), lo2(z[r].im), hi2(z[r].re), hi2(z[r].im));
     } else {
-        float2 *b = spec + (long long)x.c[1].i * g.ssi + (long long)x.c[1].j * g.ssj + (long long)f0 * g.ssf;
+        float2 *b = spec + spec_trace(g, x.c[1]) + spec_at(g, f0);
         if (x.c[0].valid) {
 #pragma unroll
             for (int r = 0; r < 8; ++r) a[r * st] = make_float2(lo2(z[r].re), lo2(z[r].im));
@@ -158,12 +166,14 @@ __device__ __forceinline__ void spec_to_smem(const FftArgs &a, const PairCtx<M> 
     bins_load<M>(B, a.spec, a.g, x, s ? S - s : S / 2, S);
     f32x2 nyq = 0;
     if (s == 0) {
-        const float2 *b = a.spec + (long long)M * a.g.ssf;
-        const float n0 = x.c[0].valid ? b[(long long)x.c[0].i * a.g.ssi + (long long)x.c[0].j * a.g.ssj].x : 0.f;
-        const float n1 = x.c[1].valid ? b[(long long)x.c[1].i * a.g.ssi + (long long)x.c[1].j * a.g.ssj].x : 0.f;
+        const float2 *b = a.spec + spec_at(a.g, M);
+        const float n0 = x.c[0].valid ? b[spec_trace(a.g, x.c[0])].x : 0.f;
+        const float n1 = x.c[1].valid ? b[spec_trace(a.g, x.c[1])].x : 0.f;
         nyq = pk2(n0, n1);
     }
-    edge_inv<M>(A, B, nyq, x.buf, s, a.tw);
+    EdgeRoots<M> t;
+    t.load(a.tw, s);
+    edge_inv<M>(A, B, nyq, x.buf, s, a.tw, t);
 }
 
 // last forward pass -> spectra in global memory
@@ -177,9 +187,9 @@ __device__ __forceinline__ void smem_to_spec(const FftArgs &a, const PairCtx<M> 
     bins_store<M>(A, a.spec, a.g, x, s, S);
     bins_store<M>(B, a.spec, a.g, x, s ? S - s : S / 2, S);
     if (s == 0) {
-        float2 *b = a.spec + (long long)M * a.g.ssf;
-        if (x.c[0].valid) b[(long long)x.c[0].i * a.g.ssi + (long long)x.c[0].j * a.g.ssj] = make_float2(lo2(nyq), 0.f);
-        if (x.c[1].valid) b[(long long)x.c[1].i * a.g.ssi + (long long)x.c[1].j * a.g.ssj] = make_float2(hi2(nyq), 0.f);
+        float2 *b = a.spec + spec_at(a.g, M);
+        if (x.c[0].valid) b[spec_trace(a.g, x.c[0])] = make_float2(lo2(nyq), 0.f);
+        if (x.c[1].valid) b[spec_trace(a.g, x.c[1])] = make_float2(hi2(nyq), 0.f);
     }
 }
 
@@ -281,7 +291,6 @@ __device__ __forceinline__ void slots_to_spec(const FftArgs &a, const PairCtx<M>
     C2 v[FFT_P];
     slots_to_regs<M>(v, ha, hb);
     fwd_first<M>(v, x.buf, x.s);
-    group_sync<M>();
     mid_passes<M, false, 1>(x.buf, x.s, a.tw);
     smem_to_spec<M>(a, x);
 }
@@ -305,8 +314,8 @@ template <int M>
 __global__ void __launch_bounds__(Team<M>::THREADS, Team<M>::MINB) k_irfft_out(FftArgs a) {
     const PairCtx<M> x = pair_ctx<M>(a.g, blockIdx.x);
     spec_to_smem<M>(a, x);
-    group_sync<M>();
     mid_passes<M, true, fft_npass(M) - 2>(x.buf, x.s, a.tw);
+    group_sync<M>();
     C2 v[FFT_P];
     inv_last<M>(v, x.buf, x.s);
 #pragma unroll
@@ -379,11 +388,15 @@ __device__ __forceinline__ void residual_body(const FftArgs &a, int bid, int nbl
     spec_to_smem<M>(a, x);
     float2 o[2][NSLOT];   // observed rows, loaded before the middle passes (their latency overlaps the rest)
 #pragma unroll
-    for (int k = 0; k < 2; ++k) time_load<M>(o[k], uo[k] ? uo[k] : a.uobs, a.nt, uo[k] != nullptr, a.vec, x.s);
-    group_sync<M>();
+    for (int k = 0; k < 2; ++k)
+        if (!Team<M>::LATE) time_load<M>(o[k], uo[k] ? uo[k] : a.uobs, a.nt, uo[k] != nullptr, a.vec, x.s);
     mid_passes<M, true, fft_npass(M) - 2>(x.buf, x.s, a.tw);
+    group_sync<M>();
     C2 v[FFT_P];
     inv_last<M>(v, x.buf, x.s);
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+        if (Team<M>::LATE) time_load<M>(o[k], uo[k] ? uo[k] : a.uobs, a.nt, uo[k] != nullptr, a.vec, x.s);
     // z = s p - o inside the window [0, nt), zero outside
     float top = 0.f;
 #pragma unroll
@@ -460,11 +473,15 @@ __device__ __forceinline__ void update_body(const FftArgs &a, int bid_in) {
     spec_to_smem<M>(a, x);
     float2 xo[2][NSLOT];   // model samples, loaded before the middle passes (their latency overlaps the rest)
 #pragma unroll
-    for (int k = 0; k < 2; ++k) time_load<M>(xo[k], a.tout + time_off<M>(a.g, x.c[k]), a.nt, x.c[k].valid, a.vec, x.s);
-    group_sync<M>();
+    for (int k = 0; k < 2; ++k)
+        if (!Team<M>::LATE) time_load<M>(xo[k], a.tout + time_off<M>(a.g, x.c[k]), a.nt, x.c[k].valid, a.vec, x.s);
     mid_passes<M, true, fft_npass(M) - 2>(x.buf, x.s, a.tw);
+    group_sync<M>();
     C2 v[FFT_P];
     inv_last<M>(v, x.buf, x.s);
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+        if (Team<M>::LATE) time_load<M>(xo[k], a.tout + time_off<M>(a.g, x.c[k]), a.nt, x.c[k].valid, a.vec, x.s);
     const float nas = -a.alpha * a.s;
 #pragma unroll
     for (int k = 0; k < 2; ++k) {

@@ -44,17 +44,18 @@ constexpr int FW_THREADS = 128, FW_ROWS = 128, FW_NB = 16, FW_KC = 16, FW_LD = F
 constexpr int FW_STAGE = (FW_ROWS + FW_NB) * FW_LD;   // float2 per stage
 constexpr size_t FW_SMEM = 2 * FW_STAGE * sizeof(float2);
 
+template <int F>
 __global__ void __launch_bounds__(FW_THREADS, 4) k_cgemm_fwd(GemmArgs a) {
     extern __shared__ __align__(16) float2 gsm[];
     const int f = blockIdx.z;
     const int v0 = blockIdx.x * FW_ROWS, b0 = blockIdx.y * FW_NB;
     if (a.nf_active > 0 && f >= a.nf_active) {
-        zero_tile(a.C + (long long)f * a.sCf, a.ldb, v0, FW_ROWS, b0, FW_NB, a.nv, a.nb);
+        zero_tile<F>(a.C + spec_bin<F>(f, a.sCf), (long long)a.ldb * F, v0, FW_ROWS, b0, FW_NB, a.nv, a.nb);
         return;
     }
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int vg = lane & 7, bg = lane >> 3;
-    const float2 *Af = a.A + (long long)f * a.sAf;
+    const float2 *Af = a.A + spec_bin<F>(f, a.sAf);
     const float2 *Df = a.Dh + (long long)f * a.sDf;
 
     // kernel row of the batch column this thread stages (one 16-byte chunk per thread per stage)
@@ -80,7 +81,7 @@ __global__ void __launch_bounds__(FW_THREADS, 4) k_cgemm_fwd(GemmArgs a) {
             const float2 *src = Af;
             if (v < a.nv && k < a.nr) {
                 bytes = (k + 1 < a.nr) ? 16 : 8;
-                src = Af + (long long)v * a.ldr + k;
+                src = Af + (long long)v * a.ldr * F + spec_col<F>(k);
             }
             cp_async16(sX + row * FW_LD + 2 * part, src, bytes);
         }
@@ -90,7 +91,7 @@ __global__ void __launch_bounds__(FW_THREADS, 4) k_cgemm_fwd(GemmArgs a) {
             const float2 *src = Df;
             if (drow >= 0 && k < a.nr) {
                 bytes = (k + 1 < a.nr) ? 16 : 8;
-                src = Df + (long long)drow * a.ldr + k;
+                src = Df + (long long)drow * a.ldd + k;
             }
             cp_async16(sD + db * FW_LD + 2 * dpart, src, bytes);
         }
@@ -136,7 +137,7 @@ __global__ void __launch_bounds__(FW_THREADS, 4) k_cgemm_fwd(GemmArgs a) {
         __syncthreads();
     }
 
-    float2 *Cf = a.C + (long long)f * a.sCf;
+    float2 *Cf = a.C + spec_bin<F>(f, a.sCf);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const int v = v0 + 32 * warp + vg + 8 * i;
@@ -144,7 +145,7 @@ __global__ void __launch_bounds__(FW_THREADS, 4) k_cgemm_fwd(GemmArgs a) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int b = b0 + bg + 4 * j;
-            if (b < a.nb) Cf[(long long)v * a.ldb + b] = acc[i][j];
+            if (b < a.nb) Cf[(long long)v * a.ldb * F + spec_col<F>(b)] = acc[i][j];
         }
     }
 }
@@ -187,7 +188,7 @@ __device__ __forceinline__ void stage_rrows(float2 *s, const float2 *Rf, int ldb
         const float2 *src = Rf;
         if (c0 + row < nc && k < nb) {
             bytes = (k + 1 < nb) ? 16 : 8;
-            src = Rf + (long long)(c0 + row) * ldb + k;
+            src = Rf + (long long)(c0 + row) * ldb * SPEC_F + spec_col(k);
         }
         cp_async16(s + row * AD_LDR + 2 * part, src, bytes);
     }
@@ -195,7 +196,7 @@ __device__ __forceinline__ void stage_rrows(float2 *s, const float2 *Rf, int ldb
 
 // stage kernel rows idx[k0 .. k0 + 16) at columns [c0, c0 + TT) into s[16][TT]
 template <int TT>
-__device__ __forceinline__ void stage_drows(float2 *s, const float2 *Df, int ldr, const int *sidx, int c0, int nc, int k0,
+__device__ __forceinline__ void stage_drows(float2 *s, const float2 *Df, int ldd, const int *sidx, int c0, int nc, int k0,
                                             int nb, int tid) {
     constexpr int NT = AdjGeom<TT>::THREADS, PARTS = TT / 2;
 #pragma unroll
@@ -208,7 +209,7 @@ __device__ __forceinline__ void stage_drows(float2 *s, const float2 *Df, int ldr
             const int srow = sidx[k0 + kk];
             if (srow >= 0) {
                 bytes = (col + 1 < nc) ? 16 : 8;
-                src = Df + (long long)srow * ldr + col;
+                src = Df + (long long)srow * ldd + col;
             }
         }
         cp_async16(s + kk * TT + 2 * part, src, bytes);
@@ -245,15 +246,16 @@ __global__ void __launch_bounds__(AdjGeom<TT>::THREADS, TT == 64 ? 3 : 8) k_cgem
     }
     const int v0 = vb * TT, r0 = rb * TT;
     if (a.nf_active > 0 && f >= a.nf_active) {
-        zero_tile(a.C + (long long)f * a.sCf, a.ldr, v0, TT, r0, TT, a.nv, a.nr);
-        if (RECIP) zero_tile(a.C + (long long)f * a.sCf, a.ldr, r0, TT, v0, TT, a.nr, a.nv);
+        const long long row = (long long)a.ldr * SPEC_F;
+        zero_tile(a.C + spec_bin(f, a.sCf), row, v0, TT, r0, TT, a.nv, a.nr);
+        if (RECIP) zero_tile(a.C + spec_bin(f, a.sCf), row, r0, TT, v0, TT, a.nr, a.nv);
         return;
     }
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int vp = lane / G::RG, rg = lane % G::RG;
     const int vl = G::WROWS * warp + 4 * vp;     // first local row of the thread
     const bool active = v0 + G::WROWS * warp < a.nv;
-    const float2 *Rf = a.A + (long long)f * a.sAf;
+    const float2 *Rf = a.A + spec_bin(f, a.sAf);
     const float2 *Df = a.Dh + (long long)f * a.sDf;
 
     for (int b = tid; b < a.nb; b += G::THREADS) {
@@ -274,10 +276,10 @@ __global__ void __launch_bounds__(AdjGeom<TT>::THREADS, TT == 64 ? 3 : 8) k_cgem
 
     for (int k0 = 0; k0 < a.nb; k0 += AD_KC) {
         stage_rrows<TT>(sRv, Rf, a.ldb, v0, a.nv, k0, a.nb, tid);
-        stage_drows<TT>(sDr, Df, a.ldr, sidx, r0, a.nr, k0, a.nb, tid);
+        stage_drows<TT>(sDr, Df, a.ldd, sidx, r0, a.nr, k0, a.nb, tid);
         if (RECIP) {
             stage_rrows<TT>(sRr, Rf, a.ldb, r0, a.nr, k0, a.nb, tid);
-            stage_drows<TT>(sDv, Df, a.ldr, sidx, v0, a.nv, k0, a.nb, tid);
+            stage_drows<TT>(sDv, Df, a.ldd, sidx, v0, a.nv, k0, a.nb, tid);
         }
         cp_async_commit();
         cp_async_wait<0>();
@@ -336,7 +338,8 @@ __global__ void __launch_bounds__(AdjGeom<TT>::THREADS, TT == 64 ? 3 : 8) k_cgem
         __syncthreads();
     }
 
-    float2 *Cf = a.C + (long long)f * a.sCf;
+    float2 *Cf = a.C + spec_bin(f, a.sCf);
+    const long long crow = (long long)a.ldr * SPEC_F;
     const bool diag = RECIP && (vb == rb);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -347,7 +350,7 @@ __global__ void __launch_bounds__(AdjGeom<TT>::THREADS, TT == 64 ? 3 : 8) k_cgem
             const float2 x0 = cscale(acc[i][2 * h], a.outscale), x1 = cscale(acc[i][2 * h + 1], a.outscale);
             if (v < a.nv) {
                 const bool w0 = r < a.nr && (!diag || v <= r), w1 = r + 1 < a.nr && (!diag || v <= r + 1);
-                float2 *dst = Cf + (long long)v * a.ldr + r;
+                float2 *dst = Cf + v * crow + spec_col(r);
                 if (w0 && w1) *reinterpret_cast<float4 *>(dst) = make_float4(x0.x, x0.y, x1.x, x1.y);
                 else {
                     if (w0) dst[0] = x0;
@@ -365,7 +368,7 @@ __global__ void __launch_bounds__(AdjGeom<TT>::THREADS, TT == 64 ? 3 : 8) k_cgem
         for (int e = tid; e < TT * TT; e += G::THREADS) {
             const int rr = e / TT, vv = e % TT;
             const int r = r0 + rr, v = v0 + vv;
-            if (v < a.nv && r < a.nr && (!diag || v < r)) Cf[(long long)r * a.ldr + v] = gsm[rr * (TT + 1) + vv];
+            if (v < a.nv && r < a.nr && (!diag || v < r)) Cf[r * crow + spec_col(v)] = gsm[rr * (TT + 1) + vv];
         }
     }
 }
@@ -388,18 +391,18 @@ __global__ void __launch_bounds__(GV_THREADS) k_gemv_fwd(GemmArgs a) {
         if (lane == 0) atomicOr(a.status, 1);
         s = -1;
     }
-    const float2 *Af = a.A + (long long)f * a.sAf;
+    const float2 *Af = a.A + spec_bin(f, a.sAf);
     float2 acc[NV];
 #pragma unroll
     for (int v = 0; v < NV; ++v) acc[v] = make_float2(0.f, 0.f);
     if (s >= 0) {
-        const float2 *d = a.Dh + (long long)f * a.sDf + (long long)s * a.ldr;
+        const float2 *d = a.Dh + (long long)f * a.sDf + (long long)s * a.ldd;
         for (int r = lane; r < a.nr; r += 32) {
             const float2 dv = __ldg(d + r);
 #pragma unroll
             for (int v = 0; v < NV; ++v) {
                 if (v < a.nv) {
-                    const float2 x = __ldg(Af + (long long)v * a.ldr + r);
+                    const float2 x = __ldg(Af + (long long)v * a.ldr * SPEC_F + spec_col(r));
                     acc[v].x = fmaf(x.x, dv.x, fmaf(-x.y, dv.y, acc[v].x));
                     acc[v].y = fmaf(x.x, dv.y, fmaf(x.y, dv.x, acc[v].y));
                 }
@@ -414,10 +417,10 @@ __global__ void __launch_bounds__(GV_THREADS) k_gemv_fwd(GemmArgs a) {
             acc[v].y += __shfl_down_sync(0xffffffffu, acc[v].y, o);
         }
     if (lane == 0) {
-        float2 *Cf = a.C + (long long)f * a.sCf;
+        float2 *Cf = a.C + spec_bin(f, a.sCf);
 #pragma unroll
         for (int v = 0; v < NV; ++v)
-            if (v < a.nv) Cf[(long long)v * a.ldb + b] = make_float2(acc[v].x * a.outscale, acc[v].y * a.outscale);
+            if (v < a.nv) Cf[(long long)v * a.ldb * SPEC_F + spec_col(b)] = make_float2(acc[v].x * a.outscale, acc[v].y * a.outscale);
     }
 }
 
@@ -437,7 +440,7 @@ __global__ void __launch_bounds__(GV_THREADS) k_gemv_adj(GemmArgs a) {
     }
     __syncthreads();
     if (r >= a.nr) return;   // after the only barrier
-    const float2 *Af = a.A + (long long)f * a.sAf;
+    const float2 *Af = a.A + spec_bin(f, a.sAf);
     const float2 *Df = a.Dh + (long long)f * a.sDf;
     float2 acc[NV];
 #pragma unroll
@@ -445,21 +448,21 @@ __global__ void __launch_bounds__(GV_THREADS) k_gemv_adj(GemmArgs a) {
     for (int b = 0; b < a.nb; ++b) {
         const int s = sidx[b];
         if (s < 0) continue;
-        const float2 d = __ldg(Df + (long long)s * a.ldr + r);
+        const float2 d = __ldg(Df + (long long)s * a.ldd + r);
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
             if (v < a.nv) {
-                const float2 c = __ldg(Af + (long long)v * a.ldb + b);
+                const float2 c = __ldg(Af + (long long)v * a.ldb * SPEC_F + spec_col(b));
                 // c * conj(d)
                 acc[v].x = fmaf(c.x, d.x, fmaf(c.y, d.y, acc[v].x));
                 acc[v].y = fmaf(c.y, d.x, fmaf(-c.x, d.y, acc[v].y));
             }
         }
     }
-    float2 *Cf = a.C + (long long)f * a.sCf;
+    float2 *Cf = a.C + spec_bin(f, a.sCf);
 #pragma unroll
     for (int v = 0; v < NV; ++v)
-        if (v < a.nv) Cf[(long long)v * a.ldr + r] = make_float2(acc[v].x * a.outscale, acc[v].y * a.outscale);
+        if (v < a.nv) Cf[(long long)v * a.ldr * SPEC_F + spec_col(r)] = make_float2(acc[v].x * a.outscale, acc[v].y * a.outscale);
 }
 
 bool gemv_supported(int nv) { return nv >= 1 && nv <= GV_MAXV; }
@@ -488,7 +491,8 @@ cudaError_t launch_gemv_adj(const GemmArgs &a, int nf, cudaStream_t st) {
 
 cudaError_t gemm_prepare() {
     cudaError_t e;
-    if ((e = cudaFuncSetAttribute(k_cgemm_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FW_SMEM))) return e;
+    if ((e = cudaFuncSetAttribute(k_cgemm_fwd<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FW_SMEM))) return e;
+    if ((e = cudaFuncSetAttribute(k_cgemm_fwd<SPEC_F>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FW_SMEM))) return e;
     if ((e = cudaFuncSetAttribute(k_cgemm_adj<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AdjGeom<64>::SMEM))) return e;
     if ((e = cudaFuncSetAttribute(k_cgemm_adj<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AdjGeom<64>::SMEM))) return e;
     if ((e = cudaFuncSetAttribute(k_cgemm_adj<32, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AdjGeom<32>::SMEM))) return e;
@@ -498,7 +502,8 @@ cudaError_t gemm_prepare() {
 
 cudaError_t launch_cgemm_fwd(const GemmArgs &a, int nf, cudaStream_t st) {
     dim3 grid((a.nv + FW_ROWS - 1) / FW_ROWS, (a.nb + FW_NB - 1) / FW_NB, nf);
-    k_cgemm_fwd<<<grid, FW_THREADS, FW_SMEM, st>>>(a);
+    if (a.plain) k_cgemm_fwd<1><<<grid, FW_THREADS, FW_SMEM, st>>>(a);
+    else k_cgemm_fwd<SPEC_F><<<grid, FW_THREADS, FW_SMEM, st>>>(a);
     return cudaGetLastError();
 }
 

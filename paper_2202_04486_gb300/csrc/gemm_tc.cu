@@ -36,8 +36,11 @@ __device__ __forceinline__ uint8_t *align1024(uint8_t *p) {
     return reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(p) + 1023) & ~uintptr_t(1023));
 }
 
-// load 8 consecutive complex values row[k .. k+8), zero past n (row may be null: all zero)
+// load the 8 complex columns k .. k+7 (k a multiple of 8) of a row in the layout of F bins, zero past n (row may be
+// null: all zero)
+template <int F = 1>
 __device__ __forceinline__ void load8(const float2 *row, int k, int n, float2 (&z)[8]) {
+    row += row ? (long long)k * (F - 1) : 0;
     if (row && k + 7 < n) {
         const float4 *p = reinterpret_cast<const float4 *>(row + k);
 #pragma unroll
@@ -54,14 +57,15 @@ __device__ __forceinline__ void load8(const float2 *row, int k, int n, float2 (&
 
 // Row v of a symmetric model's spectra, elements k .. k+8 (zero past n), when only the part on and above
 // the TR-block diagonal is stored: element r < lo = TR floor(v / TR) is read at (r, v) (column v of row r).
+// (ld: float2 of a row over its bins)
 __device__ __forceinline__ void load8_sym(const float2 *Af, long long ld, int v, int k, int n, int lo, float2 (&z)[8]) {
     if (k >= lo) {
-        load8(Af + (long long)v * ld, k, n, z);
+        load8<SPEC_F>(Af + (long long)v * ld, k, n, z);
     } else {
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int r = k + i;
-            z[i] = r < n ? __ldg(r >= lo ? Af + (long long)v * ld + r : Af + (long long)r * ld + v) : make_float2(0.f, 0.f);
+            z[i] = r < n ? __ldg(r >= lo ? Af + (long long)v * ld + spec_col(r) : Af + (long long)r * ld + spec_col(v)) : make_float2(0.f, 0.f);
         }
     }
 }
@@ -119,11 +123,12 @@ __device__ __forceinline__ void tc_fwd_body(const GemmArgs &a, int bx, int by, i
     uint8_t *sm = align1024(tc_raw);
     const int f = bz, v0 = bx * 128, b0 = by * NB;
     if (a.nf_active > 0 && f >= a.nf_active) {   // above the band limit: zero products, no TMEM
-        zero_tile(a.C + (long long)f * a.sCf, a.ldb, v0, 128, b0, NB, a.nv, a.nb);
+        zero_tile(a.C + spec_bin(f, a.sCf), (long long)a.ldb * SPEC_F, v0, 128, b0, NB, a.nv, a.nb);
         return;
     }
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const float2 *Af = a.A + (long long)f * a.sAf;
+    const float2 *Af = a.A + spec_bin(f, a.sAf);
+    const long long arow = (long long)a.ldr * SPEC_F;
     const float2 *Df = a.Dh + (long long)f * a.sDf;
 
     for (int j = tid; j < NB; j += TC_THREADS) {
@@ -171,9 +176,9 @@ __device__ __forceinline__ void tc_fwd_body(const GemmArgs &a, int bx, int by, i
             for (int i = 0; i < UA; ++i) {
                 const int u = tid + i * TC_THREADS, row = u >> 3, c = u & 7, v = v0 + row;
                 if (SYM && v < a.nv)
-                    load8_sym(Af, a.ldr, v, kc * 64 + 8 * c, a.nr, a.sym_tr * (v / a.sym_tr), z[i]);
+                    load8_sym(Af, arow, v, kc * 64 + 8 * c, a.nr, a.sym_tr * (v / a.sym_tr), z[i]);
                 else
-                    load8(v < a.nv ? Af + (long long)v * a.ldr : nullptr, kc * 64 + 8 * c, a.nr, z[i]);
+                    load8<SPEC_F>(v < a.nv ? Af + v * arow : nullptr, kc * 64 + 8 * c, a.nr, z[i]);
             }
             // stage s is free again once the MMAs of chunk kc - NSTAGE (the previous use of bars[s]) are done
             if (kc >= NSTAGE && !mbar_wait_bounded(&bars[s], ((kc - NSTAGE) / NSTAGE) & 1)) fail = 1;
@@ -187,7 +192,7 @@ __device__ __forceinline__ void tc_fwd_body(const GemmArgs &a, int bx, int by, i
         for (int u = tid; u < NB * 8; u += TC_THREADS) {
             const int row = u >> 3, c = u & 7, srow = drows[row];
             float2 z[8];
-            load8(srow >= 0 ? Df + (long long)srow * a.ldr : nullptr, kc * 64 + 8 * c, a.nr, z);
+            load8(srow >= 0 ? Df + (long long)srow * a.ldd : nullptr, kc * 64 + 8 * c, a.nr, z);
             store_planes(st + 4 * G::A_PLANE, row * 128 + ((c ^ (row & 7)) << 4), G::B_PLANE, split8(z, false));
         }
         fence_async_smem();
@@ -233,10 +238,10 @@ __device__ __forceinline__ void tc_fwd_body(const GemmArgs &a, int bx, int by, i
     tc_fence_before();
     __syncthreads();
     if (ok) {
-        float2 *Cf = a.C + (long long)f * a.sCf;
+        float2 *Cf = a.C + spec_bin(f, a.sCf);
         for (int e = tid; e < 128 * NB; e += TC_THREADS) {
             const int row = e / NB, j = e % NB, v = v0 + row, b = b0 + j;
-            if (v < a.nv && b < a.nb) Cf[(long long)v * a.ldb + b] = out[row * (NB + 1) + j];
+            if (v < a.nv && b < a.nb) Cf[(long long)v * a.ldb * SPEC_F + spec_col(b)] = out[row * (NB + 1) + j];
         }
     } else if (tid == 0) {
         atomicOr(a.status, 2);
@@ -338,14 +343,14 @@ __global__ void __launch_bounds__(TC_THREADS) k_tc_adj_images(GemmArgs a, uint8_
     if (blk < a.tiles_v) {
         // R image: residual rows cr .. cr + 127 (b contiguous), staged, then transposed and split
         const int cr = blk * 128;
-        const float2 *Rf = a.A + (long long)f * a.sAf;
+        const float2 *Rf = a.A + spec_bin(f, a.sAf);
         for (int u = tid; u < 128 * (KC / 2); u += TC_THREADS) {
             const int row = u / (KC / 2), pr = u % (KC / 2), k = k0 + 2 * pr, rr = cr + row;
             int bytes = 0;
             const float2 *src = Rf;
             if (rr < a.nv && k < a.nb) {
                 bytes = (k + 1 < a.nb) ? 16 : 8;
-                src = Rf + (long long)rr * a.ldb + k;
+                src = Rf + (long long)rr * a.ldb * SPEC_F + spec_col(k);
             }
             cp_async16_zfill(stg + row * G::SLD + 2 * pr, src, bytes);
         }
@@ -378,7 +383,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_tc_adj_images(GemmArgs a, uint8_
             const int k = u >> 4, ch = u & 15, at = ch >> 3, c = ch & 7;
             const int srow = sidx[k];
             float2 z[8];
-            load8(srow >= 0 ? Df + (long long)srow * a.ldr : nullptr, cd + 64 * at + 8 * c, a.nr, z);
+            load8(srow >= 0 ? Df + (long long)srow * a.ldd : nullptr, cd + 64 * at + 8 * c, a.nr, z);
             store_planes(dst, at * (KC * 128) + k * 128 + ((c ^ (k & 7)) << 4), G::PLANE, split8(z, true));
         }
     }
@@ -412,12 +417,13 @@ __device__ __forceinline__ void tc_adj_body(const GemmArgs &a, int bx, int by, u
     }
     const int v0 = vb * 128, r0 = rb * 128;
     if (a.nf_active > 0 && f >= a.nf_active) {   // above the band limit: zero products, no TMEM
-        zero_tile(a.C + (long long)f * a.sCf, a.ldr, v0, 128, r0, 128, a.nv, a.nr);
-        if (RECIP) zero_tile(a.C + (long long)f * a.sCf, a.ldr, r0, 128, v0, 128, a.nr, a.nv);
+        const long long row = (long long)a.ldr * SPEC_F;
+        zero_tile(a.C + spec_bin(f, a.sCf), row, v0, 128, r0, 128, a.nv, a.nr);
+        if (RECIP) zero_tile(a.C + spec_bin(f, a.sCf), row, r0, 128, v0, 128, a.nr, a.nv);
         return;
     }
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const float2 *Rf = a.A + (long long)f * a.sAf;
+    const float2 *Rf = a.A + spec_bin(f, a.sAf);
     const float2 *Df = a.Dh + (long long)f * a.sDf;
 
     if constexpr (!IMG) {
@@ -489,7 +495,7 @@ __device__ __forceinline__ void tc_adj_body(const GemmArgs &a, int bx, int by, u
             const float2 *src = Rf;
             if (rr < ncr && k < a.nb) {
                 bytes = (k + 1 < a.nb) ? 16 : 8;
-                src = Rf + (long long)rr * a.ldb + k;
+                src = Rf + (long long)rr * a.ldb * SPEC_F + spec_col(k);
             }
             cp_async16_zfill(stg + row * G::SLD + 2 * pr, src, bytes);
         }
@@ -499,7 +505,7 @@ __device__ __forceinline__ void tc_adj_body(const GemmArgs &a, int bx, int by, u
         for (int i = 0; i < UD; ++i) {
             const int u = tid + i * TC_THREADS, k = u >> 4, ch = u & 15, at = ch >> 3, c = ch & 7;
             const int srow = (k < kn) ? sidx[k0 + k] : -1;
-            load8(srow >= 0 ? Df + (long long)srow * a.ldr : nullptr, cd + 64 * at + 8 * c, ncd, zd[i]);
+            load8(srow >= 0 ? Df + (long long)srow * a.ldd : nullptr, cd + 64 * at + 8 * c, ncd, zd[i]);
         }
         // the previous products must be done reading the planes
         if (job > 0) {
@@ -550,8 +556,9 @@ __device__ __forceinline__ void tc_adj_body(const GemmArgs &a, int bx, int by, u
     tc_fence_after();
     // epilogue by the tensor memory accelerator for a tile written once (no reciprocity, or an off-diagonal
     // tile of a symmetric model's adjoint, whose mirror is not needed), in two passes of 64 columns: TMEM ->
-    // four staged boxes of 16 complex x 128 rows (128-byte swizzle: granule g of row m at g ^ (m % 8)) ->
-    // four tiled stores of the tensor map of C (clipped at nv and nr)
+    // eight staged boxes of 8 complex x 128 rows (64-byte swizzle: granule g of row m at g ^ (m / 2 % 4)) ->
+    // eight tiled stores of the tensor map of C (clipped at nv and at the last chunk of 8; the columns past nr of
+    // that chunk are padding, which no kernel reads as data)
     if (TMA && (!RECIP || (a.no_mirror && vb != rb))) {
         for (int pass = 0; pass < 2; ++pass) {
             if (ok) {
@@ -563,10 +570,10 @@ __device__ __forceinline__ void tc_adj_body(const GemmArgs &a, int bx, int by, u
                     float re[16], im[16];
                     tmem_ld16(tmem + ((uint32_t)(32 * q) << 16) + col, re);
                     tmem_ld16(tmem + ((uint32_t)(32 * q) << 16) + 128 + col, im);
-                    uint8_t *box = sm + ((32 * hc + c0) >> 4) * (128 * 128) + row * 128;
+                    uint8_t *box = sm + ((32 * hc + c0) >> 3) * (128 * 64) + row * 64;
 #pragma unroll
                     for (int g = 0; g < 8; ++g)
-                        *reinterpret_cast<float4 *>(box + ((g ^ (row & 7)) << 4)) =
+                        *reinterpret_cast<float4 *>(box + (g >> 2) * (128 * 64) + (((g & 3) ^ ((row >> 1) & 3)) << 4)) =
                             make_float4(re[2 * g] * a.outscale, im[2 * g] * a.outscale, re[2 * g + 1] * a.outscale,
                                         im[2 * g + 1] * a.outscale);
                 }
@@ -576,9 +583,9 @@ __device__ __forceinline__ void tc_adj_body(const GemmArgs &a, int bx, int by, u
             __syncthreads();
             if (ok && tid == 0) {
 #pragma unroll
-                for (int b4 = 0; b4 < 4; ++b4) {
-                    const int r = r0 + 64 * pass + 16 * b4;
-                    if (r < a.nr) tma_store_3d(tmap, sm + b4 * (128 * 128), 2 * r, v0, f);
+                for (int b8 = 0; b8 < 8; ++b8) {
+                    const int r = r0 + 64 * pass + 8 * b8;
+                    if (r < a.nr) tma_store_5d(tmap, sm + b8 * (128 * 64), 0, f % SPEC_F, r >> 3, v0, f / SPEC_F);
                 }
                 bulk_commit();
                 bulk_wait_read();   // the staging may be written again
@@ -600,7 +607,8 @@ __device__ __forceinline__ void tc_adj_body(const GemmArgs &a, int bx, int by, u
     // epilogue in two passes of 64 columns: TMEM -> shared staging [128][65] -> coalesced rows (and
     // the mirror)
     float2 *out = reinterpret_cast<float2 *>(sm);
-    float2 *Cf = a.C + (long long)f * a.sCf;
+    float2 *Cf = a.C + spec_bin(f, a.sCf);
+    const long long crow = (long long)a.ldr * SPEC_F;
     const bool diag = RECIP && vb == rb;
     for (int pass = 0; pass < 2; ++pass) {
         if (ok) {
@@ -623,13 +631,13 @@ __device__ __forceinline__ void tc_adj_body(const GemmArgs &a, int bx, int by, u
             const int rp = r0 + 64 * pass;
             for (int e = tid; e < 128 * 64; e += TC_THREADS) {
                 const int row = e >> 6, col = e & 63, v = v0 + row, r = rp + col;
-                if (v < a.nv && r < a.nr && (!diag || v <= r)) Cf[(long long)v * a.ldr + r] = out[row * 65 + col];
+                if (v < a.nv && r < a.nr && (!diag || v <= r)) Cf[v * crow + spec_col(r)] = out[row * 65 + col];
             }
             // the mirror (diagonal tiles always: their lower half is read by the update of a symmetric model)
             if (RECIP && (diag || !a.no_mirror)) {
                 for (int e = tid; e < 128 * 64; e += TC_THREADS) {
                     const int rr = e >> 7, vv = e & 127, v = v0 + vv, r = rp + rr;
-                    if (v < a.nv && r < a.nr && (!diag || v < r)) Cf[(long long)r * a.ldr + v] = out[vv * 65 + rr];
+                    if (v < a.nv && r < a.nr && (!diag || v < r)) Cf[r * crow + spec_col(v)] = out[vv * 65 + rr];
                 }
             }
         }
@@ -653,7 +661,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2) k_tc_adj(GemmArgs a) {
 }
 
 // the adjoint without reciprocity with its tile written by the tensor memory accelerator (tmap: the
-// tensor map of the gradient spectra, i.e. of the model-spectra buffer, FP32 [nf][nv][2 nr])
+// tensor map of the gradient spectra, i.e. of the model-spectra buffer)
 template <bool IMG = false>
 __global__ void __launch_bounds__(TC_THREADS, 2) k_tc_adj_tma(GemmArgs a, const __grid_constant__ CUtensorMap tmap) {
     tc_adj_body<false, false, true, IMG>(a, blockIdx.x, blockIdx.y, 0, &tmap);
@@ -693,227 +701,393 @@ __global__ void __launch_bounds__(TC_THREADS, 2) k_tc_adj_q(WorkQueue q) {
 }
 
 // ------------------------------------------------------------------------------------------------
-// forward, streamed: the product of k_tc_fwd by a persistent, warp-specialised kernel, one CTA per SM.
-// A CTA walks its tiles (f, 128 rows v, NB batch columns) chunk by chunk (64 of K = nr).
-//  * control warp (warp 16, one lane): issues four tiled copies of the tensor memory accelerator per
-//    chunk (boxes of 128 rows x 16 complex, 128-byte swizzled, zero-filled past nv and nr) into one of
-//    two staging buffers, and the MMAs of each half chunk (K = 32) once the split warps report its
-//    planes written;
-//  * split warps (0-15): convert the staged FP32 spectra and the gathered kernel rows (loaded into
-//    registers one chunk ahead) to the BF16 hi/lo planes, half by half, so the products of one half
-//    run while the other half is split; at the end of a tile they read the accumulators from TMEM and
-//    write the rows of C directly (16 consecutive complex per thread).
-// The warps meet only on mbarriers (full: copies landed; ready: planes of a half written, one arrive
-// per split warp; done: products of a half finished), every wait bounded.  Tiles are numbered
-// t = (f * gy + batch tile) * gx + v tile; the CTA takes t = blockIdx.x, blockIdx.x + gridDim.x, ...;
-// tiles of bins above the band limit are zero-filled first.
+// forward, persistent: the product of tc_fwd_body (same split, same MMAs in the same order, bit-identical) as a
+// warp-specialised kernel, one CTA per SM, fed by the tensor memory accelerator, A operand in tensor memory.
+// A unit is (two neighbouring bins, 128 rows v, NB batch columns): the SPEC_F layout holds the two bins of 8 columns
+// in one 128-byte line.  K = nr runs in chunks of 32 columns (64 KB of both bins).
+//  * copy warp (16): tiled copies of boxes of 128 rows x 8 columns x 2 bins (16 KB, 128-byte swizzle), four a chunk,
+//    into a ring of RING boxes;
+//  * split warps (0-15): thread (row, 8 columns) reads its FP32 values from the staging buffer, splits them and
+//    writes the four BF16 planes to tensor memory (tcgen05.st), so the A operand never returns to shared memory:
+//    there the product would read every plane three times, 12 x 4 KB a K step, more than the chunk itself.  The
+//    gathered kernel rows (in registers one chunk ahead) go to shared-memory planes -Bi, Br, Bi (hi and lo).  Two
+//    stages of planes.
+//  * MMA warp (17): 6 MMAs of N = 2 NB per K step of 16 and bin, Ar [Br | Bi] and Ai [-Bi | Br] with the accumulators
+//    [re | im]: the 12 products of the tile kernel in their order, in half the instructions (the one issuing
+//    thread takes about 60 cycles for each, which bound the kernel with 12).
+// The split warps also write C: the accumulators of a unit are read after the first chunk of the next one has been
+// split (for NB <= 32 there are two sets, so the next unit's products do not wait for it).
+// SYM: spectra of a symmetric model, stored on and above the sym_tr-block diagonal.  Chunks wholly below it are copied
+// as transposed boxes (8 rows x 128 columns) and read by columns; chunks that straddle it are read from global
+// memory by the threads.
+// Units go to the CTAs in rounds, so that the CTAs work on neighbouring bins at a time (contiguous ranges of units per
+// CTA: 822 against 655 us at nt 1500, 600 columns, 384 rows), rotated by one CTA a round, so that every CTA gets its
+// share of ragged last tiles (unrotated, a tile count that divides the grid gives some CTAs none: 842 us for 400
+// rows, 655 us for 384).
+// Waits (all on mbarriers, all bounded): full (a box landed), empty (a box read), aready (planes written), adone
+// (products of a stage finished), ddone (products of a unit finished), dfree (accumulators read).
 // ------------------------------------------------------------------------------------------------
-constexpr int TCS_SPLIT = 512;                 // split warps 0-15
-constexpr int TCS_THREADS = TCS_SPLIT + 32;    // + the control warp
+constexpr int TCP_SPLIT = 512;                 // split warps 0-15
+constexpr int TCP_THREADS = TCP_SPLIT + 64;    // + copy warp, MMA warp
+constexpr int TCP_KC = 32;                     // columns of a chunk
 
 template <int NB>
-struct TcFwdS {
-    static constexpr int A_PLANE = 128 * 128;
-    static constexpr int B_PLANE = NB * 128;
-    static constexpr int PLANES = 4 * A_PLANE + 4 * B_PLANE;
-    static constexpr int BOX = 128 * 128;                  // one box: 128 rows x 16 complex FP32
-    static constexpr int STG = 4 * BOX;                    // one chunk
-    static constexpr size_t SMEM = PLANES + 2 * (size_t)STG + 1024;
-    static constexpr uint32_t TMEM_COLS = 2 * NB <= 32 ? 32 : 2 * NB;
-    static_assert(PLANES % 1024 == 0, "staging boxes must stay 1024-byte aligned");
-    static_assert(NB * 4 <= TCS_SPLIT, "one kernel-row unit per split thread and half chunk");
+struct TcFwdP {
+    static constexpr int BOX = 128 * 128;                    // 128 rows x 8 columns x 2 bins
+    // boxes in flight or being read; a multiple of 4, so that a slot always belongs to the same four split warps:
+    // their wait for one round of the slot then follows their wait for the round before (a warp that skipped a
+    // round would pass the parity test of the next one at once)
+    static constexpr int RING = NB <= 32 ? 8 : 4;
+    static_assert(RING % 4 == 0, "a slot belongs to one group of split warps");
+    static constexpr int B_PLANE = NB * 128;                 // rows b: 32 k of bin 0, 32 k of bin 1
+    static constexpr int B_STAGE = 6 * B_PLANE;              // hi: -Bi, Br, Bi; lo: the same
+    static constexpr int OUT = 16 * 2048;                    // per split warp: 32 rows x 8 columns
+    static constexpr size_t SMEM = RING * (size_t)BOX + 2 * B_STAGE + OUT + 1024;
+    static constexpr int DBUF = NB <= 32 ? 2 : 1;            // sets of accumulators
+    static constexpr int D_COLS = 4 * NB;                    // two bins x (re, im)
+    static constexpr int A_COL = DBUF * D_COLS;              // planes: [stage][bin][plane][16 columns]
+    static_assert(A_COL + 256 <= 512, "accumulators and two stages of A planes fill the tensor memory");
+    static_assert(SMEM <= 232448, "one CTA per SM");
 };
 
-struct FwdTile {
-    int f, v0, b0;
+struct FwdUnit {
+    int f, v0, b0;   // first bin of the pair, first row, first batch column
 };
 template <int NB>
-__device__ __forceinline__ FwdTile fwd_tile(int t, int gx, int gy) {
+__device__ __forceinline__ FwdUnit fwd_unit(int t, int gx, int gy) {
     const int vt = t % gx, r = t / gx;
-    return FwdTile{r / gy, vt * 128, (r % gy) * NB};
+    return FwdUnit{2 * (r / gy), vt * 128, (r % gy) * NB};
 }
 
 __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(bar)) : "memory");
 }
+// A from tensor memory
+__device__ __forceinline__ void umma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem),
+        "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate));
+}
+__device__ __forceinline__ void tmem_st4(uint32_t taddr, uint4 v) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};\n" ::"r"(taddr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w));
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory"); }
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
+    uint32_t r[8];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
 
-template <int NB>
-__global__ void __launch_bounds__(TCS_THREADS, 1)
-    k_tc_fwd_stream(GemmArgs a, const __grid_constant__ CUtensorMap tmap, int gx, int gy, int n_active, int n_tiles) {
-    using G = TcFwdS<NB>;
+__device__ __forceinline__ uint4 neg_bf16x8(uint4 v) {
+    return make_uint4(v.x ^ 0x80008000u, v.y ^ 0x80008000u, v.z ^ 0x80008000u, v.w ^ 0x80008000u);
+}
+
+// which part of a symmetric model's spectra a chunk (columns k0 .. k0 + 31 of rows v0 .. v0 + 127) lies in
+enum { CH_DIRECT = 0, CH_TRANSPOSED = 1, CH_MIXED = 2 };
+template <bool SYM>
+__device__ __forceinline__ int chunk_kind(const GemmArgs &a, int v0, int k0) {
+    if (!SYM) return CH_DIRECT;
+    const int vl = min(v0 + 127, a.nv - 1);
+    if (k0 + TCP_KC <= a.sym_tr * (v0 / a.sym_tr)) return CH_TRANSPOSED;
+    return k0 >= a.sym_tr * (vl / a.sym_tr) ? CH_DIRECT : CH_MIXED;
+}
+
+template <int NB, bool SYM>
+__global__ void __launch_bounds__(TCP_THREADS, 1)
+    k_tc_fwd_p(GemmArgs a, const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap tmap_t, int gx, int gy,
+               int nf, int nf_act, int n_units) {
+    using G = TcFwdP<NB>;
     extern __shared__ uint8_t tc_raw[];
-    __shared__ uint64_t full[2];    // copies into staging buffer 0 / 1 landed
-    __shared__ uint64_t ready[2];   // planes of half 0 / 1 written (one arrive per split warp)
-    __shared__ uint64_t done[2];    // products of half 0 / 1 finished
+    __shared__ uint64_t full[G::RING], empty[G::RING], aready[2], adone[2], ddone[G::DBUF], dfree[G::DBUF], probe;
     __shared__ uint32_t tmem_holder;
-    __shared__ int fail, s_issued, s_last[2];
-    uint8_t *planes = align1024(tc_raw);
-    uint8_t *stg0 = planes + G::PLANES;
+    __shared__ int fail, s_copies, s_mma;      // copies and stages of products issued, for the failure path
+    uint8_t *stg0 = align1024(tc_raw);
+    uint8_t *bpl0 = stg0 + G::RING * G::BOX;
+    uint8_t *out0 = bpl0 + 2 * G::B_STAGE;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
-    for (int t = n_active + blockIdx.x; t < n_tiles; t += gridDim.x) {   // above the band limit
-        const FwdTile T = fwd_tile<NB>(t, gx, gy);
-        zero_tile(a.C + (long long)T.f * a.sCf, a.ldb, T.v0, 128, T.b0, NB, a.nv, a.nb);
-    }
-    const int my_tiles = (int)blockIdx.x < n_active ? (n_active - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
-    if (my_tiles == 0) return;
-    const int nk = (a.nr + 63) / 64;
-    const int nchunks = my_tiles * nk;
+    // bins above the band limit: zero products (pairs that hold an active bin are handled with their unit)
+    if (nf_act < nf)
+        for (int t = gx * gy * ((nf_act + 1) / 2) + blockIdx.x; t < gx * gy * ((nf + 1) / 2); t += gridDim.x) {
+            const FwdUnit U = fwd_unit<NB>(t, gx, gy);
+            for (int f = U.f; f < min(U.f + 2, nf); ++f)
+                zero_tile(a.C + spec_bin(f, a.sCf), (long long)a.ldb * SPEC_F, U.v0, 128, U.b0, NB, a.nv, a.nb);
+        }
+    const int rounds = n_units / (int)gridDim.x;   // whole rounds; unit i of this CTA is i gridDim + (blockIdx + i) % gridDim
+    const int my_units = rounds + (((int)blockIdx.x + rounds) % (int)gridDim.x < n_units % (int)gridDim.x ? 1 : 0);
+    if (my_units == 0) return;
+    const int nk = (a.nr + TCP_KC - 1) / TCP_KC;
 
     if (tid == 0) {
-        for (int i = 0; i < 2; ++i) {
+        for (int i = 0; i < G::RING; ++i) {
             mbar_init(&full[i], 1);
-            mbar_init(&ready[i], TCS_SPLIT / 32);
-            mbar_init(&done[i], 1);
+            mbar_init(&empty[i], 4);   // the four split warps that read the box
         }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&aready[i], TCP_SPLIT / 32);
+            mbar_init(&adone[i], 1);
+        }
+        for (int i = 0; i < G::DBUF; ++i) {
+            mbar_init(&ddone[i], 1);
+            mbar_init(&dfree[i], TCP_SPLIT / 32);
+        }
+        mbar_init(&probe, 1);
         fail = 0;
-        s_issued = 0;
-        s_last[0] = s_last[1] = -1;
+        s_copies = s_mma = 0;
         fence_mbar_init();
     }
-    if (warp == 0) tmem_alloc(&tmem_holder, G::TMEM_COLS);
+    if (warp == 0) tmem_alloc(&tmem_holder, 512);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_holder;
+    // failure-path check: before any copy or product, wait on a barrier that nothing arrives on for a short limit
+    if (a.wait_probe > 0) {
+        if (tid == 0 && !mbar_wait_limit(&probe, 0, a.wait_probe)) fail = 1;
+        __syncthreads();
+    }
+    volatile int *vfail = &fail;
+    auto unit_at = [&](int u) { return fwd_unit<NB>(u * (int)gridDim.x + (int)((blockIdx.x + u) % gridDim.x), gx, gy); };
 
-    if (warp == TCS_SPLIT / 32) {
-        // ---------------- control warp ----------------
+    if (*vfail) {
+        // nothing was issued
+    } else if (warp == TCP_SPLIT / 32) {
+        // ---------------- copy warp ----------------
         if (lane == 0) {
-            constexpr uint32_t idp = umma_idesc(128, NB, 0, 0, 0), idn = umma_idesc(128, NB, 0, 0, 1);
-            auto issue = [&](int g) {   // four boxes of chunk g into staging buffer g & 1
-                const FwdTile T = fwd_tile<NB>((int)blockIdx.x + (g / nk) * (int)gridDim.x, gx, gy);
-                const int k0 = (g % nk) * 64;
-                uint8_t *stg = stg0 + (g & 1) * G::STG;
-                mbar_arrive_expect_tx(&full[g & 1], (uint32_t)G::STG);
-#pragma unroll
-                for (int j = 0; j < 4; ++j) tma_load_3d(stg + j * G::BOX, &tmap, 2 * k0 + 32 * j, T.v0, T.f, &full[g & 1]);
-                s_issued = g + 1;
-            };
-            issue(0);
-            if (nchunks > 1) issue(1);
-            for (int g = 0; g < nchunks; ++g) {
-                const int kc = g % nk;
-                for (int h = 0; h < 2; ++h) {
-                    if (!mbar_wait_bounded(&ready[h], g & 1)) {
-                        fail = 1;
-                        break;
-                    }
-                    tc_fence_after();
-#pragma unroll
-                    for (int k2 = 0; k2 < 2; ++k2) {
-                        const int ks = 2 * h + k2;
-                        uint64_t ad[4], bd[4];
-#pragma unroll
-                        for (int p = 0; p < 4; ++p) {
-                            ad[p] = umma_desc(smem_u32(planes + p * G::A_PLANE + ks * 32), 16, 1024);
-                            bd[p] = umma_desc(smem_u32(planes + 4 * G::A_PLANE + p * G::B_PLANE + ks * 32), 16, 1024);
+            int n = 0, slot = 0, round = 0;   // box, its ring slot, times around the ring
+            for (int u = 0; u < my_units && !*vfail; ++u) {
+                const FwdUnit U = unit_at(u);
+                const int pr = (U.f % SPEC_F) / 2, fb = U.f / SPEC_F;
+                for (int kc = 0; kc < nk && !*vfail; ++kc) {
+                    const int k0 = kc * TCP_KC, kind = chunk_kind<SYM>(a, U.v0, k0);
+                    for (int j = 0; j < 4; ++j) {
+                        if (round > 0 && !mbar_wait_bounded(&empty[slot], (round - 1) & 1)) fail = 1;
+                        if (*vfail) break;
+                        if (SYM && kind == CH_MIXED) {
+                            mbar_arrive(&full[slot]);
+                        } else {
+                            mbar_arrive_expect_tx(&full[slot], (uint32_t)G::BOX);
+                            if (SYM && kind == CH_TRANSPOSED) tma_load_5d(stg0 + slot * G::BOX, &tmap_t, 0, pr, U.v0 / 8, k0 + 8 * j, fb, &full[slot]);
+                            else tma_load_5d(stg0 + slot * G::BOX, &tmap, 0, pr, k0 / 8 + j, U.v0, fb, &full[slot]);
                         }
-                        mma_complex_split(tmem, tmem + NB, ad, bd, idp, idn, (kc > 0 || ks > 0) ? 1u : 0u);
+                        s_copies = ++n;
+                        if (++slot == G::RING) {
+                            slot = 0;
+                            ++round;
+                        }
                     }
-                    umma_commit(&done[h]);
-                    s_last[h] = g;
                 }
-                if (*(volatile int *)&fail) break;
-                if (g + 2 < nchunks) issue(g + 2);   // staging buffer g & 1: both halves split
+            }
+        }
+    } else if (warp == TCP_SPLIT / 32 + 1) {
+        // ---------------- MMA warp ----------------
+        if (lane == 0) {
+            constexpr uint32_t id = umma_idesc(128, 2 * NB, 0, 0, 0);
+            const uint64_t bd0 = umma_desc(smem_u32(bpl0), 16, 1024);
+            constexpr uint64_t PL = G::B_PLANE >> 4;
+            int g = 0;
+            for (int u = 0; u < my_units; ++u) {
+                const int db = u % G::DBUF;
+                if (u >= G::DBUF && !mbar_wait_bounded(&dfree[db], (u / G::DBUF - 1) & 1)) fail = 1;
+                for (int kc = 0; kc < nk; ++kc, ++g) {
+                    const int s = g & 1;
+                    if (!*vfail && !mbar_wait_bounded(&aready[s], (g / 2) & 1)) fail = 1;
+                    if (*vfail) break;
+                    tc_fence_after();
+                    const uint64_t bs = bd0 + (uint64_t)s * (G::B_STAGE >> 4);
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {   // the two bins
+                        const uint32_t d = tmem + db * G::D_COLS + h * 2 * NB;
+#pragma unroll
+                        for (int ks = 0; ks < 2; ++ks) {
+                            const uint32_t ad = tmem + G::A_COL + s * 128 + h * 64 + ks * 8;   // re hi, re lo, im hi, im lo 16 apart
+                            const uint64_t bd = bs + h * 4 + ks * 2;                          // planes -Bi, Br, Bi of hi, then of lo
+                            umma_bf16_ts(d, ad, bd + PL, id, (kc > 0 || ks > 0) ? 1u : 0u);
+                            umma_bf16_ts(d, ad, bd + 4 * PL, id, 1);
+                            umma_bf16_ts(d, ad + 16, bd + PL, id, 1);
+                            umma_bf16_ts(d, ad + 32, bd, id, 1);
+                            umma_bf16_ts(d, ad + 32, bd + 3 * PL, id, 1);
+                            umma_bf16_ts(d, ad + 48, bd, id, 1);
+                        }
+                    }
+                    umma_commit(&adone[s]);
+                    if (kc == nk - 1) umma_commit(&ddone[db]);
+                    s_mma = g + 1;
+                }
+                if (*vfail) break;
             }
         }
     } else {
         // ---------------- split warps ----------------
-        auto load_b = [&](int g, float2 (&zb)[2][8]) {
-            // thread u < 4 NB: kernel row u / 4, 8 complex at columns 8 (4h + u % 4) of halves h = 0, 1
-            // (an index out of range sets status bit 1 and gives a zero row)
-            if (tid >= NB * 4) return;
-            const FwdTile T = fwd_tile<NB>((int)blockIdx.x + (g / nk) * (int)gridDim.x, gx, gy);
-            const int k0 = (g % nk) * 64, row = tid >> 2, c = tid & 3, b = T.b0 + row;
-            const float2 *Df = a.Dh + (long long)T.f * a.sDf;
-            int s = -1;
-            if (b < a.nb) {
-                s = a.idx[b];
-                if (s < 0 || s >= a.ns) {
-                    atomicOr(a.status, 1);
-                    s = -1;
-                }
+        const int q = warp & 3, cc = warp >> 2, m = 32 * q + lane;   // rows 32q .., columns 8cc .. of a chunk
+        const uint32_t lanes = (uint32_t)(32 * q) << 16;
+        auto failed = [&] { return __any_sync(0xffffffffu, *vfail) != 0; };   // warp-uniform
+        // thread u < 8 NB: kernel row u / 8, bin (u % 8) / 4, columns 8 (u % 4) .. of a chunk
+        const bool has_b = tid < NB * 8;
+        const int brow = tid >> 3, bc = tid & 7;
+        const float2 *brp = nullptr;   // this thread's kernel row, for the unit of the next load
+        auto b_row = [&](const FwdUnit &U) {
+            brp = nullptr;
+            if (!has_b || U.b0 + brow >= a.nb) return;
+            const int s = a.idx[U.b0 + brow], f = U.f + (bc >> 2);
+            if (s < 0 || s >= a.ns) {
+                atomicOr(a.status, 1);
+                return;
             }
-            const float2 *rowp = s >= 0 ? Df + (long long)s * a.ldr : nullptr;
-            load8(rowp, k0 + 8 * c, a.nr, zb[0]);
-            load8(rowp, k0 + 32 + 8 * c, a.nr, zb[1]);
+            if (f < nf_act) brp = a.Dh + (long long)f * a.sDf + (long long)s * a.ldd;
         };
-        float2 zb[2][8];
-        load_b(0, zb);
-        for (int g = 0; g < nchunks; ++g) {
-            const int kc = g % nk;
-            const uint8_t *stg = stg0 + (g & 1) * G::STG;
-            if (!mbar_wait_bounded(&full[g & 1], (g >> 1) & 1)) fail = 1;   // chunk g staged
-            for (int h = 0; h < 2 && !*(volatile int *)&fail; ++h) {
-                if (g > 0 && !mbar_wait_bounded(&done[h], (g - 1) & 1)) {     // bytes of half h free
-                    fail = 1;
-                    break;
-                }
-                tc_fence_after();
-                // units (row m, 8 complex c), c in 4h .. 4h+3: box c / 2, granules 4 (c % 2) .. +3 of
-                // the row, each stored at granule ^ (m % 8)
-                const int m = tid & 127, c = 4 * h + (tid >> 7);
-                const uint8_t *row = stg + (c >> 1) * G::BOX + m * 128;
-                float2 z[8];
+        auto epilogue = [&](int u) {
+            const FwdUnit U = unit_at(u);
+            const int db = u % G::DBUF;
+            if (!mbar_wait_bounded(&ddone[db], (u / G::DBUF) & 1)) fail = 1;
+            if (failed()) return;
+            tc_fence_after();
+            uint8_t *out = out0 + warp * 2048;
+            // 8 columns of one bin at a time: TMEM -> 32 rows x 64 bytes -> rows of C
+            for (int e = cc; e < 2 * (NB / 8); e += 4) {
+                const int h = e & 1, c0 = (e >> 1) * 8, f = U.f + h;
+                float re[8], im[8];
+                const uint32_t d = tmem + lanes + db * G::D_COLS + h * 2 * NB + c0;
+                tmem_ld8(d, re);
+                tmem_ld8(d + NB, im);
+                const bool live = f < nf_act;   // (a band limit may cut the pair)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const float4 w = *reinterpret_cast<const float4 *>(row + (((4 * (c & 1) + j) ^ (m & 7)) << 4));
-                    z[2 * j] = make_float2(w.x, w.y);
-                    z[2 * j + 1] = make_float2(w.z, w.w);
+                for (int j = 0; j < 4; ++j)
+                    *reinterpret_cast<float4 *>(out + lane * 64 + ((j ^ ((lane >> 1) & 3)) << 4)) =
+                        live ? make_float4(re[2 * j], im[2 * j], re[2 * j + 1], im[2 * j + 1]) : make_float4(0.f, 0.f, 0.f, 0.f);
+                __syncwarp();
+                if (f < nf) {
+                    const int b = U.b0 + c0 + 2 * (lane & 3);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int row = 8 * i + (lane >> 2), v = U.v0 + 32 * q + row;
+                        const float4 w = *reinterpret_cast<const float4 *>(out + row * 64 + (((lane & 3) ^ ((row >> 1) & 3)) << 4));
+                        float2 *dst = a.C + spec_bin(f, a.sCf) + (long long)v * a.ldb * SPEC_F + spec_col(b);
+                        if (v < a.nv) {
+                            if (b + 1 < a.nb) *reinterpret_cast<float4 *>(dst) = w;
+                            else if (b < a.nb) *dst = make_float2(w.x, w.y);
+                        }
+                    }
                 }
-                store_planes(planes, m * 128 + ((c ^ (m & 7)) << 4), G::A_PLANE, split8(z, false));
-                if (tid < NB * 4) {
-                    const int brow = tid >> 2, bc = 4 * h + (tid & 3);
-                    store_planes(planes + 4 * G::A_PLANE, brow * 128 + ((bc ^ (brow & 7)) << 4), G::B_PLANE,
-                                 split8(zb[h], false));
+                __syncwarp();
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&dfree[db]);
+        };
+
+        float2 zb[8];
+        FwdUnit U = unit_at(0);
+        b_row(U);
+        load8(brp, 8 * (bc & 3), a.nr, zb);
+        int g = 0, slot = cc, round = 0;   // chunk, ring slot of this warp's box, times around the ring
+        for (int u = 0; u < my_units; ++u) {
+            for (int kc = 0; kc < nk; ++kc, ++g) {
+                const int s = g & 1, k0 = kc * TCP_KC;
+                const int kind = chunk_kind<SYM>(a, U.v0, k0);
+                const uint8_t *box = stg0 + slot * G::BOX;
+                const int left = a.nr - (k0 + 8 * cc);   // columns of this thread inside the matrix (past it: padding)
+                float2 z[2][8];
+                if (!mbar_wait_bounded(&full[slot], round & 1)) fail = 1;
+                if (!SYM || kind == CH_DIRECT) {
+                    const uint8_t *row = box + m * 128;
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const float4 w = *reinterpret_cast<const float4 *>(row + ((j ^ (m & 7)) << 4));
+                        z[j >> 2][2 * (j & 3)] = make_float2(w.x, w.y);
+                        z[j >> 2][2 * (j & 3) + 1] = make_float2(w.z, w.w);
+                    }
+                } else if (kind == CH_TRANSPOSED) {
+                    // row k of the box: 128 columns v in chunks of 8, both bins
+                    const int x = (m >> 3) & 7;
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            z[h][i] = *reinterpret_cast<const float2 *>(box + i * 2048 + (m >> 3) * 128 +
+                                                                        (((h * 4 + ((m & 7) >> 1)) ^ x) << 4) + (m & 1) * 8);
+                } else {
+                    const int v = U.v0 + m;
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) z[h][i] = make_float2(0.f, 0.f);
+                    if (v < a.nv) {
+                        const int lo = a.sym_tr * (v / a.sym_tr);
+                        for (int h = 0; h < 2; ++h)   // (the second bin of the last pair lies in the padding of its block)
+                            load8_sym(a.A + spec_bin(U.f + h, a.sAf), (long long)a.ldr * SPEC_F, v, k0 + 8 * cc, a.nr, lo, z[h]);
+                    }
                 }
+                if (left < 8) {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            if (i >= left) z[h][i] = make_float2(0.f, 0.f);
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&empty[slot]);   // the box has been read
+                slot += 4;
+                if (slot >= G::RING) {
+                    slot -= G::RING;
+                    ++round;
+                }
+                if (g >= 2 && !mbar_wait_bounded(&adone[s], (g / 2 - 1) & 1)) fail = 1;   // planes of stage s free
+                if (failed()) break;
+                tc_fence_after();
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const Chunk4 c = split8(z[h], false);
+                    const uint32_t col = tmem + lanes + G::A_COL + s * 128 + h * 64 + (cc >> 1) * 8 + (cc & 1) * 4;
+                    tmem_st4(col, c.rh);
+                    tmem_st4(col + 16, c.rl);
+                    tmem_st4(col + 32, c.ih);
+                    tmem_st4(col + 48, c.il);
+                }
+                if (has_b) {
+                    const Chunk4 c = split8(zb, false);
+                    uint8_t *p = bpl0 + s * G::B_STAGE + brow * 128 + ((bc ^ (brow & 7)) << 4);
+                    *reinterpret_cast<uint4 *>(p) = neg_bf16x8(c.ih);
+                    *reinterpret_cast<uint4 *>(p + G::B_PLANE) = c.rh;
+                    *reinterpret_cast<uint4 *>(p + 2 * G::B_PLANE) = c.ih;
+                    *reinterpret_cast<uint4 *>(p + 3 * G::B_PLANE) = neg_bf16x8(c.il);
+                    *reinterpret_cast<uint4 *>(p + 4 * G::B_PLANE) = c.rl;
+                    *reinterpret_cast<uint4 *>(p + 5 * G::B_PLANE) = c.il;
+                }
+                tmem_wait_st();
                 fence_async_smem();
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&ready[h]);
-            }
-            if (*(volatile int *)&fail) break;
-            if (g + 1 < nchunks) load_b(g + 1, zb);
-            if (kc == nk - 1) {
-                // the tile's epilogue: done[1] of this chunk follows every earlier product
-                if (!mbar_wait_bounded(&done[1], g & 1)) {
-                    fail = 1;
-                    break;
+                if (lane == 0) mbar_arrive(&aready[s]);
+                // kernel rows of the next chunk
+                if (kc + 1 < nk) {
+                    load8(brp, k0 + TCP_KC + 8 * (bc & 3), a.nr, zb);
+                } else if (u + 1 < my_units) {
+                    U = unit_at(u + 1);
+                    b_row(U);
+                    load8(brp, 8 * (bc & 3), a.nr, zb);
                 }
-                tc_fence_after();
-                const FwdTile T = fwd_tile<NB>((int)blockIdx.x + (g / nk) * (int)gridDim.x, gx, gy);
-                const int q = warp & 3, cc = warp >> 2;   // TMEM lanes 32q.., columns 16cc..
-                if (16 * cc < NB) {
-                    const int v = T.v0 + 32 * q + lane, c0 = 16 * cc;
-                    float re[16], im[16];
-                    tmem_ld16(tmem + ((uint32_t)(32 * q) << 16) + c0, re);
-                    tmem_ld16(tmem + ((uint32_t)(32 * q) << 16) + NB + c0, im);
-                    if (v < a.nv) {
-                        float2 *Crow = a.C + (long long)T.f * a.sCf + (long long)v * a.ldb + T.b0 + c0;
-#pragma unroll
-                        for (int j = 0; j < 16; ++j)
-                            if (T.b0 + c0 + j < a.nb) Crow[j] = make_float2(re[j], im[j]);
-                    }
-                }
-                tc_fence_before();   // the next tile's first products overwrite the accumulators
+                if (kc == 0 && u > 0) epilogue(u - 1);
             }
+            if (failed()) break;
         }
+        if (!failed()) epilogue(my_units - 1);
     }
     __syncthreads();
-    if (fail) {
-        // copies and products still in flight get one more bounded wait before the CTA frees TMEM
-        // and exits
-        if (tid == 0) {
-            for (int i = max(0, s_issued - 2); i < s_issued; ++i) mbar_wait_bounded(&full[i & 1], (i >> 1) & 1);
-            for (int h = 0; h < 2; ++h)
-                if (s_last[h] >= 0) mbar_wait_bounded(&done[h], s_last[h] & 1);
-            atomicOr(a.status, 2);
-        }
+    if (fail && tid == 0) {
+        // copies and products still in flight get one more bounded wait before the CTA frees TMEM and exits
+        for (int i = max(0, s_copies - G::RING); i < s_copies; ++i) mbar_wait_bounded(&full[i % G::RING], (i / G::RING) & 1);
+        for (int i = max(0, s_mma - 2); i < s_mma; ++i) mbar_wait_bounded(&adone[i & 1], (i / 2) & 1);
+        atomicOr(a.status, 2);
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem, G::TMEM_COLS);
+    if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -925,9 +1099,12 @@ cudaError_t tc_prepare() {
     if ((e = cudaFuncSetAttribute(k_tc_fwd<16, TC_FWD_STAGES, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcFwd<16, TC_FWD_STAGES>::SMEM))) return e;
     if ((e = cudaFuncSetAttribute(k_tc_fwd<32, TC_FWD_STAGES, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcFwd<32, TC_FWD_STAGES>::SMEM))) return e;
     if ((e = cudaFuncSetAttribute(k_tc_fwd<64, TC_FWD_STAGES, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcFwd<64, TC_FWD_STAGES>::SMEM))) return e;
-    if ((e = cudaFuncSetAttribute(k_tc_fwd_stream<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcFwdS<16>::SMEM))) return e;
-    if ((e = cudaFuncSetAttribute(k_tc_fwd_stream<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcFwdS<32>::SMEM))) return e;
-    if ((e = cudaFuncSetAttribute(k_tc_fwd_stream<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcFwdS<64>::SMEM))) return e;
+    if ((e = cudaFuncSetAttribute(k_tc_fwd_p<16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcFwdP<16>::SMEM))) return e;
+    if ((e = cudaFuncSetAttribute(k_tc_fwd_p<16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcFwdP<16>::SMEM))) return e;
+    if ((e = cudaFuncSetAttribute(k_tc_fwd_p<32, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcFwdP<32>::SMEM))) return e;
+    if ((e = cudaFuncSetAttribute(k_tc_fwd_p<32, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcFwdP<32>::SMEM))) return e;
+    if ((e = cudaFuncSetAttribute(k_tc_fwd_p<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcFwdP<64>::SMEM))) return e;
+    if ((e = cudaFuncSetAttribute(k_tc_fwd_p<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcFwdP<64>::SMEM))) return e;
     if ((e = cudaFuncSetAttribute(k_tc_adj<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcAdj::SMEM))) return e;
     if ((e = cudaFuncSetAttribute(k_tc_adj<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcAdj::SMEM))) return e;
     if ((e = cudaFuncSetAttribute(k_tc_adj_tma<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcAdj::SMEM))) return e;
@@ -959,10 +1136,10 @@ cudaError_t launch_tc_fwd(const GemmArgs &a, int nf, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-// Tensor map of the model spectra [nf][nv][ldr] complex, seen as FP32 [nf][nv][2 nr] (the padding
-// column of an odd nr lies outside it): boxes of 32 floats x 128 rows x 1 bin, 128-byte swizzle,
-// zero fill outside the tensor.  The encoder is taken from the driver at run time.
-cudaError_t tc_encode_fwd_map(void *map_out, const float2 *Xh, int nr, int nv, int ldr, int nf) {
+// Tensor maps of the model spectra in the SPEC_F layout, seen as FP32 [nf / F][nv][ceil(nr / 8)][F / BB][16 BB] with
+// BB bins in a box: boxes of 8 columns x BB bins times `cblk` column blocks times `rows` rows, swizzled over their
+// 64 BB bytes, zero fill outside the tensor (the padding columns of the last block of 8 lie inside it).
+static cudaError_t encode_map(void *map_out, const float2 *Xh, int nr, int nv, int ldr, int nf, int bb, int cblk, int rows) {
     static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
     if (!encode) {
         void *fn = nullptr;
@@ -972,32 +1149,44 @@ cudaError_t tc_encode_fwd_map(void *map_out, const float2 *Xh, int nr, int nv, i
         if (q != cudaDriverEntryPointSuccess || !fn) return cudaErrorNotSupported;
         encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
     }
-    const cuuint64_t dims[3] = {(cuuint64_t)2 * nr, (cuuint64_t)nv, (cuuint64_t)nf};
-    const cuuint64_t strides[2] = {(cuuint64_t)ldr * 8, (cuuint64_t)nv * ldr * 8};
-    const cuuint32_t box[3] = {32, 128, 1}, estr[3] = {1, 1, 1};
-    const CUresult r = encode(reinterpret_cast<CUtensorMap *>(map_out), CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3,
+    const cuuint64_t row = (cuuint64_t)ldr * SPEC_F * 8;
+    const cuuint64_t dims[5] = {(cuuint64_t)16 * bb, (cuuint64_t)SPEC_F / bb, (cuuint64_t)(nr + 7) / 8, (cuuint64_t)nv, (cuuint64_t)spec_blocks(nf)};
+    const cuuint64_t strides[4] = {(cuuint64_t)64 * bb, 64 * SPEC_F, row, row * nv};
+    const cuuint32_t box[5] = {(cuuint32_t)16 * bb, 1, (cuuint32_t)cblk, (cuuint32_t)rows, 1}, estr[5] = {1, 1, 1, 1, 1};
+    const CUresult r = encode(reinterpret_cast<CUtensorMap *>(map_out), CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 5,
                               const_cast<float2 *>(Xh), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                              CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                              bb == 2 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-cudaError_t launch_tc_fwd_stream(const GemmArgs &a, const void *map, int nf, cudaStream_t st) {
+cudaError_t tc_encode_maps(TcMaps *m, const float2 *Xh, int nr, int nv, int ldr, int nf) {
+    cudaError_t e = encode_map(m->fwd, Xh, nr, nv, ldr, nf, 2, 1, 128);
+    if (e == cudaSuccess) e = encode_map(m->fwd_t, Xh, nr, nv, ldr, nf, 2, 16, 8);
+    if (e == cudaSuccess) e = encode_map(m->adj, Xh, nr, nv, ldr, nf, 1, 1, 128);
+    return e;
+}
+
+template <int NB>
+static cudaError_t launch_fwd_p(const GemmArgs &a, const TcMaps &maps, int nf, int sms, cudaStream_t st) {
+    CUtensorMap m, mt;
+    memcpy(&m, maps.fwd, sizeof(m));
+    memcpy(&mt, maps.fwd_t, sizeof(mt));
+    const int gx = (a.nv + 127) / 128, gy = (a.nb + NB - 1) / NB;
+    const int nf_act = (a.nf_active > 0 && a.nf_active < nf) ? a.nf_active : nf;
+    const int n_units = (nf_act + 1) / 2 * gx * gy;
+    const int grid = std::max(1, std::min(std::max(n_units, (nf + 1) / 2 * gx * gy), sms));
+    if (a.sym_tr > 0) k_tc_fwd_p<NB, true><<<grid, TCP_THREADS, TcFwdP<NB>::SMEM, st>>>(a, m, mt, gx, gy, nf, nf_act, n_units);
+    else k_tc_fwd_p<NB, false><<<grid, TCP_THREADS, TcFwdP<NB>::SMEM, st>>>(a, m, mt, gx, gy, nf, nf_act, n_units);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_tc_fwd_p(const GemmArgs &a, const TcMaps &maps, int nf, cudaStream_t st) {
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    CUtensorMap tmap;
-    memcpy(&tmap, map, sizeof(tmap));
-    const int gx = (a.nv + 127) / 128;
-    const int nb_tile = a.nb <= 16 ? 16 : a.nb <= 32 ? 32 : 64;
-    const int gy = (a.nb + nb_tile - 1) / nb_tile;
-    const int nf_act = (a.nf_active > 0 && a.nf_active < nf) ? a.nf_active : nf;
-    const int n_active = nf_act * gx * gy, n_tiles = nf * gx * gy;
-    const int grid = std::max(1, std::min(n_tiles, sms));
-    if (nb_tile == 16) k_tc_fwd_stream<16><<<grid, TCS_THREADS, TcFwdS<16>::SMEM, st>>>(a, tmap, gx, gy, n_active, n_tiles);
-    else if (nb_tile == 32) k_tc_fwd_stream<32><<<grid, TCS_THREADS, TcFwdS<32>::SMEM, st>>>(a, tmap, gx, gy, n_active, n_tiles);
-    else k_tc_fwd_stream<64><<<grid, TCS_THREADS, TcFwdS<64>::SMEM, st>>>(a, tmap, gx, gy, n_active, n_tiles);
-    return cudaGetLastError();
+    return a.nb <= 16 ? launch_fwd_p<16>(a, maps, nf, sms, st) : a.nb <= 32 ? launch_fwd_p<32>(a, maps, nf, sms, st) : launch_fwd_p<64>(a, maps, nf, sms, st);
 }
 
 int tc_fwd_queue_nb(int nb) { return nb <= 16 ? 16 : nb <= 32 ? 32 : 64; }

@@ -145,7 +145,7 @@ extern "C" int mdc_forward_static(int nt, int nr, int nv, int ns, float scale, c
     // kernel spectra of every source: D [ns][nr][nt] -> Dh [nf][ns][ldr]
     a.g.ni = nr; a.g.nj = ns; a.g.ti_log2 = ti_log2(nr);
     a.g.tsi = nt; a.g.tsj = (long long)nr * nt;
-    a.g.ssi = 1; a.g.ssj = ldr; a.g.ssf = (long long)ns * ldr;
+    a.g.fl2 = 0; a.g.ssj = ldr; a.g.ssf = (long long)ns * ldr;
     a.tin = D;
     a.vec = time_vec(nt, D);
     a.spec = Dh;
@@ -160,7 +160,8 @@ extern "C" int mdc_forward_static(int nt, int nr, int nv, int ns, float scale, c
     GemmArgs g;
     memset(&g, 0, sizeof(g));
     g.A = Xh; g.Dh = Dh; g.idx = idx; g.C = Uh;
-    g.nv = nv; g.nr = nr; g.ns = ns; g.nb = nb; g.ldr = ldr; g.ldb = ldb;
+    g.nv = nv; g.nr = nr; g.ns = ns; g.nb = nb; g.ldr = ldr; g.ldb = ldb; g.ldd = ldr;
+    g.plain = 1;
     g.sAf = (long long)nv * ldr; g.sDf = (long long)ns * ldr; g.sCf = (long long)nv * ldb;
     g.outscale = 1.f;
     g.status = status;
@@ -169,7 +170,7 @@ extern "C" int mdc_forward_static(int nt, int nr, int nv, int ns, float scale, c
     FftArgs o = a;
     o.g.ni = nb; o.g.nj = nv; o.g.ti_log2 = ti_log2(nb);
     o.g.tsi = (long long)nv * nt; o.g.tsj = nt;
-    o.g.ssi = 1; o.g.ssj = ldb; o.g.ssf = (long long)nv * ldb;
+    o.g.ssj = ldb; o.g.ssf = (long long)nv * ldb;
     o.tin = nullptr;
     o.tout = U;
     o.vec = time_vec(nt, U);

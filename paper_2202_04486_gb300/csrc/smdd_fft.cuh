@@ -116,10 +116,7 @@ __device__ __forceinline__ C2 ldsC(const float4 *p) {
     return C2{v.x, v.y};
 }
 __device__ __forceinline__ void stsC(float4 *p, C2 v) { *reinterpret_cast<ulonglong2 *>(p) = make_ulonglong2(v.re, v.im); }
-__device__ __forceinline__ W2 ldtw(const float2 *p) {
-    const float2 v = __ldg(p);
-    return W2{dup2(v.x), dup2(v.y)};
-}
+__device__ __forceinline__ W2 wdup(float2 v) { return W2{dup2(v.x), dup2(v.y)}; }
 __device__ __forceinline__ W2 wmul(W2 a, W2 b) {
     return W2{fma2(a.im, neg2(b.im), mul2(a.re, b.re)), fma2(a.re, b.im, mul2(a.im, b.re))};
 }
@@ -305,16 +302,28 @@ __host__ __device__ inline void tw_angle(int M, int i, int &num, int &den) {
     }
 }
 
-// z[r] *= w^r (INV: conj(w)^r), r = 1 .. R - 1, with the root w^{tw_root(i)} at tw[i NS]
-template <int R, int NS, bool INV>
-__device__ __forceinline__ void twiddles(C2 *z, const float2 *__restrict__ tw) {
-    const W2 w1 = ldtw(tw), w2 = ldtw(tw + NS), w3 = ldtw(tw + 2 * NS);
+// The roots w^{tw_root(i)} of one butterfly, loaded ahead of their use (before the barrier in front of the pass, so
+// that the latency of the table loads overlaps it).
+template <int R>
+struct Roots {
+    float2 w[tw_roots(R)];
+    template <int NS>
+    __device__ __forceinline__ void load(const float2 *__restrict__ tw) {
+#pragma unroll
+        for (int i = 0; i < tw_roots(R); ++i) w[i] = __ldg(tw + i * NS);
+    }
+};
+
+// z[r] *= w^r (INV: conj(w)^r), r = 1 .. R - 1
+template <int R, bool INV>
+__device__ __forceinline__ void twiddles(C2 *z, const Roots<R> &t) {
+    const W2 w1 = wdup(t.w[0]), w2 = wdup(t.w[1]), w3 = wdup(t.w[2]);
     z[1] = ctw2<INV>(z[1], w1);
     z[2] = ctw2<INV>(z[2], w2);
     z[3] = ctw2<INV>(z[3], w3);
 #pragma unroll
     for (int i = 1; i < R / 4; ++i) {
-        const W2 w = ldtw(tw + (2 + i) * NS);
+        const W2 w = wdup(t.w[2 + i]);
         z[4 * i] = ctw2<INV>(z[4 * i], w);
         z[4 * i + 1] = ctw2<INV>(z[4 * i + 1], wmul(w, w1));
         z[4 * i + 2] = ctw2<INV>(z[4 * i + 2], wmul(w, w2));
@@ -325,20 +334,10 @@ __device__ __forceinline__ void twiddles(C2 *z, const float2 *__restrict__ tw) {
 // Launch geometry for complex length M: T = M/16 threads per pair of traces, PL pairs interleaved in the lanes,
 // G such groups in a CTA (4 for the lengths whose group is at most a warp: with one, the CTA's fixed work -- the
 // loss reduction and its atomic above all -- costs a third of the residual step at nt 30 to 128).
-#ifndef SMDD_FFT_MINB_1024
-#define SMDD_FFT_MINB_1024 2
-#endif
-#ifndef SMDD_FFT_MINB_1536
-#define SMDD_FFT_MINB_1536 1
-#endif
-#ifndef SMDD_FFT_PL_1536
-#define SMDD_FFT_PL_1536 4
-#endif
-
 template <int M>
 struct Team {
     static constexpr int T = M / FFT_P;
-    static constexpr int PL = M == 4096 ? 2 : M == 1536 ? SMDD_FFT_PL_1536 : 4;
+    static constexpr int PL = M == 4096 ? 2 : 4;
     static constexpr int GT = PL * T;                    // threads of a group
     static constexpr int G = M <= 128 ? 4 : 1;           // groups in a CTA
     static constexpr int THREADS = GT * G;
@@ -346,10 +345,12 @@ struct Team {
     static constexpr int R1 = fft_radix(M, 0), L1 = M / R1;
     static constexpr int ELEMS = R1 * (L1 + 1);          // elements of a pair's buffer (padded)
     static constexpr size_t SMEM = (size_t)ELEMS * PL * G * 16;
-    // resident CTAs per SM asked of the compiler: at most 128 registers per thread
-    static constexpr int MINB = M == 1024 ? SMDD_FFT_MINB_1024
-                              : M == 1536 ? SMDD_FFT_MINB_1536
-                              : THREADS >= 512 ? 1 : 512 / THREADS;
+    // resident CTAs per SM asked of the compiler: 512 threads at 128 registers.  At M = 1536 two CTAs of 384 threads
+    // at 80 registers, although they spill: one CTA leaves the SM idle while it waits for its tile (transform alone
+    // 1410 -> 1090 us, update 2560 -> 2440 us at nt 1500, 600 x 400); the samples that the update or the residual
+    // needs after the inverse transform are then loaded after it (LATE), not held through it.
+    static constexpr int MINB = M == 1536 ? 2 : THREADS >= 512 ? 1 : 512 / THREADS;
+    static constexpr bool LATE = M == 1536;
 };
 
 // Synchronise the threads of a group (a group lies in one warp, or the CTA is one group).
@@ -415,28 +416,33 @@ __device__ __forceinline__ void inv_last(C2 (&a)[FFT_P], const float4 *buf, int 
     }
 }
 
-// middle pass p, in place (a length whose butterflies do not divide by the threads has a partial last round)
+// middle pass p, in place (a length whose butterflies do not divide by the threads has a partial last round); the
+// barrier before it is inside, behind the loads of the roots
 template <int M, bool INV, int p>
 __device__ __forceinline__ void mid_pass(float4 *buf, int s, const float2 *__restrict__ tw) {
     constexpr int R = fft_radix(M, p), L = fft_left(M, p), NS = fft_span(M, p), T = Team<M>::T, PL = Team<M>::PL;
     constexpr int NB = M / R, NQ = (NB + T - 1) / T;
     static_assert(T % L == 0 && L % 4 == 0, "every round of a thread has the same jj");
     const int jj = s % L;
+    Roots<R> t[NQ];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q)
+        t[q].template load<NS>(tw + tw_off(M, p) + ((NB % T == 0 || s + T * q < NB) ? s / L + q * (T / L) : 0));
+    group_sync<M>();
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
         if (NB % T == 0 || s + T * q < NB) {
             const int kk = s / L + q * (T / L);
             float4 *b = buf + (mix<PL>(jj) + digit_off<M>(kk, p)) * PL;
-            const float2 *w = tw + tw_off(M, p) + kk;
             C2 x[R];
 #pragma unroll
             for (int r = 0; r < R; ++r) x[r] = ldsC(b + r * L * PL);
             if constexpr (!INV) {
-                twiddles<R, NS, false>(x, w);
+                twiddles<R, false>(x, t[q]);
                 dftRp<R, false, false>(x);
             } else {
                 dftRp<R, true, false>(x);
-                twiddles<R, NS, true>(x, w);
+                twiddles<R, true>(x, t[q]);
             }
 #pragma unroll
             for (int r = 0; r < R; ++r) stsC(b + r * L * PL, x[r]);
@@ -446,10 +452,9 @@ __device__ __forceinline__ void mid_pass(float4 *buf, int s, const float2 *__res
 
 template <int M, bool INV, int p>
 __device__ __forceinline__ void mid_passes(float4 *buf, int s, const float2 *__restrict__ tw) {
-    // forward: p = 1 .. npass - 2; inverse: p = npass - 2 .. 1; a barrier after each
+    // forward: p = 1 .. npass - 2; inverse: p = npass - 2 .. 1
     if constexpr (p >= 1 && p <= fft_npass(M) - 2) {
         mid_pass<M, INV, p>(buf, s, tw);
-        group_sync<M>();
         mid_passes<M, INV, INV ? p - 1 : p + 1>(buf, s, tw);
     }
 }
@@ -479,11 +484,25 @@ __device__ __forceinline__ void real_post(C2 &x, C2 &y, W2 w) {
 // The bins of thread s: A[r] = bin s + r S and B[r] = bin S - s + r S (S/2 + r S for s = 0), r < 8, S = M / 8; for
 // s = 0 also bin M (its real part goes to `nyq`).
 //
+// roots of the edge pass: of the butterflies of A and B, and of the real-signal processing
+template <int M>
+struct EdgeRoots {
+    Roots<8> a, b;
+    float2 n;   // w_N^s
+    __device__ __forceinline__ void load(const float2 *__restrict__ tw, int s) {
+        constexpr int S = M / 8, P = fft_npass(M) - 1;
+        n = __ldg(tw + twn_off(M) + s);
+        a.template load<S>(tw + tw_off(M, P) + s);
+        b.template load<S>(tw + tw_off(M, P) + (s ? S - s : S / 2));
+    }
+};
+
 // inverse: A, B hold the spectrum; real pre-processing, radix-8 inverse butterflies, twiddles, store
 template <int M>
-__device__ __forceinline__ void edge_inv(C2 (&A)[8], C2 (&B)[8], f32x2 nyq, float4 *buf, int s, const float2 *__restrict__ tw) {
+__device__ __forceinline__ void edge_inv(C2 (&A)[8], C2 (&B)[8], f32x2 nyq, float4 *buf, int s, const float2 *__restrict__ tw,
+                                         const EdgeRoots<M> &t) {
     constexpr int S = M / 8, PL = Team<M>::PL, P = fft_npass(M) - 1;
-    const W2 wn = ldtw(tw + twn_off(M) + s);   // w_N^s
+    const W2 wn = wdup(t.n);
     if (s != 0) {
         real_pre(A[0], B[7], wn);
         real_pre(A[1], B[6], rot16<1>(wn));
@@ -502,31 +521,32 @@ __device__ __forceinline__ void edge_inv(C2 (&A)[8], C2 (&B)[8], f32x2 nyq, floa
         real_pre(A[3], A[5], rot16<3>(wn));
         A[4] = C2{add2(A[4].re, A[4].re), neg2(add2(A[4].im, A[4].im))};
         // B: k = S/2 + r S pairs with S/2 + (7 - r) S
-        const W2 wh = ldtw(tw + twn_off(M) + S / 2);
+        const W2 wh = wdup(__ldg(tw + twn_off(M) + S / 2));
         real_pre(B[0], B[7], wh);
         real_pre(B[1], B[6], rot16<1>(wh));
         real_pre(B[2], B[5], rot16<2>(wh));
         real_pre(B[3], B[4], rot16<3>(wh));
     }
-    const float2 *w = tw + tw_off(M, P);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         C2(&z)[8] = h ? B : A;
         const int u = h ? (s ? S - s : S / 2) : s;
         dft8p<true, false>(z);
-        twiddles<8, S, true>(z, w + u);
+        twiddles<8, true>(z, h ? t.b : t.a);
         float4 *b = buf + digit_off<M>(u, P) * PL;
 #pragma unroll
         for (int r = 0; r < 8; ++r) stsC(b + mix<PL>(r) * PL, z[r]);
     }
 }
 
-// forward: load, twiddles, radix-8 butterflies, real post-processing; on return A, B hold the spectrum, nyq the
+// forward (the barrier in front of it inside): load, twiddles, radix-8 butterflies, real post-processing; on return A, B hold the spectrum, nyq the
 // real part of bin M for s = 0
 template <int M>
 __device__ __forceinline__ void edge_fwd(C2 (&A)[8], C2 (&B)[8], f32x2 &nyq, const float4 *buf, int s, const float2 *__restrict__ tw) {
     constexpr int S = M / 8, PL = Team<M>::PL, P = fft_npass(M) - 1;
-    const float2 *w = tw + tw_off(M, P);
+    EdgeRoots<M> t;
+    t.load(tw, s);
+    group_sync<M>();
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         C2(&z)[8] = h ? B : A;
@@ -534,10 +554,10 @@ __device__ __forceinline__ void edge_fwd(C2 (&A)[8], C2 (&B)[8], f32x2 &nyq, con
         const float4 *b = buf + digit_off<M>(u, P) * PL;
 #pragma unroll
         for (int r = 0; r < 8; ++r) z[r] = ldsC(b + mix<PL>(r) * PL);
-        twiddles<8, S, false>(z, w + u);
+        twiddles<8, false>(z, h ? t.b : t.a);
         dft8p<false, false>(z);
     }
-    const W2 wn = ldtw(tw + twn_off(M) + s);   // w_N^s
+    const W2 wn = wdup(t.n);
     nyq = 0;
     if (s != 0) {
         real_post(A[0], B[7], wn);
@@ -555,7 +575,7 @@ __device__ __forceinline__ void edge_fwd(C2 (&A)[8], C2 (&B)[8], f32x2 &nyq, con
         real_post(A[2], A[6], rot16<2>(wn));
         real_post(A[3], A[5], rot16<3>(wn));
         A[4].im = neg2(A[4].im);
-        const W2 wh = ldtw(tw + twn_off(M) + S / 2);
+        const W2 wh = wdup(__ldg(tw + twn_off(M) + S / 2));
         real_post(B[0], B[7], wh);
         real_post(B[1], B[6], rot16<1>(wh));
         real_post(B[2], B[5], rot16<2>(wh));

@@ -13,14 +13,31 @@ namespace smdd {
 
 enum Stage { ST_RFFT = 0, ST_GEMM_FWD = 1, ST_RESID = 2, ST_GEMM_ADJ = 3, ST_UPDATE = 4, ST_IRFFT_OUT = 5, ST_SETUP = 6 };
 
+// Layout of the spectra of a model ([nv][nr]) or of a batch ([nv][nb]): SPEC_F bins and 8 columns (receivers, batch
+// entries) interleaved, [f / F][row][column / 8][f % F][column % 8] with F = SPEC_F, rows of ld (a multiple of 8)
+// columns.  The trace kernels move the bins of 8 columns: F x 64 contiguous bytes per access; the products read and
+// write 64-byte chunks of one bin, whose neighbours in a 128-byte line belong to bins that run at the same time.
+// With F = 1 (rows of one bin contiguous) the trace kernels' 64-byte segments, each in another 2 MB page for
+// larger problems, cap their rate: 4.7 TB/s at nf 1025, 301 x 304 and 3.6 TB/s at nf 1537, 600 x 600 for a plain
+// read and write, against 6.3 and 5.0 TB/s with F = 4.  (The kernel spectra [f][source][receiver], read by rows, and
+// the static entry point's arrays keep F = 1.)
+constexpr int SPEC_F = 4;
+// column k of a row, and bin f of a row (blk: float2 of one block of F bins)
+template <int F = SPEC_F>
+__host__ __device__ __forceinline__ constexpr int spec_col(int k) { return k + (k & ~7) * (F - 1); }
+template <int F = SPEC_F>
+__host__ __device__ __forceinline__ constexpr long long spec_bin(int f, long long blk) { return (long long)(f / F) * blk + (f % F) * 8; }
+__host__ __device__ constexpr int spec_blocks(int nf) { return (nf + SPEC_F - 1) / SPEC_F; }
+
 // A 2-D grid of time traces and the matching spectra.  Trace (i, j), i < ni, j < nj:
 //   time samples at  tin/tout + i*tsi + j*tsj + t          (floats),  t < nt
-//   spectrum bin f at spec + f*ssf + i*ssi + j*ssj           (float2), f <= M
+//   spectrum bin f at spec + (f / F)*ssf + (f % F)*8 + col(i) + j*ssj   (float2), f <= M, col as spec_col, F = 1 << fl2
 // A CTA owns TR traces: 2^ti_log2 consecutive i times TR >> ti_log2 consecutive j.
 struct TraceGrid {
     int ni, nj, ti_log2;
     long long tsi, tsj;
-    long long ssi, ssj, ssf;
+    long long ssj, ssf;
+    int fl2;
     // 1: only the tiles on or above the block diagonal of a square grid (ni == nj, CTAs of TR traces along
     // i): tile (bi, j) for bi >= j / TR, bi fastest (a symmetric model, see sym_tile_to_full)
     int sym = 0;
@@ -62,8 +79,10 @@ struct GemmArgs {
     const float2 *Dh;        // kernel spectra [nf][ns][ldr]
     const int32_t *idx;
     float2 *C;               // forward: Uh; adjoint: Gh
-    int nv, nr, ns, nb, ldr, ldb;
-    long long sAf, sDf, sCf; // per-frequency strides (float2)
+    int nv, nr, ns, nb;
+    int ldr, ldb, ldd;       // columns per row: model, batch and kernel spectra
+    long long sAf, sDf, sCf; // strides (float2) of a block of bins of A and C, of a bin of Dh
+    int plain;               // forward: A and C in the F = 1 layout (the static entry point)
     float outscale;
     int tiles_v, tiles_r;    // adjoint tile grid
     int *status;
@@ -81,11 +100,13 @@ struct GemmArgs {
 
 // Zero the output tile [r0, r0+nrows) x [c0, c0+ncols) of a CTA whose frequency bin lies above the
 // band limit (inside the matrix bounds rmax x cmax; leading dimension ld).
+// (C: row 0 of the bin, ld: float2 of a row over its bins)
+template <int F = SPEC_F>
 __device__ __forceinline__ void zero_tile(float2 *C, long long ld, int r0, int nrows, int c0, int ncols, int rmax,
                                           int cmax) {
     for (int e = threadIdx.x; e < nrows * ncols; e += blockDim.x) {
         const int i = e / ncols, j = e % ncols, r = r0 + i, c = c0 + j;
-        if (r < rmax && c < cmax) C[(long long)r * ld + c] = make_float2(0.f, 0.f);
+        if (r < rmax && c < cmax) C[(long long)r * ld + spec_col<F>(c)] = make_float2(0.f, 0.f);
     }
 }
 
@@ -102,7 +123,7 @@ struct WorkQueue {
 
 // Symmetric model: X^[f][v][r] <- X^[f][r][v] for every r < TR floor(v / TR) (the part of the spectra below
 // the TR-block diagonal, which the update of a symmetric model leaves unwritten); n = nr = nv
-cudaError_t launch_mirror_lower(float2 *spec, int n, int ld, long long ssf, int nf, int TR, cudaStream_t st);
+cudaError_t launch_mirror_lower(float2 *spec, int n, int ld, int nf, int TR, cudaStream_t st);
 // Number of tiles of the upper enumeration of a square grid of n x n traces with TR traces per CTA along
 // i: row j holds the tiles bi = j / TR .. ceil(n / TR) - 1.
 __host__ __device__ inline long long sym_tiles(int n, int TR) {
@@ -149,12 +170,16 @@ cudaError_t launch_gemv_adj(const GemmArgs &a, int nf, cudaStream_t st);
 // split-BF16 tensor-core products (tcgen05)
 cudaError_t tc_prepare();
 cudaError_t launch_tc_fwd(const GemmArgs &a, int nf, cudaStream_t st);
-// streamed forward product fed by the tensor memory accelerator: map = 128-byte tensor map of the
-// model spectra written by tc_encode_fwd_map (64-byte aligned host memory)
-cudaError_t tc_encode_fwd_map(void *map_out, const float2 *Xh, int nr, int nv, int ldr, int nf);
-cudaError_t launch_tc_fwd_stream(const GemmArgs &a, const void *map, int nf, cudaStream_t st);
-// map (or null): the 128-byte tensor map of the output (tc_encode_fwd_map of the model-spectra buffer):
-// the tile without reciprocity is then written by the tensor memory accelerator
+// tensor maps of the model-spectra buffer (the forward product's boxes, direct and transposed, and the adjoint's
+// output boxes); encoded once per split-BF16 plan
+struct TcMaps {
+    alignas(64) unsigned char fwd[128], fwd_t[128], adj[128];
+};
+cudaError_t tc_encode_maps(TcMaps *m, const float2 *Xh, int nr, int nv, int ldr, int nf);
+// persistent forward product fed by the tensor memory accelerator
+cudaError_t launch_tc_fwd_p(const GemmArgs &a, const TcMaps &maps, int nf, cudaStream_t st);
+// map (or null): the tensor map of the output boxes (TcMaps::adj): tiles written once are then stored by the tensor
+// memory accelerator
 cudaError_t launch_tc_adj(const GemmArgs &a, bool recip, int nf, cudaStream_t st, const void *map = nullptr);
 // Operand images of the split-BF16 adjoint (bytes for a problem; 0 where the batch needs more than two K
 // chunks), and their construction for one step (residual spectra and gathered kernel rows of a.idx).

@@ -61,15 +61,18 @@ __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::
 
 // Wait for the given phase parity of an mbarrier, giving up after `limit` SM clock cycles.
 // Returns false on timeout (the caller records the error and finishes without the result).
+__device__ __forceinline__ bool mbar_try(uint64_t *bar, uint32_t parity) {
+    uint32_t done;
+    asm volatile(
+        "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(done) : "r"(smem_u32(bar)), "r"(parity) : "memory");
+    return done != 0;
+}
 __device__ __forceinline__ bool mbar_wait_limit(uint64_t *bar, uint32_t parity, long long limit) {
-    uint32_t done = 0;
+    if (mbar_try(bar, parity)) return true;   // (the clock is read only where the wait has to go on)
     const long long t0 = clock64();
-    while (!done) {
-        asm volatile(
-            "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
-            : "=r"(done) : "r"(smem_u32(bar)), "r"(parity) : "memory");
-        if (!done && clock64() - t0 > limit) return false;
-    }
+    while (!mbar_try(bar, parity))
+        if (clock64() - t0 > limit) return false;
     return true;
 }
 
@@ -83,24 +86,24 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t by
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
 }
 
-// Tiled copy of one box of a 3D tensor by the tensor memory accelerator into this CTA's shared memory
+// Tiled copy of one box of a 5D tensor by the tensor memory accelerator into this CTA's shared memory
 // (coordinates innermost first; x times the element size a multiple of 16 bytes); completion counted
 // on the mbarrier.  tmap: address of a tensor map in the kernel's parameter space.
-__device__ __forceinline__ void tma_load_3d(void *smem_dst, const void *tmap, int x, int y, int z, uint64_t *bar) {
+__device__ __forceinline__ void tma_load_5d(void *smem_dst, const void *tmap, int x, int y, int z, int w, int u, uint64_t *bar) {
     asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];\n" ::"r"(
+        "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, %6}], [%7];\n" ::"r"(
             smem_u32(smem_dst)),
-        "l"(reinterpret_cast<uint64_t>(tmap)), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
+        "l"(reinterpret_cast<uint64_t>(tmap)), "r"(x), "r"(y), "r"(z), "r"(w), "r"(u), "r"(smem_u32(bar))
         : "memory");
 }
 
-// Tiled store of one box of a 3D tensor from this CTA's shared memory by the tensor memory accelerator
+// Tiled store of one box of a 5D tensor from this CTA's shared memory by the tensor memory accelerator
 // (coordinates innermost first, never negative; x times the element size a multiple of 16 bytes; parts
 // of the box outside the tensor are not written), as one bulk async-group operation of this thread.
-__device__ __forceinline__ void tma_store_3d(const void *tmap, const void *smem_src, int x, int y, int z) {
-    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];\n" ::"l"(
+__device__ __forceinline__ void tma_store_5d(const void *tmap, const void *smem_src, int x, int y, int z, int w, int u) {
+    asm volatile("cp.async.bulk.tensor.5d.global.shared::cta.bulk_group [%0, {%1, %2, %3, %4, %5}], [%6];\n" ::"l"(
                      reinterpret_cast<uint64_t>(tmap)),
-                 "r"(x), "r"(y), "r"(z), "r"(smem_u32(smem_src))
+                 "r"(x), "r"(y), "r"(z), "r"(w), "r"(u), "r"(smem_u32(smem_src))
                  : "memory");
 }
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;\n" ::: "memory"); }
@@ -131,14 +134,18 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// x = hi + lo with hi = bf16(x), lo = bf16(x - hi): the compensated (split) BF16 representation
-__device__ __forceinline__ void split_bf16(float x, __nv_bfloat16 &hi, __nv_bfloat16 &lo) {
-    hi = __float2bfloat16_rn(x);
-    lo = __float2bfloat16_rn(x - __bfloat162float(hi));
+// x = hi + lo with hi = bf16(x), lo = bf16(x - hi): the compensated (split) BF16 representation of two values, packed
+// (a in the low half).  Two conversions, two unpackings and two subtractions a pair: the packed conversion runs on
+// the ALU pipe, where single ones take the quarter-rate pipe (forward product at nt 1500, 600 x 384: 560
+// instructions a warp and chunk with those).
+__device__ __forceinline__ uint32_t cvt_bf16x2(float a, float b) {
+    uint32_t d;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(b), "f"(a));
+    return d;
 }
-
-__device__ __forceinline__ uint32_t pack_bf16x2(__nv_bfloat16 lo_elem, __nv_bfloat16 hi_elem) {
-    return (uint32_t)__bfloat16_as_ushort(lo_elem) | ((uint32_t)__bfloat16_as_ushort(hi_elem) << 16);
+__device__ __forceinline__ void split_bf16x2(float a, float b, uint32_t &hi, uint32_t &lo) {
+    hi = cvt_bf16x2(a, b);
+    lo = cvt_bf16x2(a - __uint_as_float(hi << 16), b - __uint_as_float(hi & 0xffff0000u));
 }
 
 // 8 complex values -> one 16-byte chunk in each of the four planes (re hi, re lo, im hi, im lo);
@@ -147,17 +154,18 @@ struct Chunk4 {
     uint4 rh, rl, ih, il;
 };
 __device__ __forceinline__ Chunk4 split8(const float2 (&z)[8], bool conj) {
-    __nv_bfloat16 rh[8], rl[8], ih[8], il[8];
+    uint32_t rh[4], rl[4], ih[4], il[4];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        split_bf16(z[i].x, rh[i], rl[i]);
-        split_bf16(conj ? -z[i].y : z[i].y, ih[i], il[i]);
+    for (int i = 0; i < 4; ++i) {
+        const float2 p = z[2 * i], q = z[2 * i + 1];
+        split_bf16x2(p.x, q.x, rh[i], rl[i]);
+        split_bf16x2(conj ? -p.y : p.y, conj ? -q.y : q.y, ih[i], il[i]);
     }
     Chunk4 c;
-    c.rh = make_uint4(pack_bf16x2(rh[0], rh[1]), pack_bf16x2(rh[2], rh[3]), pack_bf16x2(rh[4], rh[5]), pack_bf16x2(rh[6], rh[7]));
-    c.rl = make_uint4(pack_bf16x2(rl[0], rl[1]), pack_bf16x2(rl[2], rl[3]), pack_bf16x2(rl[4], rl[5]), pack_bf16x2(rl[6], rl[7]));
-    c.ih = make_uint4(pack_bf16x2(ih[0], ih[1]), pack_bf16x2(ih[2], ih[3]), pack_bf16x2(ih[4], ih[5]), pack_bf16x2(ih[6], ih[7]));
-    c.il = make_uint4(pack_bf16x2(il[0], il[1]), pack_bf16x2(il[2], il[3]), pack_bf16x2(il[4], il[5]), pack_bf16x2(il[6], il[7]));
+    c.rh = make_uint4(rh[0], rh[1], rh[2], rh[3]);
+    c.rl = make_uint4(rl[0], rl[1], rl[2], rl[3]);
+    c.ih = make_uint4(ih[0], ih[1], ih[2], ih[3]);
+    c.il = make_uint4(il[0], il[1], il[2], il[3]);
     return c;
 }
 
