@@ -344,24 +344,6 @@ __device__ __forceinline__ double block_sum(double v, double *red) {
     return s;   // valid in thread 0
 }
 
-// Sum of squares of FP32 values to FP64 accuracy without the FP64 unit, which runs at 1/64 of the FP32 rate
-// here: each square is split exactly into p + e (e by a fused multiply-add) and the p are added with their
-// rounding errors kept, so a thread's sum carries about 2^-46 of relative error.  Both members of a pair at once.
-// Values whose squares or their errors could leave the FP32 range (|x| above 2^60, or all below 2^-40) take
-// the FP64 unit.
-struct SumSq {
-    f32x2 hi = 0, lo = 0;
-    __device__ __forceinline__ void add(f32x2 x) {
-        const f32x2 p = mul2(x, x), e = fma2(x, x, neg2(p));
-        const f32x2 t = add2(hi, p), z = sub2(t, hi);
-        lo = add2(lo, add2(e, add2(sub2(hi, sub2(t, z)), sub2(p, z))));
-        hi = t;
-    }
-    __device__ __forceinline__ double total() const {
-        return ((double)lo2(hi) + (double)hi2(hi)) + ((double)lo2(lo) + (double)hi2(lo));
-    }
-};
-
 // Residual step: R = s * irfft(Uh)[0:nt] - U_obs[row], loss partial 1/2 sum R^2 (FP64), Rh = rfft(R)
 // written in place over Uh.  Trace grid: i = batch entry b, j = virtual source v.
 // tile bid of nblk tiles; the last tile to finish (atomic ticket) sums the partials of all nblk
@@ -411,7 +393,7 @@ __device__ __forceinline__ void residual_body(const FftArgs &a, int bid, int nbl
         }
     }
     double l2;
-    if (top <= 0x1p60f && (top >= 0x1p-40f || top == 0.f)) {   // (a NaN passes and reaches the sum)
+    if (SumSq::in_range(top)) {   // (a NaN passes and reaches the sum)
         SumSq q;
 #pragma unroll
         for (int i = 0; i < NSLOT; ++i) {

@@ -8,6 +8,7 @@
 #include <cmath>
 #include <cstring>
 
+#include "smdd_fft.cuh"
 #include "smdd_internal.h"
 
 namespace smdd {
@@ -30,15 +31,21 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-// one FP64 partial of sum(a^2) per block (fixed assignment of elements to blocks and threads)
-__global__ void __launch_bounds__(VEC_THREADS) k_sumsq_partials(const float *__restrict__ a, long long n,
-                                                                  double *__restrict__ partials) {
-    __shared__ double red[VEC_THREADS / 32];
-    double s = 0.0;
-    for (long long i = blockIdx.x * (long long)VEC_THREADS + threadIdx.x; i < n; i += (long long)gridDim.x * VEC_THREADS) {
-        const double x = a[i];
-        s += x * x;
+// Element-wise passes.  Four elements per thread and access where every vector is 16-byte aligned (a tail and
+// unaligned vectors element by element), and the norm of what a pass writes in the same pass: one FP64 partial of the
+// sum of squares per block (fixed assignment of elements to blocks and threads).
+__device__ __forceinline__ void add_squares(SumSq &q, double &d, float4 v) {
+    const float top = fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)));
+    if (SumSq::in_range(top)) {
+        q.add(pk2(v.x, v.y));
+        q.add(pk2(v.z, v.w));
+    } else {
+        d += (double)v.x * v.x + (double)v.y * v.y + (double)v.z * v.z + (double)v.w * v.w;
     }
+}
+
+__device__ __forceinline__ void block_partial(double s, double *partials) {
+    __shared__ double red[VEC_THREADS / 32];
     s = warp_sum(s);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
     __syncthreads();
@@ -49,16 +56,54 @@ __global__ void __launch_bounds__(VEC_THREADS) k_sumsq_partials(const float *__r
     }
 }
 
-// the norm from the partials, in block order, then the scalar step `what`:
+// y = t - coef y (coef: alpha or beta of the scalars, or 1, by `which` = 0, 1, 2; 3: y = t), t muted, and the partials
+// of sum(y^2)
+__global__ void __launch_bounds__(VEC_THREADS) k_combine_norm(float *__restrict__ y, const float *__restrict__ t, long long n, int vec,
+                                                                const LsqrScalars *sc, int which, const int32_t *__restrict__ mute,
+                                                                int nt, double *__restrict__ partials) {
+    const float cf = which == 0 ? (float)sc->alpha : which == 1 ? (float)sc->beta : 1.f;
+    const long long first = blockIdx.x * (long long)VEC_THREADS + threadIdx.x, step = (long long)gridDim.x * VEC_THREADS;
+    SumSq q;
+    double d = 0.0;
+    auto muted = [&](float x, long long i) { return (mute && (int)(i % nt) < mute[i / nt]) ? 0.f : x; };
+    const long long n4 = vec ? n / 4 : 0;
+    for (long long i = first; i < n4; i += step) {
+        float4 a = reinterpret_cast<const float4 *>(t)[i];
+        if (mute) a = make_float4(muted(a.x, 4 * i), muted(a.y, 4 * i + 1), muted(a.z, 4 * i + 2), muted(a.w, 4 * i + 3));
+        if (which < 3) {
+            const float4 b = reinterpret_cast<const float4 *>(y)[i];
+            a = make_float4(a.x - cf * b.x, a.y - cf * b.y, a.z - cf * b.z, a.w - cf * b.w);
+        }
+        reinterpret_cast<float4 *>(y)[i] = a;
+        add_squares(q, d, a);
+    }
+    for (long long i = 4 * n4 + first; i < n; i += step) {
+        float a = muted(t[i], i);
+        if (which < 3) a = a - cf * y[i];
+        y[i] = a;
+        add_squares(q, d, make_float4(a, 0.f, 0.f, 0.f));
+    }
+    block_partial(q.total() + d, partials);
+}
+
+// the norm from the partials (summed in a fixed order), then the scalar step `what`:
 //   0: beta_1 = ||u||, phi_bar = beta                       (start)
 //   1: alpha_1 = ||v||, rho_bar = alpha                     (start)
 //   2: beta = ||u||                                          (iteration, after u = A v - alpha u)
 //   3: alpha = ||v||, then the plane rotation; norms[it] = phi_bar   (iteration, after v = A^T u - beta v)
-__global__ void k_norm_step(const double *__restrict__ partials, int nparts, LsqrScalars *sc, int what,
-                            double *norms, int it) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+constexpr int NORM_THREADS = 256;
+
+__global__ void __launch_bounds__(NORM_THREADS) k_norm_step(const double *__restrict__ partials, int nparts, LsqrScalars *sc, int what,
+                                                              double *norms, int it) {
+    __shared__ double red[NORM_THREADS / 32];
     double t = 0.0;
-    for (int b = 0; b < nparts; ++b) t += partials[b];
+    for (int b = threadIdx.x; b < nparts; b += NORM_THREADS) t += partials[b];
+    t = warp_sum(t);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = t;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    t = 0.0;
+    for (int w = 0; w < NORM_THREADS / 32; ++w) t += red[w];
     const double nrm = sqrt(t);
     sc->inv = nrm > 0.0 ? 1.0 / nrm : 0.0;
     if (what == 0) {
@@ -84,58 +129,44 @@ __global__ void k_norm_step(const double *__restrict__ partials, int nparts, Lsq
     }
 }
 
-// a *= inv (the reciprocal of the last norm)
-__global__ void __launch_bounds__(VEC_THREADS) k_scale_inv(float *__restrict__ a, long long n, const LsqrScalars *sc) {
+// a *= inv (the reciprocal of the last norm), and a copy to w (or null)
+__global__ void __launch_bounds__(VEC_THREADS) k_scale_inv(float *__restrict__ a, float *__restrict__ w, long long n, const LsqrScalars *sc) {
     const float inv = (float)sc->inv;
-    for (long long i = blockIdx.x * (long long)VEC_THREADS + threadIdx.x; i < n; i += (long long)gridDim.x * VEC_THREADS)
-        a[i] *= inv;
-}
-
-// y = t - coef * y   (coef = alpha or beta from the scalars; which = 0: alpha, 1: beta), optional
-// causality mute on model-layout vectors (traces of nt samples, mute[trace])
-__global__ void __launch_bounds__(VEC_THREADS) k_sub_scaled(float *__restrict__ y, const float *__restrict__ t, long long n,
-                                                              const LsqrScalars *sc, int which, const int32_t *__restrict__ mute,
-                                                              int nt) {
-    const float cf = (float)(which ? sc->beta : sc->alpha);
-    for (long long i = blockIdx.x * (long long)VEC_THREADS + threadIdx.x; i < n; i += (long long)gridDim.x * VEC_THREADS) {
-        float tv = t[i];
-        if (mute && (int)(i % nt) < mute[i / nt]) tv = 0.f;
-        y[i] = tv - cf * y[i];
+    const long long first = blockIdx.x * (long long)VEC_THREADS + threadIdx.x, step = (long long)gridDim.x * VEC_THREADS;
+    for (long long i = first; i < n / 4; i += step) {
+        float4 v = reinterpret_cast<const float4 *>(a)[i];
+        v = make_float4(v.x * inv, v.y * inv, v.z * inv, v.w * inv);
+        reinterpret_cast<float4 *>(a)[i] = v;
+        if (w) reinterpret_cast<float4 *>(w)[i] = v;
     }
-}
-
-// u = b - u  (start: the residual of x0)
-__global__ void __launch_bounds__(VEC_THREADS) k_rsub(float *__restrict__ u, const float *__restrict__ b, long long n) {
-    for (long long i = blockIdx.x * (long long)VEC_THREADS + threadIdx.x; i < n; i += (long long)gridDim.x * VEC_THREADS)
-        u[i] = b[i] - u[i];
-}
-
-// v = g (with the mute)
-__global__ void __launch_bounds__(VEC_THREADS) k_first_v(float *__restrict__ v, const float *__restrict__ g, long long n,
-                                                           const int32_t *__restrict__ mute, int nt) {
-    for (long long i = blockIdx.x * (long long)VEC_THREADS + threadIdx.x; i < n; i += (long long)gridDim.x * VEC_THREADS) {
-        float gv = g[i];
-        if (mute && (int)(i % nt) < mute[i / nt]) gv = 0.f;
-        v[i] = gv;
+    for (long long i = (n & ~3LL) + first; i < n; i += step) {
+        a[i] *= inv;
+        if (w) w[i] = a[i];
     }
 }
 
 // v *= inv; then x += cx w; w = v - cw w   (the normalisation of v fused with the solution update)
 __global__ void __launch_bounds__(VEC_THREADS) k_update_xw(float *__restrict__ x, float *__restrict__ w, float *__restrict__ v,
-                                                             long long n, const LsqrScalars *sc) {
+                                                             long long n, int vec, const LsqrScalars *sc) {
     const float inv = (float)sc->inv, cx = (float)sc->cx, cw = (float)sc->cw;
-    for (long long i = blockIdx.x * (long long)VEC_THREADS + threadIdx.x; i < n; i += (long long)gridDim.x * VEC_THREADS) {
-        const float vv = v[i] * inv;
-        const float wv = w[i];
-        v[i] = vv;
-        x[i] = fmaf(cx, wv, x[i]);
-        w[i] = fmaf(-cw, wv, vv);
+    const long long first = blockIdx.x * (long long)VEC_THREADS + threadIdx.x, step = (long long)gridDim.x * VEC_THREADS;
+    auto one = [&](float &xv, float &wv, float &vv) {
+        vv *= inv;
+        xv = fmaf(cx, wv, xv);
+        wv = fmaf(-cw, wv, vv);
+    };
+    const long long n4 = vec ? n / 4 : 0;
+    for (long long i = first; i < n4; i += step) {
+        float4 a = reinterpret_cast<const float4 *>(x)[i], b = reinterpret_cast<const float4 *>(w)[i], c = reinterpret_cast<const float4 *>(v)[i];
+        one(a.x, b.x, c.x);
+        one(a.y, b.y, c.y);
+        one(a.z, b.z, c.z);
+        one(a.w, b.w, c.w);
+        reinterpret_cast<float4 *>(x)[i] = a;
+        reinterpret_cast<float4 *>(w)[i] = b;
+        reinterpret_cast<float4 *>(v)[i] = c;
     }
-}
-
-__global__ void __launch_bounds__(VEC_THREADS) k_copy(float *__restrict__ y, const float *__restrict__ x, long long n) {
-    for (long long i = blockIdx.x * (long long)VEC_THREADS + threadIdx.x; i < n; i += (long long)gridDim.x * VEC_THREADS)
-        y[i] = x[i];
+    for (long long i = 4 * n4 + first; i < n; i += step) one(x[i], w[i], v[i]);
 }
 
 }  // namespace
@@ -181,42 +212,35 @@ cudaError_t lsqr_run(LsqrWork &wk, float *x, const float *b, long long nd, long 
                      const OperatorFn &apply_adj, long long *launches) {
     LsqrScalars *sc = reinterpret_cast<LsqrScalars *>(wk.scalars);
     long long nl = 0;
-    auto norm_step = [&](const float *a, long long n, int what, int it) {
-        k_sumsq_partials<<<VEC_BLOCKS, VEC_THREADS, 0, st>>>(a, n, wk.partials);
-        k_norm_step<<<1, 32, 0, st>>>(wk.partials, VEC_BLOCKS, sc, what, norms, it);
+    const auto aligned = [](const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0 ? 1 : 0; };
+    // y = t - coef y (or y = t) with its norm, and the scalar step `what`
+    auto combine = [&](float *y, const float *t, long long n, int which, const int32_t *m, int what, int it) {
+        k_combine_norm<<<VEC_BLOCKS, VEC_THREADS, 0, st>>>(y, t, n, aligned(y) && aligned(t), sc, which, m, nt, wk.partials);
+        k_norm_step<<<1, NORM_THREADS, 0, st>>>(wk.partials, VEC_BLOCKS, sc, what, norms, it);
         nl += 2;
         return cudaGetLastError();
     };
     cudaError_t e;
     // u = b - A x0; beta = ||u||; u /= beta
     if ((e = apply_fwd(x, wk.u))) return e;
-    k_rsub<<<VEC_BLOCKS, VEC_THREADS, 0, st>>>(wk.u, b, nd);
-    ++nl;
-    if ((e = norm_step(wk.u, nd, 0, 0))) return e;
-    k_scale_inv<<<VEC_BLOCKS, VEC_THREADS, 0, st>>>(wk.u, nd, sc);
+    if ((e = combine(wk.u, b, nd, 2, nullptr, 0, 0))) return e;
+    k_scale_inv<<<VEC_BLOCKS, VEC_THREADS, 0, st>>>(wk.u, nullptr, nd, sc);
     ++nl;
     // v = C A^T u; alpha = ||v||; v /= alpha; w = v
     if ((e = apply_adj(wk.u, wk.g))) return e;
-    k_first_v<<<VEC_BLOCKS, VEC_THREADS, 0, st>>>(wk.v, wk.g, nm, mute, nt);
+    if ((e = combine(wk.v, wk.g, nm, 3, mute, 1, 0))) return e;
+    k_scale_inv<<<VEC_BLOCKS, VEC_THREADS, 0, st>>>(wk.v, wk.w, nm, sc);
     ++nl;
-    if ((e = norm_step(wk.v, nm, 1, 0))) return e;
-    k_scale_inv<<<VEC_BLOCKS, VEC_THREADS, 0, st>>>(wk.v, nm, sc);
-    k_copy<<<VEC_BLOCKS, VEC_THREADS, 0, st>>>(wk.w, wk.v, nm);
-    nl += 2;
     for (int it = 1; it <= n_iter; ++it) {
         // u = A v - alpha u; beta = ||u||; u /= beta
         if ((e = apply_fwd(wk.v, wk.t))) return e;
-        k_sub_scaled<<<VEC_BLOCKS, VEC_THREADS, 0, st>>>(wk.u, wk.t, nd, sc, 0, nullptr, nt);
-        ++nl;
-        if ((e = norm_step(wk.u, nd, 2, it))) return e;
-        k_scale_inv<<<VEC_BLOCKS, VEC_THREADS, 0, st>>>(wk.u, nd, sc);
+        if ((e = combine(wk.u, wk.t, nd, 0, nullptr, 2, it))) return e;
+        k_scale_inv<<<VEC_BLOCKS, VEC_THREADS, 0, st>>>(wk.u, nullptr, nd, sc);
         ++nl;
         // v = C A^T u - beta v; alpha = ||v||; rotation; v /= alpha; x, w updates
         if ((e = apply_adj(wk.u, wk.g))) return e;
-        k_sub_scaled<<<VEC_BLOCKS, VEC_THREADS, 0, st>>>(wk.v, wk.g, nm, sc, 1, mute, nt);
-        ++nl;
-        if ((e = norm_step(wk.v, nm, 3, it))) return e;
-        k_update_xw<<<VEC_BLOCKS, VEC_THREADS, 0, st>>>(x, wk.w, wk.v, nm, sc);
+        if ((e = combine(wk.v, wk.g, nm, 1, mute, 3, it))) return e;
+        k_update_xw<<<VEC_BLOCKS, VEC_THREADS, 0, st>>>(x, wk.w, wk.v, nm, aligned(x), sc);
         ++nl;
     }
     if (launches) *launches += nl;

@@ -88,6 +88,25 @@ __device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
     return d;
 }
 
+// Sum of squares of FP32 values to FP64 accuracy without the FP64 unit, which runs at 1/64 of the FP32 rate
+// here: each square is split exactly into p + e (e by a fused multiply-add) and the p are added with their
+// rounding errors kept, so a thread's sum carries about 2^-46 of relative error.  Both members of a pair at once.
+// Values whose squares or their errors could leave the FP32 range (a largest |x| above 2^60 or below 2^-50) take
+// the FP64 unit.
+struct SumSq {
+    f32x2 hi = 0, lo = 0;
+    static __device__ __forceinline__ bool in_range(float top) { return top <= 0x1p60f && (top >= 0x1p-50f || top == 0.f); }
+    __device__ __forceinline__ void add(f32x2 x) {
+        const f32x2 p = mul2(x, x), e = fma2(x, x, neg2(p));
+        const f32x2 t = add2(hi, p), z = sub2(t, hi);
+        lo = add2(lo, add2(e, add2(sub2(hi, sub2(t, z)), sub2(p, z))));
+        hi = t;
+    }
+    __device__ __forceinline__ double total() const {
+        return ((double)lo2(hi) + (double)hi2(hi)) + ((double)lo2(lo) + (double)hi2(lo));
+    }
+};
+
 // a complex value of two traces, and a twiddle held twice
 struct C2 {
     f32x2 re, im;
