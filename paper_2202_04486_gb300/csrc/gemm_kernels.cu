@@ -11,6 +11,8 @@
 // Gh_f^T[v][r] = sum_b conj(Dh_f[idx_b][v]) Rh_f[r][b], the symmetric part is one product with
 // inner dimension 2 nb, A' = [Rh | conj(Dh_B)^T], B' = [conj(Dh_B) ; Rh^T], evaluated on the upper
 // triangle of tiles only and mirrored into the lower triangle through shared memory.
+#include <climits>
+
 #include "smdd_fft.cuh"
 #include "smdd_internal.h"
 
@@ -33,7 +35,9 @@ __device__ __forceinline__ void cmac(float2 &acc, float2 a, float2 b) {
 }
 
 // ------------------------------------------------------------------------------------------------
-// forward: C[f][v][b] = sum_r A[f][v][r] * Dh[f][idx_b][r]
+// forward, few rows (scalar products, 4 x 4 outputs per thread): C[f][v][b] = sum_r A[f][v][r] * Dh[f][idx_b][r]
+// With at most 64 rows a product is a chain of latencies; the longer chunk (16) through cp.async has fewer of them:
+// 8.4 us at nf 129, 32 x 32, batch 8, against 11 us for the packed tiles below.
 // CTA: 4 warps, 128 rows v x 16 batch columns, one frequency.  Lane (vg = lane & 7, bg = lane >> 3)
 // of warp w owns rows v0 + 32w + vg + 8i and columns b0 + bg + 4j (i, j < 4): a 4 x 4 complex register
 // tile.  K (= nr) streams in chunks of 16 through a two-stage cp.async pipeline; every operand load is
@@ -45,7 +49,7 @@ constexpr int FW_STAGE = (FW_ROWS + FW_NB) * FW_LD;   // float2 per stage
 constexpr size_t FW_SMEM = 2 * FW_STAGE * sizeof(float2);
 
 template <int F>
-__global__ void __launch_bounds__(FW_THREADS, 4) k_cgemm_fwd(GemmArgs a) {
+__global__ void __launch_bounds__(FW_THREADS, 4) k_cgemm_fwd_small(GemmArgs a) {
     extern __shared__ __align__(16) float2 gsm[];
     const int f = blockIdx.z;
     const int v0 = blockIdx.x * FW_ROWS, b0 = blockIdx.y * FW_NB;
@@ -154,7 +158,10 @@ __global__ void __launch_bounds__(FW_THREADS, 4) k_cgemm_fwd(GemmArgs a) {
 // adjoint: C[f][v][r] = outscale * sum_k A'[v][k] B'[k][r]
 //   k < nb :  A' = Rh[f][v][k],            B' = conj(Dh[f][idx_k][r])
 //   k >= nb (reciprocity only, k' = k - nb):  A' = conj(Dh[f][idx_k'][v]),  B' = Rh[f][r][k']
-// CTA tile TT x TT (TT = 64 or 32).  A warp covers 4*VPN rows x TT columns: lane (vp = lane / RG,
+// 32 x 32 tiles with scalar products (4 x 4 outputs per thread, chunks of 16): finer at triangular and ragged edges
+// than the packed 64 x 64 tiles below.  With reciprocity both halves of a chunk are staged at once, one latency: 107
+// us against 130 us at nf 513, 201 x 201, batch 16 (1057 and 1118 us at batch 201).
+// CTA tile TT x TT.  A warp covers 4*VPN rows x TT columns: lane (vp = lane / RG,
 // rg = lane % RG) owns rows v0 + 4*VPN*w + 4vp + {0,1,2,3} and columns r0 + {2rg, 2rg+1, 2rg+TT/2,
 // 2rg+TT/2+1}.  Operands are staged by cp.async in their global layouts -- residual-spectrum rows [v][k]
 // and kernel-spectrum rows [k][r] -- and conjugated when used; chunks of 16 k per half.  Warps whose
@@ -162,8 +169,8 @@ __global__ void __launch_bounds__(FW_THREADS, 4) k_cgemm_fwd(GemmArgs a) {
 // ------------------------------------------------------------------------------------------------
 constexpr int AD_KC = 16, AD_LDR = AD_KC + 2, AD_MAXNB = 1024;
 
-template <int TT>
-struct AdjGeom {
+struct AdjS {
+    static constexpr int TT = 32;
     static constexpr int RG = TT / 4;             // lanes along r
     static constexpr int VPN = 32 / RG;           // lane groups along v
     static constexpr int WROWS = 4 * VPN;         // rows per warp
@@ -177,9 +184,8 @@ struct AdjGeom {
 };
 
 // stage rows [c0, c0 + TT) x k [k0, k0 + 16) of Rh (row pitch ldb) into s[TT][AD_LDR]
-template <int TT>
 __device__ __forceinline__ void stage_rrows(float2 *s, const float2 *Rf, int ldb, int c0, int nc, int k0, int nb, int tid) {
-    constexpr int NT = AdjGeom<TT>::THREADS;
+    constexpr int TT = AdjS::TT, NT = AdjS::THREADS;
 #pragma unroll
     for (int u = 0; u < TT * AD_KC / 2 / NT; ++u) {
         const int c = tid + u * NT, row = c >> 3, part = c & 7;
@@ -195,10 +201,9 @@ __device__ __forceinline__ void stage_rrows(float2 *s, const float2 *Rf, int ldb
 }
 
 // stage kernel rows idx[k0 .. k0 + 16) at columns [c0, c0 + TT) into s[16][TT]
-template <int TT>
 __device__ __forceinline__ void stage_drows(float2 *s, const float2 *Df, int ldd, const int *sidx, int c0, int nc, int k0,
                                             int nb, int tid) {
-    constexpr int NT = AdjGeom<TT>::THREADS, PARTS = TT / 2;
+    constexpr int TT = AdjS::TT, NT = AdjS::THREADS, PARTS = TT / 2;
 #pragma unroll
     for (int u = 0; u < AD_KC * TT / 2 / NT; ++u) {
         const int c = tid + u * NT, kk = c / PARTS, part = c % PARTS;
@@ -224,9 +229,10 @@ __device__ __forceinline__ void cmac_c(float2 &acc, float2 a, float2 b) {
     acc.y = fmaf(-a.x, b.y, acc.y);
 }
 
-template <int TT, bool RECIP>
-__global__ void __launch_bounds__(AdjGeom<TT>::THREADS, TT == 64 ? 3 : 8) k_cgemm_adj(GemmArgs a) {
-    using G = AdjGeom<TT>;
+template <bool RECIP>
+__global__ void __launch_bounds__(AdjS::THREADS, 8) k_cgemm_adj_small(GemmArgs a) {
+    using G = AdjS;
+    constexpr int TT = G::TT;
     extern __shared__ __align__(16) float2 gsm[];
     float2 *sRv = gsm;                  // [TT][AD_LDR]  Rh rows of the v block
     float2 *sDr = sRv + G::RROWS;       // [16][TT]      kernel rows at the r block
@@ -275,11 +281,11 @@ __global__ void __launch_bounds__(AdjGeom<TT>::THREADS, TT == 64 ? 3 : 8) k_cgem
         for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
 
     for (int k0 = 0; k0 < a.nb; k0 += AD_KC) {
-        stage_rrows<TT>(sRv, Rf, a.ldb, v0, a.nv, k0, a.nb, tid);
-        stage_drows<TT>(sDr, Df, a.ldd, sidx, r0, a.nr, k0, a.nb, tid);
+        stage_rrows(sRv, Rf, a.ldb, v0, a.nv, k0, a.nb, tid);
+        stage_drows(sDr, Df, a.ldd, sidx, r0, a.nr, k0, a.nb, tid);
         if (RECIP) {
-            stage_rrows<TT>(sRr, Rf, a.ldb, r0, a.nr, k0, a.nb, tid);
-            stage_drows<TT>(sDv, Df, a.ldd, sidx, v0, a.nv, k0, a.nb, tid);
+            stage_rrows(sRr, Rf, a.ldb, r0, a.nr, k0, a.nb, tid);
+            stage_drows(sDv, Df, a.ldd, sidx, v0, a.nv, k0, a.nb, tid);
         }
         cp_async_commit();
         cp_async_wait<0>();
@@ -358,6 +364,324 @@ __global__ void __launch_bounds__(AdjGeom<TT>::THREADS, TT == 64 ? 3 : 8) k_cgem
                 }
             }
             if (RECIP) {   // mirror buffer (r, v); operands are dead after the final barrier
+                gsm[rr * (TT + 1) + vv] = x0;
+                gsm[(rr + 1) * (TT + 1) + vv] = x1;
+            }
+        }
+    }
+    if (RECIP && (diag || !a.no_mirror)) {   // diagonal tiles always mirror (see GemmArgs::no_mirror)
+        __syncthreads();
+        for (int e = tid; e < TT * TT; e += G::THREADS) {
+            const int rr = e / TT, vv = e % TT;
+            const int r = r0 + rr, v = v0 + vv;
+            if (v < a.nv && r < a.nr && (!diag || v < r)) Cf[r * crow + spec_col(v)] = gsm[rr * (TT + 1) + vv];
+        }
+    }
+}
+
+// ------------------------------------------------------------------------------------------------
+// Tile products on the CUDA cores.  A thread owns 8 x 4 complex outputs, the 8 as four pairs of packed FP32 values
+// (fma.f32x2: two multiply-adds in one issue slot; the arithmetic rate is that of scalar instructions, but the
+// operand loads and duplications then fit in the freed slots): pair p holds i = 2 ti + 2 WTI p and i + 1, so that the
+// lanes of a row store 64 contiguous bytes of the output.  Operands lie in shared memory as separate real and
+// imaginary planes [k][i] and [k][j]: an LDS.64 of the i operand is a packed pair, the j operand is duplicated
+// into pairs in registers (24 cycles of the shared-memory pipe and 64 packed multiply-adds a k and warp; with 4 x 4 outputs the shared-memory pipe, at
+// four cycles an LDS.128, would be as busy as the arithmetic).  Chunks of 8 k, double buffered, the next chunk's
+// global loads in registers while one is multiplied: one barrier a chunk.
+//   FORM 0: c += a b            (forward:  a = model spectra, b = kernel rows)
+//   FORM 1: c += conj(a) b      (adjoint:  a = kernel rows, b = residual spectra)
+//   FORM 2: c += a conj(b)      (its transpose, for the reciprocity half)
+// A warp covers 8 WTI x 4 (32 / WTI) outputs; warps whose outputs all lie outside the matrix skip the products.
+// ------------------------------------------------------------------------------------------------
+template <int WTI_, int NWI_, int NWJ_, int KC_ = 8>
+struct SimtGeom {
+    static constexpr int WTI = WTI_, NWI = NWI_, NWJ = NWJ_, KC = KC_;
+    static constexpr int WI = 8 * WTI, WJ = 4 * (32 / WTI);      // outputs of a warp
+    static constexpr int BI = WI * NWI, BJ = WJ * NWJ;           // outputs of the CTA
+    static constexpr int THREADS = 32 * NWI * NWJ;
+    // row pitches: 16-byte multiples whose double is 8 mod 32 words, so the transposing stores of 4 k pairs x 8 rows
+    // fall on distinct banks (8 x 4 for KC = 16: two to a bank)
+    static constexpr int PI = BI + 4, PJ = BJ + 4;
+    static constexpr int STAGE = 2 * KC * (PI + PJ);          // floats: Ar, Ai, Br, Bi
+    static constexpr size_t SMEM = 2 * STAGE * sizeof(float);
+    // LDG.128 units (two complex values) of a chunk per thread
+    static constexpr int UI = (BI * KC / 2 + THREADS - 1) / THREADS, UJ = (BJ * KC / 2 + THREADS - 1) / THREADS;
+    static constexpr int MINB = (UI > 4 ? 384 : 512) / THREADS;   // resident CTAs: 168 or 128 registers per thread
+};
+
+struct SimtAcc {
+    f32x2 re[4][4], im[4][4];   // [pair of i][j]
+    __device__ __forceinline__ void zero() {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) re[i][j] = im[i][j] = 0;
+    }
+};
+
+// one chunk: planes of stage s; ia, jb: the thread's first i and j of the tile
+template <class G, int FORM>
+__device__ __forceinline__ void simt_chunk(SimtAcc &c, const float *st, int ia, int jb) {
+    constexpr int KC = G::KC;
+    const float *pa = st + ia, *pb = st + 2 * KC * G::PI + jb;
+#pragma unroll
+    for (int k = 0; k < KC; ++k) {
+        f32x2 ar[4], ai[4];
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+            ar[p] = *reinterpret_cast<const f32x2 *>(pa + k * G::PI + 2 * G::WTI * p);
+            ai[p] = *reinterpret_cast<const f32x2 *>(pa + (KC + k) * G::PI + 2 * G::WTI * p);
+        }
+        const float4 b4 = *reinterpret_cast<const float4 *>(pb + k * G::PJ), d4 = *reinterpret_cast<const float4 *>(pb + (KC + k) * G::PJ);
+        const float br[4] = {b4.x, b4.y, b4.z, b4.w}, bi[4] = {d4.x, d4.y, d4.z, d4.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const f32x2 r = dup2(br[j]), i = dup2(bi[j]), n = dup2(FORM == 1 ? -br[j] : -bi[j]);
+#pragma unroll
+            for (int p = 0; p < 4; ++p) {
+                c.re[p][j] = fma2(ar[p], r, c.re[p][j]);
+                c.re[p][j] = fma2(ai[p], FORM == 0 ? n : i, c.re[p][j]);
+                c.im[p][j] = fma2(ar[p], FORM == 2 ? n : i, c.im[p][j]);
+                c.im[p][j] = fma2(ai[p], FORM == 1 ? n : r, c.im[p][j]);
+            }
+        }
+    }
+}
+
+// An operand whose rows hold k contiguously (rows of the layout of F bins: row x at base + x ld): unit c of a chunk is
+// (row c / (KC / 2), columns k0 + 2 (c % (KC / 2)), + 1); rows past n and columns past nk are zero.
+template <int F>
+__device__ __forceinline__ float4 krow_load(const float2 *base, long long ld, int x, int n, int k, int nk) {
+    if (x >= n || k >= nk) return make_float4(0.f, 0.f, 0.f, 0.f);
+    const float2 *p = base + (long long)x * ld + spec_col<F>(k);
+    if (k + 1 < nk) return __ldg(reinterpret_cast<const float4 *>(p));
+    const float2 v = __ldg(p);
+    return make_float4(v.x, v.y, 0.f, 0.f);
+}
+template <int P, int KC>
+__device__ __forceinline__ void krow_store(float *pl, int c, float4 v) {   // pl: real plane; the imaginary one follows
+    float *q = pl + 2 * (c % (KC / 2)) * P + c / (KC / 2);
+    q[0] = v.x;
+    q[P] = v.z;
+    q[KC * P] = v.y;
+    q[(KC + 1) * P] = v.w;
+}
+// An operand given by rows k (kernel spectra): unit c is (k = c / (B / 2), columns x0 + 2 (c % (B / 2)), + 1)
+__device__ __forceinline__ float4 xrow_load(const float2 *row, int x, int n) {   // row may be null: zero
+    if (!row || x >= n) return make_float4(0.f, 0.f, 0.f, 0.f);
+    if (x + 1 < n) return __ldg(reinterpret_cast<const float4 *>(row + x));
+    const float2 v = __ldg(row + x);
+    return make_float4(v.x, v.y, 0.f, 0.f);
+}
+template <int P, int B, int KC>
+__device__ __forceinline__ void xrow_store(float *pl, int c, float4 v) {
+    float *q = pl + (c / (B / 2)) * P + 2 * (c % (B / 2));
+    *reinterpret_cast<float2 *>(q) = make_float2(v.x, v.z);
+    *reinterpret_cast<float2 *>(q + KC * P) = make_float2(v.y, v.w);
+}
+
+// ------------------------------------------------------------------------------------------------
+// forward: C[f][v][b] = sum_r A[f][v][r] * Dh[f][idx_b][r]   (i = v, j = b, k = r)
+// ------------------------------------------------------------------------------------------------
+template <class G, int F>
+__global__ void __launch_bounds__(G::THREADS, G::MINB) k_cgemm_fwd(GemmArgs a) {
+    extern __shared__ __align__(16) float ssm[];
+    __shared__ int srow[G::BJ];
+    const int f = blockIdx.z, v0 = blockIdx.x * G::BI, b0 = blockIdx.y * G::BJ;
+    if (a.nf_active > 0 && f >= a.nf_active) {
+        zero_tile<F>(a.C + spec_bin<F>(f, a.sCf), (long long)a.ldb * F, v0, G::BI, b0, G::BJ, a.nv, a.nb);
+        return;
+    }
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int wi = (warp % G::NWI) * G::WI, wj = (warp / G::NWI) * G::WJ;
+    const int ia = wi + 2 * (lane % G::WTI), jb = wj + 4 * (lane / G::WTI);
+    const float2 *Af = a.A + spec_bin<F>(f, a.sAf);
+    const float2 *Df = a.Dh + (long long)f * a.sDf;
+    for (int j = tid; j < G::BJ; j += G::THREADS) {
+        int s = -1;
+        if (b0 + j < a.nb) {
+            s = a.idx[b0 + j];
+            if (s < 0 || s >= a.ns) {
+                atomicOr(a.status, 1);
+                s = -1;
+            }
+        }
+        srow[j] = s;
+    }
+    __syncthreads();
+    const long long arow = (long long)a.ldr * F;
+    constexpr int H = G::KC / 2;   // units of a row and chunk
+    float4 ra[G::UI], rb[G::UJ];
+    auto load = [&](int k0) {
+#pragma unroll
+        for (int u = 0; u < G::UI; ++u) {
+            const int c = tid + u * G::THREADS;
+            if (c < G::BI * H) ra[u] = krow_load<F>(Af, arow, v0 + c / H, a.nv, k0 + 2 * (c % H), a.nr);
+        }
+#pragma unroll
+        for (int u = 0; u < G::UJ; ++u) {
+            const int c = tid + u * G::THREADS;
+            if (c < G::BJ * H) rb[u] = krow_load<1>(Df, a.ldd, srow[c / H], srow[c / H] < 0 ? INT_MIN : INT_MAX, k0 + 2 * (c % H), a.nr);
+        }
+    };
+    auto store = [&](int s) {
+        float *pa = ssm + s * G::STAGE, *pb = pa + 2 * G::KC * G::PI;
+#pragma unroll
+        for (int u = 0; u < G::UI; ++u)
+            if (tid + u * G::THREADS < G::BI * H) krow_store<G::PI, G::KC>(pa, tid + u * G::THREADS, ra[u]);
+#pragma unroll
+        for (int u = 0; u < G::UJ; ++u)
+            if (tid + u * G::THREADS < G::BJ * H) krow_store<G::PJ, G::KC>(pb, tid + u * G::THREADS, rb[u]);
+    };
+    SimtAcc c;
+    c.zero();
+    const bool active = v0 + wi < a.nv && b0 + wj < a.nb;
+    const int nk = (a.nr + G::KC - 1) / G::KC;
+    load(0);
+    store(0);
+    __syncthreads();
+    for (int kc = 0; kc < nk; ++kc) {
+        if (kc + 1 < nk) load((kc + 1) * G::KC);
+        if (active) simt_chunk<G, 0>(c, ssm + (kc & 1) * G::STAGE, ia, jb);
+        if (kc + 1 < nk) store((kc + 1) & 1);
+        __syncthreads();
+    }
+    float2 *Cf = a.C + spec_bin<F>(f, a.sCf);
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int v = v0 + ia + 2 * G::WTI * p + e;
+            if (v >= a.nv) continue;
+#pragma unroll
+            for (int j = 0; j < 4; j += 2) {
+                const int b = b0 + jb + j;
+                const float2 x = e ? make_float2(hi2(c.re[p][j]), hi2(c.im[p][j])) : make_float2(lo2(c.re[p][j]), lo2(c.im[p][j]));
+                const float2 y = e ? make_float2(hi2(c.re[p][j + 1]), hi2(c.im[p][j + 1])) : make_float2(lo2(c.re[p][j + 1]), lo2(c.im[p][j + 1]));
+                float2 *dst = Cf + (long long)v * a.ldb * F + spec_col<F>(b);
+                if (b + 1 < a.nb) *reinterpret_cast<float4 *>(dst) = make_float4(x.x, x.y, y.x, y.y);
+                else if (b < a.nb) *dst = x;
+            }
+        }
+}
+
+// ------------------------------------------------------------------------------------------------
+// adjoint: C[f][v][r] = outscale * sum_k A'[v][k] B'[k][r]   (i = r, j = v)
+//   first half:   Rh[f][v][k] conj(Dh[f][idx_k][r])
+//   second half:  conj(Dh[f][idx_k][v]) Rh[f][r][k]      (reciprocity)
+// Tiles of 64 x 64 (four warps); with reciprocity the upper-triangular ones, mirrored through shared memory.
+// ------------------------------------------------------------------------------------------------
+using AdjGeom64 = SimtGeom<4, 2, 2>;
+template <class G>
+constexpr size_t adj_smem() {   // the operands, or the mirror buffer
+    const size_t mirror = G::BI * (G::BI + 1) * sizeof(float2);
+    return G::SMEM > mirror ? G::SMEM : mirror;
+}
+
+template <class G, bool RECIP>
+__global__ void __launch_bounds__(G::THREADS, 512 / G::THREADS) k_cgemm_adj(GemmArgs a) {
+    constexpr int TT = G::BI, KC = G::KC, H = KC / 2;
+    static_assert(G::BI == G::BJ, "square tiles");
+    extern __shared__ __align__(16) float ssm[];
+    __shared__ int sidx[AD_MAXNB];
+    const int f = blockIdx.y;
+    int vb, rb_;
+    if (RECIP) {   // upper-triangular tile enumeration: vb <= rb
+        int t = blockIdx.x, row = 0, len = a.tiles_v;
+        while (t >= len) { t -= len; ++row; --len; }
+        vb = row;
+        rb_ = row + t;
+    } else {
+        vb = blockIdx.x / a.tiles_r;
+        rb_ = blockIdx.x % a.tiles_r;
+    }
+    const int v0 = vb * TT, r0 = rb_ * TT;
+    const long long crow = (long long)a.ldr * SPEC_F, brow = (long long)a.ldb * SPEC_F;
+    float2 *Cf = a.C + spec_bin(f, a.sCf);
+    if (a.nf_active > 0 && f >= a.nf_active) {
+        zero_tile(Cf, crow, v0, TT, r0, TT, a.nv, a.nr);
+        if (RECIP) zero_tile(Cf, crow, r0, TT, v0, TT, a.nr, a.nv);
+        return;
+    }
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int wi = (warp % G::NWI) * G::WI, wj = (warp / G::NWI) * G::WJ;
+    const int ia = wi + 2 * (lane % G::WTI), jb = wj + 4 * (lane / G::WTI);
+    const float2 *Rf = a.A + spec_bin(f, a.sAf);
+    const float2 *Df = a.Dh + (long long)f * a.sDf;
+    for (int b = tid; b < a.nb; b += G::THREADS) {
+        int s = a.idx[b];
+        if (s < 0 || s >= a.ns) {
+            atomicOr(a.status, 1);
+            s = -1;
+        }
+        sidx[b] = s;
+    }
+    __syncthreads();
+    constexpr int NH = RECIP ? 2 : 1;
+    float4 ra[G::UI], rb[G::UJ];
+    // job = (chunk, half): half 0: i from kernel rows, j from residual rows; half 1: i from residual rows, j from kernel rows
+    auto load = [&](int job) {
+        const int k0 = (job / NH) * KC, half = job % NH;
+#pragma unroll
+        for (int u = 0; u < G::UI; ++u) {
+            const int c = tid + u * G::THREADS, kk = k0 + c / (TT / 2), x = 2 * (c % (TT / 2));
+            const int s = kk < a.nb ? sidx[kk] : -1;
+            const float2 *row = s >= 0 ? Df + (long long)s * a.ldd : nullptr;
+            const int xr = (half ? r0 : v0) + c / H, nx = half ? a.nr : a.nv;
+            const float4 d = xrow_load(row, (half ? v0 : r0) + x, half ? a.nv : a.nr);
+            const float4 q = krow_load<SPEC_F>(Rf, brow, xr, nx, k0 + 2 * (c % H), a.nb);
+            ra[u] = d;
+            rb[u] = q;
+        }
+    };
+    auto store = [&](int job) {
+        const int half = job % NH;
+        float *pi = ssm + (job & 1) * G::STAGE, *pj = pi + 2 * KC * G::PI;
+#pragma unroll
+        for (int u = 0; u < G::UI; ++u) {
+            const int c = tid + u * G::THREADS;
+            xrow_store<G::PI, TT, KC>(half ? pj : pi, c, ra[u]);
+            krow_store<G::PJ, KC>(half ? pi : pj, c, rb[u]);
+        }
+    };
+    static_assert(G::UI == G::UJ && G::PI == G::PJ && G::UI * G::THREADS == TT * KC / 2, "both operands are staged alike");
+    SimtAcc c;
+    c.zero();
+    const bool diag = RECIP && (vb == rb_);
+    // (the outputs of a diagonal tile below the diagonal are the mirrored ones)
+    const bool active = r0 + wi < a.nr && v0 + wj < a.nv && !(diag && wi + G::WI <= wj);
+    const int njobs = (a.nb + KC - 1) / KC * NH;
+    load(0);
+    store(0);
+    __syncthreads();
+    for (int job = 0; job < njobs; ++job) {
+        if (job + 1 < njobs) load(job + 1);
+        if (active) {
+            if (!RECIP || job % 2 == 0) simt_chunk<G, 1>(c, ssm + (job & 1) * G::STAGE, ia, jb);
+            else simt_chunk<G, 2>(c, ssm + (job & 1) * G::STAGE, ia, jb);
+        }
+        if (job + 1 < njobs) store(job + 1);
+        __syncthreads();
+    }
+    float2 *gsm = reinterpret_cast<float2 *>(ssm);   // mirror buffer (r, v); the operands are dead
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int vv = jb + j, v = v0 + vv;
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+            const int rr = ia + 2 * G::WTI * p, r = r0 + rr;
+            const float2 x0 = cscale(make_float2(lo2(c.re[p][j]), lo2(c.im[p][j])), a.outscale);
+            const float2 x1 = cscale(make_float2(hi2(c.re[p][j]), hi2(c.im[p][j])), a.outscale);
+            if (v < a.nv) {
+                const bool w0 = r < a.nr && (!diag || v <= r), w1 = r + 1 < a.nr && (!diag || v <= r + 1);
+                float2 *dst = Cf + v * crow + spec_col(r);
+                if (w0 && w1) *reinterpret_cast<float4 *>(dst) = make_float4(x0.x, x0.y, x1.x, x1.y);
+                else {
+                    if (w0) dst[0] = x0;
+                    if (w1) dst[1] = x1;
+                }
+            }
+            if (RECIP) {
                 gsm[rr * (TT + 1) + vv] = x0;
                 gsm[(rr + 1) * (TT + 1) + vv] = x1;
             }
@@ -489,44 +813,55 @@ cudaError_t launch_gemv_adj(const GemmArgs &a, int nf, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-cudaError_t gemm_prepare() {
-    cudaError_t e;
-    if ((e = cudaFuncSetAttribute(k_cgemm_fwd<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FW_SMEM))) return e;
-    if ((e = cudaFuncSetAttribute(k_cgemm_fwd<SPEC_F>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FW_SMEM))) return e;
-    if ((e = cudaFuncSetAttribute(k_cgemm_adj<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AdjGeom<64>::SMEM))) return e;
-    if ((e = cudaFuncSetAttribute(k_cgemm_adj<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AdjGeom<64>::SMEM))) return e;
-    if ((e = cudaFuncSetAttribute(k_cgemm_adj<32, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AdjGeom<32>::SMEM))) return e;
-    if ((e = cudaFuncSetAttribute(k_cgemm_adj<32, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AdjGeom<32>::SMEM))) return e;
-    return cudaSuccess;
+// forward tiles: 64 x 64 (batches over 32), 128 x 32, 128 x 16 (batches up to 16): the narrowest block of the batch that
+// leaves no warp without columns
+using FwdGeom64 = SimtGeom<4, 2, 2>;
+using FwdGeom32 = SimtGeom<4, 4, 1>;
+using FwdGeom16 = SimtGeom<8, 2, 1>;
+static_assert(adj_smem<AdjGeom64>() <= 49152 - AD_MAXNB * 4 && FwdGeom64::SMEM <= 40960 && FwdGeom32::SMEM <= 40960 &&
+                  FwdGeom16::SMEM <= 40960 && FW_SMEM <= 49152 && AdjS::SMEM <= 49152 - AD_MAXNB * 4,
+              "no opt-in to more shared memory");
+
+cudaError_t gemm_prepare() { return cudaSuccess; }
+
+template <class G>
+static void launch_fwd(const GemmArgs &a, int nf, cudaStream_t st) {
+    const dim3 grid((a.nv + G::BI - 1) / G::BI, (a.nb + G::BJ - 1) / G::BJ, nf);
+    if (a.plain) k_cgemm_fwd<G, 1><<<grid, G::THREADS, G::SMEM, st>>>(a);
+    else k_cgemm_fwd<G, SPEC_F><<<grid, G::THREADS, G::SMEM, st>>>(a);
 }
 
+// measured (us, packed tiles against the scalar kernel): 814 / 1296 (nf 1025, 301 x 301, batch 64), 237 / 304 (nf 1025, 237 x
+// 133, batch 27), 88 / 94 (nf 513, 201 x 201, batch 16), 11 / 8.4 (nf 129, 32 x 32, batch 8)
 cudaError_t launch_cgemm_fwd(const GemmArgs &a, int nf, cudaStream_t st) {
-    dim3 grid((a.nv + FW_ROWS - 1) / FW_ROWS, (a.nb + FW_NB - 1) / FW_NB, nf);
-    if (a.plain) k_cgemm_fwd<1><<<grid, FW_THREADS, FW_SMEM, st>>>(a);
-    else k_cgemm_fwd<SPEC_F><<<grid, FW_THREADS, FW_SMEM, st>>>(a);
+    if (a.nv <= 64) {
+        const dim3 grid((a.nv + FW_ROWS - 1) / FW_ROWS, (a.nb + FW_NB - 1) / FW_NB, nf);
+        if (a.plain) k_cgemm_fwd_small<1><<<grid, FW_THREADS, FW_SMEM, st>>>(a);
+        else k_cgemm_fwd_small<SPEC_F><<<grid, FW_THREADS, FW_SMEM, st>>>(a);
+    } else if (a.nb <= 16) launch_fwd<FwdGeom16>(a, nf, st);
+    else if (a.nb <= 32) launch_fwd<FwdGeom32>(a, nf, st);
+    else launch_fwd<FwdGeom64>(a, nf, st);
     return cudaGetLastError();
 }
 
-template <int TT>
-static void launch_adj_tt(const GemmArgs &a0, bool recip, int nf, cudaStream_t st) {
+// tile = 0: the scalar 32-wide tiles with reciprocity up to 512 columns and for matrices of one packed tile, else the
+// packed 64-wide ones (us, scalar 32 / packed 64: 1320 / 974 at nf 1025, 301 x 301, batch 64; 145 / 98 at nf 513, 256 x 256,
+// batch 16; 275 / 240 at nf 1025, 237 x 133, batch 27; with reciprocity 107 / 130 at nf 513, 201 x 201, batch 16); 32 or 64:
+// as given
+cudaError_t launch_cgemm_adj(const GemmArgs &a0, bool recip, int nf, cudaStream_t st, int tile) {
     GemmArgs a = a0;
-    a.tiles_v = (a.nv + TT - 1) / TT;
-    a.tiles_r = (a.nr + TT - 1) / TT;
-    if (recip) {
-        const int ntiles = a.tiles_v * (a.tiles_v + 1) / 2;
-        k_cgemm_adj<TT, true><<<dim3(ntiles, nf), AdjGeom<TT>::THREADS, AdjGeom<TT>::SMEM, st>>>(a);
+    if (tile == 0) tile = (recip && a.nv <= 512) || (a.nv <= 64 && a.nr <= 64) ? 32 : 64;
+    a.tiles_v = (a.nv + tile - 1) / tile;
+    a.tiles_r = (a.nr + tile - 1) / tile;
+    const dim3 grid(recip ? a.tiles_v * (a.tiles_v + 1) / 2 : a.tiles_v * a.tiles_r, nf);
+    using G = AdjGeom64;
+    if (tile == 32) {
+        if (recip) k_cgemm_adj_small<true><<<grid, AdjS::THREADS, AdjS::SMEM, st>>>(a);
+        else k_cgemm_adj_small<false><<<grid, AdjS::THREADS, AdjS::SMEM, st>>>(a);
     } else {
-        k_cgemm_adj<TT, false><<<dim3(a.tiles_v * a.tiles_r, nf), AdjGeom<TT>::THREADS, AdjGeom<TT>::SMEM, st>>>(a);
+        if (recip) k_cgemm_adj<G, true><<<grid, G::THREADS, adj_smem<G>(), st>>>(a);
+        else k_cgemm_adj<G, false><<<grid, G::THREADS, adj_smem<G>(), st>>>(a);
     }
-}
-
-cudaError_t launch_cgemm_adj(const GemmArgs &a, bool recip, int nf, cudaStream_t st, int tile) {
-    // 32-wide tiles waste less of the (triangular, ragged) output at moderate sizes; 64-wide tiles
-    // re-use each staged operand for twice the products when the matrices are large (tile = 0: choose
-    // by that rule; 32 or 64: as given)
-    if (tile == 0) tile = (a.nv <= 512 && a.nr <= 512) ? 32 : 64;
-    if (tile == 32) launch_adj_tt<32>(a, recip, nf, st);
-    else launch_adj_tt<64>(a, recip, nf, st);
     return cudaGetLastError();
 }
 
