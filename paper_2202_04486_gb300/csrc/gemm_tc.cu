@@ -406,7 +406,9 @@ __device__ __forceinline__ void tc_adj_body(const GemmArgs &a, int bx, int by, u
     float2 *stg = reinterpret_cast<float2 *>(sm + G::OPER);
     const int f = by;
     int vb, rb;
-    if (RECIP) {
+    if (RECIP && a.diag_only) {
+        vb = rb = bx;
+    } else if (RECIP) {
         int t = bx, row = 0, len = a.tiles_v;
         while (t >= len) { t -= len; ++row; --len; }
         vb = row;
@@ -1091,6 +1093,216 @@ __global__ void __launch_bounds__(TCP_THREADS, 1)
 }
 
 // ------------------------------------------------------------------------------------------------
+// adjoint, persistent: the product of tc_adj_body from the operand images (same MMAs in the same order, bit-identical) for
+// tiles that are written once: every tile without reciprocity, the off-diagonal ones of a symmetric model (OFF; its
+// diagonal tiles, with their mirror, run on k_tc_adj_sym_tma).  One CTA per SM walks its tiles; its roles overlap from
+// tile to tile, where the tile kernel runs load, products and stores of a tile one after the other (15 000 cycles a tile
+// at two CTAs per SM for 3 700 cycles of output at the HBM rate, nt 1024, 301 x 301, batch 32):
+//  * copy warp (8): the two images of a job (a K chunk, a half) by bulk copies of 32 KB into one of two stages;
+//  * MMA warp (9): the products of a job; two sets of accumulators fill the tensor memory;
+//  * store warps (0-7): 16 columns of 32 rows at a time, tensor memory -> the warp's own staging (two buffers of two
+//    boxes of 8 columns x 32 rows, 64-byte swizzle) -> tiled stores (clipped at nv and the last chunk of 8 of nr).
+// Tiles go to the CTAs in rounds rotated by one CTA a round, as the forward product's units.
+// ------------------------------------------------------------------------------------------------
+constexpr int TAP_STORE = 256;                 // store warps 0-7
+constexpr int TAP_THREADS = TAP_STORE + 64;    // + copy warp, MMA warp
+constexpr int TAP_STAGE = 2 * TC_ADJ_IMG;      // operand planes of a job
+constexpr int TAP_OUT = 8 * 8192;
+constexpr size_t TAP_SMEM = 2 * (size_t)TAP_STAGE + TAP_OUT + 1024;
+
+__device__ __forceinline__ void bulk_load(void *smem_dst, const void *src, uint32_t bytes, uint64_t *bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(smem_u32(smem_dst)),
+                 "l"(src), "r"(bytes), "r"(smem_u32(bar))
+                 : "memory");
+}
+// at most one of this thread's committed bulk stores still reads its shared-memory source
+__device__ __forceinline__ void bulk_wait_read1() { asm volatile("cp.async.bulk.wait_group.read 1;\n" ::: "memory"); }
+
+// tile t of nf bins: the bins of a block of SPEC_F fastest (their outputs share 256-byte lines, written by neighbouring
+// CTAs at a time), then the tiles of a bin
+template <bool OFF>
+__device__ __forceinline__ void adj_tile(const GemmArgs &a, int t, int tiles, int nf, int &f, int &vb, int &rb) {
+    const int whole = nf / SPEC_F * SPEC_F * tiles;   // tiles of the whole blocks
+    int x;
+    if (t < whole) {
+        x = t / SPEC_F;
+        f = x / tiles * SPEC_F + t % SPEC_F;
+    } else {
+        x = t - whole;
+        f = nf / SPEC_F * SPEC_F + x / tiles;
+    }
+    x %= tiles;
+    if (OFF) {   // vb < rb
+        int len = a.tiles_v - 1;
+        vb = 0;
+        while (x >= len) { x -= len; ++vb; --len; }
+        rb = vb + 1 + x;
+    } else {
+        vb = x / a.tiles_r;
+        rb = x % a.tiles_r;
+    }
+}
+
+template <bool OFF>
+__global__ void __launch_bounds__(TAP_THREADS, 1)
+    k_tc_adj_p(GemmArgs a, const __grid_constant__ CUtensorMap tmap, int tiles, int nf, int nf_act) {
+    using G = TcAdj;
+    constexpr int KC = G::KC;
+    extern __shared__ uint8_t tc_raw[];
+    __shared__ uint64_t full[2], adone[2], ddone[2], dfree[2], probe;
+    __shared__ uint32_t tmem_holder;
+    __shared__ int fail, s_copies, s_mma;
+    uint8_t *op0 = align1024(tc_raw), *out0 = op0 + 2 * TAP_STAGE;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+
+    for (int t = blockIdx.x; t < (nf - nf_act) * tiles; t += gridDim.x) {   // above the band limit
+        int f, vb, rb;
+        adj_tile<OFF>(a, t, tiles, nf - nf_act, f, vb, rb);
+        f += nf_act;
+        const long long row = (long long)a.ldr * SPEC_F;
+        zero_tile(a.C + spec_bin(f, a.sCf), row, vb * 128, 128, rb * 128, 128, a.nv, a.nr);
+        if (OFF) zero_tile(a.C + spec_bin(f, a.sCf), row, rb * 128, 128, vb * 128, 128, a.nr, a.nv);
+    }
+    const int n_tiles = nf_act * tiles, rounds = n_tiles / (int)gridDim.x;
+    const int my_tiles = rounds + (((int)blockIdx.x + rounds) % (int)gridDim.x < n_tiles % (int)gridDim.x ? 1 : 0);
+    if (my_tiles == 0) return;
+    auto tile_at = [&](int u, int &f, int &vb, int &rb) {
+        adj_tile<OFF>(a, u * (int)gridDim.x + (int)((blockIdx.x + u) % gridDim.x), tiles, nf_act, f, vb, rb);
+    };
+    constexpr int NH = OFF ? 2 : 1;
+    const int njobs = a.img_nkc * NH;
+
+    if (tid == 0) {
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&full[i], 1);
+            mbar_init(&adone[i], 1);
+            mbar_init(&ddone[i], 1);
+            mbar_init(&dfree[i], TAP_STORE / 32);
+        }
+        mbar_init(&probe, 1);
+        fail = 0;
+        s_copies = s_mma = 0;
+        fence_mbar_init();
+    }
+    if (warp == 0) tmem_alloc(&tmem_holder, 512);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tmem_holder;
+    if (a.wait_probe > 0) {   // failure-path check, before any copy or product
+        if (tid == 0 && !mbar_wait_limit(&probe, 0, a.wait_probe)) fail = 1;
+        __syncthreads();
+    }
+    volatile int *vfail = &fail;
+
+    if (*vfail) {
+        // nothing was issued
+    } else if (warp == TAP_STORE / 32) {
+        // ---------------- copy warp ----------------
+        if (lane == 0) {
+            const int nbl = a.tiles_v + a.tiles_r;
+            int g = 0;
+            for (int u = 0; u < my_tiles && !*vfail; ++u) {
+                int f, vb, rb;
+                tile_at(u, f, vb, rb);
+                for (int job = 0; job < njobs; ++job, ++g) {
+                    const int s = g & 1, kc = job / NH, half = job % NH;
+                    if (g >= 2 && !mbar_wait_bounded(&adone[s], (g / 2 - 1) & 1)) fail = 1;
+                    if (*vfail) break;
+                    const uint8_t *base = a.img + ((long long)f * a.img_nkc + kc) * nbl * (long long)TC_ADJ_IMG;
+                    uint8_t *op = op0 + s * TAP_STAGE;
+                    mbar_arrive_expect_tx(&full[s], TAP_STAGE);
+                    bulk_load(op, base + (long long)(half ? a.tiles_v + vb : vb) * TC_ADJ_IMG, TC_ADJ_IMG, &full[s]);
+                    bulk_load(op + TC_ADJ_IMG, base + (long long)(half ? rb : a.tiles_v + rb) * TC_ADJ_IMG, TC_ADJ_IMG, &full[s]);
+                    s_copies = g + 1;
+                }
+            }
+        }
+    } else if (warp == TAP_STORE / 32 + 1) {
+        // ---------------- MMA warp ----------------
+        if (lane == 0) {
+            constexpr uint32_t idp = umma_idesc(128, 128, 1, 1, 0), idn = umma_idesc(128, 128, 1, 1, 1);
+            const uint64_t a0 = umma_desc(smem_u32(op0), KC * 128, 1024), b0 = umma_desc(smem_u32(op0 + TC_ADJ_IMG), KC * 128, 1024);
+            constexpr uint64_t PL = G::PLANE >> 4;
+            int g = 0;
+            for (int u = 0; u < my_tiles; ++u) {
+                const int db = u & 1;
+                if (u >= 2 && !mbar_wait_bounded(&dfree[db], (u / 2 - 1) & 1)) fail = 1;
+                for (int job = 0; job < njobs; ++job, ++g) {
+                    const int s = g & 1, kn = min(KC, a.nb - (job / NH) * KC);
+                    if (!*vfail && !mbar_wait_bounded(&full[s], (g / 2) & 1)) fail = 1;
+                    if (*vfail) break;
+                    tc_fence_after();
+                    const uint32_t d_re = tmem + db * 256, d_im = d_re + 128;
+                    for (int ks = 0; ks < (kn + 15) / 16; ++ks) {
+                        const uint64_t o = (uint64_t)(s * (TAP_STAGE >> 4) + ks * (16 * 128 >> 4));
+                        const uint64_t ad[4] = {a0 + o, a0 + o + PL, a0 + o + 2 * PL, a0 + o + 3 * PL};
+                        const uint64_t bd[4] = {b0 + o, b0 + o + PL, b0 + o + 2 * PL, b0 + o + 3 * PL};
+                        mma_complex_split(d_re, d_im, ad, bd, idp, idn, (job > 0 || ks > 0) ? 1u : 0u);
+                    }
+                    umma_commit(&adone[s]);
+                    if (job == njobs - 1) umma_commit(&ddone[db]);
+                    s_mma = g + 1;
+                }
+                if (*vfail) break;
+            }
+        }
+    } else {
+        // ---------------- store warps ----------------
+        auto failed = [&] { return __any_sync(0xffffffffu, *vfail) != 0; };   // warp-uniform
+        const int q = warp & 3, hc = warp >> 2;   // rows 32q .., columns 64hc .. of a tile
+        uint8_t *out = out0 + warp * 8192;
+        int nst = 0;   // stores of this warp so far: they alternate between its two buffers
+        for (int u = 0; u < my_tiles; ++u) {
+            int f, vb, rb;
+            tile_at(u, f, vb, rb);
+            const int db = u & 1, v = vb * 128 + 32 * q;
+            if (!mbar_wait_bounded(&ddone[db], (u / 2) & 1)) fail = 1;
+            if (failed()) break;
+            tc_fence_after();
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const int col = 64 * hc + 16 * c, r = rb * 128 + col;
+                if (v >= a.nv || r >= a.nr) continue;   // warp-uniform
+                float re[16], im[16];
+                const uint32_t d = tmem + ((uint32_t)(32 * q) << 16) + db * 256 + col;
+                tmem_ld16(d, re);
+                tmem_ld16(d + 128, im);
+                uint8_t *buf = out + (nst++ & 1) * 4096;
+                if (lane == 0) bulk_wait_read1();   // the store before the last one has read this buffer
+                __syncwarp();
+#pragma unroll
+                for (int g8 = 0; g8 < 8; ++g8)
+                    *reinterpret_cast<float4 *>(buf + (g8 >> 2) * 2048 + lane * 64 + (((g8 & 3) ^ ((lane >> 1) & 3)) << 4)) =
+                        make_float4(re[2 * g8] * a.outscale, im[2 * g8] * a.outscale, re[2 * g8 + 1] * a.outscale,
+                                    im[2 * g8 + 1] * a.outscale);
+                fence_async_smem();
+                __syncwarp();
+                if (lane == 0) {
+                    tma_store_5d(&tmap, buf, 0, f % SPEC_F, r >> 3, v, f / SPEC_F);
+                    if (r + 8 < a.nr) tma_store_5d(&tmap, buf + 2048, 0, f % SPEC_F, (r >> 3) + 1, v, f / SPEC_F);
+                    bulk_commit();
+                }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&dfree[db]);
+        }
+        if (lane == 0) bulk_wait_all();
+    }
+    __syncthreads();
+    if (fail && tid == 0) {
+        // copies and products still in flight get one more bounded wait before the CTA frees TMEM and exits
+        for (int i = max(0, s_copies - 2); i < s_copies; ++i) mbar_wait_bounded(&full[i & 1], (i / 2) & 1);
+        for (int i = max(0, s_mma - 2); i < s_mma; ++i) mbar_wait_bounded(&adone[i & 1], (i / 2) & 1);
+        atomicOr(a.status, 2);
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) tmem_dealloc(tmem, 512);
+}
+
+// ------------------------------------------------------------------------------------------------
 cudaError_t tc_prepare() {
     cudaError_t e;
     if ((e = cudaFuncSetAttribute(k_tc_fwd<16, TC_FWD_STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcFwd<16, TC_FWD_STAGES>::SMEM))) return e;
@@ -1113,6 +1325,8 @@ cudaError_t tc_prepare() {
     if ((e = cudaFuncSetAttribute(k_tc_adj_tma<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcAdj::SMEM))) return e;
     if ((e = cudaFuncSetAttribute(k_tc_adj_sym_tma<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcAdj::SMEM))) return e;
     if ((e = cudaFuncSetAttribute(k_tc_adj_sym_tma<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcAdj::SMEM))) return e;
+    if ((e = cudaFuncSetAttribute(k_tc_adj_p<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TAP_SMEM))) return e;
+    if ((e = cudaFuncSetAttribute(k_tc_adj_p<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TAP_SMEM))) return e;
     if ((e = cudaFuncSetAttribute(k_tc_fwd_q<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcFwd<16, 1>::SMEM))) return e;
     if ((e = cudaFuncSetAttribute(k_tc_fwd_q<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcFwd<32, 1>::SMEM))) return e;
     if ((e = cudaFuncSetAttribute(k_tc_fwd_q<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcFwd<64, 1>::SMEM))) return e;
@@ -1164,6 +1378,7 @@ cudaError_t tc_encode_maps(TcMaps *m, const float2 *Xh, int nr, int nv, int ldr,
     cudaError_t e = encode_map(m->fwd, Xh, nr, nv, ldr, nf, 2, 1, 128);
     if (e == cudaSuccess) e = encode_map(m->fwd_t, Xh, nr, nv, ldr, nf, 2, 16, 8);
     if (e == cudaSuccess) e = encode_map(m->adj, Xh, nr, nv, ldr, nf, 1, 1, 128);
+    if (e == cudaSuccess) e = encode_map(m->adj32, Xh, nr, nv, ldr, nf, 1, 1, 32);
     return e;
 }
 
@@ -1217,11 +1432,35 @@ cudaError_t launch_tc_adj_queue(bool recip, const WorkQueue &q, cudaStream_t st)
     return cudaGetLastError();
 }
 
-cudaError_t launch_tc_adj(const GemmArgs &a0, bool recip, int nf, cudaStream_t st, const void *map) {
+cudaError_t launch_tc_adj(const GemmArgs &a0, bool recip, int nf, cudaStream_t st, const TcMaps *maps) {
+    const void *map = maps ? maps->adj : nullptr;
     GemmArgs a = a0;
     a.tiles_v = (a.nv + 127) / 128;
     a.tiles_r = (a.nr + 127) / 128;
     const bool img = a.img != nullptr;
+    // (a symmetric model of two tile rows has one off-diagonal tile a bin: not worth a launch of its own, 105 against 97 us
+    // at nf 513, 201 x 201)
+    if (img && maps && (!recip || (a.no_mirror && a.tiles_v > 2))) {
+        int dev = 0, sms = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return e;
+        CUtensorMap m32;
+        memcpy(&m32, maps->adj32, sizeof(m32));
+        const int nf_act = (a.nf_active > 0 && a.nf_active < nf) ? a.nf_active : nf;
+        const int tiles = recip ? a.tiles_v * (a.tiles_v - 1) / 2 : a.tiles_v * a.tiles_r;
+        const int grid = std::max(1, std::min(nf * tiles, sms));
+        if (!recip) {
+            k_tc_adj_p<false><<<grid, TAP_THREADS, TAP_SMEM, st>>>(a, m32, tiles, nf, nf_act);
+        } else {
+            if (tiles > 0) k_tc_adj_p<true><<<grid, TAP_THREADS, TAP_SMEM, st>>>(a, m32, tiles, nf, nf_act);
+            a.diag_only = 1;
+            CUtensorMap tmap;
+            memcpy(&tmap, map, sizeof(tmap));
+            k_tc_adj_sym_tma<true><<<dim3(a.tiles_v, nf), TC_THREADS, TcAdj::SMEM, st>>>(a, tmap);
+        }
+        return cudaGetLastError();
+    }
     if (recip && map && a.no_mirror) {
         CUtensorMap tmap;
         memcpy(&tmap, map, sizeof(tmap));

@@ -93,6 +93,7 @@ struct GemmArgs {
                              // at (r, v)
     const uint8_t *img;      // adjoint, split-BF16 tile kernel: the operand images of k_tc_adj_images (or null:
     int img_nkc;             // the kernel splits its operands itself), their K chunks (32 batch entries each)
+    int diag_only;           // adjoint tile kernel with reciprocity: only the diagonal tiles
     int no_mirror;           // adjoint with reciprocity: skip the mirrored copy of the off-diagonal tiles (the
                              // update of a symmetric model reads the upper tiles and the diagonal ones only;
                              // a diagonal tile still mirrors its upper half, so it stays exactly symmetric)
@@ -173,14 +174,14 @@ cudaError_t launch_tc_fwd(const GemmArgs &a, int nf, cudaStream_t st);
 // tensor maps of the model-spectra buffer (the forward product's boxes, direct and transposed, and the adjoint's
 // output boxes); encoded once per split-BF16 plan
 struct TcMaps {
-    alignas(64) unsigned char fwd[128], fwd_t[128], adj[128];
+    alignas(64) unsigned char fwd[128], fwd_t[128], adj[128], adj32[128];
 };
 cudaError_t tc_encode_maps(TcMaps *m, const float2 *Xh, int nr, int nv, int ldr, int nf);
 // persistent forward product fed by the tensor memory accelerator
 cudaError_t launch_tc_fwd_p(const GemmArgs &a, const TcMaps &maps, int nf, cudaStream_t st);
-// map (or null): the tensor map of the output boxes (TcMaps::adj): tiles written once are then stored by the tensor
-// memory accelerator
-cudaError_t launch_tc_adj(const GemmArgs &a, bool recip, int nf, cudaStream_t st, const void *map = nullptr);
+// maps (or null): tiles written once are then stored by the tensor memory accelerator, and computed by the persistent
+// kernel where the operand images are given
+cudaError_t launch_tc_adj(const GemmArgs &a, bool recip, int nf, cudaStream_t st, const TcMaps *maps = nullptr);
 // Operand images of the split-BF16 adjoint (bytes for a problem; 0 where the batch needs more than two K
 // chunks), and their construction for one step (residual spectra and gathered kernel rows of a.idx).
 size_t tc_adj_image_bytes(int nv, int nr, int nb, int nf);

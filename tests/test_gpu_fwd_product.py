@@ -1,4 +1,4 @@
-"""The persistent split-BF16 forward product at the edges of its tiles: rows around 128, columns around the chunk of
+"""The persistent split-BF16 products at the edges of its tiles: rows around 128, columns around the chunk of
 32 and the block of 8, batch blocks of 16 / 32 / 64 and beyond, the last pair of bins and band limits that cut a pair,
 and the transposed read of a symmetric model (chunks below, across and above the block diagonal).
 
@@ -39,7 +39,7 @@ def test_forward_at_tile_edges(nt, nr, nv, ns, nb):
     seed = nt + nr + nv
     D = synth.random_traces((ns, nr, nt), seed).astype(np.float32).astype(np.float64)
     X = synth.random_traces((nv, nr, nt), seed + 1).astype(np.float32).astype(np.float64)
-    idx = synth.random_indices(ns, nb, seed + 2)
+    idx = synth.random_indices(ns, nb, seed + 2, replace=True)
     plan = binding.MDCPlan(_cuda(D), nv, nb_max=nb, precision=binding.MDC_PREC_BF16X3)
     U = plan.forward(_cuda(X), _cuda(idx, torch.int32)).double().cpu().numpy()
     assert plan.sync_status() == binding.MDC_OK
@@ -76,3 +76,20 @@ def test_transposed_read_of_a_symmetric_model(n, nb):
         out.append(X.cpu().numpy())
         plan.close()
     assert np.array_equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("nt,nr,nv,ns,nb", [
+    (33, 1, 1, 3, 1), (64, 127, 7, 9, 16), (100, 128, 31, 40, 17), (128, 129, 130, 40, 32), (130, 257, 33, 70, 33),
+    (64, 300, 400, 80, 64), (64, 65, 60, 90, 65),
+])
+def test_adjoint_at_tile_edges(nt, nr, nv, ns, nb):
+    """The persistent adjoint (tiles of 128 x 128, one or two K chunks of 32; batch 65 runs on the tile kernel)."""
+    seed = nt + nr + nv
+    D = synth.random_traces((ns, nr, nt), seed).astype(np.float32).astype(np.float64)
+    R = synth.random_traces((nb, nv, nt), seed + 1).astype(np.float32).astype(np.float64)
+    idx = synth.random_indices(ns, nb, seed + 2, replace=True)
+    plan = binding.MDCPlan(_cuda(D), nv, nb_max=nb, precision=binding.MDC_PREC_BF16X3)
+    G = plan.adjoint(_cuda(R), _cuda(idx, torch.int32)).double().cpu().numpy()
+    assert plan.sync_status() == binding.MDC_OK
+    assert oracle.rel_l2(G, oracle.mdc_adjoint_fft(D, R, idx)) <= REL_L2
+    plan.close()
