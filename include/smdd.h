@@ -236,18 +236,18 @@ int mdc_forward_static(int nt, int nr, int nv, int ns, float scale, const float 
  * A plan made with MDC_PREC_BF16X3 may run the FP32 FMA kernels for a product (they are more
  * accurate than the split-BF16 bound); the tensor-core kernels are allowed for such plans only.
  * ------------------------------------------------------------------------------------------- */
-#define MDC_GEMM_SIMT    0   /* FP32 FMA kernels on the CUDA cores (adjoint: tile chosen by size) */
-#define MDC_GEMM_SIMT32  1   /* adjoint only: FP32 FMA, 32 x 32 output tiles */
-#define MDC_GEMM_SIMT64  2   /* adjoint only: FP32 FMA, 64 x 64 output tiles */
+#define MDC_GEMM_SIMT    0   /* FP32 FMA kernels on the CUDA cores (tiles chosen by size) */
+#define MDC_GEMM_SIMT32  1   /* adjoint only: FP32 FMA, 32 x 32 output tiles (scalar) */
+#define MDC_GEMM_SIMT64  2   /* adjoint only: FP32 FMA, 64 x 64 output tiles (packed pairs) */
 #define MDC_GEMM_TC      3   /* split-BF16 tcgen05 kernels (MDC_PREC_BF16X3 plans only) */
 #define MDC_GEMM_GEMV    4   /* FP32 matrix-vector kernels for few virtual sources (nv <= 8): a warp or a
                                 thread streams each gathered kernel row once.  Used where allowed: with
                                 a band limit, and for the adjoint with reciprocity, the call runs
                                 MDC_GEMM_SIMT instead. */
-#define MDC_GEMM_TC_STREAM 5 /* forward only: the split-BF16 tcgen05 product as a persistent kernel (one
-                                CTA per SM) fed by tiled copies of the tensor memory accelerator
-                                (MDC_PREC_BF16X3 plans only; MDC_ERR_UNSUPPORTED where the driver
-                                gives no tensor-map encoder) */
+#define MDC_GEMM_TC_STREAM 5 /* forward only: the split-BF16 tcgen05 product as the persistent kernel (one
+                                CTA per SM) fed by tiled copies of the tensor memory accelerator, which
+                                MDC_GEMM_TC runs too where it can (MDC_PREC_BF16X3 plans only;
+                                MDC_ERR_UNSUPPORTED where the driver gives no tensor-map encoder) */
 
 typedef struct {
     int fft_variant;   /* 0, 1 or 2: accepted and read back (1 as 0 for the lengths 128, 1024 and 8192, 2 as 0
@@ -343,7 +343,7 @@ int mdc_batch_destroy(mdc_batch_t batch);
  * second of SM clock); a CTA whose wait gives up records MDC_ERR_TIMEOUT in the plan's status word,
  * writes no products, lets products still in flight finish (one more bounded wait), frees its tensor
  * memory and returns, so the context stays usable.  With cycles > 0 every CTA of the tile kernels
- * (MDC_GEMM_TC; the streamed forward kernel ignores it) first waits on an mbarrier that nothing arrives
+ * and of the persistent kernels (MDC_GEMM_TC; MDC_GEMM_TC_STREAM ignores it) first waits on an mbarrier that nothing arrives
  * on, for `cycles` SM clock cycles, before any copy or product is issued, and then takes that path: the
  * call's products are not written (the spectral workspaces keep their previous contents) and
  * mdc_plan_sync_status returns MDC_ERR_TIMEOUT.  0 (the default) turns it off.
