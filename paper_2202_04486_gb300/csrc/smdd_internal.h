@@ -63,6 +63,7 @@ struct FftArgs {
     unsigned int *counter;
     double *loss;
     int *status;
+    int ahead;               // update: tile bid + ahead is fetched into L2 while tile bid is transformed (0: none)
     // update: Nesterov velocity (null for SGD), momentum, causality mute (first kept sample per
     // model trace, [nv][nr]; null for none)
     float *vel;
