@@ -813,10 +813,11 @@ cudaError_t launch_gemv_adj(const GemmArgs &a, int nf, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-// forward tiles: 64 x 64 (batches over 32), 128 x 32, 128 x 16 (batches up to 16): the narrowest block of the batch that
-// leaves no warp without columns
+// forward tiles: 64 x 64 (batches over 32), 64 x 32 (one CTA of 128 x 32 up to 128 rows), 128 x 16 (batches up to 16): the
+// narrowest block of the batch that leaves no warp without columns
 using FwdGeom64 = SimtGeom<4, 2, 2>;
-using FwdGeom32 = SimtGeom<4, 4, 1>;
+using FwdGeom32 = SimtGeom<4, 2, 1>;
+using FwdGeom32R = SimtGeom<4, 4, 1>;
 using FwdGeom16 = SimtGeom<8, 2, 1>;
 static_assert(adj_smem<AdjGeom64>() <= 49152 - AD_MAXNB * 4 && FwdGeom64::SMEM <= 40960 && FwdGeom32::SMEM <= 40960 &&
                   FwdGeom16::SMEM <= 40960 && FW_SMEM <= 49152 && AdjS::SMEM <= 49152 - AD_MAXNB * 4,
@@ -831,14 +832,15 @@ static void launch_fwd(const GemmArgs &a, int nf, cudaStream_t st) {
     else k_cgemm_fwd<G, SPEC_F><<<grid, G::THREADS, G::SMEM, st>>>(a);
 }
 
-// measured (us, packed tiles against the scalar kernel): 814 / 1296 (nf 1025, 301 x 301, batch 64), 237 / 304 (nf 1025, 237 x
-// 133, batch 27), 88 / 94 (nf 513, 201 x 201, batch 16), 11 / 8.4 (nf 129, 32 x 32, batch 8)
+// measured (us, packed tiles against the scalar kernel): 814 / 1296 (nf 1025, 301 x 301, batch 64), 228 / 304 (nf 1025, 237 x
+// 133, batch 27; 240 with 128-row tiles, as 510 and 439 at 301 x 301, batch 32, and 19.5 against 21.1 at 100 x 100), 88 / 94 (nf 513, 201 x 201, batch 16), 11 / 8.4 (nf 129, 32 x 32, batch 8)
 cudaError_t launch_cgemm_fwd(const GemmArgs &a, int nf, cudaStream_t st) {
     if (a.nv <= 64) {
         const dim3 grid((a.nv + FW_ROWS - 1) / FW_ROWS, (a.nb + FW_NB - 1) / FW_NB, nf);
         if (a.plain) k_cgemm_fwd_small<1><<<grid, FW_THREADS, FW_SMEM, st>>>(a);
         else k_cgemm_fwd_small<SPEC_F><<<grid, FW_THREADS, FW_SMEM, st>>>(a);
     } else if (a.nb <= 16) launch_fwd<FwdGeom16>(a, nf, st);
+    else if (a.nb <= 32 && a.nv <= 128) launch_fwd<FwdGeom32R>(a, nf, st);
     else if (a.nb <= 32) launch_fwd<FwdGeom32>(a, nf, st);
     else launch_fwd<FwdGeom64>(a, nf, st);
     return cudaGetLastError();
