@@ -846,13 +846,19 @@ cudaError_t launch_cgemm_fwd(const GemmArgs &a, int nf, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-// tile = 0: the scalar 32-wide tiles with reciprocity up to 512 columns and for matrices of one packed tile, else the
-// packed 64-wide ones (us, scalar 32 / packed 64: 1320 / 974 at nf 1025, 301 x 301, batch 64; 145 / 98 at nf 513, 256 x 256,
+// tile = 0: the scalar 32-wide tiles with reciprocity up to 512 columns, for matrices of one packed tile, and where tiles of
+// 64 would pad the output 1.5 times as much as tiles of 32 (150 x 65, batch 10, nf 513: 29 us against 37; at 150 x 150, 1.44
+// times, batch 40, the packed ones stay ahead), else the packed
+// 64-wide ones (us, scalar 32 / packed 64: 1320 / 974 at nf 1025, 301 x 301, batch 64; 145 / 98 at nf 513, 256 x 256,
 // batch 16; 275 / 240 at nf 1025, 237 x 133, batch 27; with reciprocity 107 / 130 at nf 513, 201 x 201, batch 16); 32 or 64:
 // as given
 cudaError_t launch_cgemm_adj(const GemmArgs &a0, bool recip, int nf, cudaStream_t st, int tile) {
     GemmArgs a = a0;
-    if (tile == 0) tile = (recip && a.nv <= 512) || (a.nv <= 64 && a.nr <= 64) ? 32 : 64;
+    if (tile == 0) {
+        auto padded = [](int n, int t) { return (double)((n + t - 1) / t * t); };
+        const double p32 = padded(a.nv, 32) * padded(a.nr, 32), p64 = padded(a.nv, 64) * padded(a.nr, 64);
+        tile = (recip && a.nv <= 512) || (a.nv <= 64 && a.nr <= 64) || p64 > 1.5 * p32 ? 32 : 64;
+    }
     a.tiles_v = (a.nv + tile - 1) / tile;
     a.tiles_r = (a.nr + tile - 1) / tile;
     const dim3 grid(recip ? a.tiles_v * (a.tiles_v + 1) / 2 : a.tiles_v * a.tiles_r, nf);
