@@ -34,15 +34,32 @@ __device__ __forceinline__ double warp_sum(double v) {
 // Element-wise passes.  Four elements per thread and access where every vector is 16-byte aligned (a tail and
 // unaligned vectors element by element), and the norm of what a pass writes in the same pass: one FP64 partial of the
 // sum of squares per block (fixed assignment of elements to blocks and threads).
-__device__ __forceinline__ void add_squares(SumSq &q, double &d, float4 v) {
-    const float top = fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)));
-    if (SumSq::in_range(top)) {
-        q.add(pk2(v.x, v.y));
-        q.add(pk2(v.z, v.w));
-    } else {
-        d += (double)v.x * v.x + (double)v.y * v.y + (double)v.z * v.z + (double)v.w * v.w;
+//
+// A thread's share of a long vector has hundreds of squares in each half of its FP32 pair, so the pair goes to the FP64
+// sum every NORM_RUN accesses: with two squares a half and access, 2 NORM_RUN squares of at most 2^120 (SumSq::in_range)
+// stay below 2^125, inside the FP32 range, whatever the length of the vector.
+constexpr int NORM_RUN = 16;
+
+struct NormSum {
+    SumSq q;
+    double d = 0.0;
+    int run = 0;
+    __device__ __forceinline__ void add(float4 v) {
+        const float top = fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)));
+        if (SumSq::in_range(top)) {
+            q.add(pk2(v.x, v.y));
+            q.add(pk2(v.z, v.w));
+        } else {
+            d += (double)v.x * v.x + (double)v.y * v.y + (double)v.z * v.z + (double)v.w * v.w;
+        }
+        if (++run == NORM_RUN) {
+            d += q.total();
+            q = SumSq();
+            run = 0;
+        }
     }
-}
+    __device__ __forceinline__ double total() const { return q.total() + d; }
+};
 
 __device__ __forceinline__ void block_partial(double s, double *partials) {
     __shared__ double red[VEC_THREADS / 32];
@@ -63,8 +80,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_combine_norm(float *__restrict_
                                                                 int nt, double *__restrict__ partials) {
     const float cf = which == 0 ? (float)sc->alpha : which == 1 ? (float)sc->beta : 1.f;
     const long long first = blockIdx.x * (long long)VEC_THREADS + threadIdx.x, step = (long long)gridDim.x * VEC_THREADS;
-    SumSq q;
-    double d = 0.0;
+    NormSum sum;
     auto muted = [&](float x, long long i) { return (mute && (int)(i % nt) < mute[i / nt]) ? 0.f : x; };
     const long long n4 = vec ? n / 4 : 0;
     for (long long i = first; i < n4; i += step) {
@@ -75,15 +91,15 @@ __global__ void __launch_bounds__(VEC_THREADS) k_combine_norm(float *__restrict_
             a = make_float4(a.x - cf * b.x, a.y - cf * b.y, a.z - cf * b.z, a.w - cf * b.w);
         }
         reinterpret_cast<float4 *>(y)[i] = a;
-        add_squares(q, d, a);
+        sum.add(a);
     }
     for (long long i = 4 * n4 + first; i < n; i += step) {
         float a = muted(t[i], i);
         if (which < 3) a = a - cf * y[i];
         y[i] = a;
-        add_squares(q, d, make_float4(a, 0.f, 0.f, 0.f));
+        sum.add(make_float4(a, 0.f, 0.f, 0.f));
     }
-    block_partial(q.total() + d, partials);
+    block_partial(sum.total(), partials);
 }
 
 // the norm from the partials (summed in a fixed order), then the scalar step `what`:
