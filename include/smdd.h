@@ -129,7 +129,7 @@ typedef struct {
 } smdd_params;
 
 /* One stochastic MDD step on the batch idx (Eq. 6 and the SGD update):
- *   R = P_B X - U_obs[idx],  loss = 1/2 ||R||^2 (accumulated in float64),
+ *   R = P_B X - U_obs[idx],  loss = 1/2 ||R||^2 (summed to float64 accuracy),
  *   g = P_B^H R,  X <- X - alpha * C(g),  C = C_r (reciprocity flag) or the identity.
  *   X     : [nv][nr][nt] device float32, updated in place.
  *   U_obs : [ns][nv][nt] (or [nb][nv][nt] with SMDD_UOBS_GATHERED) device float32.

@@ -1,5 +1,5 @@
 // Trace-parallel FFT kernels of the MDC hot path: model / residual / kernel spectra (rfft), the
-// residual step (inverse FFT, causal window, subtraction of the observed data, FP64 loss, forward FFT),
+// residual step (inverse FFT, causal window, subtraction of the observed data, loss to FP64 accuracy, forward FFT),
 // the SGD update (inverse FFT of the gradient spectrum, window, X <- X - alpha g, optional forward FFT
 // of the new model) and plain inverse transforms for the operator outputs.
 //
@@ -363,7 +363,7 @@ __device__ __forceinline__ double block_sum(double v, double *red) {
     return s;   // valid in thread 0
 }
 
-// Residual step: R = s * irfft(Uh)[0:nt] - U_obs[row], loss partial 1/2 sum R^2 (FP64), Rh = rfft(R)
+// Residual step: R = s * irfft(Uh)[0:nt] - U_obs[row], loss partial 1/2 sum R^2 (SumSq, then FP64), Rh = rfft(R)
 // written in place over Uh.  Trace grid: i = batch entry b, j = virtual source v.
 // tile bid of nblk tiles; the last tile to finish (atomic ticket) sums the partials of all nblk
 template <int M>
@@ -413,7 +413,8 @@ __device__ __forceinline__ void residual_body(const FftArgs &a, int bid, int nbl
     }
     double l2;
     if (SumSq::in_range(top)) {   // (a NaN passes and reaches the sum)
-        SumSq q;
+        static_assert(2 * NSLOT <= SumSq::SQUARES, "one sum for a thread's samples");
+        SumSq q(SumSq::pow2(top));
 #pragma unroll
         for (int i = 0; i < NSLOT; ++i) {
             const C2 z = join(o[0][i], o[1][i]);

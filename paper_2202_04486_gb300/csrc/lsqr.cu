@@ -1,8 +1,8 @@
 // Full-gradient MDD by LSQR (Paige & Saunders 1982), the baseline the paper compares stochastic MDD
 // against: every source at once, on the preconditioned operator A = P C (Eq. 3-4).
 //
-// The vectors are FP32 device arrays, every norm is reduced in FP64 with a fixed order (per-block
-// partials, then one block), and the scalar recurrence of the bidiagonalisation and of the plane
+// The vectors are FP32 device arrays, every norm is reduced in FP64 with a fixed order (runs of a thread's
+// elements in FP32 words that are no less exact, SumSq; then threads, blocks and one block over them in FP64), and the scalar recurrence of the bidiagonalisation and of the plane
 // rotations runs on the device (one thread), so an iteration is a fixed sequence of launches with no
 // host round trip.  The operator's forward and adjoint are the plan's own kernels with nb = ns.
 #include <cmath>
@@ -35,27 +35,40 @@ __device__ __forceinline__ double warp_sum(double v) {
 // unaligned vectors element by element), and the norm of what a pass writes in the same pass: one FP64 partial of the
 // sum of squares per block (fixed assignment of elements to blocks and threads).
 //
-// A thread's share of a long vector has hundreds of squares in each half of its FP32 pair, so the pair goes to the FP64
-// sum every NORM_RUN accesses: with two squares a half and access, 2 NORM_RUN squares of at most 2^120 (SumSq::in_range)
-// stay below 2^125, inside the FP32 range, whatever the length of the vector.
-constexpr int NORM_RUN = 16;
+// A thread's share of a long vector has hundreds of squares in each half of its FP32 pair, so the sum in the pair goes
+// to the FP64 sum after the NORM_RUN groups (eight squares a half and group) that SumSq takes, and when a larger value
+// than its bound comes.  Groups of 16 elements, whose loads are all issued before the first is used: one range check a
+// group, and the loads do not wait for the sum of the elements before (with groups of 4: +38 us a pass at 4.6e7 elements).
+constexpr int NORM_GROUP = 4;   // accesses of four elements
+constexpr int NORM_RUN = SumSq::SQUARES / (2 * NORM_GROUP);
 
 struct NormSum {
-    SumSq q;
+    SumSq q{0.f};
+    float bound = 0.f;
     double d = 0.0;
     int run = 0;
-    __device__ __forceinline__ void add(float4 v) {
-        const float top = fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)));
-        if (SumSq::in_range(top)) {
-            q.add(pk2(v.x, v.y));
-            q.add(pk2(v.z, v.w));
+    __device__ __forceinline__ void add(const float4 (&v)[NORM_GROUP]) {
+        float top = 0.f;
+#pragma unroll
+        for (int u = 0; u < NORM_GROUP; ++u)
+            top = fmaxf(top, fmaxf(fmaxf(fabsf(v[u].x), fabsf(v[u].y)), fmaxf(fabsf(v[u].z), fabsf(v[u].w))));
+        if (SumSq::in_range(top)) {   // (a NaN passes and reaches the sum)
+            if (run == NORM_RUN || SumSq::pow2(top) > bound) {
+                d += q.total();
+                bound = fmaxf(bound, SumSq::pow2(top));
+                q = SumSq(bound);
+                run = 0;
+            }
+            ++run;
+#pragma unroll
+            for (int u = 0; u < NORM_GROUP; ++u) {
+                q.add(pk2(v[u].x, v[u].y));
+                q.add(pk2(v[u].z, v[u].w));
+            }
         } else {
-            d += (double)v.x * v.x + (double)v.y * v.y + (double)v.z * v.z + (double)v.w * v.w;
-        }
-        if (++run == NORM_RUN) {
-            d += q.total();
-            q = SumSq();
-            run = 0;
+#pragma unroll
+            for (int u = 0; u < NORM_GROUP; ++u)
+                d += (double)v[u].x * v[u].x + (double)v[u].y * v[u].y + (double)v[u].z * v[u].z + (double)v[u].w * v[u].w;
         }
     }
     __device__ __forceinline__ double total() const { return q.total() + d; }
@@ -83,21 +96,43 @@ __global__ void __launch_bounds__(VEC_THREADS) k_combine_norm(float *__restrict_
     NormSum sum;
     auto muted = [&](float x, long long i) { return (mute && (int)(i % nt) < mute[i / nt]) ? 0.f : x; };
     const long long n4 = vec ? n / 4 : 0;
-    for (long long i = first; i < n4; i += step) {
-        float4 a = reinterpret_cast<const float4 *>(t)[i];
-        if (mute) a = make_float4(muted(a.x, 4 * i), muted(a.y, 4 * i + 1), muted(a.z, 4 * i + 2), muted(a.w, 4 * i + 3));
-        if (which < 3) {
-            const float4 b = reinterpret_cast<const float4 *>(y)[i];
-            a = make_float4(a.x - cf * b.x, a.y - cf * b.y, a.z - cf * b.z, a.w - cf * b.w);
+    for (long long i = first; i < n4; i += NORM_GROUP * step) {
+        float4 a[NORM_GROUP], b[NORM_GROUP];
+#pragma unroll
+        for (int u = 0; u < NORM_GROUP; ++u) {
+            const long long j = i + u * step;
+            a[u] = b[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (j < n4) {
+                a[u] = reinterpret_cast<const float4 *>(t)[j];
+                if (which < 3) b[u] = reinterpret_cast<const float4 *>(y)[j];
+            }
         }
-        reinterpret_cast<float4 *>(y)[i] = a;
+#pragma unroll
+        for (int u = 0; u < NORM_GROUP; ++u) {
+            const long long j = i + u * step;
+            if (j >= n4) continue;
+            if (mute) a[u] = make_float4(muted(a[u].x, 4 * j), muted(a[u].y, 4 * j + 1), muted(a[u].z, 4 * j + 2), muted(a[u].w, 4 * j + 3));
+            if (which < 3) a[u] = make_float4(a[u].x - cf * b[u].x, a[u].y - cf * b[u].y, a[u].z - cf * b[u].z, a[u].w - cf * b[u].w);
+            reinterpret_cast<float4 *>(y)[j] = a[u];
+        }
         sum.add(a);
     }
-    for (long long i = 4 * n4 + first; i < n; i += step) {
-        float a = muted(t[i], i);
-        if (which < 3) a = a - cf * y[i];
-        y[i] = a;
-        sum.add(make_float4(a, 0.f, 0.f, 0.f));
+    for (long long i = 4 * n4 + first; i < n; i += NORM_GROUP * step) {   // the tail, or unaligned vectors
+        float a[NORM_GROUP];
+        float4 g[NORM_GROUP];
+#pragma unroll
+        for (int u = 0; u < NORM_GROUP; ++u) a[u] = i + u * step < n ? t[i + u * step] : 0.f;
+#pragma unroll
+        for (int u = 0; u < NORM_GROUP; ++u) {
+            const long long j = i + u * step;
+            if (j < n) {
+                a[u] = muted(a[u], j);
+                if (which < 3) a[u] = a[u] - cf * y[j];
+                y[j] = a[u];
+            }
+            g[u] = make_float4(a[u], 0.f, 0.f, 0.f);
+        }
+        sum.add(g);
     }
     block_partial(sum.total(), partials);
 }
