@@ -700,13 +700,40 @@ __global__ void __launch_bounds__(G::THREADS, 512 / G::THREADS) k_cgemm_adj(Gemm
 // ------------------------------------------------------------------------------------------------
 // Few virtual sources (nv <= 8, the matrix-vector regime of a single-virtual-source inversion): the
 // products are bound by reading the batch rows of Dh once, so a warp streams one kernel row against
-// the nv model rows (forward) or a thread owns one receiver and walks the batch (adjoint).
+// the nv model rows (forward) or a thread owns one receiver and walks the batch (adjoint).  The operand that every
+// kernel row meets again -- the model rows, or the residuals' coefficients -- is staged in shared memory by the CTA, and
+// eight loads of kernel rows are on their way at a time.  (Read from the SPEC_F layout for every kernel row, a warp's
+// access touches four half lines: 231 and 222 us at nf 513, 600 x 8, batch 100,
+// against 136 and 84.)
 // ------------------------------------------------------------------------------------------------
 constexpr int GV_THREADS = 256, GV_MAXV = 8;
+constexpr int GV_KC = 256;   // columns of a chunk of the model rows (forward)
+constexpr int GV_BC = 128;   // batch entries of a chunk of the coefficients (adjoint)
 
-// forward: C[f][v][b] = sum_r A[f][v][r] Dh[f][idx_b][r]; one warp per batch entry b
 template <int NV>
-__global__ void __launch_bounds__(GV_THREADS) k_gemv_fwd(GemmArgs a) {
+__device__ __forceinline__ void gemv_reduce(float2 (&acc)[NV]) {   // over the lanes, to lane 0
+#pragma unroll
+    for (int v = 0; v < NV; ++v)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            acc[v].x += __shfl_down_sync(0xffffffffu, acc[v].x, o);
+            acc[v].y += __shfl_down_sync(0xffffffffu, acc[v].y, o);
+        }
+}
+template <int NV>
+__device__ __forceinline__ void gemv_put(const GemmArgs &a, int f, int b, const float2 (&acc)[NV]) {
+    float2 *Cf = a.C + spec_bin(f, a.sCf);
+#pragma unroll
+    for (int v = 0; v < NV; ++v)
+        if (v < a.nv) Cf[(long long)v * a.ldb * SPEC_F + spec_col(b)] = make_float2(acc[v].x * a.outscale, acc[v].y * a.outscale);
+}
+
+// forward: C[f][v][b] = sum_r A[f][v][r] Dh[f][idx_b][r]; one warp per batch entry b.  Short rows (up to GV_SHORT columns, four
+// accesses a lane and row): both operands from global memory, no barrier
+constexpr int GV_SHORT = 128;
+
+template <int NV>
+__global__ void __launch_bounds__(GV_THREADS) k_gemv_fwd_short(GemmArgs a) {
     const int f = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int b = blockIdx.y * (GV_THREADS / 32) + warp;
     if (b >= a.nb) return;   // warp-uniform; no barrier in this kernel
@@ -733,34 +760,125 @@ __global__ void __launch_bounds__(GV_THREADS) k_gemv_fwd(GemmArgs a) {
             }
         }
     }
-#pragma unroll
-    for (int v = 0; v < NV; ++v)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            acc[v].x += __shfl_down_sync(0xffffffffu, acc[v].x, o);
-            acc[v].y += __shfl_down_sync(0xffffffffu, acc[v].y, o);
+    gemv_reduce<NV>(acc);
+    if (lane == 0) gemv_put<NV>(a, f, b, acc);
+}
+
+// longer rows: the model rows staged; 2^split_log2 warps per batch entry, which take the groups of 32 columns in turn (one
+// warp in batches of 8 and more; in smaller ones the CTA's warps share the rows)
+template <int NV>
+__global__ void __launch_bounds__(GV_THREADS, NV <= 2 ? 6 : NV == 4 ? 5 : 4) k_gemv_fwd(GemmArgs a, int split_log2) {
+    constexpr int WARPS = GV_THREADS / 32, G = GV_KC / 32, ROW = GV_KC / 2;
+    constexpr int ST = (NV * ROW + GV_THREADS - 1) / GV_THREADS;   // staged units (two columns) of a thread
+    __shared__ float4 rows[2][NV][ROW];
+    __shared__ float2 part[WARPS][NV];
+    const int f = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int wb = WARPS >> split_log2, split = 1 << split_log2, p = warp / wb;
+    const int b = blockIdx.y * wb + warp % wb;
+    int s = -1;   // a warp past the batch helps to stage
+    if (b < a.nb) {
+        s = a.idx[b];
+        if (s < 0 || s >= a.ns) {
+            if (lane == 0) atomicOr(a.status, 1);
+            s = -1;
         }
-    if (lane == 0) {
-        float2 *Cf = a.C + spec_bin(f, a.sCf);
-#pragma unroll
-        for (int v = 0; v < NV; ++v)
-            if (v < a.nv) Cf[(long long)v * a.ldb * SPEC_F + spec_col(b)] = make_float2(acc[v].x * a.outscale, acc[v].y * a.outscale);
     }
+    const float2 *Af = a.A + spec_bin(f, a.sAf);
+    const float2 *d = a.Dh + (long long)f * a.sDf + (long long)(s < 0 ? 0 : s) * a.ldd;
+    float4 st[ST];
+    auto fetch = [&](int k0) {
+#pragma unroll
+        for (int u = 0; u < ST; ++u) {
+            const int e = threadIdx.x + u * GV_THREADS, v = e / ROW, c = e % ROW;
+            if (v < NV) st[u] = krow_load<SPEC_F>(Af, (long long)a.ldr * SPEC_F, v, a.nv, k0 + 2 * c, a.nr);
+        }
+    };
+    auto put = [&](int buf) {
+#pragma unroll
+        for (int u = 0; u < ST; ++u) {
+            const int e = threadIdx.x + u * GV_THREADS, v = e / ROW, c = e % ROW;
+            if (v < NV) rows[buf][v][c] = st[u];
+        }
+    };
+    float2 dv[G];
+    auto load = [&](int k0) {
+#pragma unroll
+        for (int i = 0; i < G; ++i) {
+            const int r = k0 + lane + 32 * i;
+            dv[i] = s >= 0 && r < a.nr && (i & (split - 1)) == p ? __ldg(d + r) : make_float2(0.f, 0.f);
+        }
+    };
+    float2 acc[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) acc[v] = make_float2(0.f, 0.f);
+    fetch(0);
+    load(0);
+    put(0);
+    __syncthreads();
+    int buf = 0;
+    for (int k0 = 0; k0 < a.nr; k0 += GV_KC, buf ^= 1) {
+        const bool more = k0 + GV_KC < a.nr;
+        if (more) fetch(k0 + GV_KC);
+        if (s >= 0) {
+#pragma unroll
+            for (int i = 0; i < G; ++i) {
+                if (k0 + 32 * i < a.nr && (i & (split - 1)) == p) {   // (columns past nr are zero in both operands)
+#pragma unroll
+                    for (int v = 0; v < NV; ++v) {
+                        if (v < a.nv) {
+                            const float2 x = reinterpret_cast<const float2 *>(rows[buf][v])[lane + 32 * i];
+                            acc[v].x = fmaf(x.x, dv[i].x, fmaf(-x.y, dv[i].y, acc[v].x));
+                            acc[v].y = fmaf(x.x, dv[i].y, fmaf(x.y, dv[i].x, acc[v].y));
+                        }
+                    }
+                }
+            }
+        }
+        if (more) {
+            load(k0 + GV_KC);
+            put(buf ^ 1);
+            __syncthreads();
+        }
+    }
+    gemv_reduce<NV>(acc);
+    if (split > 1) {
+        if (lane == 0) {
+#pragma unroll
+            for (int v = 0; v < NV; ++v) part[warp][v] = acc[v];
+        }
+        __syncthreads();
+        if (p == 0 && lane == 0)
+            for (int q = 1; q < split; ++q)
+#pragma unroll
+                for (int v = 0; v < NV; ++v) acc[v] = cadd(acc[v], part[warp + q * wb][v]);
+    }
+    if (b < a.nb && p == 0 && lane == 0) gemv_put<NV>(a, f, b, acc);
 }
 
 // adjoint (no reciprocity): C[f][v][r] = outscale * sum_b A[f][v][b] conj(Dh[f][idx_b][r]); one thread
 // per receiver r, the batch walked in order (the coefficients are warp-uniform broadcasts)
+constexpr int GV_FEW = 8;
+
 template <int NV>
-__global__ void __launch_bounds__(GV_THREADS) k_gemv_adj(GemmArgs a) {
-    __shared__ int sidx[AD_MAXNB];
+__device__ __forceinline__ void gemv_store(const GemmArgs &a, int f, int r, const float2 (&acc)[NV]) {
+    float2 *Cf = a.C + spec_bin(f, a.sCf);
+#pragma unroll
+    for (int v = 0; v < NV; ++v)
+        if (v < a.nv) Cf[(long long)v * a.ldr * SPEC_F + spec_col(r)] = make_float2(acc[v].x * a.outscale, acc[v].y * a.outscale);
+}
+
+// batches below GV_FEW, whose chain of latencies bounds them: coefficients from global memory, beside the kernel rows
+template <int NV>
+__global__ void __launch_bounds__(GV_THREADS) k_gemv_adj_few(GemmArgs a) {
+    __shared__ int sidx[GV_FEW];
     const int f = blockIdx.x, r = blockIdx.y * GV_THREADS + threadIdx.x;
-    for (int b = threadIdx.x; b < a.nb; b += GV_THREADS) {
-        int s = a.idx[b];
+    if (threadIdx.x < a.nb) {
+        int s = a.idx[threadIdx.x];
         if (s < 0 || s >= a.ns) {
             atomicOr(a.status, 1);
             s = -1;
         }
-        sidx[b] = s;
+        sidx[threadIdx.x] = s;
     }
     __syncthreads();
     if (r >= a.nr) return;   // after the only barrier
@@ -783,10 +901,66 @@ __global__ void __launch_bounds__(GV_THREADS) k_gemv_adj(GemmArgs a) {
             }
         }
     }
-    float2 *Cf = a.C + spec_bin(f, a.sCf);
+    gemv_store<NV>(a, f, r, acc);
+}
+
+// larger batches: the coefficients staged, eight kernel rows on their way at a time
+template <int NV>
+__global__ void __launch_bounds__(GV_THREADS) k_gemv_adj(GemmArgs a) {
+    constexpr int UB = 8;
+    __shared__ int sidx[GV_BC];
+    __shared__ __align__(16) float2 coef[GV_BC][NV];
+    const int f = blockIdx.x, r = blockIdx.y * GV_THREADS + threadIdx.x;
+    const float2 *Af = a.A + spec_bin(f, a.sAf);
+    const float2 *Df = a.Dh + (long long)f * a.sDf + r;
+    float2 acc[NV];
 #pragma unroll
-    for (int v = 0; v < NV; ++v)
-        if (v < a.nv) Cf[(long long)v * a.ldr * SPEC_F + spec_col(r)] = make_float2(acc[v].x * a.outscale, acc[v].y * a.outscale);
+    for (int v = 0; v < NV; ++v) acc[v] = make_float2(0.f, 0.f);
+    for (int b0 = 0; b0 < a.nb; b0 += GV_BC) {
+        const int n = min(GV_BC, a.nb - b0);
+        if (b0 > 0) __syncthreads();   // the last chunk has been read
+        if (threadIdx.x < GV_BC) {
+            int s = -1;
+            if (threadIdx.x < n) {
+                s = a.idx[b0 + threadIdx.x];
+                if (s < 0 || s >= a.ns) {
+                    atomicOr(a.status, 1);
+                    s = -1;
+                }
+            }
+            sidx[threadIdx.x] = s;
+        }
+        for (int e = threadIdx.x; e < a.nv * GV_BC; e += GV_THREADS) {
+            const int v = e / GV_BC, b = e % GV_BC;
+            if (b < n) coef[b][v] = __ldg(Af + (long long)v * a.ldb * SPEC_F + spec_col(b0 + b));
+        }
+        __syncthreads();
+        if (r < a.nr) {
+#pragma unroll 1
+            for (int bb = 0; bb < n; bb += UB) {   // (entries past the batch have no source)
+                float2 d[UB];
+#pragma unroll
+                for (int j = 0; j < UB; ++j) {
+                    const int s = sidx[bb + j];
+                    d[j] = s >= 0 ? __ldg(Df + (long long)s * a.ldd) : make_float2(0.f, 0.f);
+                }
+#pragma unroll
+                for (int j = 0; j < UB; ++j) {
+                    if (sidx[bb + j] < 0) continue;
+#pragma unroll
+                    for (int v = 0; v < NV; ++v) {
+                        if (v < a.nv) {
+                            const float2 c = coef[bb + j][v];
+                            // c * conj(d)
+                            acc[v].x = fmaf(c.x, d[j].x, fmaf(c.y, d[j].y, acc[v].x));
+                            acc[v].y = fmaf(c.y, d[j].x, fmaf(-c.x, d[j].y, acc[v].y));
+                        }
+                    }
+                }
+            }
+        }
+    }
+    if (r < a.nr) gemv_store<NV>(a, f, r, acc);
 }
 
 bool gemv_supported(int nv) { return nv >= 1 && nv <= GV_MAXV; }
@@ -794,11 +968,20 @@ bool gemv_supported(int nv) { return nv >= 1 && nv <= GV_MAXV; }
 cudaError_t launch_gemv_fwd(const GemmArgs &a, int nf, cudaStream_t st) {
     if (!gemv_supported(a.nv) || nf < 1) return cudaErrorInvalidValue;
     if (a.nf_active > 0 && a.nf_active < nf) return cudaErrorInvalidValue;   // band limits use the tiled kernels
-    const dim3 grid(nf, (a.nb + GV_THREADS / 32 - 1) / (GV_THREADS / 32));
-    if (a.nv == 1) k_gemv_fwd<1><<<grid, GV_THREADS, 0, st>>>(a);
-    else if (a.nv <= 2) k_gemv_fwd<2><<<grid, GV_THREADS, 0, st>>>(a);
-    else if (a.nv <= 4) k_gemv_fwd<4><<<grid, GV_THREADS, 0, st>>>(a);
-    else k_gemv_fwd<8><<<grid, GV_THREADS, 0, st>>>(a);
+    constexpr int WARPS = GV_THREADS / 32;
+    int split = 0;   // (log2)
+    if (a.nr > GV_SHORT)
+        while (WARPS >> split > 1 && (WARPS >> (split + 1)) >= a.nb) ++split;
+    const int wb = WARPS >> split;
+    const dim3 grid(nf, (a.nb + wb - 1) / wb);
+    auto go = [&](auto kern, auto shorter) {
+        if (a.nr > GV_SHORT) kern<<<grid, GV_THREADS, 0, st>>>(a, split);
+        else shorter<<<grid, GV_THREADS, 0, st>>>(a);
+    };
+    if (a.nv == 1) go(k_gemv_fwd<1>, k_gemv_fwd_short<1>);
+    else if (a.nv <= 2) go(k_gemv_fwd<2>, k_gemv_fwd_short<2>);
+    else if (a.nv <= 4) go(k_gemv_fwd<4>, k_gemv_fwd_short<4>);
+    else go(k_gemv_fwd<8>, k_gemv_fwd_short<8>);
     return cudaGetLastError();
 }
 
@@ -806,10 +989,14 @@ cudaError_t launch_gemv_adj(const GemmArgs &a, int nf, cudaStream_t st) {
     if (!gemv_supported(a.nv) || nf < 1 || a.nb > AD_MAXNB) return cudaErrorInvalidValue;
     if (a.nf_active > 0 && a.nf_active < nf) return cudaErrorInvalidValue;
     const dim3 grid(nf, (a.nr + GV_THREADS - 1) / GV_THREADS);
-    if (a.nv == 1) k_gemv_adj<1><<<grid, GV_THREADS, 0, st>>>(a);
-    else if (a.nv <= 2) k_gemv_adj<2><<<grid, GV_THREADS, 0, st>>>(a);
-    else if (a.nv <= 4) k_gemv_adj<4><<<grid, GV_THREADS, 0, st>>>(a);
-    else k_gemv_adj<8><<<grid, GV_THREADS, 0, st>>>(a);
+    auto go = [&](auto kern, auto few) {
+        if (a.nb >= GV_FEW) kern<<<grid, GV_THREADS, 0, st>>>(a);
+        else few<<<grid, GV_THREADS, 0, st>>>(a);
+    };
+    if (a.nv == 1) go(k_gemv_adj<1>, k_gemv_adj_few<1>);
+    else if (a.nv <= 2) go(k_gemv_adj<2>, k_gemv_adj_few<2>);
+    else if (a.nv <= 4) go(k_gemv_adj<4>, k_gemv_adj_few<4>);
+    else go(k_gemv_adj<8>, k_gemv_adj_few<8>);
     return cudaGetLastError();
 }
 
