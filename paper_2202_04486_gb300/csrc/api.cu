@@ -986,7 +986,8 @@ int mdc_plan_autotune(mdc_plan_t p, int nb, int flags, int reps, mdc_config *bes
     }
     if (rc == MDC_OK) {
         double tbest = 1e300;
-        const int cand[4] = {MDC_GEMM_SIMT32, MDC_GEMM_SIMT64, MDC_GEMM_TC, MDC_GEMM_GEMV};
+        // (MDC_GEMM_SIMT: for few rows its rule takes tiles that neither of the named ones is)
+        const int cand[5] = {MDC_GEMM_SIMT, MDC_GEMM_SIMT32, MDC_GEMM_SIMT64, MDC_GEMM_TC, MDC_GEMM_GEMV};
         for (int c : cand) {
             if (c == MDC_GEMM_TC && p->prec != MDC_PREC_BF16X3) continue;
             if (c == MDC_GEMM_GEMV && (!gemv_supported(p->nv) || recip)) continue;

@@ -158,10 +158,12 @@ __global__ void __launch_bounds__(FW_THREADS, 4) k_cgemm_fwd_small(GemmArgs a) {
 // adjoint: C[f][v][r] = outscale * sum_k A'[v][k] B'[k][r]
 //   k < nb :  A' = Rh[f][v][k],            B' = conj(Dh[f][idx_k][r])
 //   k >= nb (reciprocity only, k' = k - nb):  A' = conj(Dh[f][idx_k'][v]),  B' = Rh[f][r][k']
-// 32 x 32 tiles with scalar products (4 x 4 outputs per thread, chunks of 16): finer at triangular and ragged edges
-// than the packed 64 x 64 tiles below.  With reciprocity both halves of a chunk are staged at once, one latency: 107
-// us against 130 us at nf 513, 201 x 201, batch 16 (1057 and 1118 us at batch 201).
-// CTA tile TT x TT.  A warp covers 4*VPN rows x TT columns: lane (vp = lane / RG,
+// TV x TT tiles with scalar products (4 x 4 outputs per thread, chunks of 16).  32 x 32: finer at triangular and ragged
+// edges than the packed 64 x 64 tiles below.  With reciprocity both halves of a chunk are staged at once, one latency: 107
+// us against 130 us at nf 513, 201 x 201, batch 16 (1057 and 1118 us at batch 201).  16 x 64: a warp covers 8 rows x 64
+// columns, against 16 x 32, so that few rows leave fewer outputs of a warp unused (us, 32 x 32 / 16 x 64, batch 64: 74 / 54 at nf 257,
+// 600 columns x 8 rows; 154 / 97 at nf 1025, 300 x 16).
+// A warp covers 4*VPN rows x TT columns: lane (vp = lane / RG,
 // rg = lane % RG) owns rows v0 + 4*VPN*w + 4vp + {0,1,2,3} and columns r0 + {2rg, 2rg+1, 2rg+TT/2,
 // 2rg+TT/2+1}.  Operands are staged by cp.async in their global layouts -- residual-spectrum rows [v][k]
 // and kernel-spectrum rows [k][r] -- and conjugated when used; chunks of 16 k per half.  Warps whose
@@ -169,25 +171,27 @@ __global__ void __launch_bounds__(FW_THREADS, 4) k_cgemm_fwd_small(GemmArgs a) {
 // ------------------------------------------------------------------------------------------------
 constexpr int AD_KC = 16, AD_LDR = AD_KC + 2, AD_MAXNB = 1024;
 
+template <int TV_, int TT_, bool RECIP>
 struct AdjS {
-    static constexpr int TT = 32;
+    static constexpr int TV = TV_, TT = TT_;
+    static_assert(!RECIP || TV == TT, "mirrored tiles are square");
     static constexpr int RG = TT / 4;             // lanes along r
     static constexpr int VPN = 32 / RG;           // lane groups along v
     static constexpr int WROWS = 4 * VPN;         // rows per warp
-    static constexpr int WARPS = TT / WROWS;
+    static constexpr int WARPS = TV / WROWS;
     static constexpr int THREADS = 32 * WARPS;
-    static constexpr int RROWS = TT * AD_LDR;     // float2: residual rows of one block
+    static constexpr int RROWS = TV * AD_LDR;     // float2: residual rows of one block
     static constexpr int DROWS = AD_KC * TT;      // float2: kernel rows at one block's columns
-    static constexpr size_t SMEM_OPER = 2 * (RROWS + DROWS) * sizeof(float2);
-    static constexpr size_t SMEM_MIRROR = TT * (TT + 1) * sizeof(float2);
+    static constexpr size_t SMEM_OPER = (RECIP ? 2 : 1) * (RROWS + DROWS) * sizeof(float2);
+    static constexpr size_t SMEM_MIRROR = RECIP ? TT * (TT + 1) * sizeof(float2) : 0;
     static constexpr size_t SMEM = SMEM_OPER > SMEM_MIRROR ? SMEM_OPER : SMEM_MIRROR;
 };
 
-// stage rows [c0, c0 + TT) x k [k0, k0 + 16) of Rh (row pitch ldb) into s[TT][AD_LDR]
+// stage rows [c0, c0 + ROWS) x k [k0, k0 + 16) of Rh (row pitch ldb) into s[ROWS][AD_LDR], by NT threads
+template <int ROWS, int NT>
 __device__ __forceinline__ void stage_rrows(float2 *s, const float2 *Rf, int ldb, int c0, int nc, int k0, int nb, int tid) {
-    constexpr int TT = AdjS::TT, NT = AdjS::THREADS;
 #pragma unroll
-    for (int u = 0; u < TT * AD_KC / 2 / NT; ++u) {
+    for (int u = 0; u < ROWS * AD_KC / 2 / NT; ++u) {
         const int c = tid + u * NT, row = c >> 3, part = c & 7;
         const int k = k0 + 2 * part;
         int bytes = 0;
@@ -201,9 +205,10 @@ __device__ __forceinline__ void stage_rrows(float2 *s, const float2 *Rf, int ldb
 }
 
 // stage kernel rows idx[k0 .. k0 + 16) at columns [c0, c0 + TT) into s[16][TT]
+template <int TT, int NT>
 __device__ __forceinline__ void stage_drows(float2 *s, const float2 *Df, int ldd, const int *sidx, int c0, int nc, int k0,
                                             int nb, int tid) {
-    constexpr int TT = AdjS::TT, NT = AdjS::THREADS, PARTS = TT / 2;
+    constexpr int PARTS = TT / 2;
 #pragma unroll
     for (int u = 0; u < AD_KC * TT / 2 / NT; ++u) {
         const int c = tid + u * NT, kk = c / PARTS, part = c % PARTS;
@@ -229,14 +234,14 @@ __device__ __forceinline__ void cmac_c(float2 &acc, float2 a, float2 b) {
     acc.y = fmaf(-a.x, b.y, acc.y);
 }
 
-template <bool RECIP>
-__global__ void __launch_bounds__(AdjS::THREADS, 8) k_cgemm_adj_small(GemmArgs a) {
-    using G = AdjS;
-    constexpr int TT = G::TT;
+template <int TV, int TT, bool RECIP>
+__global__ void __launch_bounds__(64, 8) k_cgemm_adj_small(GemmArgs a) {
+    using G = AdjS<TV, TT, RECIP>;
+    static_assert(G::THREADS == 64, "two warps");
     extern __shared__ __align__(16) float2 gsm[];
-    float2 *sRv = gsm;                  // [TT][AD_LDR]  Rh rows of the v block
+    float2 *sRv = gsm;                  // [TV][AD_LDR]  Rh rows of the v block
     float2 *sDr = sRv + G::RROWS;       // [16][TT]      kernel rows at the r block
-    float2 *sRr = sDr + G::DROWS;       // [TT][AD_LDR]  Rh rows of the r block (reciprocity)
+    float2 *sRr = sDr + G::DROWS;       // [TV][AD_LDR]  Rh rows of the r block (reciprocity)
     float2 *sDv = sRr + G::RROWS;       // [16][TT]      kernel rows at the v block (reciprocity)
     __shared__ int sidx[AD_MAXNB];
     const int f = blockIdx.y;
@@ -250,11 +255,11 @@ __global__ void __launch_bounds__(AdjS::THREADS, 8) k_cgemm_adj_small(GemmArgs a
         vb = blockIdx.x / a.tiles_r;
         rb = blockIdx.x % a.tiles_r;
     }
-    const int v0 = vb * TT, r0 = rb * TT;
+    const int v0 = vb * TV, r0 = rb * TT;
     if (a.nf_active > 0 && f >= a.nf_active) {
         const long long row = (long long)a.ldr * SPEC_F;
-        zero_tile(a.C + spec_bin(f, a.sCf), row, v0, TT, r0, TT, a.nv, a.nr);
-        if (RECIP) zero_tile(a.C + spec_bin(f, a.sCf), row, r0, TT, v0, TT, a.nr, a.nv);
+        zero_tile(a.C + spec_bin(f, a.sCf), row, v0, TV, r0, TT, a.nv, a.nr);
+        if (RECIP) zero_tile(a.C + spec_bin(f, a.sCf), row, r0, TT, v0, TV, a.nr, a.nv);
         return;
     }
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -281,11 +286,11 @@ __global__ void __launch_bounds__(AdjS::THREADS, 8) k_cgemm_adj_small(GemmArgs a
         for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
 
     for (int k0 = 0; k0 < a.nb; k0 += AD_KC) {
-        stage_rrows(sRv, Rf, a.ldb, v0, a.nv, k0, a.nb, tid);
-        stage_drows(sDr, Df, a.ldd, sidx, r0, a.nr, k0, a.nb, tid);
+        stage_rrows<TV, G::THREADS>(sRv, Rf, a.ldb, v0, a.nv, k0, a.nb, tid);
+        stage_drows<TT, G::THREADS>(sDr, Df, a.ldd, sidx, r0, a.nr, k0, a.nb, tid);
         if (RECIP) {
-            stage_rrows(sRr, Rf, a.ldb, r0, a.nr, k0, a.nb, tid);
-            stage_drows(sDv, Df, a.ldd, sidx, v0, a.nv, k0, a.nb, tid);
+            stage_rrows<TV, G::THREADS>(sRr, Rf, a.ldb, r0, a.nr, k0, a.nb, tid);
+            stage_drows<TT, G::THREADS>(sDv, Df, a.ldd, sidx, v0, a.nv, k0, a.nb, tid);
         }
         cp_async_commit();
         cp_async_wait<0>();
@@ -1000,14 +1005,14 @@ cudaError_t launch_gemv_adj(const GemmArgs &a, int nf, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-// forward tiles: 64 x 64 (batches over 32), 64 x 32 (one CTA of 128 x 32 up to 128 rows), 128 x 16 (batches up to 16): the
-// narrowest block of the batch that leaves no warp without columns
-using FwdGeom64 = SimtGeom<4, 2, 2>;
-using FwdGeom32 = SimtGeom<4, 2, 1>;
-using FwdGeom32R = SimtGeom<4, 4, 1>;
-using FwdGeom16 = SimtGeom<8, 2, 1>;
+// forward tiles
+using FwdGeom64 = SimtGeom<4, 2, 2>;    // 64 x 64
+using FwdGeom32 = SimtGeom<4, 2, 1>;    // 64 x 32
+using FwdGeom32R = SimtGeom<4, 4, 1>;   // 128 x 32
+using FwdGeom16 = SimtGeom<8, 2, 1>;    // 128 x 16
 static_assert(adj_smem<AdjGeom64>() <= 49152 - AD_MAXNB * 4 && FwdGeom64::SMEM <= 40960 && FwdGeom32::SMEM <= 40960 &&
-                  FwdGeom16::SMEM <= 40960 && FW_SMEM <= 49152 && AdjS::SMEM <= 49152 - AD_MAXNB * 4,
+                  FwdGeom16::SMEM <= 40960 && FW_SMEM <= 49152 && AdjS<32, 32, true>::SMEM <= 49152 - AD_MAXNB * 4 &&
+                  AdjS<16, 64, false>::SMEM <= 49152 - AD_MAXNB * 4,
               "no opt-in to more shared memory");
 
 cudaError_t gemm_prepare() { return cudaSuccess; }
@@ -1019,43 +1024,89 @@ static void launch_fwd(const GemmArgs &a, int nf, cudaStream_t st) {
     else k_cgemm_fwd<G, SPEC_F><<<grid, G::THREADS, G::SMEM, st>>>(a);
 }
 
-// measured (us, packed tiles against the scalar kernel): 814 / 1296 (nf 1025, 301 x 301, batch 64), 228 / 304 (nf 1025, 237 x
-// 133, batch 27; 240 with 128-row tiles, as 510 and 439 at 301 x 301, batch 32, and 19.5 against 21.1 at 100 x 100), 88 / 94 (nf 513, 201 x 201, batch 16), 11 / 8.4 (nf 129, 32 x 32, batch 8)
+// outputs that tiles of geometry G compute for a product, padding included
+template <class G>
+static double padded_outputs(const GemmArgs &a) {
+    return (double)((a.nv + G::BI - 1) / G::BI * G::BI) * ((a.nb + G::BJ - 1) / G::BJ * G::BJ);
+}
+
+// The geometry by the rows nv and the batch nb; us measured at nf 257, 300 columns unless stated (scalar / 128 x 16 /
+// 128 x 32 / 64 x 32 / 64 x 64):
+//   nb <= 16, nv <= 128: scalar          (100 rows, batch 16: 39.5 / 45.5 / 65 / 65 / 69; 32: 8.4 against 11 at nf 129)
+//   nb <= 16, more rows: 128 x 16        (200, 16: 76 / 71 / - / 113 / 124)
+//   up to 32 rows:       64 x 64         (24, 24: 40 / 64 / 41 / 41 / 37; 24, 64: 69 / 112 / 45 / 62 / 39)
+//   nb <= 32, up to 64:  64 x 32         (48, 32: 65 / 64 / 62 / 43 / 59)
+//   nb <= 32, up to 128: 128 x 32        (100 x 100, batch 32: 19.5 against 21.1 for 64 x 32)
+//   nb <= 32, more rows: 64 x 32         (301, 32, nf 1025: 439 against 510 for 128 x 32)
+//   larger batches: the least padded outputs, weighted by the time per output of the tiles (16 columns 1.3, 32 columns
+//   1.1 times that of 64 x 64)           (128, 48: 108 / 98 / 117 / 115 / 108; 256, 80: - / 265 / - / 287 / 320;
+//                                         301, 80: - / 363 / - / 336 / 393; 301, 64: - / - / - / 238 / 225)
 cudaError_t launch_cgemm_fwd(const GemmArgs &a, int nf, cudaStream_t st) {
-    if (a.nv <= 64) {
+    if (a.nb <= 16 && a.nv <= 128) {
         const dim3 grid((a.nv + FW_ROWS - 1) / FW_ROWS, (a.nb + FW_NB - 1) / FW_NB, nf);
         if (a.plain) k_cgemm_fwd_small<1><<<grid, FW_THREADS, FW_SMEM, st>>>(a);
         else k_cgemm_fwd_small<SPEC_F><<<grid, FW_THREADS, FW_SMEM, st>>>(a);
-    } else if (a.nb <= 16) launch_fwd<FwdGeom16>(a, nf, st);
-    else if (a.nb <= 32 && a.nv <= 128) launch_fwd<FwdGeom32R>(a, nf, st);
-    else if (a.nb <= 32) launch_fwd<FwdGeom32>(a, nf, st);
-    else launch_fwd<FwdGeom64>(a, nf, st);
+    } else if (a.nb <= 16) {
+        launch_fwd<FwdGeom16>(a, nf, st);
+    } else if (a.nv <= 32) {
+        launch_fwd<FwdGeom64>(a, nf, st);
+    } else if (a.nb <= 32) {
+        if (a.nv > 64 && a.nv <= 128) launch_fwd<FwdGeom32R>(a, nf, st);
+        else launch_fwd<FwdGeom32>(a, nf, st);
+    } else {
+        const double w16 = 1.3 * padded_outputs<FwdGeom16>(a), w32 = 1.1 * padded_outputs<FwdGeom32>(a), w64 = padded_outputs<FwdGeom64>(a);
+        if (w64 <= w32 && w64 <= w16) launch_fwd<FwdGeom64>(a, nf, st);
+        else if (w32 <= w16) launch_fwd<FwdGeom32>(a, nf, st);
+        else launch_fwd<FwdGeom16>(a, nf, st);
+    }
     return cudaGetLastError();
 }
 
-// tile = 0: the scalar 32-wide tiles with reciprocity up to 512 columns, for matrices of one packed tile, and where tiles of
-// 64 would pad the output 1.5 times as much as tiles of 32 (150 x 65, batch 10, nf 513: 29 us against 37; at 150 x 150, 1.44
-// times, batch 40, the packed ones stay ahead), else the packed
-// 64-wide ones (us, scalar 32 / packed 64: 1320 / 974 at nf 1025, 301 x 301, batch 64; 145 / 98 at nf 513, 256 x 256,
-// batch 16; 275 / 240 at nf 1025, 237 x 133, batch 27; with reciprocity 107 / 130 at nf 513, 201 x 201, batch 16); 32 or 64:
-// as given
+// tile = 0, by the sizes (us at nf 257 unless stated):
+//  * reciprocity: the packed 64-wide tiles unless their upper triangle has more than 1.2 times the outputs of the scalar
+//    32-wide ones (scalar / packed: 201 columns, batch 16, nf 513, 1.43 times: 107 / 130; 210, batch 32, 1.43: 103 / 116;
+//    400, batch 16, 1.23: 185 / 187; 128, batch 16, 1.20: 31.0 / 29.7; 192, batch 32, 1.14: 82 / 78; 256, batch 32, 1.11:
+//    131 / 118; 512, batch 64, 1.06: 848 / 720);
+//  * up to 16 rows and more than 64 columns: the scalar 16 x 64 tiles (scalar 32 x 32 / 16 x 64, batch 64: 17.7 / 16.2 at
+//    65 columns x 4 rows, 47 / 34 at 300 x 8, 122 / 81 at 1000 x 16; batch 8: 7.7 / 7.8, 14.3 / 10.3, 26.7 / 18.5);
+//  * matrices of one packed tile, and where tiles of 64 would pad the output 1.5 times as much as tiles of 32: the scalar
+//    32-wide ones (150 x 65, batch 10, nf 513: 29 against 37; at 150 x 150, 1.44 times, batch 40, the packed ones stay ahead);
+//  * else the packed 64-wide ones (scalar 32 / packed 64: 1320 / 974 at nf 1025, 301 x 301, batch 64; 145 / 98 at nf 513,
+//    256 x 256, batch 16; 275 / 240 at nf 1025, 237 x 133, batch 27).
+// 32 or 64: the scalar 32-wide or the packed 64-wide tiles
 cudaError_t launch_cgemm_adj(const GemmArgs &a0, bool recip, int nf, cudaStream_t st, int tile) {
     GemmArgs a = a0;
-    if (tile == 0) {
-        auto padded = [](int n, int t) { return (double)((n + t - 1) / t * t); };
-        const double p32 = padded(a.nv, 32) * padded(a.nr, 32), p64 = padded(a.nv, 64) * padded(a.nr, 64);
-        tile = (recip && a.nv <= 512) || (a.nv <= 64 && a.nr <= 64) || p64 > 1.5 * p32 ? 32 : 64;
+    auto tiles = [](int n, int t) { return (n + t - 1) / t; };
+    auto grid = [&](int tv, int tr) {
+        a.tiles_v = tiles(a.nv, tv);
+        a.tiles_r = tiles(a.nr, tr);
+        return dim3(recip ? a.tiles_v * (a.tiles_v + 1) / 2 : a.tiles_v * a.tiles_r, nf);
+    };
+    if (tile == 0 && !recip && a.nv <= 16 && a.nr > 64) {
+        using F = AdjS<16, 64, false>;
+        const dim3 g = grid(16, 64);
+        k_cgemm_adj_small<16, 64, false><<<g, F::THREADS, F::SMEM, st>>>(a);
+        return cudaGetLastError();
     }
-    a.tiles_v = (a.nv + tile - 1) / tile;
-    a.tiles_r = (a.nr + tile - 1) / tile;
-    const dim3 grid(recip ? a.tiles_v * (a.tiles_v + 1) / 2 : a.tiles_v * a.tiles_r, nf);
-    using G = AdjGeom64;
-    if (tile == 32) {
-        if (recip) k_cgemm_adj_small<true><<<grid, AdjS::THREADS, AdjS::SMEM, st>>>(a);
-        else k_cgemm_adj_small<false><<<grid, AdjS::THREADS, AdjS::SMEM, st>>>(a);
+    bool scalar = tile == 32;
+    if (tile == 0 && recip) {
+        const double t32 = tiles(a.nv, 32), t64 = tiles(a.nv, 64);
+        scalar = 4 * t64 * (t64 + 1) > 1.2 * t32 * (t32 + 1);
+    } else if (tile == 0) {
+        scalar = (a.nv <= 64 && a.nr <= 64) ||
+                 4. * tiles(a.nv, 64) * tiles(a.nr, 64) > 1.5 * tiles(a.nv, 32) * tiles(a.nr, 32);
+    }
+    if (scalar) {
+        using F = AdjS<32, 32, false>;
+        using R = AdjS<32, 32, true>;
+        const dim3 g = grid(32, 32);
+        if (recip) k_cgemm_adj_small<32, 32, true><<<g, R::THREADS, R::SMEM, st>>>(a);
+        else k_cgemm_adj_small<32, 32, false><<<g, F::THREADS, F::SMEM, st>>>(a);
     } else {
-        if (recip) k_cgemm_adj<G, true><<<grid, G::THREADS, adj_smem<G>(), st>>>(a);
-        else k_cgemm_adj<G, false><<<grid, G::THREADS, adj_smem<G>(), st>>>(a);
+        using G = AdjGeom64;
+        const dim3 g = grid(64, 64);
+        if (recip) k_cgemm_adj<G, true><<<g, G::THREADS, adj_smem<G>(), st>>>(a);
+        else k_cgemm_adj<G, false><<<g, G::THREADS, adj_smem<G>(), st>>>(a);
     }
     return cudaGetLastError();
 }
