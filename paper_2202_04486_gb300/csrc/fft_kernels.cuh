@@ -467,9 +467,23 @@ __global__ void __launch_bounds__(Team<M>::THREADS, Team<M>::MINB) k_residual(Ff
 // spectra below the block diagonal are left to launch_mirror_lower or to the transposed read of the
 // forward product.  Traces of the diagonal blocks run in both orders (their mirrors are in the same
 // block row and column), so every element of X is written once.
-template <int M, bool KEEP, bool EXT>
+//
+// EXT: 0 SGD, 1 SGD with the causality mute, 2 with a velocity or Adam moments (and the mute).  (The mute without the code
+// of the others: update 1200 -> 1030 us at nt 1500, 300 x 300, 330 -> 243 us at nt 1024, 201 x 201.)
+//
+// At M = 1536 a thread with a velocity or moments has 24 to 32 more values to hold than 80 registers take: one CTA per SM
+// at 168 registers there, without spills and with the model loaded early (two CTAs at 80 registers spill 468 to 716 bytes a
+// thread; us at nt 1500, two / one CTA: 300 x 300 N-SGD 1389 / 1366, Adam 1730 / 1630; 600 x 600 symmetric N-SGD 3611 /
+// 3121, Adam 4939 / 3779).
+template <int M, int EXT>
+constexpr bool one_cta() { return M == 1536 && EXT == 2; }
+template <int M, int EXT>
+constexpr int update_minb() { return one_cta<M, EXT>() ? 1 : Team<M>::MINB; }
+
+template <int M, bool KEEP, int EXT>
 __device__ __forceinline__ void update_body(const FftArgs &a, int bid_in) {
     constexpr int TR = Team<M>::TR;
+    constexpr bool LATE = Team<M>::LATE && !one_cta<M, EXT>();
     const int bid = a.g.sym ? sym_tile_to_full(a.g, TR, bid_in) : bid_in;
     const PairCtx<M> x = pair_ctx<M>(a.g, bid);
     spec_to_smem<M>(a, x);
@@ -480,14 +494,14 @@ __device__ __forceinline__ void update_body(const FftArgs &a, int bid_in) {
     float2 xo[2][NSLOT];   // model samples, loaded before the middle passes (their latency overlaps the rest)
 #pragma unroll
     for (int k = 0; k < 2; ++k)
-        if (!Team<M>::LATE) time_load<M>(xo[k], a.tout + time_off<M>(a.g, x.c[k]), a.nt, x.c[k].valid, a.vec, x.s);
+        if (!LATE) time_load<M>(xo[k], a.tout + time_off<M>(a.g, x.c[k]), a.nt, x.c[k].valid, a.vec, x.s);
     mid_passes<M, true, fft_npass(M) - 2>(x.buf, x.s, a.tw);
     group_sync<M>();
     C2 v[FFT_P];
     inv_last<M>(v, x.buf, x.s);
 #pragma unroll
     for (int k = 0; k < 2; ++k)
-        if (Team<M>::LATE) time_load<M>(xo[k], a.tout + time_off<M>(a.g, x.c[k]), a.nt, x.c[k].valid, a.vec, x.s);
+        if (LATE) time_load<M>(xo[k], a.tout + time_off<M>(a.g, x.c[k]), a.nt, x.c[k].valid, a.vec, x.s);
     const float nas = -a.alpha * a.s;
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
@@ -496,7 +510,7 @@ __device__ __forceinline__ void update_body(const FftArgs &a, int bid_in) {
         // the mirror trace (r, v) of a trace above the block diagonal
         const bool mir = a.g.sym && c.valid && c.i / TR > c.j / TR;
         const long long moff = mir ? (long long)c.j * a.g.tsi + (long long)c.i * a.g.tsj : 0;
-        if constexpr (!EXT) {
+        if constexpr (EXT == 0) {
             // SGD: X <- X - alpha g
 #pragma unroll
             for (int i = 0; i < NSLOT; ++i) {
@@ -512,22 +526,22 @@ __device__ __forceinline__ void update_body(const FftArgs &a, int bid_in) {
             // m <- b1 m + (1-b1) g, v <- b2 v + (1-b2) g^2, X <- X - alpha (c1 m) / (sqrt(c2 v) + eps)
             const int first = (a.mute && c.valid) ? __ldg(a.mute + (long long)c.j * a.g.ni + c.i) : 0;
             float2 m0[NSLOT], m1[NSLOT];   // velocity, or the moments
-            if (a.adam_m) {
+            if (EXT == 2 && a.adam_m) {
                 time_load<M>(m0, a.adam_m + off, a.nt, c.valid, a.vec, x.s);
                 time_load<M>(m1, a.adam_v + off, a.nt, c.valid, a.vec, x.s);
-            } else if (a.vel) {
+            } else if (EXT == 2 && a.vel) {
                 time_load<M>(m0, a.vel + off, a.nt, c.valid, a.vec, x.s);
             }
             auto sample = [&](int t, float g0, float xv, float &p, float &q) {
                 float z;
-                if (a.adam_m) {
+                if (EXT == 2 && a.adam_m) {
                     const float g = (t >= first) ? a.s * g0 : 0.f;
                     p = fmaf(a.beta1, p, (1.f - a.beta1) * g);
                     q = fmaf(a.beta2, q, (1.f - a.beta2) * (g * g));
                     z = xv - a.alpha * (p * a.c1) / (sqrtf(q * a.c2) + a.eps);
                 } else {
                     const float st = (t >= first) ? nas * g0 : 0.f;
-                    if (a.vel) {
+                    if (EXT == 2 && a.vel) {
                         p = fmaf(a.mu, p, st);
                         z = fmaf(a.mu, p, xv + st);
                     } else {
@@ -544,17 +558,17 @@ __device__ __forceinline__ void update_body(const FftArgs &a, int bid_in) {
                                        sample(i0 + 1, g.y, xo[k][i].y, m0[i].y, m1[i].y));
             }
             if (c.valid) {
-                if (a.adam_m) {
+                if (EXT == 2 && a.adam_m) {
                     time_store<M>(m0, a.adam_m + off, a.nt, a.vec, x.s);
                     time_store<M>(m1, a.adam_v + off, a.nt, a.vec, x.s);
-                } else if (a.vel) {
+                } else if (EXT == 2 && a.vel) {
                     time_store<M>(m0, a.vel + off, a.nt, a.vec, x.s);
                 }
                 if (mir) {   // the mirror trace of the velocity or of the moments
-                    if (a.adam_m) {
+                    if (EXT == 2 && a.adam_m) {
                         time_store<M>(m0, a.adam_m + moff, a.nt, a.vec, x.s);
                         time_store<M>(m1, a.adam_v + moff, a.nt, a.vec, x.s);
-                    } else if (a.vel) {
+                    } else if (EXT == 2 && a.vel) {
                         time_store<M>(m0, a.vel + moff, a.nt, a.vec, x.s);
                     }
                 }
@@ -566,8 +580,8 @@ __device__ __forceinline__ void update_body(const FftArgs &a, int bid_in) {
     if constexpr (KEEP) slots_to_spec<M>(a, x, xo[0], xo[1]);
 }
 
-template <int M, bool KEEP, bool EXT>
-__global__ void __launch_bounds__(Team<M>::THREADS, Team<M>::MINB) k_update(FftArgs a) {
+template <int M, bool KEEP, int EXT>
+__global__ void __launch_bounds__(Team<M>::THREADS, update_minb<M, EXT>()) k_update(FftArgs a) {
     update_body<M, KEEP, EXT>(a, blockIdx.x);
 }
 
@@ -604,7 +618,7 @@ __global__ void __launch_bounds__(Team<M>::THREADS, Team<M>::MINB) k_update_q(Wo
     while (queue_next(q, m, tile) >= 0) {
         queue_args(args + m, sa);
         __syncthreads();
-        update_body<M, true, false>(sa, tile);
+        update_body<M, true, 0>(sa, tile);
     }
 }
 
@@ -637,8 +651,9 @@ struct FftLaunch {
 template <int M>
 cudaError_t FftLaunch<M>::prepare() {
     const void *kernels[] = {(const void *)k_rfft<M>, (const void *)k_irfft_out<M>, (const void *)k_residual<M>,
-                             (const void *)k_update<M, false, false>, (const void *)k_update<M, true, false>,
-                             (const void *)k_update<M, false, true>, (const void *)k_update<M, true, true>,
+                             (const void *)k_update<M, false, 0>, (const void *)k_update<M, true, 0>,
+                             (const void *)k_update<M, false, 1>, (const void *)k_update<M, true, 1>,
+                             (const void *)k_update<M, false, 2>, (const void *)k_update<M, true, 2>,
                              (const void *)k_rfft_q<M>, (const void *)k_residual_q<M>, (const void *)k_update_q<M>};
     for (const void *k : kernels) {
         const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Team<M>::SMEM);
@@ -675,12 +690,12 @@ cudaError_t FftLaunch<M>::residual(const FftArgs &a, int nblocks_expected, cudaS
 
 template <int M>
 cudaError_t FftLaunch<M>::update(bool keep, const FftArgs &a, cudaStream_t st) {
-    const bool ext = a.vel || a.mute || a.adam_m;
     const int nb = blocks_for<M>(a.g);
     if (nb < 0) return cudaErrorInvalidValue;
     if (nb == 0) return cudaSuccess;
-    auto kern = ext ? (keep ? k_update<M, true, true> : k_update<M, false, true>)
-                    : (keep ? k_update<M, true, false> : k_update<M, false, false>);
+    auto kern = (a.vel || a.adam_m) ? (keep ? k_update<M, true, 2> : k_update<M, false, 2>)
+                : a.mute            ? (keep ? k_update<M, true, 1> : k_update<M, false, 1>)
+                                    : (keep ? k_update<M, true, 0> : k_update<M, false, 0>);
     FftArgs b = a;
     b.ahead = prefetches<M>() ? 152 * Team<M>::MINB : 0;   // the CTAs resident at a time
     kern<<<nb, Team<M>::THREADS, Team<M>::SMEM, st>>>(b);
