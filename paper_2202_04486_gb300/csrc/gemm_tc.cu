@@ -1434,28 +1434,47 @@ cudaError_t launch_tc_adj_queue(bool recip, const WorkQueue &q, cudaStream_t st)
     return cudaGetLastError();
 }
 
+// Which products the persistent adjoint takes (K products a tile and its mirror: the batch, twice with reciprocity):
+//  * enough tiles for its roles to overlap from tile to tile: two a CTA; sixteen with reciprocity, where the diagonal tiles
+//    take a launch of their own (persistent / tile kernel, us, batch 16: 23.6 / 22.0 at nf 257, 128 x 128; symmetric
+//    83.6 / 78.5 at nf 257, 300 x 300, 148.9 / 143.1 at nf 513, 300 x 300, 205 / 210 at nf 513, 400 x 400);
+//  * and work that hides the writes: two jobs a tile (K > 32: 505 / 650 at nf 1025, 300 x 600, batch 64), or operand images
+//    that stay in seven eighths of the L2 (117 / 126 at nf 257, 300 x 600, batch 32; 135 MB of them at nf 513: 254 / 221,
+//    batch 16), or output tiles with half as much padding again as
+//    outputs, which the tile kernel computes and the persistent one skips (265 / 284 at nf 1025, 301 x 301, batch 32).
+//    Otherwise the output bounds both, and the tile kernel's CTAs, which start in the order of the bins, keep the four
+//    64-byte pieces of a 256-byte line closer together in time than CTAs that walk lists of tiles (541 / 421 at nf 1025,
+//    300 x 600, 764 / 691 at 600 x 600, batch 8; four or two bins of a line on one CTA in turn: 459 and 455, 730 and 721).
+static bool adj_persistent(const GemmArgs &a, bool recip, int tiles, int nf, int sms, int l2) {
+    if ((long long)tiles * nf < (recip ? 16LL : 2LL) * sms) return false;
+    const double images = (double)nf * a.img_nkc * (a.tiles_v + a.tiles_r) * TC_ADJ_IMG;
+    const double padded = 128.0 * 128.0 * a.tiles_v * a.tiles_r;
+    return a.nb * (recip ? 2 : 1) > TcAdj::KC || images <= 0.875 * l2 || padded >= 1.5 * a.nv * a.nr;
+}
+
 cudaError_t launch_tc_adj(const GemmArgs &a0, bool recip, int nf, cudaStream_t st, const TcMaps *maps) {
     const void *map = maps ? maps->adj : nullptr;
     GemmArgs a = a0;
     a.tiles_v = (a.nv + 127) / 128;
     a.tiles_r = (a.nr + 127) / 128;
     const bool img = a.img != nullptr;
-    // (a symmetric model of two tile rows has one off-diagonal tile a bin: not worth a launch of its own, 105 against 97 us
-    // at nf 513, 201 x 201)
-    if (img && maps && (!recip || (a.no_mirror && a.tiles_v > 2))) {
-        int dev = 0, sms = 0;
+    const int tiles = recip ? a.tiles_v * (a.tiles_v - 1) / 2 : a.tiles_v * a.tiles_r;   // of the persistent kernel
+    int dev = 0, sms = 0, l2 = 0;
+    if (img && maps && (!recip || a.no_mirror)) {
         cudaError_t e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev);
         if (e != cudaSuccess) return e;
+    }
+    if (sms > 0 && adj_persistent(a, recip, tiles, nf, sms, l2)) {
         CUtensorMap m32;
         memcpy(&m32, maps->adj32, sizeof(m32));
         const int nf_act = (a.nf_active > 0 && a.nf_active < nf) ? a.nf_active : nf;
-        const int tiles = recip ? a.tiles_v * (a.tiles_v - 1) / 2 : a.tiles_v * a.tiles_r;
-        const int grid = std::max(1, std::min(nf * tiles, sms));
+        const int grid = std::min(nf * tiles, sms);
         if (!recip) {
             k_tc_adj_p<false><<<grid, TAP_THREADS, TAP_SMEM, st>>>(a, m32, tiles, nf, nf_act);
         } else {
-            if (tiles > 0) k_tc_adj_p<true><<<grid, TAP_THREADS, TAP_SMEM, st>>>(a, m32, tiles, nf, nf_act);
+            k_tc_adj_p<true><<<grid, TAP_THREADS, TAP_SMEM, st>>>(a, m32, tiles, nf, nf_act);
             a.diag_only = 1;
             CUtensorMap tmap;
             memcpy(&tmap, map, sizeof(tmap));
