@@ -986,9 +986,10 @@ int mdc_plan_autotune(mdc_plan_t p, int nb, int flags, int reps, mdc_config *bes
     }
     if (rc == MDC_OK) {
         double tbest = 1e300;
-        // (MDC_GEMM_SIMT: for few rows its rule takes tiles that neither of the named ones is)
         const int cand[5] = {MDC_GEMM_SIMT, MDC_GEMM_SIMT32, MDC_GEMM_SIMT64, MDC_GEMM_TC, MDC_GEMM_GEMV};
         for (int c : cand) {
+            // (MDC_GEMM_SIMT only where its rule takes tiles that neither of the named ones is)
+            if (c == MDC_GEMM_SIMT && !cgemm_adj_few_rows(p->nv, p->nr, recip)) continue;
             if (c == MDC_GEMM_TC && p->prec != MDC_PREC_BF16X3) continue;
             if (c == MDC_GEMM_GEMV && (!gemv_supported(p->nv) || recip)) continue;
             p->gemm_adj = c;

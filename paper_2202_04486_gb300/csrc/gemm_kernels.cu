@@ -1074,6 +1074,8 @@ cudaError_t launch_cgemm_fwd(const GemmArgs &a, int nf, cudaStream_t st) {
 //  * else the packed 64-wide ones (scalar 32 / packed 64: 1320 / 974 at nf 1025, 301 x 301, batch 64; 145 / 98 at nf 513,
 //    256 x 256, batch 16; 275 / 240 at nf 1025, 237 x 133, batch 27).
 // 32 or 64: the scalar 32-wide or the packed 64-wide tiles
+bool cgemm_adj_few_rows(int nv, int nr, bool recip) { return !recip && nv <= 16 && nr > 64; }
+
 cudaError_t launch_cgemm_adj(const GemmArgs &a0, bool recip, int nf, cudaStream_t st, int tile) {
     GemmArgs a = a0;
     auto tiles = [](int n, int t) { return (n + t - 1) / t; };
@@ -1082,7 +1084,7 @@ cudaError_t launch_cgemm_adj(const GemmArgs &a0, bool recip, int nf, cudaStream_
         a.tiles_r = tiles(a.nr, tr);
         return dim3(recip ? a.tiles_v * (a.tiles_v + 1) / 2 : a.tiles_v * a.tiles_r, nf);
     };
-    if (tile == 0 && !recip && a.nv <= 16 && a.nr > 64) {
+    if (tile == 0 && cgemm_adj_few_rows(a.nv, a.nr, recip)) {
         using F = AdjS<16, 64, false>;
         const dim3 g = grid(16, 64);
         k_cgemm_adj_small<16, 64, false><<<g, F::THREADS, F::SMEM, st>>>(a);

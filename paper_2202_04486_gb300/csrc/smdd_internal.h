@@ -163,6 +163,7 @@ cudaError_t launch_queue_update(int M, const WorkQueue &q, cudaStream_t st);
 
 cudaError_t launch_cgemm_fwd(const GemmArgs &a, int nf, cudaStream_t st);
 cudaError_t launch_cgemm_adj(const GemmArgs &a, bool recip, int nf, cudaStream_t st, int tile = 0);
+bool cgemm_adj_few_rows(int nv, int nr, bool recip);   // launch_cgemm_adj with tile 0 takes tiles of its own
 cudaError_t gemm_prepare();
 // few virtual sources (nv <= 8): matrix-vector kernels; no band limit, no reciprocity (adjoint)
 bool gemv_supported(int nv);
