@@ -246,8 +246,9 @@ int mdc_forward_static(int nt, int nr, int nv, int ns, float scale, const float 
                                 MDC_GEMM_SIMT instead. */
 #define MDC_GEMM_TC_STREAM 5 /* forward only: the split-BF16 tcgen05 product as the persistent kernel (one
                                 CTA per SM) fed by tiled copies of the tensor memory accelerator, which
-                                MDC_GEMM_TC runs too where it can (MDC_PREC_BF16X3 plans only;
-                                MDC_ERR_UNSUPPORTED where the driver gives no tensor-map encoder) */
+                                MDC_GEMM_TC runs too unless the product is so small that its tiles
+                                all run at once in one step (MDC_PREC_BF16X3 plans only; MDC_ERR_UNSUPPORTED
+                                where the driver gives no tensor-map encoder) */
 
 typedef struct {
     int fft_variant;   /* 0, 1 or 2: accepted and read back (1 as 0 for the lengths 128, 1024 and 8192, 2 as 0

@@ -252,7 +252,8 @@ int gemm_forward(mdc_plan_s *p, const int32_t *idx, int nb, cudaStream_t st) {
     if (p->gemm_fwd == MDC_GEMM_TC_STREAM) g.wait_probe = 0;   // (the failure-path check is MDC_GEMM_TC's)
     if (p->gemm_fwd == MDC_GEMM_TC || p->gemm_fwd == MDC_GEMM_TC_STREAM)
         return launch_stage(p, ST_GEMM_FWD, st, [&] {
-            return p->xh_map_ok ? launch_tc_fwd_p(g, p->maps, p->nf, st) : launch_tc_fwd(g, p->nf, st);
+            return p->xh_map_ok ? launch_tc_fwd_p(g, p->maps, p->nf, p->gemm_fwd == MDC_GEMM_TC_STREAM, st)
+                                : launch_tc_fwd(g, p->nf, st);
         });
     if (p->gemm_fwd == MDC_GEMM_GEMV && gemv_supported(p->nv) && p->nf_active == 0)
         return launch_stage(p, ST_GEMM_FWD, st, [&] { return launch_gemv_fwd(g, p->nf, st); });

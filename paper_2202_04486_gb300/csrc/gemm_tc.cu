@@ -1398,11 +1398,16 @@ static cudaError_t launch_fwd_p(const GemmArgs &a, const TcMaps &maps, int nf, i
     return cudaGetLastError();
 }
 
-cudaError_t launch_tc_fwd_p(const GemmArgs &a, const TcMaps &maps, int nf, cudaStream_t st) {
+// Tiles of one K chunk that all run at once, one CTA each, take the tile kernel: one bin a CTA, where the persistent
+// kernel's units are two bins with nothing after them to overlap with (us, tile / persistent, nf 129: 9.7 / 10.8 at 64 x 64,
+// batch 16, 12.1 / 14.1, batch 64; with two chunks, 100 x 100, batch 4, 14.3 / 13.5; at 257 bins, where some SMs get
+// two tiles, the persistent kernel is level or ahead).  The results are the same bits.
+cudaError_t launch_tc_fwd_p(const GemmArgs &a, const TcMaps &maps, int nf, bool always, cudaStream_t st) {
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
+    if (!always && a.nr <= 64 && tc_fwd_tiles(a, nf) <= sms) return launch_tc_fwd(a, nf, st);
     return a.nb <= 16 ? launch_fwd_p<16>(a, maps, nf, sms, st) : a.nb <= 32 ? launch_fwd_p<32>(a, maps, nf, sms, st) : launch_fwd_p<64>(a, maps, nf, sms, st);
 }
 

@@ -179,8 +179,9 @@ struct TcMaps {
     alignas(64) unsigned char fwd[128], fwd_t[128], adj[128], adj32[128];
 };
 cudaError_t tc_encode_maps(TcMaps *m, const float2 *Xh, int nr, int nv, int ldr, int nf);
-// persistent forward product fed by the tensor memory accelerator
-cudaError_t launch_tc_fwd_p(const GemmArgs &a, const TcMaps &maps, int nf, cudaStream_t st);
+// persistent forward product fed by the tensor memory accelerator; the tile kernel where its tiles all run at once (unless
+// `always`)
+cudaError_t launch_tc_fwd_p(const GemmArgs &a, const TcMaps &maps, int nf, bool always, cudaStream_t st);
 // maps (or null): tiles written once are then stored by the tensor memory accelerator, and computed by the persistent
 // kernel where the operand images are given
 cudaError_t launch_tc_adj(const GemmArgs &a, bool recip, int nf, cudaStream_t st, const TcMaps *maps = nullptr);
