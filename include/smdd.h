@@ -271,7 +271,8 @@ int mdc_plan_get_config(mdc_plan_t plan, mdc_config *cfg);
 int mdc_plan_set_config(mdc_plan_t plan, const mdc_config *cfg);
 /* Autotune: time every candidate of each choice on this plan's sizes, with batch size nb and the
  * step flags (SMDD_RECIPROCITY changes the adjoint), reps timed launches each after one warm-up, and
- * keep the fastest.  best (host, may be NULL) receives the chosen configuration.
+ * keep the fastest (MDC_GEMM_TC_STREAM is no candidate: MDC_GEMM_TC runs the same kernel where it is
+ * the faster one).  best (host, may be NULL) receives the chosen configuration.
  * Uses temporary device memory (cudaMalloc), overwrites the plan's spectral workspaces, synchronises
  * the stream, and must not be called during a stream capture. */
 int mdc_plan_autotune(mdc_plan_t plan, int nb, int flags, int reps, mdc_config *best, void *stream);

@@ -974,10 +974,11 @@ int mdc_plan_autotune(mdc_plan_t p, int nb, int flags, int reps, mdc_config *bes
     int best_f = old_f, best_a = old_a;
     if (rc == MDC_OK) {
         double tbest = 1e300;
-        const int cand[4] = {MDC_GEMM_SIMT, MDC_GEMM_TC, MDC_GEMM_TC_STREAM, MDC_GEMM_GEMV};
+        // (not MDC_GEMM_TC_STREAM: MDC_GEMM_TC runs the same kernel wherever it is the faster one, and only MDC_GEMM_TC
+        // honours the failure-path check)
+        const int cand[3] = {MDC_GEMM_SIMT, MDC_GEMM_TC, MDC_GEMM_GEMV};
         for (int c : cand) {
-            if ((c == MDC_GEMM_TC || c == MDC_GEMM_TC_STREAM) && p->prec != MDC_PREC_BF16X3) continue;
-            if (c == MDC_GEMM_TC_STREAM && !p->xh_map_ok) continue;
+            if (c == MDC_GEMM_TC && p->prec != MDC_PREC_BF16X3) continue;
             if (c == MDC_GEMM_GEMV && !gemv_supported(p->nv)) continue;
             p->gemm_fwd = c;
             const double t = time_it([&] { return gemm_forward(p, didx, nb, st); });
