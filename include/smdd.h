@@ -76,7 +76,9 @@ typedef enum { MDC_PREC_FP32 = 0, MDC_PREC_BF16X3 = 1 } mdc_precision;
  *   D       : device pointer, [ns][nr][nt] float32, read during this call only.
  *   precision : MDC_PREC_FP32 or MDC_PREC_BF16X3 (see mdc_precision).
  *   stream  : stream for the precompute; the call returns after it has been enqueued.
- * Allocates about 8*nf*(ns+nv)*nr + 8*nf*nv*nb_max bytes of device memory (nf = nfft/2+1). */
+ * Allocates about 8*nf*(ns*nr + nv*nr8 + nv*nb8) bytes of device memory (nf = nfft/2+1; nr8, nb8: nr and nb_max
+ * rounded up to multiples of 8, in rows of the model and of the batch spectra), and for MDC_PREC_BF16X3 with
+ * nb_max <= 64 another 32768*nf*ceil(nb_max/32)*(ceil(nv/128)+ceil(nr/128)) where they can be had. */
 int mdc_plan_create(mdc_plan_t *out, int nt, int nr, int nv, int ns, int nb_max, int nfft,
                     float scale, const float *D, int precision, void *stream);
 
@@ -324,7 +326,7 @@ int mdc_batch_create(mdc_batch_t *out, const smdd_member *members, int n, int n_
  *                        holding step w of every member that has one (members have ceil(ns/nb) steps);
  *                        each stage of a wave -- the model transform (wave 0), the forward product, the
  *                        residual step, the adjoint product, the update -- is one launch per kernel family
- *                        (FFT length and variant; product kernel) of CTAs resident on every SM, which take
+ *                        (FFT length; product kernel) of CTAs resident on every SM, which take
  *                        (problem, tile) items from a queue in device memory by atomic counter until it is
  *                        empty.  The same steps and arithmetic as the branch layout (results equal bit for
  *                        bit).  n_branches is ignored.  Every member's plan must be MDC_PREC_BF16X3 with

@@ -77,7 +77,7 @@ struct FftArgs {
 
 struct GemmArgs {
     const float2 *A;         // forward: model spectra Xh; adjoint: residual spectra Rh
-    const float2 *Dh;        // kernel spectra [nf][ns][ldr]
+    const float2 *Dh;        // kernel spectra [nf][ns][ldd]
     const int32_t *idx;
     float2 *C;               // forward: Uh; adjoint: Gh
     int nv, nr, ns, nb;
