@@ -91,6 +91,7 @@ struct mdc_plan_s {
     // kernel configuration (see mdc_config)
     int fft_variant = 0;         // accepted and reported; the trace kernels are the same for every value
     int fft_prefetch = 0;        // likewise
+    int upd_ahead = 0;           // FftArgs::ahead of the update
     int gemm_fwd = MDC_GEMM_SIMT;
     int gemm_adj = MDC_GEMM_SIMT;
     int nf_active = 0;           // band limit of the products (0: every bin)
@@ -457,6 +458,7 @@ int mdc_plan_create(mdc_plan_t *out, int nt, int nr, int nv, int ns, int nb_max,
     if (cudaMemsetAsync(p->Xh, 0, szX, st) != cudaSuccess) rc = MDC_ERR_CUDA;
     if (cudaMemsetAsync(p->Uh, 0, szU, st) != cudaSuccess) rc = MDC_ERR_CUDA;
     if (rc == MDC_OK && (fft_prepare(M) != cudaSuccess || gemm_prepare() != cudaSuccess)) rc = MDC_ERR_CUDA;
+    p->upd_ahead = fft_update_ahead(M);
     if (rc == MDC_OK && precision == MDC_PREC_BF16X3 && tc_prepare() != cudaSuccess) rc = MDC_ERR_CUDA;
     if (rc == MDC_OK && precision == MDC_PREC_BF16X3)   // without a map, MDC_GEMM_TC_STREAM is unsupported
         p->xh_map_ok = tc_encode_maps(&p->maps, p->Xh, nr, nv, p->ldr, p->nf) == cudaSuccess;
@@ -675,6 +677,7 @@ int step_impl(mdc_plan_t p, float *X, const float *U_obs, const int32_t *idx, in
         FftArgs a = base_fft(p);
         a.g = mg;
         if (sym) a.g.sym = 1;
+        a.ahead = p->upd_ahead;
         a.tout = X;
         a.vec = time_vec(p->nt, X);
         for (const float *q : {vel, adam.m, adam.v})

@@ -66,6 +66,8 @@ cudaError_t launch_update(int M, bool keep, const FftArgs &a, cudaStream_t st) {
     SMDD_SWITCH_M(M, cudaErrorInvalidValue, FftLaunch<MM>::update(keep, a, st))
 }
 
+int fft_update_ahead(int M) { SMDD_SWITCH_M(M, 0, FftLaunch<MM>::update_ahead()) }
+
 cudaError_t launch_queue_rfft(int M, const WorkQueue &q, cudaStream_t st) {
     SMDD_SWITCH_M(M, cudaErrorInvalidValue, FftLaunch<MM>::queue_rfft(q, st))
 }

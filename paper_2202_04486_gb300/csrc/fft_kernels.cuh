@@ -160,9 +160,9 @@ __device__ __forceinline__ void bulk_prefetch_l2(const void *p, unsigned bytes) 
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(p), "r"(bytes) : "memory");
 }
 
-// The spectra of tile bid + `ahead` (about the CTAs resident on the GPU, so the tile that starts when this one ends)
+// The spectra of tile bid + `ahead` (the CTAs resident on the GPU, so about the tile that starts when this one ends)
 // into L2, 256 contiguous bytes of four bins at a time, while this tile is transformed.  Only for 256 <= M <= 512 and whole tiles of
-// 8 columns: update 432 -> 409 us at nt 512, 400 x 400, 478 -> 454 us at nt 256, 600 x 600; at M = 1024 and 1536, whose tiles
+// 8 columns: update 432 -> 409 us at nt 512, 400 x 400, 478 -> 462 us at nt 256, 600 x 600; at M = 1024 and 1536, whose tiles
 // take longer, 1 % slower to 5 % faster by shape, at M = 128 no change.
 template <int M>
 constexpr bool prefetches() { return M >= 256 && M <= 512; }
@@ -642,6 +642,7 @@ struct FftLaunch {
     static cudaError_t irfft_out(const FftArgs &a, cudaStream_t st);
     static cudaError_t residual(const FftArgs &a, int nblocks_expected, cudaStream_t st);
     static cudaError_t update(bool keep, const FftArgs &a, cudaStream_t st);
+    static int update_ahead();
     static cudaError_t queue_rfft(const WorkQueue &q, cudaStream_t st);
     static cudaError_t queue_residual(const WorkQueue &q, cudaStream_t st);
     static cudaError_t queue_update(const WorkQueue &q, cudaStream_t st);
@@ -696,10 +697,18 @@ cudaError_t FftLaunch<M>::update(bool keep, const FftArgs &a, cudaStream_t st) {
     auto kern = (a.vel || a.adam_m) ? (keep ? k_update<M, true, 2> : k_update<M, false, 2>)
                 : a.mute            ? (keep ? k_update<M, true, 1> : k_update<M, false, 1>)
                                     : (keep ? k_update<M, true, 0> : k_update<M, false, 0>);
-    FftArgs b = a;
-    b.ahead = prefetches<M>() ? 152 * Team<M>::MINB : 0;   // the CTAs resident at a time
-    kern<<<nb, Team<M>::THREADS, Team<M>::SMEM, st>>>(b);
+    kern<<<nb, Team<M>::THREADS, Team<M>::SMEM, st>>>(a);
     return cudaGetLastError();
+}
+
+template <int M>
+int FftLaunch<M>::update_ahead() {
+    int dev = 0, sms = 0, ctas = 0;
+    if (!prefetches<M>() || cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, k_update<M, true, 0>, Team<M>::THREADS, Team<M>::SMEM) != cudaSuccess)
+        return 0;
+    return sms * ctas;
 }
 
 // work-queue launches: resident CTAs on every SM take (problem, tile) items until the queue is empty

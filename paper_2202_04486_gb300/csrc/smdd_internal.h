@@ -146,6 +146,7 @@ cudaError_t launch_update(int M, bool keep_xhat, const FftArgs &a, cudaStream_t 
 int fft_blocks(int M, const TraceGrid &g);
 int fft_traces_per_cta(int M);
 cudaError_t fft_prepare(int M);                                // opt-in to the dynamic shared memory of size M
+int fft_update_ahead(int M);                                   // FftArgs::ahead for the current device (after fft_prepare)
 int fft_tw_size(int M);                                        // entries of the twiddle tables
 void fft_tw_fill(int M, std::vector<float2> &tw);              // host: the tables, rounded once from double
 // alignment class of time traces (FftArgs::vec): every trace starts on a 16-byte (2) or 8-byte (1) boundary
