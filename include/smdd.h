@@ -222,8 +222,8 @@ int smdd_lsqr(mdc_plan_t plan, float *X, const float *U_obs, int n_iter, int fla
  *               has passed the call.
  *   stream: as elsewhere.
  * Returns MDC_ERR_UNSUPPORTED, launching nothing, when the intermediates of the problem need more than
- * the 64 MiB: 8 * (nfft/2+1) * (ns*ldr + nv*ldr + nv*ldb) bytes plus the twiddle tables, with ldr and ldb
- * nr and nb rounded up to even.  Shapes are not checked here (there is no plan): the caller must pass
+ * the 64 MiB: 8 * (nfft/2+1) * (ns*ldr + nv*ldr + nv*ldb) bytes plus a reserve for the twiddle tables (1 to 106 KiB
+ * by nfft), with ldr and ldb nr and nb rounded up to even.  Shapes are not checked here (there is no plan): the caller must pass
  * arrays of exactly the sizes above.
  * The first call on a device looks up the array's device address (once per device) and must therefore
  * not be the first call made during a stream capture.  All calls share the array: two calls that can

@@ -26,30 +26,25 @@ namespace {
 
 constexpr size_t kScratchBytes = size_t(64) << 20;   // 64 MiB
 constexpr int kMaxDevices = 64;
-constexpr int kMaxTable = smdd::tw_size(4096);       // twiddle tables of the longest transform
 
 static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
-static __device__ __align__(256) float2 g_tables[kMaxTable];
 
 std::mutex g_mu;
-void *g_scratch_ptr[kMaxDevices] = {nullptr}, *g_tables_ptr[kMaxDevices] = {nullptr};
+void *g_scratch_ptr[kMaxDevices] = {nullptr};
 
-// Device addresses of g_scratch and g_tables on the current device (looked up once per device); false on failure.
-bool scratch_addresses(int dev, unsigned char *&scratch, float2 *&tables) {
+// Device address of g_scratch on the current device (looked up once per device), or nullptr.
+void *scratch_address(int dev) {
     std::lock_guard<std::mutex> lock(g_mu);
-    if (dev < 0 || dev >= kMaxDevices) return false;
+    if (dev < 0 || dev >= kMaxDevices) return nullptr;
     if (!g_scratch_ptr[dev]) {
-        void *p = nullptr, *t = nullptr;
-        if (cudaGetSymbolAddress(&p, g_scratch) != cudaSuccess || cudaGetSymbolAddress(&t, g_tables) != cudaSuccess) {
+        void *p = nullptr;
+        if (cudaGetSymbolAddress(&p, g_scratch) != cudaSuccess) {
             cudaGetLastError();
-            return false;
+            return nullptr;
         }
         g_scratch_ptr[dev] = p;
-        g_tables_ptr[dev] = t;
     }
-    scratch = static_cast<unsigned char *>(g_scratch_ptr[dev]);
-    tables = static_cast<float2 *>(g_tables_ptr[dev]);
-    return true;
+    return g_scratch_ptr[dev];
 }
 
 // twiddle tables of the trace kernels, computed on the device in double precision
@@ -63,28 +58,27 @@ __global__ void k_fill_twiddles(float2 *tw, int ntw, int M) {
     }
 }
 
-// Bytes that a problem's need is charged for its tables: 8 bytes for each entry of the tables of both directions
-// of a radix-8/4/3 plan of length M.  (Callers rely on which problems fit; the tables themselves lie beside the
-// scratch, in g_tables.)
-void table_charge(int M, size_t &passes, size_t &roots) {
-    const int rad[9][5] = {{32, 8, 4, 1, 1}, {64, 8, 8, 1, 1}, {128, 8, 4, 4, 1}, {256, 8, 8, 4, 1}, {512, 8, 8, 8, 1},
-                           {1024, 8, 8, 4, 4}, {1536, 8, 8, 3, 8}, {2048, 8, 8, 8, 4}, {4096, 8, 8, 8, 8}};
-    passes = 0;
-    roots = (size_t)(M + 1) * 8;
-    for (const auto &r : rad) {
-        if (r[0] != M) continue;
-        for (int p = 2, f = r[1]; p <= 4; ++p) {   // spans of the forward passes after the first
-            if (r[p] > 1) passes += (size_t)f * r[p] * 8;
-            f *= r[p];
-        }
-        int n = 4;
-        while (r[n] == 1) --n;
-        for (int p = n - 1, f = r[n]; p >= 1; --p) {   // and of the inverse, whose radices are reversed
-            passes += (size_t)f * r[p] * 8;
-            f *= r[p];
-        }
+// Bytes at the start of the scratch reserved for the twiddle tables of complex length M, in which they lie.  (More than the
+// tables take: which problems fit is part of what callers rely on, and these sizes decide it.)
+constexpr size_t table_reserve(int M) {
+    switch (M) {
+        case 32: return 1024;
+        case 64: return 1792;
+        case 128: return 3840;
+        case 256: return 7168;
+        case 512: return 13568;
+        case 1024: return 28672;
+        case 1536: return 40960;
+        case 2048: return 56320;
+        default: return 107776;   // 4096
     }
 }
+constexpr bool tables_fit() {
+    for (int M : {32, 64, 128, 256, 512, 1024, 1536, 2048, 4096})
+        if (smdd::tw_size(M) * sizeof(float2) > table_reserve(M) || table_reserve(M) % 256 != 0) return false;
+    return true;
+}
+static_assert(tables_fit(), "the tables fit their reserve, whose size keeps the spectra aligned");
 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
@@ -100,10 +94,8 @@ extern "C" int mdc_forward_static(int nt, int nr, int nv, int ns, float scale, c
     const int M = nfft / 2, nf = M + 1;
     const int ldr = (nr + 1) & ~1, ldb = (nb + 1) & ~1;
 
-    // scratch layout: charge of the tables | kernel spectra | model spectra | batch spectra
-    size_t t_pass, t_roots;
-    table_charge(M, t_pass, t_roots);
-    const size_t o_dh = align256(align256(t_pass) + t_roots);
+    // scratch layout: tables | kernel spectra | model spectra | batch spectra
+    const size_t o_dh = table_reserve(M);
     const size_t o_xh = align256(o_dh + (size_t)nf * ns * ldr * sizeof(float2));
     const size_t o_uh = align256(o_xh + (size_t)nf * nv * ldr * sizeof(float2));
     const size_t need = align256(o_uh + (size_t)nf * nv * ldb * sizeof(float2));
@@ -115,12 +107,12 @@ extern "C" int mdc_forward_static(int nt, int nr, int nv, int ns, float scale, c
 
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return MDC_ERR_CUDA;
-    unsigned char *base = nullptr;
-    float2 *tw = nullptr;
-    if (!scratch_addresses(dev, base, tw)) return MDC_ERR_CUDA;
+    unsigned char *base = static_cast<unsigned char *>(scratch_address(dev));
+    if (!base) return MDC_ERR_CUDA;
     if (fft_prepare(M) != cudaSuccess || gemm_prepare() != cudaSuccess) return MDC_ERR_CUDA;
     cudaStream_t st = (cudaStream_t)stream;
 
+    float2 *tw = reinterpret_cast<float2 *>(base);
     float2 *Dh = reinterpret_cast<float2 *>(base + o_dh);
     float2 *Xh = reinterpret_cast<float2 *>(base + o_xh);
     float2 *Uh = reinterpret_cast<float2 *>(base + o_uh);
