@@ -706,10 +706,10 @@ __global__ void __launch_bounds__(G::THREADS, 512 / G::THREADS) k_cgemm_adj(Gemm
 // Few virtual sources (nv <= 8, the matrix-vector regime of a single-virtual-source inversion): the
 // products are bound by reading the batch rows of Dh once, so a warp streams one kernel row against
 // the nv model rows (forward) or a thread owns one receiver and walks the batch (adjoint).  The operand that every
-// kernel row meets again -- the model rows, or the residuals' coefficients -- is staged in shared memory by the CTA, and
-// eight loads of kernel rows are on their way at a time.  (Read from the SPEC_F layout for every kernel row, a warp's
-// access touches four half lines: 231 and 222 us at nf 513, 600 x 8, batch 100,
-// against 136 and 84.)
+// kernel row meets again -- the model rows, or the residuals' coefficients -- is staged in shared memory by the CTA or shared
+// by two kernel rows of a warp, and several loads of kernel rows are on their way at a time.  (Read from the SPEC_F
+// layout for every kernel row, a warp's access touches four half lines: 231 and 222 us at nf 513, 600 x 8, batch 100,
+// against 136 and 84 staged.)
 // ------------------------------------------------------------------------------------------------
 constexpr int GV_THREADS = 256, GV_MAXV = 8;
 constexpr int GV_KC = 256;   // columns of a chunk of the model rows (forward)
@@ -733,46 +733,67 @@ __device__ __forceinline__ void gemv_put(const GemmArgs &a, int f, int b, const 
         if (v < a.nv) Cf[(long long)v * a.ldb * SPEC_F + spec_col(b)] = make_float2(acc[v].x * a.outscale, acc[v].y * a.outscale);
 }
 
-// forward: C[f][v][b] = sum_r A[f][v][r] Dh[f][idx_b][r]; one warp per batch entry b.  Short rows (up to GV_SHORT columns, four
-// accesses a lane and row): both operands from global memory, no barrier
-constexpr int GV_SHORT = 128;
-
-template <int NV>
-__global__ void __launch_bounds__(GV_THREADS) k_gemv_fwd_short(GemmArgs a) {
+// forward: C[f][v][b] = sum_r A[f][v][r] Dh[f][idx_b][r].  Both operands from global memory, no barrier; a warp takes BW
+// neighbouring batch entries at once, which share its loads of the model rows
+template <int NV, int BW>
+__global__ void __launch_bounds__(GV_THREADS) k_gemv_fwd_direct(GemmArgs a) {
+    constexpr int UNROLL = NV == 2 ? 1 : 2;   // (two rows: 9.8 us unrolled against 8.3 at nf 257, 60 columns, batch 64)
     const int f = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int b = blockIdx.y * (GV_THREADS / 32) + warp;
+    const int b = (blockIdx.y * (GV_THREADS / 32) + warp) * BW;
     if (b >= a.nb) return;   // warp-uniform; no barrier in this kernel
-    int s = a.idx[b];
-    if (s < 0 || s >= a.ns) {
-        if (lane == 0) atomicOr(a.status, 1);
-        s = -1;
+    const float2 *Af = a.A + spec_bin(f, a.sAf), *Df = a.Dh + (long long)f * a.sDf;
+    const float2 *d[BW];
+    bool have[BW];
+#pragma unroll
+    for (int j = 0; j < BW; ++j) {
+        int s = -1;
+        if (b + j < a.nb) {
+            s = a.idx[b + j];
+            if (s < 0 || s >= a.ns) {
+                if (lane == 0) atomicOr(a.status, 1);
+                s = -1;
+            }
+        }
+        have[j] = s >= 0;
+        d[j] = Df + (long long)(s < 0 ? 0 : s) * a.ldd;   // (row 0 for an entry without a source, whose sum is dropped)
     }
-    const float2 *Af = a.A + spec_bin(f, a.sAf);
-    float2 acc[NV];
+    float2 acc[BW][NV];
 #pragma unroll
-    for (int v = 0; v < NV; ++v) acc[v] = make_float2(0.f, 0.f);
-    if (s >= 0) {
-        const float2 *d = a.Dh + (long long)f * a.sDf + (long long)s * a.ldd;
-        for (int r = lane; r < a.nr; r += 32) {
-            const float2 dv = __ldg(d + r);
+    for (int j = 0; j < BW; ++j)
 #pragma unroll
-            for (int v = 0; v < NV; ++v) {
-                if (v < a.nv) {
-                    const float2 x = __ldg(Af + (long long)v * a.ldr * SPEC_F + spec_col(r));
-                    acc[v].x = fmaf(x.x, dv.x, fmaf(-x.y, dv.y, acc[v].x));
-                    acc[v].y = fmaf(x.x, dv.y, fmaf(x.y, dv.x, acc[v].y));
+        for (int v = 0; v < NV; ++v) acc[j][v] = make_float2(0.f, 0.f);
+#pragma unroll UNROLL
+    for (int r = lane; r < a.nr; r += 32) {
+        float2 dv[BW];
+#pragma unroll
+        for (int j = 0; j < BW; ++j) dv[j] = __ldg(d[j] + r);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            if (NV <= 2 || v < a.nv) {   // (one or two rows: exactly as many; the loads of a round are issued together)
+                const float2 x = __ldg(Af + (long long)v * a.ldr * SPEC_F + spec_col(r));
+#pragma unroll
+                for (int j = 0; j < BW; ++j) {
+                    acc[j][v].x = fmaf(x.x, dv[j].x, fmaf(-x.y, dv[j].y, acc[j][v].x));
+                    acc[j][v].y = fmaf(x.x, dv[j].y, fmaf(x.y, dv[j].x, acc[j][v].y));
                 }
             }
         }
     }
-    gemv_reduce<NV>(acc);
-    if (lane == 0) gemv_put<NV>(a, f, b, acc);
+#pragma unroll
+    for (int j = 0; j < BW; ++j) {
+        gemv_reduce<NV>(acc[j]);
+        if (!have[j]) {
+#pragma unroll
+            for (int v = 0; v < NV; ++v) acc[j][v] = make_float2(0.f, 0.f);
+        }
+        if (lane == 0 && b + j < a.nb) gemv_put<NV>(a, f, b + j, acc[j]);
+    }
 }
 
-// longer rows: the model rows staged; 2^split_log2 warps per batch entry, which take the groups of 32 columns in turn (one
+// The model rows staged; 2^split_log2 warps per batch entry, which take the groups of 32 columns in turn (one
 // warp in batches of 8 and more; in smaller ones the CTA's warps share the rows)
 template <int NV>
-__global__ void __launch_bounds__(GV_THREADS, NV <= 2 ? 6 : NV == 4 ? 5 : 4) k_gemv_fwd(GemmArgs a, int split_log2) {
+__global__ void __launch_bounds__(GV_THREADS, NV == 2 ? 6 : NV == 4 ? 5 : 4) k_gemv_fwd(GemmArgs a, int split_log2) {
     constexpr int WARPS = GV_THREADS / 32, G = GV_KC / 32, ROW = GV_KC / 2;
     constexpr int ST = (NV * ROW + GV_THREADS - 1) / GV_THREADS;   // staged units (two columns) of a thread
     __shared__ float4 rows[2][NV][ROW];
@@ -970,23 +991,34 @@ __global__ void __launch_bounds__(GV_THREADS) k_gemv_adj(GemmArgs a) {
 
 bool gemv_supported(int nv) { return nv >= 1 && nv <= GV_MAXV; }
 
+// Which forward kernel (us, direct with one entry a warp / with two / staged; batch 100 unless stated):
+//  * rows of at most 128 columns, and one row: direct (nf 257, 60 x 8: 22.3 / 25 / 25; nf 513, 600 x 1: 51 / 50 / 53; nf 1025,
+//    180 x 1: 41 / 37 / 42, batch 32: 14.2 / 12.3 / 16.2);
+//  * three or four rows, batches of 16 and more: direct, two entries (nf 513, 600 x 3: 107 / 70 / 79; nf 1025, 180 x 3: 84 / 60 / 63);
+//  * else staged (nf 1025, 180 x 2: 59 / 57 / 47; 180 x 8: 141 / 154 / 109; nf 513, 600 x 8, batch 1: 16 / 28 / 12).
 cudaError_t launch_gemv_fwd(const GemmArgs &a, int nf, cudaStream_t st) {
     if (!gemv_supported(a.nv) || nf < 1) return cudaErrorInvalidValue;
     if (a.nf_active > 0 && a.nf_active < nf) return cudaErrorInvalidValue;   // band limits use the tiled kernels
     constexpr int WARPS = GV_THREADS / 32;
+    const bool many = a.nb >= 16;
+    if (a.nr <= 128 || a.nv == 1 || (a.nv <= 4 && a.nv > 2 && many)) {
+        const int bw = many && ((a.nv == 1 && a.nr <= 256) || (a.nv > 2 && a.nv <= 4)) ? 2 : 1;
+        const dim3 grid(nf, (a.nb + WARPS * bw - 1) / (WARPS * bw));
+        if (a.nv == 1 && bw == 2) k_gemv_fwd_direct<1, 2><<<grid, GV_THREADS, 0, st>>>(a);
+        else if (a.nv == 1) k_gemv_fwd_direct<1, 1><<<grid, GV_THREADS, 0, st>>>(a);
+        else if (a.nv == 2) k_gemv_fwd_direct<2, 1><<<grid, GV_THREADS, 0, st>>>(a);
+        else if (a.nv <= 4 && bw == 2) k_gemv_fwd_direct<4, 2><<<grid, GV_THREADS, 0, st>>>(a);
+        else if (a.nv <= 4) k_gemv_fwd_direct<4, 1><<<grid, GV_THREADS, 0, st>>>(a);
+        else k_gemv_fwd_direct<8, 1><<<grid, GV_THREADS, 0, st>>>(a);
+        return cudaGetLastError();
+    }
     int split = 0;   // (log2)
-    if (a.nr > GV_SHORT)
-        while (WARPS >> split > 1 && (WARPS >> (split + 1)) >= a.nb) ++split;
+    while (WARPS >> split > 1 && (WARPS >> (split + 1)) >= a.nb) ++split;
     const int wb = WARPS >> split;
     const dim3 grid(nf, (a.nb + wb - 1) / wb);
-    auto go = [&](auto kern, auto shorter) {
-        if (a.nr > GV_SHORT) kern<<<grid, GV_THREADS, 0, st>>>(a, split);
-        else shorter<<<grid, GV_THREADS, 0, st>>>(a);
-    };
-    if (a.nv == 1) go(k_gemv_fwd<1>, k_gemv_fwd_short<1>);
-    else if (a.nv <= 2) go(k_gemv_fwd<2>, k_gemv_fwd_short<2>);
-    else if (a.nv <= 4) go(k_gemv_fwd<4>, k_gemv_fwd_short<4>);
-    else go(k_gemv_fwd<8>, k_gemv_fwd_short<8>);
+    if (a.nv == 2) k_gemv_fwd<2><<<grid, GV_THREADS, 0, st>>>(a, split);
+    else if (a.nv <= 4) k_gemv_fwd<4><<<grid, GV_THREADS, 0, st>>>(a, split);
+    else k_gemv_fwd<8><<<grid, GV_THREADS, 0, st>>>(a, split);
     return cudaGetLastError();
 }
 
