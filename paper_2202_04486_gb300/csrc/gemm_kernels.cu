@@ -35,9 +35,10 @@ __device__ __forceinline__ void cmac(float2 &acc, float2 a, float2 b) {
 }
 
 // ------------------------------------------------------------------------------------------------
-// forward, few rows (scalar products, 4 x 4 outputs per thread): C[f][v][b] = sum_r A[f][v][r] * Dh[f][idx_b][r]
-// With at most 64 rows a product is a chain of latencies; the longer chunk (16) through cp.async has fewer of them:
-// 8.4 us at nf 129, 32 x 32, batch 8, against 11 us for the packed tiles below.
+// forward, batches up to 16 and up to 128 rows (scalar products, 4 x 4 outputs per thread):
+//   C[f][v][b] = sum_r A[f][v][r] * Dh[f][idx_b][r]
+// Such a product is a chain of latencies; the longer chunk (16) through cp.async has fewer of them: 8.4 us at nf 129,
+// 32 x 32, batch 8, against 11 us for the packed tiles below.
 // CTA: 4 warps, 128 rows v x 16 batch columns, one frequency.  Lane (vg = lane & 7, bg = lane >> 3)
 // of warp w owns rows v0 + 32w + vg + 8i and columns b0 + bg + 4j (i, j < 4): a 4 x 4 complex register
 // tile.  K (= nr) streams in chunks of 16 through a two-stage cp.async pipeline; every operand load is

@@ -7,8 +7,8 @@
 // (re*re - im*im, re*im + im*re), the subtraction through the negate-B bit of the instruction
 // descriptor.  So each K-step of 16 issues 12 MMAs of M = 128 rows into two accumulators (re, im).
 //
-// Tile kernels (work-queue epochs, the mirrored tiles of reciprocity steps, and where no tensor maps are to be had): the
-// CUDA threads of a CTA load the FP32 complex spectra (coalesced rows), split them and store the
+// Tile kernels (work-queue epochs, the mirrored tiles of reciprocity steps, the products that launch_tc_fwd_p and
+// adj_persistent leave to them, and where no tensor maps are to be had): the CUDA threads of a CTA load the FP32 complex spectra (coalesced rows), split them and store the
 // four BF16 planes (re hi, re lo, im hi, im lo) in the 128-byte swizzled layouts of tc_common.cuh -- or,
 // for the adjoint of a plan that holds them, copy the planes from operand images split once per step
 // (k_tc_adj_images); thread 0 issues the MMAs and commits them to an mbarrier.  The persistent kernels k_tc_fwd_p and
@@ -1096,7 +1096,7 @@ __global__ void __launch_bounds__(TCP_THREADS, 1)
 
 // ------------------------------------------------------------------------------------------------
 // adjoint, persistent: the product of tc_adj_body from the operand images (same MMAs in the same order, bit-identical) for
-// tiles that are written once: every tile without reciprocity, the off-diagonal ones of a symmetric model (OFF; its
+// tiles that are written once, where it is the faster kernel (adj_persistent): every tile without reciprocity, the off-diagonal ones of a symmetric model (OFF; its
 // diagonal tiles, with their mirror, run on k_tc_adj_sym_tma).  One CTA per SM walks its tiles; its roles overlap from
 // tile to tile, where the tile kernel runs load, products and stores of a tile one after the other (15 000 cycles a tile
 // at two CTAs per SM for 3 700 cycles of output at the HBM rate, nt 1024, 301 x 301, batch 32):

@@ -1,10 +1,10 @@
 // Full-gradient MDD by LSQR (Paige & Saunders 1982), the baseline the paper compares stochastic MDD
 // against: every source at once, on the preconditioned operator A = P C (Eq. 3-4).
 //
-// The vectors are FP32 device arrays, every norm is reduced in FP64 with a fixed order (runs of a thread's
-// elements in FP32 words that are no less exact, SumSq; then threads, blocks and one block over them in FP64), and the scalar recurrence of the bidiagonalisation and of the plane
-// rotations runs on the device (one thread), so an iteration is a fixed sequence of launches with no
-// host round trip.  The operator's forward and adjoint are the plan's own kernels with nb = ns.
+// The vectors are FP32 device arrays, every norm is reduced in a fixed order to FP64 accuracy (runs of a thread's
+// elements in FP32 words that are no less exact, SumSq; then threads, blocks and one block over them in FP64), and
+// the scalar recurrence of the bidiagonalisation and of the plane rotations runs on the device (one thread), so an
+// iteration is a fixed sequence of launches with no host round trip.  The operator's forward and adjoint are the plan's own kernels with nb = ns.
 #include <cmath>
 #include <cstring>
 
